@@ -608,3 +608,57 @@ def test_gpu_quantizer_full_size_layer(stb):
     got, W, xn = _gpu_quantize(stb, torch, n, m, N, seed)
     torch.cuda.synchronize()
     _same_logical(got, wl.as_logical(wl.quantized_layer(n, m, N, seed)))
+
+
+def _shaped_weights(kind, n, m, seed):
+    """Weights on which the quantizer's decisions tie or its special cases arise."""
+    W = si.dense_weight(n, m, seed).astype(np.float32)
+    if kind == "levels":                    # few distinct values: many break-points with the same partition, equal errors
+        W = np.clip(np.round(W / 0.01), -8, 7) * 0.01
+    elif kind == "zero block":              # a block and some rows without a weight
+        W[:, :128] = 0.0
+        W[:3] = 0.0
+    elif kind == "duplicate columns":       # equal scores inside a group: ties go to the lower column
+        W[:, 1::2] = W[:, ::2]
+    elif kind == "tiny":                    # subnormal fp16 weights
+        W = W * 1e-5
+    return W.astype(np.float16)
+
+
+@pytest.mark.parametrize("kind", ["dense", "levels", "zero block", "duplicate columns", "tiny"])
+@pytest.mark.parametrize("n,m", [(1, 128), (33, 256), (129, 384), (65, 1280)])
+def test_gpu_quantizer_ties_edges_and_layouts(stb, kind, n, m):
+    """stb_quantize where its filters leave more than one candidate (ties), at the edges of its 32-, 64- and 128-row and
+    256-column pieces, and on rows that are not 16-byte aligned: every field equal to the oracle's."""
+    import torch
+    N, seed = 4 + (n + m // 128) % 3, 3100 + n
+    W, xn = _shaped_weights(kind, n, m, seed), si.calib_norms(m, seed)
+    if kind == "duplicate columns":
+        xn[1::2] = xn[::2]
+    L, _, _ = oracle.quantize(W.astype(np.float64), xn, N)
+    wide = torch.zeros(n, m + 3, dtype=torch.float16, device="cuda")
+    wide[:, 1:m + 1] = torch.from_numpy(W).cuda()
+    for Wd in (torch.from_numpy(W).cuda(), wide[:, 1:m + 1]):
+        got = stb.quantize(Wd, torch.from_numpy(xn).cuda(), N)
+        torch.cuda.synchronize()
+        _same_logical(got, L)
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6])
+def test_dequant_row_stride_and_base(stb, N):
+    """stb_dequant into a matrix whose rows or base address do not allow 16-byte stores, and into one that does."""
+    import torch
+    n, m = 37, 384
+    L = _quantized(n, m, N, 3200 + N)
+    What = oracle.decode(L)
+    layer = stb.pack_numpy(_fields(L))
+    for dt in (torch.float32, torch.float16):
+        want = torch.from_numpy(What).to(dt)
+        for ld, off in ((m, 0), (m + 8, 0), (m + 8, 8), (m + 3, 0), (m + 8, 1)):
+            out = torch.full((n, ld), 7.0, dtype=dt, device="cuda")
+            view = torch.as_strided(out, (n, m), (ld, 1), off)
+            if off + m > ld:
+                continue
+            stb.dequant(layer, dtype=dt, out=view)
+            assert torch.equal(view.cpu(), want)
+            assert bool((out[:, off + m:] == 7.0).all())

@@ -22,42 +22,47 @@ __global__ void header_kernel(int n, int m, int N, const uint64_t* __restrict__ 
   BlockInfo* bi = reinterpret_cast<BlockInfo*>(packed + sizeof(Header));
   ResidWord* rwt = reinterpret_cast<ResidWord*>(packed + rwtab_offset(nblk));
   __shared__ int bad;
-  __shared__ uint32_t total;
+  __shared__ uint32_t wsum[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-    uint64_t lo = salient[2 * b], hi = salient[2 * b + 1];
+  // one block per thread, 256 at a time: a scan over the CTA numbers the residual words, everything a block needs then
+  // leaves from registers (walking the blocks' words through global memory took 8 us at 32 blocks)
+  uint32_t total = 0;
+  for (int b0 = 0; b0 < nblk; b0 += 256) {
+    const int b = b0 + (int)threadIdx.x;
+    uint64_t lo = 0, hi = 0;
+    if (b < nblk) { lo = salient[2 * b]; hi = salient[2 * b + 1]; }
     int ns = __popcll(lo) + __popcll(hi);
     if (ns > kMaxSalient) { bad = 1; ns = kMaxSalient; }
-    bi[b].salient[0] = lo;
-    bi[b].salient[1] = hi;
-    bi[b].nsal = (uint32_t)ns;
-    bi[b].nrw = (uint32_t)resid_words_for(ns);
-    bi[b].pad = 0;
-    int q = 0;
-    for (int h = 0; h < 2; ++h) {
-      uint64_t mk = h ? hi : lo;
-      while (mk && q < kMaxSalient) {
-        bi[b].cols[q++] = (uint8_t)(__ffsll((long long)mk) - 1 + 64 * h);
-        mk &= mk - 1;
+    const uint32_t nrw = (uint32_t)resid_words_for(ns);
+    uint32_t incl = nrw;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d); if (lane >= d) incl += o; }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t off = total + incl - nrw;
+    for (int k = 0; k < 8; ++k) { if (k < warp) off += wsum[k]; total += wsum[k]; }
+    __syncthreads();
+    if (b >= nblk) continue;
+    uint4* d = reinterpret_cast<uint4*>(bi + b);
+    d[0] = make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+    d[1] = make_uint4((uint32_t)ns, off, nrw, 0u);
+    uint32_t cols[kMaxResidWords];
+#pragma unroll
+    for (int wq = 0; wq < kMaxResidWords; ++wq) {
+      cols[wq] = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (lo) { cols[wq] |= (uint32_t)(__ffsll((long long)lo) - 1) << (8 * k); lo &= lo - 1; }
+        else if (hi) { cols[wq] |= (uint32_t)(__ffsll((long long)hi) + 63) << (8 * k); hi &= hi - 1; }
       }
+      if ((uint32_t)wq < nrw) *reinterpret_cast<uint2*>(rwt + off + wq) = make_uint2(8u * (uint32_t)b + (uint32_t)wq, cols[wq]);
     }
-    for (; q < kMaxSalient; ++q) bi[b].cols[q] = 0;
+    d[2] = make_uint4(cols[0], cols[1], cols[2], cols[3]);
+    d[3] = make_uint4(cols[4], cols[5], cols[6], cols[7]);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t off = 0;
-    for (int b = 0; b < nblk; ++b) { bi[b].rw_off = off; off += bi[b].nrw; }
-    total = off;
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-    for (uint32_t wq = 0; wq < bi[b].nrw; ++wq) {
-      ResidWord e;
-      e.block_wq = 8u * (uint32_t)b + wq;
-      for (int k = 0; k < 4; ++k) e.cols[k] = bi[b].cols[4 * wq + k];
-      rwt[bi[b].rw_off + wq] = e;
-    }
   if (threadIdx.x == 0) {
     const int ntile = (n + kTileRows - 1) / kTileRows;
     const uint32_t tb = tile_bytes(N);

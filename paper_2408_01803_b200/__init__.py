@@ -1,6 +1,6 @@
 """Python binding of libstb.so: the N:M structured-binary linear layer on B200 (sm_100a).
 
-Argument marshalling only: every step of the path (pack, dequant, GEMV, GEMM, layer stack)
+Argument marshalling only (through ctypes, and natively for the calls of a decode or prefill loop): every step of the path (pack, dequant, GEMV, GEMM, layer stack)
 runs in the CUDA kernels behind the C ABI declared in include/stb.h.  torch is used for
 device memory and streams.  There is no CPU fallback: the shared library is loaded on the
 first call of any function here, and a missing library raises ImportError at that point
@@ -15,6 +15,7 @@ from dataclasses import dataclass
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libstb.so")
+BIND_PATH = os.path.join(_HERE, "_stb_bind.so")
 
 STB_OK, STB_ERR_ARG, STB_ERR_SHAPE, STB_ERR_NM, STB_ERR_SIZE = 0, 1, 2, 3, 4
 STB_ERR_UNSUPPORTED, STB_ERR_CORRUPT, STB_ERR_TIMEOUT, STB_ERR_CUDA = 5, 6, 7, 8
@@ -101,6 +102,28 @@ class _LazyLib:
 _lib = _LazyLib()
 
 
+_bind = None
+
+
+def _fast():
+    """The native host path of the calls that a decode or prefill loop makes (csrc/stb_bind.cpp).  It takes the plain cases
+    and hands everything else to the `_..._py` form of the call below."""
+    global _bind
+    if _bind is None:
+        import torch  # noqa: F401  (its libraries first)
+        from importlib.machinery import ExtensionFileLoader
+        from importlib.util import module_from_spec, spec_from_loader
+        if not os.path.exists(BIND_PATH):
+            raise ImportError("_stb_bind.so is not built (%s): run `python -m paper_2408_01803_b200.build`" % BIND_PATH)
+        mod = module_from_spec(spec_from_loader("_stb_bind", ExtensionFileLoader("_stb_bind", BIND_PATH)))
+        mod.__loader__.exec_module(mod)
+        names = ("stb_gemv", "stb_gemm_workspace", "stb_gemm", "stb_gemm_f16_workspace", "stb_gemm_f16", "stb_layer_stack", "stb_layer_stack_resident")
+        mod.start(*[C.cast(getattr(_lib, nm), C.c_void_p).value for nm in names], _check, _gemv_py, _gemm_py, _gemm_f16_py, _layer_stack_py,
+                  _layer_stack_resident_py)
+        _bind = mod
+    return _bind
+
+
 def status_str(status: int) -> str:
     return _lib.stb_status_str(int(status)).decode()
 
@@ -184,6 +207,10 @@ def dequant(layer: PackedLayer, dtype=None, out=None, stream=None):
 
 def gemv(layer: PackedLayer, x, out=None, out_dtype=None, stream=None):
     """stb_gemv: x fp16 [batch][m] (or [m]) -> y [batch][n] fp32 (or fp16)."""
+    return (_bind or _fast()).gemv(layer, x, out, out_dtype, stream)
+
+
+def _gemv_py(layer: PackedLayer, x, out=None, out_dtype=None, stream=None):
     import torch
     x2 = x if x.dim() == 2 else x.unsqueeze(0)
     assert x2.dtype == torch.float16 and x2.is_cuda and x2.stride(1) == 1
@@ -215,6 +242,10 @@ def gemm_workspace(n, m, N, T, minimum=False) -> int:
 
 def gemm(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, stream=None):
     """stb_gemm: X bf16 [T][m] -> Y [T][n] fp32 (or bf16)."""
+    return (_bind or _fast()).gemm(layer, X, out, out_dtype, ws, stream)
+
+
+def _gemm_py(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, stream=None):
     import torch
     assert X.dtype == torch.bfloat16 and X.is_cuda and X.dim() == 2 and X.stride(1) == 1
     T = X.shape[0]
@@ -238,6 +269,10 @@ def gemm_f16_workspace(n, m, N, T) -> int:
 
 def gemm_f16(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, stream=None):
     """stb_gemm_f16: X fp16 [T][m] -> Y [T][n] fp32 (or fp16); exact fp16 scales, the small token tile for T <= 64."""
+    return (_bind or _fast()).gemm_f16(layer, X, out, out_dtype, ws, stream)
+
+
+def _gemm_f16_py(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, stream=None):
     import torch
     assert X.dtype == torch.float16 and X.is_cuda and X.dim() == 2 and X.stride(1) == 1
     T = X.shape[0]
@@ -292,6 +327,10 @@ def make_steps(steps):
 
 def layer_stack(steps, dev_status=None, stream=None, marshalled=None):
     """stb_layer_stack over a list of (PackedLayer, x, out) triples (or a pre-marshalled array)."""
+    return (_bind or _fast()).layer_stack(steps, dev_status, stream, marshalled)
+
+
+def _layer_stack_py(steps, dev_status=None, stream=None, marshalled=None):
     arr = marshalled if marshalled is not None else make_steps(steps)
     _check(_lib.stb_layer_stack(arr, len(arr), _ptr(dev_status), _stream(stream)), "stb_layer_stack")
 
@@ -317,6 +356,10 @@ def resident_workspace(marshalled, device="cuda"):
 def layer_stack_resident(steps, ws, dev_status=None, stream=None, marshalled=None, selftest=False):
     """stb_layer_stack_resident over a list of (PackedLayer, x, out) triples (or a pre-marshalled array);
     ws from resident_workspace().  selftest=True runs the wait self-test instead."""
+    return (_bind or _fast()).layer_stack_resident(steps, ws, dev_status, stream, marshalled, selftest)
+
+
+def _layer_stack_resident_py(steps, ws, dev_status=None, stream=None, marshalled=None, selftest=False):
     arr = marshalled if marshalled is not None else make_steps(steps)
     fn = _lib.stb_layer_stack_resident_wait_selftest if selftest else _lib.stb_layer_stack_resident
     _check(fn(arr, len(arr), _ptr(ws), ws.numel(), _ptr(dev_status), _stream(stream)), "stb_layer_stack_resident")

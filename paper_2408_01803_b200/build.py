@@ -1,15 +1,18 @@
-"""Builds the CUDA library (libstb.so) for sm_100a with nvcc, in-tree."""
+"""Builds the CUDA library (libstb.so) for sm_100a with nvcc, and the native host path of its Python calls (_stb_bind.so)
+with g++ against the installed torch, in-tree."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstb.so")
+BIND = os.path.join(HERE, "_stb_bind.so")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
          "-Xcompiler", "-fPIC"]
 
@@ -31,8 +34,34 @@ def _headers_mtime() -> float:
     return max(os.path.getmtime(h) for h in hs)
 
 
+def _torch_dir() -> str:
+    """Where torch is installed (found without importing it)."""
+    from importlib.util import find_spec
+    return os.path.dirname(find_spec("torch").origin)
+
+
+def build_bind(force: bool = False) -> str:
+    """Compile csrc/stb_bind.cpp into _stb_bind.so."""
+    src = os.path.join(CSRC, "stb_bind.cpp")
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(HERE, "..", "include", "stb.h")))
+    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= newest:
+        return BIND
+    torch_dir = _torch_dir()
+    inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+    tmp = BIND + ".tmp%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", tmp, src, "-I" + sysconfig.get_paths()["include"], "-I" + inc,
+           "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), "-I" + cuda, "-D_GLIBCXX_USE_CXX11_ABI=1",
+           "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
+    os.replace(tmp, BIND)
+    return BIND
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every csrc/*.cu for sm_100a (one nvcc per file, in parallel) and link libstb.so."""
+    """Compile every csrc/*.cu for sm_100a (one nvcc per file, in parallel), link libstb.so, and build _stb_bind.so."""
     os.makedirs(OBJ, exist_ok=True)
     hm = _headers_mtime()
     todo, objs = [], []
@@ -50,6 +79,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
         return r.stderr
 
+    pool = ThreadPoolExecutor(max_workers=1)
+    bind = pool.submit(build_bind, force)
     if todo:
         with ThreadPoolExecutor(max_workers=min(8, len(todo))) as ex:
             for log in ex.map(compile_one, todo):
@@ -59,6 +90,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + ".tmp%d" % os.getpid()
         subprocess.check_call([nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs + ["-lcuda"])
         os.replace(tmp, LIB)
+    bind.result()
+    pool.shutdown()
     return LIB
 
 

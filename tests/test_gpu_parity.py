@@ -662,3 +662,34 @@ def test_dequant_row_stride_and_base(stb, N):
             stb.dequant(layer, dtype=dt, out=view)
             assert torch.equal(view.cpu(), want)
             assert bool((out[:, off + m:] == 7.0).all())
+
+
+@pytest.mark.parametrize("call,dtype,rows", [("gemv", "float16", 3), ("gemv", "float16", 1), ("gemm", "bfloat16", 70), ("gemm_f16", "float16", 20)])
+def test_native_host_path_equals_the_python_form(stb, call, dtype, rows):
+    """gemv / gemm / gemm_f16 through the native host path: the Python form's results for every way of giving the output, a
+    given stream, a vector, a strided input; and its errors."""
+    import torch
+    n, m, N = 100, 256, 5
+    layer = stb.pack_numpy(si.logical_layer(n, m, N, 3300))
+    t16 = getattr(torch, dtype)
+    wide = torch.from_numpy(si.activations(rows, m + 8, 3301).astype(np.float32)).to(t16).cuda()
+    fast, plain = getattr(stb, call), getattr(stb, "_%s_py" % call)
+    for x in (wide[:, :m].contiguous(), wide[:, :m]):
+        for kw in ({}, {"out_dtype": t16}, {"out": torch.zeros(rows, n, device="cuda")}, {"out": torch.zeros(rows, n + 4, dtype=t16, device="cuda")[:, :n]}):
+            want = plain(layer, x, **{k: v.clone() if k == "out" else v for k, v in kw.items()})
+            got = fast(layer, x, **kw)
+            assert got.dtype == want.dtype and torch.equal(got, want)
+            if "out" in kw:
+                assert got is kw["out"]
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    got = fast(layer, wide[:, :m], stream=s)
+    torch.cuda.synchronize()
+    assert torch.equal(got, plain(layer, wide[:, :m]))
+    if call == "gemv":
+        v = fast(layer, wide[0, :m])
+        assert v.shape == (n,) and torch.equal(v, plain(layer, wide[0, :m]))
+    with pytest.raises(AssertionError):
+        fast(layer, wide[:, :m].float())
+    with pytest.raises(stb.StbError):
+        fast(stb.PackedLayer(n, m, 9, layer.buf, layer.dev_status), wide[:, :m])

@@ -8,26 +8,35 @@
 //     warps as equal contiguous runs.  When whole row tiles can be dealt with little imbalance (at least 85 % of
 //     the SM time used) every CTA gets whole row tiles and no sum crosses CTAs; otherwise the ranges are equal
 //     in tiles and a row tile may straddle CTAs.
-//   * Each warp streams its tiles through a private ring in shared memory with 1-D bulk copies (mbarrier
-//     completion, bounded waits) and runs ahead into its range of the NEXT phase: packed weights never depend on
-//     activations, so the stream does not stop at a phase boundary.
-//   * Decode and multiply per tile are those of stb_gemv: 6:8 keeps the weights in rank order and lets
-//     mma.sp.m16n8k32 place them (activations from an image of x in operand order in shared memory, built once
-//     per phase and CTA); 4:8 and 5:8 (and 6:8 when the image does not fit or for more than two batch rows)
-//     decode to position order for mma.m16n8k16 with the activations read through L1.
+//   * Each warp's tiles stream through a private ring in shared memory (two slots of up to two tiles and their
+//     residual records, two 1-D bulk copies each, mbarrier completion, bounded waits).  A seventeenth warp issues the
+//     copies, one lane per ring, and runs ahead into the NEXT phases: packed weights never depend on activations, so the
+//     stream does not stop at a phase boundary.  It also works out where a chunk belongs (row tile, first block, residual
+//     words, end of a run) and leaves that beside the slot, so that the other warps only wait, decode and multiply.
+//   * Decode and multiply per tile: 6:8 keeps the weights in rank order and lets mma.sp.m16n8k32 place them
+//     (activations from an image of x in operand order in shared memory, built once per phase and CTA); 4:8 and 5:8
+//     (and 6:8 when the image does not fit) decode to position order for mma.m16n8k16 with the activations from a
+//     plain copy in shared memory, or through L1 when that does not fit either.
 //   * A step may take x = silu(in) * in2 (the gated activation between gate / up and down of an MLP): the CTA forms
-//     it while it stages the activations in shared memory, in operand order (6:8, up to two batch rows) or as a
-//     plain fp16 copy (everything else), and the tiles and the residual term read it from there.
-//   * The residual term of the salient columns (Eq. 4) is applied per span of up to five blocks from the span's
-//     records of the residual stream, brought into shared memory by one bulk copy while the span's tiles run.
+//     it while it stages the activations.
+//   * The residual term of the salient columns (Eq. 4): a block's record of the residual stream comes with its tile,
+//     four residual words (16 salient slots) of a chunk per tensor-core step; the activations behind every residual
+//     word of the phase are gathered into shared memory while x is staged.
 //   * Partial sums: a warp that covers a whole row tile writes y itself; the others leave their head / tail
-//     pieces in shared memory and the CTA adds them in tile order at the end of the phase; a row tile that
-//     straddles CTAs goes through partial tiles in the caller's workspace, summed in CTA order by whichever
-//     CTA arrives last (a counter per row tile).  Every sum has a fixed order: results are reproducible.
+//     pieces in shared memory and the CTA adds them in tile order at the end of the phase; of a row tile that
+//     straddles CTAs the later ones hand their sums to the first through the caller's workspace, every value beside a tag
+//     of the launch and phase (one 8-byte store, no fence, no counter), and the first adds them in CTA order.  Every
+//     sum has a fixed order: results are reproducible.
 //   * A phase may read what an earlier phase wrote: a CTA starts a phase's arithmetic only when the count of
 //     finished row tiles (one counter in the workspace, bumped once per CTA and phase) has reached the total
 //     of all earlier phases.  The poll is bounded; when it or an mbarrier wait runs out, an abort flag makes
 //     every CTA leave, STB_ERR_TIMEOUT is reported and the last CTA out restores the workspace to zero.
+//
+// What bounds it: in the tile loop instruction issue, the integer ALU first (2 warp-instructions per clock and SM; the decode
+// alone takes 126 / 145 / 118 clocks per tile and SM at N = 6 / 5 / 4, with the waits, residual words and copies 180 / 193 /
+// 170); between phases, latencies: the spread of the warps' ends, the sums, one trip through L2 for the count of finished row
+// tiles and one for the activations.  13B block at 5:8, batch 1: 106.4 -> 92.5 us, 7B MLP at 6:8: 44.5 -> 42.3 us, 32 7B
+// layers: 2040 -> 1905 us against one copy per five-block span issued by the decoding warps themselves.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -42,18 +51,22 @@ namespace stb {
 __device__ const Meta6Joint g_meta6_joint = make_meta6_joint();
 
 constexpr int kSWarps = 16;
-constexpr int kSThreads = kSWarps * 32;
+constexpr int kSThreads = kSWarps * 32;       // the decoding warps; the copies are issued by one warp of a fifth warpgroup,
+constexpr int kSAllThreads = kSThreads + 128; // which gives registers up to the other four: 640 x 96 at launch, then
+constexpr int kDecodeRegs = 104, kFeedRegs = 64;   // 512 x 104 + 128 x 64 of them
+static_assert(kSThreads * kDecodeRegs + 128 * kFeedRegs <= kSAllThreads * 96, "register split within the launch's total");
 constexpr int kMaxPhases = 64;                // per launch; longer lists run as several launches
 constexpr int kMaxFusedSteps = 4;
-constexpr int kSDepth = 2, kSChunk = 2;       // ring: slots per warp, tiles per bulk copy
-static_assert(kSDepth == 2, "the warp state keeps the two slots' chunk sizes in two registers");
-constexpr uint32_t kSlotBytes = 4096;         // two tiles of at most 1920 bytes
-constexpr int kSpan = 5;                      // blocks per residual span
-constexpr uint32_t kStageBytes = 2048;        // per warp: the span's residual records (<= 5 x 320) + its word table
-constexpr uint32_t kStageTab = 1664;
+constexpr int kSDepth = 2, kSChunk = 2;       // ring: slots per warp, tiles per slot
+constexpr uint32_t kSlotTiles = kSChunk * 1920;                    // tiles (at most 1920 bytes each) ...
+constexpr uint32_t kSlotBytes = kSlotTiles + kSChunk * (kResidA2Bytes + kMaxResidWords * kResidWordBytes);   // ... and records
+static_assert(kSlotBytes % 128 == 0, "slots stay 128-byte aligned");
 constexpr long long kSWaitLimit = 2000000000ll;        // about a second of SM clocks
 constexpr long long kSSelftestLimit = 100000ll;
 constexpr uint32_t kImgWordsPerBlock = 96;    // 6:8 operand-order image: words per block and batch row
+constexpr uint32_t kXPad = 64;                // bytes between the rows of the plain copy beyond 2 m: the eight lane groups' loads do not conflict
+constexpr uint32_t kPosCopies = 16;           // copies of a position table, lane-minor: the look-ups of 16 lanes never conflict
+constexpr uint32_t kPosBytes = kPosTableEntries * kPosCopies * 8;
 
 struct StackPhase {
   const uint8_t* packed[kMaxFusedSteps];
@@ -66,47 +79,59 @@ struct StackPhase {
   uint32_t ldx;
   int32_t m;
   uint8_t N, batch, count, f16_mask;          // f16_mask bit i: step i writes fp16
-  uint8_t use_image, aligned, pad[2];         // use_image: 0 activations from global memory, 1 operand-order image (6:8),
-                                              // 2 plain fp16 copy in shared memory; aligned: CTA ranges are whole row tiles
+  uint8_t use_image, aligned, gather, pad;    // use_image: 0 activations from global memory, 1 operand-order image (6:8),
+                                              // 2 plain fp16 copy in shared memory; aligned: CTA ranges are whole row tiles;
+                                              // gather: the residual words' activations fit shared memory
   uint32_t done_before;                       // row tiles finished by all earlier phases of this launch
 };
 
 struct StackParams {
   StackPhase ph[kMaxPhases];
   int32_t nphase;
-  uint32_t image_bytes;                       // shared memory set aside for the staged activations
+  // shared memory plan (byte offsets; see SSmem for what comes before)
+  uint32_t pos_off[3];                        // position tables of N = 4, 5, 6, 0 where no phase needs one
+  uint32_t use_meta6;
+  uint32_t ring_off, pdata_off, xs_off, cols_off, x_off, x_bytes;
+  uint32_t pos_row;                           // bytes from one entry of a position table to the next
   uint32_t part_floats;                       // floats per partial slot: 32 rows x largest batch
   uint32_t max_share;                         // most CTAs that share one row tile
-  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left, [4..] per row tile arrivals
-  float* gpart;                               // partial tiles of row tiles that straddle CTAs
+  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left, [4] launches so far
+  uint2* gpart;                               // sums handed on for row tiles that straddle CTAs: { value, tag }
   int* dev_status;
   long long wait_limit;
   int32_t copies_off;
 };
 
-// shared memory plan
+// shared memory: joint 6:8 metadata table first (784 x 16 B, at offset 0: a pair field of a tile is the shared-memory
+// address of its entry), when a phase needs it; then, from `base`:
 struct SSmem {
-  static constexpr uint32_t meta6 = 0;                               // joint 6:8 metadata table, 784 x 16 B, at offset 0: a pair
-                                                                     // field of a tile is the shared-memory address of its entry
-  static constexpr uint32_t pos = kMasks6 * kMasks6 * 16;            // 3 x 576 B position tables (N = 4, 5, 6)
-  static constexpr uint32_t bars = pos + 3 * 576;                    // ring barriers: 16 warps x 2 + 16 stage barriers
-  static constexpr uint32_t ctl = bars + 8 * (kSWarps * kSDepth + kSWarps);   // control words
-  static constexpr uint32_t slots = ctl + 64;                        // partial slot descriptors: 32 x 16 B
-  static constexpr uint32_t ring = 15360;
-  static constexpr uint32_t stage = ring + kSWarps * kSDepth * kSlotBytes;
-  static constexpr uint32_t pdata = stage + kSWarps * kStageBytes;
+  static constexpr uint32_t meta6_bytes = kMasks6 * kMasks6 * 16;
+  static constexpr uint32_t full = 0;                                          // ring barriers, 16 warps x 2: copies landed ...
+  static constexpr uint32_t empty = full + 8 * kSWarps * kSDepth;              // ... and slot read
+  static constexpr uint32_t ctl = empty + 8 * kSWarps * kSDepth;               // control words
+  static constexpr uint32_t slots = ctl + 64;                                  // row tiles of the partial slots: 32 x 4 B
+  static constexpr uint32_t chunks = slots + 2 * kSWarps * 4;                  // what each ring slot holds: 32 x 16 B
+  static constexpr uint32_t zero = chunks + kSWarps * kSDepth * 16;            // 384 bytes of zeros: the activations of lanes beyond the batch
+  static constexpr uint32_t range = zero + 384;                                // this CTA's tiles of every phase
+  static constexpr uint32_t nrw = range + 32 * kMaxPhases;                     // residual words per row tile of every step
+  static constexpr uint32_t bytes = nrw + 4 * kMaxPhases * kMaxFusedSteps;
 };
-static_assert(SSmem::slots + 32 * 16 <= SSmem::ring && SSmem::ring % 128 == 0, "control area overflows");
 
-struct PartSlot { int32_t R, lo, hi, pad; };   // row tile (phase-wide number) or -1, block range [lo, hi)
+// A CTA's share of a phase: tiles [lo, hi), the row tiles that lie inside it as a whole, and the row tile of its first tile.
+// Where the first or the last row tile straddles CTAs: the CTA where it begins, and how many share it.
+struct CtaRange { int32_t lo, hi, whole, first, head_cta, head_share, tail_cta, tail_share; };
 
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// a value and its tag in one 8-byte access: whoever sees the tag sees the value
+__device__ __forceinline__ void st_tagged(uint2* p, float v, uint32_t tag) {
+  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(__float_as_uint(v)), "r"(tag) : "memory");
+}
+__device__ __forceinline__ uint2 ld_tagged(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
 }
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const void* p) {
   unsigned long long v;
@@ -119,19 +144,8 @@ __device__ __forceinline__ uint32_t hmul2_bits(uint32_t a, uint32_t b) {
   asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
-// Coherent loads of activations (written by this kernel, so never through the read-only path); the address may be
-// global or shared memory.
-__device__ __forceinline__ uint4 ld_v4(const void* p) {
-  uint4 v;
-  asm volatile("ld.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t ld_u16(const void* p) {
-  unsigned short v;
-  asm volatile("ld.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint4 ldg_v4_coherent(const void* p) {      // the same from global memory
+// Coherent loads of activations (written by this kernel, so never through the read-only path)
+__device__ __forceinline__ uint4 ldg_v4_coherent(const void* p) {
   uint4 v;
   asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
@@ -141,27 +155,44 @@ __device__ __forceinline__ uint32_t ldg_u16_coherent(const void* p) {
   asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
   return v;
 }
+// silu(a) b = a b / (1 + exp(-a)) in fp32: one reciprocal and one correction of the quotient (Markstein's: the remainder
+// by a fused multiply-add), within an ulp of the divided form without its slow path.  exp is held below 2^116: there
+// the quotient is far below the smallest fp16 value anyway.
+__device__ __forceinline__ float silu_mul(float a, float b) {
+  const float d = 1.0f + __expf(fminf(-a, 80.0f));
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+  const float q = a * r;
+  return fmaf(fmaf(-d, q, a), r, q) * b;
+}
 // fp16 pair (bits) of silu(a) * b per half, in fp32, rounded to nearest even
 __device__ __forceinline__ uint32_t silu_mul_bits(uint32_t a, uint32_t b) {
   const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&a)), fb = __half22float2(*reinterpret_cast<const __half2*>(&b));
-  const __half2 r = __floats2half2_rn(fa.x / (1.0f + __expf(-fa.x)) * fb.x, fa.y / (1.0f + __expf(-fa.y)) * fb.y);
+  const __half2 r = __floats2half2_rn(silu_mul(fa.x, fb.x), silu_mul(fa.y, fb.y));
   return *reinterpret_cast<const uint32_t*>(&r);
 }
-// the staged form of eight activations: as they are, or silu(in) * in2
-__device__ __forceinline__ uint4 staged_x(const __half* x, const __half* x2, size_t off) {
-  uint4 v = ldg_v4_coherent(x + off);
-  if (x2) {
-    const uint4 w = ldg_v4_coherent(x2 + off);
-    v.x = silu_mul_bits(v.x, w.x); v.y = silu_mul_bits(v.y, w.y); v.z = silu_mul_bits(v.z, w.z); v.w = silu_mul_bits(v.w, w.w);
-  }
-  return v;
+// where column c of block b stands in the staged activations of a batch row, in halves: in operand order (6:8), word
+// ((t 2 + sl) 3 + i) 4 + u of a block = operand register u of chunk i of step sl of lane t, or plainly
+__device__ __forceinline__ uint32_t image_word(uint32_t b, uint32_t group) {
+  return b * kImgWordsPerBlock + (4u * (group & 1u) + ((group >> 2) & 1u)) * 12u + 2u * (group >> 3) + ((group >> 1) & 1u);
 }
-// Activation of column c (0..127) of block blk from the operand-order image of one batch row (see the image build).
-__device__ __forceinline__ uint32_t image_x(const uint32_t* img_row, uint32_t blk, uint32_t c) {
-  const uint32_t Gp = c >> 3, pr = (c >> 1) & 3u;
-  const uint32_t* d = img_row + blk * kImgWordsPerBlock + (4u * (Gp & 1u) + ((Gp >> 2) & 1u)) * 12u + 2u * (Gp >> 3) + ((Gp >> 1) & 1u);
-  const uint32_t w = d[pr < 3u ? 4u * pr : 32u];
-  return (c & 1u) ? (w >> 16) : (w & 0xFFFFu);
+__device__ __forceinline__ uint32_t staged_index(bool image, uint32_t b, uint32_t c) {
+  const uint32_t pr = (c >> 1) & 3u;
+  return image ? 2u * (image_word(b, c >> 3) + (pr < 3u ? 4u * pr : 32u)) + (c & 1u) : b * (uint32_t)kBlock + c;
+}
+// the activations of a residual word's four columns (the bytes of `cols`), as two fp16 pairs
+__device__ __forceinline__ uint2 word_x(const __half* x, const __half* x2, uint32_t cols) {
+  uint32_t v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = ldg_u16_coherent(x + ((cols >> (8 * k)) & 0xFFu));
+  uint2 r = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+  if (x2) {
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = ldg_u16_coherent(x2 + ((cols >> (8 * k)) & 0xFFu));
+    r.x = silu_mul_bits(r.x, w[0] | (w[1] << 16)); r.y = silu_mul_bits(r.y, w[2] | (w[3] << 16));
+  }
+  return r;
 }
 
 // Dealing the T = R nb tiles of a phase (R row tiles of nb blocks) to G CTAs.
@@ -184,16 +215,11 @@ __host__ __device__ __forceinline__ void cta_range(int R, int nb, bool aligned, 
 }
 // the CTA that owns tile L (not aligned)
 __host__ __device__ __forceinline__ int owner_of(long long L, long long T, int Ge) { return (int)(((L + 1) * Ge - 1) / T); }
-
-__device__ __forceinline__ void warp_range(const StackPhase& q, int nb, int cta, int G, int warp, int& lo, int& hi) {
-  const int R = q.tile_start[q.count];
-  const int Ge = dealt_ctas(R, nb, q.aligned != 0, G);
-  lo = hi = 0;
-  if (cta >= Ge) return;
-  int cl, ch;
-  cta_range(R, nb, q.aligned != 0, Ge, cta, cl, ch);
-  lo = cl + (int)(((long long)(ch - cl) * warp) >> 4);
-  hi = cl + (int)(((long long)(ch - cl) * (warp + 1)) >> 4);
+// a warp's run of its CTA's range
+__device__ __forceinline__ void warp_range(const CtaRange& r, int warp, int& lo, int& hi) {
+  const int len = r.hi - r.lo;
+  lo = r.lo + (int)(((long long)len * warp) >> 4);
+  hi = r.lo + (int)(((long long)len * (warp + 1)) >> 4);
 }
 static_assert(kSWarps == 16, "warp_range divides by 16 with a shift");
 
@@ -205,60 +231,146 @@ __device__ __forceinline__ int step_of(const StackPhase& q, int R) {
   return i;
 }
 
-// The producer side of a warp's ring: a walk through the warp's tiles of all phases in chunks of up to kSChunk
-// tiles that never cross a packed buffer.  Between chunks it only bumps a pointer and two counters.
+// What is in a ring slot: x = tiles (bits 0..1), residual words of the first block (from bit 8) and of all (from bit 16), flags;
+// y = first block; z = number of the first residual word (counted through the phase where its activations are gathered);
+// w = row tile (numbered through the phase).
+constexpr uint32_t kSegEnd = 1u << 24;        // the warp's tiles of this row tile end with the chunk ...
+constexpr uint32_t kSegWhole = 1u << 25;      // ... and were all of it
+constexpr uint32_t kSegLeads = 1u << 26;      // ... or began with its first block
+constexpr uint32_t kRunEnd = 1u << 27;        // the warp's run of the phase ends with the chunk
+
+// The copies of one ring: a walk through the warp's tiles of all phases in chunks of up to kSChunk tiles that never cross a
+// row tile.  Between chunks it only bumps pointers; the word counts of the next chunk's blocks (which give the size of
+// their residual records) are loaded when the previous chunk is issued.
 struct TileWalk {
   int phase;              // current phase (== nphase: finished)
-  const uint8_t* src;     // next tile
-  int left_range;         // tiles left in the warp's range of this phase
-  int left_step;          // tiles left in the packed buffer `src` points into
-  int step;
+  int left;               // tiles left in the warp's run of this phase
+  int step, R;            // step, and row tile (numbered through the phase)
+  int blk, first;         // next block of the row tile, and the run's first block of it
   uint32_t tb;            // tile bytes of this phase
-  __device__ void enter(const StackParams& P, int ph, int cta, int G, int warp) {
-    phase = ph;
-    while (phase < P.nphase) {
-      const StackPhase& q = P.ph[phase];
-      const int nb = q.m / kBlock;
-      int lo, hi;
-      warp_range(q, nb, cta, G, warp, lo, hi);
-      if (lo < hi) {
-        tb = tile_bytes(q.N);
-        left_range = hi - lo;
-        step = step_of(q, lo / nb);
-        left_step = q.tile_start[step + 1] * nb - lo;
-        src = q.packed[step] + tiles_offset(nb) + (size_t)(lo - q.tile_start[step] * nb) * tb;
-        return;
-      }
-      ++phase;
-    }
+  uint32_t words;         // residual words of the phase's earlier steps (0 without gathering)
+  const uint8_t* src;     // next tile
+  const uint8_t* rec;     // next residual record
+  uint4 ba, bb;           // second 16 bytes of the BlockInfo of blocks blk, blk + 1: { nsal, rw_off, nrw, - }
+
+  __device__ __forceinline__ int count(int nb) const { return min(min(kSChunk, left), nb - blk); }
+  __device__ __forceinline__ void load_info(const StackPhase& q) {
+    const uint4* bi = reinterpret_cast<const uint4*>(q.packed[step] + sizeof(Header)) + 4 * blk + 1;
+    ba = __ldg(bi);
+    bb = make_uint4(0, 0, 0, 0);
+    if (count(q.m / kBlock) > 1) bb = __ldg(bi + 4);
   }
-  // next chunk: source address, bytes per tile and number of tiles (0 when the walk is over)
-  __device__ int next(const StackParams& P, int cta, int G, int warp, const uint8_t*& chunk_src, uint32_t& chunk_tb) {
-    if (phase >= P.nphase) return 0;
-    int cnt = kSChunk;
-    if (cnt > left_range) cnt = left_range;
-    if (cnt > left_step) cnt = left_step;
-    chunk_src = src; chunk_tb = tb;
-    src += (size_t)cnt * tb;
-    left_range -= cnt; left_step -= cnt;
-    if (left_range == 0) enter(P, phase + 1, cta, G, warp);
-    else if (left_step == 0) {
+  // row tile R, block blk of step `step`; the residual record's place needs the block's first word number
+  __device__ __forceinline__ void locate(const StackPhase& q, const uint32_t* nrw) {
+    const int nb = q.m / kBlock, rt = R - q.tile_start[step], ntile = q.tile_start[step + 1] - q.tile_start[step];
+    const uint8_t* tiles = q.packed[step] + tiles_offset(nb);
+    load_info(q);
+    src = tiles + ((size_t)rt * nb + blk) * tb;
+    rec = tiles + (size_t)tb * nb * ntile + (size_t)rt * resid_rt_bytes(nb, nrw[step]) + kResidA2Bytes * (uint32_t)blk;
+    words = 0;
+    if (q.gather)
+      for (int k = 0; k < step; ++k) words += nrw[k];
+    rec += (size_t)kResidWordBytes * ba.y;
+  }
+  __device__ __forceinline__ void enter(const StackParams& P, const CtaRange* range, const uint32_t* nrw, int ph, int warp) {
+    for (phase = ph; phase < P.nphase; ++phase) {
       const StackPhase& q = P.ph[phase];
+      const CtaRange r = range[phase];
+      int lo, hi;
+      warp_range(r, warp, lo, hi);
+      if (lo >= hi) continue;
       const int nb = q.m / kBlock;
-      ++step;
-      src = q.packed[step] + tiles_offset(nb);
-      left_step = (q.tile_start[step + 1] - q.tile_start[step]) * nb;
+      tb = tile_bytes(q.N);
+      left = hi - lo;
+      R = r.first + (int)((uint32_t)(lo - r.first * nb) / (uint32_t)nb);
+      blk = first = lo - R * nb;
+      step = step_of(q, R);
+      locate(q, nrw + phase * kMaxFusedSteps);
+      return;
     }
-    return cnt;
   }
 };
 
+// The copying warp: lane w feeds the ring of warp w.  A slot is refilled when its reader has arrived on its empty barrier;
+// the wait has no limit of its own (a reader may be waiting for other CTAs) but ends with the CTA's failed flag.
+__device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, uint8_t* base, volatile int* ctl) {
+  const int w = threadIdx.x & 31;
+  const CtaRange* range = reinterpret_cast<const CtaRange*>(base + SSmem::range);
+  const uint32_t* nrw = reinterpret_cast<const uint32_t*>(base + SSmem::nrw);
+  if (w >= kSWarps) return;
+  TileWalk t;
+  t.enter(P, range, nrw, 0, w);
+  const uint32_t full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)w, empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)w;
+  const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)w * kSDepth * kSlotBytes;
+  uint4* chunk = reinterpret_cast<uint4*>(base + SSmem::chunks) + kSDepth * w;
+  uint32_t k = 0;                                     // chunks issued
+  while (t.phase < P.nphase) {
+    const uint32_t slot = k % kSDepth;
+    if (k >= kSDepth && !mbar_try_wait(empty + 8u * slot, (k / kSDepth - 1u) & 1u)) {
+      if (ctl[0]) return;
+      __nanosleep(20);
+      continue;
+    }
+    const StackPhase& q = P.ph[t.phase];
+    const int nb = q.m / kBlock, cnt = t.count(nb);
+    const uint32_t na = t.ba.z, nw = na + t.bb.z;
+    const bool seg_end = t.blk + cnt == nb || t.left == cnt;
+    uint4 c;
+    c.x = (uint32_t)cnt | (na << 8) | (nw << 16);
+    if (seg_end) c.x |= kSegEnd | (t.first == 0 ? (t.blk + cnt == nb ? kSegWhole : kSegLeads) : 0u);
+    if (t.left == cnt) c.x |= kRunEnd;
+    c.y = (uint32_t)t.blk; c.z = t.words + t.ba.y; c.w = (uint32_t)t.R;
+    chunk[slot] = c;                                  // (seen by the reader through the full barrier)
+    const uint32_t tile_b = (uint32_t)cnt * t.tb, rec_b = (uint32_t)cnt * kResidA2Bytes + nw * kResidWordBytes;
+    const uint32_t bar = full + 8u * slot, dst = ring + slot * kSlotBytes;
+    mbar_expect_tx(bar, tile_b + rec_b);
+    // copies off (the wait self-test): the barrier is armed but nothing will ever complete it
+    if (!P.copies_off) {
+      bulk_g2s(dst, t.src, tile_b, bar);
+      bulk_g2s(dst + kSlotTiles, t.rec, rec_b, bar);
+    }
+    ++k;
+    t.left -= cnt; t.blk += cnt;
+    if (t.left == 0) t.enter(P, range, nrw, t.phase + 1, w);
+    else {
+      t.src += tile_b; t.rec += rec_b;
+      if (t.blk == nb) {
+        t.blk = t.first = 0; ++t.R;
+        if (t.R == q.tile_start[t.step + 1]) { ++t.step; t.locate(q, nrw + t.phase * kMaxFusedSteps); }
+        else t.load_info(q);
+      } else t.load_info(q);
+    }
+  }
+}
+
+// What a decoding warp carries through the whole kernel: the slot it reads next and the phase parity of its barrier.
+struct WarpState {
+  uint32_t slot, parity;
+  bool failed;                        // a wait ran out, or the CTA was told to stop
+};
+struct WarpEnv {
+  const StackParams* P;
+  uint8_t* smem;
+  uint8_t* base;
+  uint8_t* ring;                      // of this warp
+  const uint4* chunk;
+  uint32_t full, empty;
+  int warp, lane, g, t;
+};
+__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSThreads) : "memory"); }
+
 // ------------------------------------------------------------------------------------------
-// One 32 x 128 tile at 6:8 through the sparse instruction, activations from the image (see stb_gemv.cu).
-__device__ __forceinline__ void tile_sp6(const LaneTile<6>& lt, const uint32_t (&fld)[8], const uint8_t* smem, const uint32_t* xi0,
-                                         bool xlive, float (&acc)[2][4]) {
+// One 32 x 128 tile at 6:8 through the sparse instruction: the weights stay in rank order and the instruction places
+// them (stb_decode.cuh, meta6_nibble).  x: the lane's place in the operand-order image.
+struct Tile6 { LaneTile<6> lt; uint32_t fld[8]; };
+__device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, Tile6& d) {
+  load_lane_tile<6>(tile, lane, d.lt, true);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) d.fld[k] = *reinterpret_cast<const uint16_t*>(tile + lane * 16 + 2 * k);
+}
+__device__ __forceinline__ void tile_mul(const Tile6& d, const uint8_t* smem, const uint8_t* x, float (&acc)[2][4]) {
   FastRows<6> fr;
-  fr.init(lt, lt.A, lt.B);
+  fr.init(d.lt, d.lt.A, d.lt.B);
   // Metadata: fld[4 bb + tq] is the pair field (= the address of the joint-table entry) of slot 2 h + bb of lane tq of
   // the quad, for the two rows whose metadata this lane supplies; word i of the entries, shifted to the lane's
   // nibble and added (multiply-adds: the integer pipe is the busy one), is the metadata of chunk i.
@@ -267,7 +379,7 @@ __device__ __forceinline__ void tile_sp6(const LaneTile<6>& lt, const uint32_t (
   for (int bb = 0; bb < 2; ++bb) {
     uint4 en[4];
 #pragma unroll
-    for (int tq = 0; tq < 4; ++tq) en[tq] = *reinterpret_cast<const uint4*>(smem + SSmem::meta6 + fld[4 * bb + tq]);
+    for (int tq = 0; tq < 4; ++tq) en[tq] = *reinterpret_cast<const uint4*>(smem + d.fld[4 * bb + tq]);
     E[bb][0] = ((en[3].x * 16u + en[2].x) * 16u + en[1].x) * 16u + en[0].x;
     E[bb][1] = ((en[3].y * 16u + en[2].y) * 16u + en[1].y) * 16u + en[0].y;
     E[bb][2] = ((en[3].z * 16u + en[2].z) * 16u + en[1].z) * 16u + en[0].z;
@@ -277,10 +389,7 @@ __device__ __forceinline__ void tile_sp6(const LaneTile<6>& lt, const uint32_t (
 #pragma unroll
   for (int sl = 0; sl < 2; ++sl)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      bxs[sl][i] = make_uint4(0, 0, 0, 0);
-      if (xlive) bxs[sl][i] = *reinterpret_cast<const uint4*>(xi0 + sl * 12 + 4 * i);
-    }
+    for (int i = 0; i < 3; ++i) bxs[sl][i] = *reinterpret_cast<const uint4*>(x + sl * 48 + 16 * i);
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt) {
     uint32_t XLh[2][2], XHh[2][2];
@@ -305,25 +414,38 @@ __device__ __forceinline__ void tile_sp6(const LaneTile<6>& lt, const uint32_t (
   }
 }
 
-// One tile in position order (N = 4, 5, 6): byte-permute decode into m16n8k16 operands; activations of batch row g
-// through L1 (xrow = x + g ldx + 8 t + 128 b, or null for lanes beyond the batch).
+// One tile in position order (N = 4, 5, 6): byte-permute decode into m16n8k16 operands.  The position selectors are looked
+// up by keep-mask index: where a lane's mask bytes are its slots' indices they are loaded one by one (the load pipe has
+// room, the integer pipe has not), and each of 16 lanes has a copy of the table in its own pair of banks.
+template <int N>
+struct TileD { LaneTile<N> lt; uint2 P[16]; };
+template <int N>
+__device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, const uint8_t* ptab, uint32_t prow, TileD<N>& d) {
+  load_lane_tile<N>(tile, lane, d.lt);
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const uint32_t idx = mask_pairs(N) ? keep_index_of(d.lt.mask, u >> 2, u & 3) : (uint32_t)tile[lane * 16 + u];
+    d.P[u] = *reinterpret_cast<const uint2*>(ptab + idx * prow);
+  }
+}
+// x: the lane's activations of the block, in shared memory (kStaged) or global
 template <int N, bool kStaged>
-__device__ __forceinline__ void tile_dense(const LaneTile<N>& lt, const uint2* ptab, const __half* xrow, float (&acc)[2][4]) {
+__device__ __forceinline__ void tile_mul(const TileD<N>& d, const uint8_t* x, float (&acc)[2][4]) {
   FastRows<N> fr;
-  fr.init(lt, lt.A, lt.B);
+  fr.init(d.lt, d.lt.A, d.lt.B);
   uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
   if (N == 5) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) fr.high(j, 0, XL[j], XH[j]);
   }
-  uint2 P[16];
-#pragma unroll
-  for (int u = 0; u < 16; ++u) P[u] = ptab[keep_index_of(lt.mask, u >> 2, u & 3)];
   uint4 xf[4];
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
-    xf[s] = make_uint4(0, 0, 0, 0);
-    if (xrow) xf[s] = kStaged ? ld_v4(xrow + s * 32) : ldg_v4_coherent(xrow + s * 32);
+    if (kStaged) xf[s] = *reinterpret_cast<const uint4*>(x + s * 64);
+    else {
+      xf[s] = make_uint4(0, 0, 0, 0);
+      if (x) xf[s] = ldg_v4_coherent(x + s * 64);
+    }
   }
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
@@ -331,7 +453,7 @@ __device__ __forceinline__ void tile_dense(const LaneTile<N>& lt, const uint2* p
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (N == 6 && (s & 1) == 0) fr.high(j, s >> 1, XL[j], XH[j]);
-      fr.slot2(j, s, P[4 * j + s].x, P[4 * j + s].y, XL[j], XH[j], f[j]);
+      fr.slot2(j, s, d.P[4 * j + s].x, d.P[4 * j + s].y, XL[j], XH[j], f[j]);
     }
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
@@ -341,321 +463,331 @@ __device__ __forceinline__ void tile_dense(const LaneTile<N>& lt, const uint2* p
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// What a warp carries through the whole kernel.
-struct WarpState {
-  TileWalk prod;                      // producer side of the ring
-  int chunk_cnt0, chunk_cnt1;         // tiles of the chunk in ring slot 0 / 1
-  uint32_t consumed;                  // chunks consumed (slot = consumed % kSDepth, barrier parity = consumed / kSDepth)
-  int cur_in;                         // tile inside the current chunk
-  uint32_t stage_use;                 // residual stage copies issued (barrier parity)
-  bool failed;                        // a wait ran out, or the CTA was told to stop
-};
-
-struct WarpEnv {
-  const StackParams* P;
-  uint8_t* smem;
-  uint8_t* ring;
-  uint8_t* stage;
-  uint32_t bar0, bar_stage;
-  int cta, G, warp, lane, g, t;
-};
-
-__device__ __forceinline__ void ring_issue(const WarpEnv& E, WarpState& W, int slot) {
-  const uint8_t* src = nullptr;
-  uint32_t tb = 0;
-  const int cnt = W.prod.next(*E.P, E.cta, E.G, E.warp, src, tb);
-  if (slot == 0) W.chunk_cnt0 = cnt; else W.chunk_cnt1 = cnt;
-  if (cnt > 0 && E.lane == 0) {
-    const uint32_t bytes = (uint32_t)cnt * tb;
-    fence_async_smem();
-    mbar_expect_tx(E.bar0 + 8u * slot, bytes);
-    if (!E.P->copies_off) bulk_g2s(smem_u32(E.ring + (size_t)slot * kSlotBytes), src, bytes, E.bar0 + 8u * slot);
+// Residual term of a chunk: its residual words, four (16 salient slots) per tensor-core step, lane t the t-th.  rec: the
+// chunk's records; na / nw: words of its first block / of all; xw: activations of the chunk's first word for the lane's
+// batch row, xw_step bytes per word.  kGather false: they are fetched one by one (word table entry, then x).
+template <bool kGather>
+__device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint32_t nw, int g, int t, const uint8_t* xw, uint32_t xw_step,
+                                          const ResidWord* rwt, const __half* xg, const __half* xg2, float (&acc)[2][4]) {
+#pragma unroll 1
+  for (uint32_t k0 = 0; k0 < nw; k0 += 4u) {
+    const uint32_t kk = k0 + (uint32_t)t, k = min(kk, nw - 1u);
+    const bool second = k >= na;
+    // records: a_sal2 of the 32 rows, then the block's words
+    const uint8_t* r = rec + k * kResidWordBytes + (second ? 2u * kResidA2Bytes : kResidA2Bytes);
+    uint32_t rw = *reinterpret_cast<const uint32_t*>(r + 4 * g);
+    const uint2 a2 = *reinterpret_cast<const uint2*>(rec + (second ? kResidA2Bytes + na * kResidWordBytes : 0u) + 8 * g);
+    if (kk >= nw) rw = 0x55555555u;
+    // operand registers of the lane's four rows: the two-bit codes pick the high byte of +1, 0 or -1 (one byte
+    // permute per row), two more spread them to fp16 pairs, and one fp16 multiply per register (not on the
+    // busy integer pipe) scales them by the row's a_sal2: exact, the factors are +-1 and 0
+    uint32_t fa[4][2];
+    const uint32_t code_lo = rw & 0x33333333u, code_hi = (rw >> 2) & 0x33333333u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t codes = (j & 2) ? code_hi : code_lo;
+      const uint32_t unit = prmt(0x00BC003Cu, 0u, (j & 1) ? (codes >> 16) : codes);          // high bytes of +1, 0, -1, 0 by code
+      const uint32_t s2 = prmt((j & 2) ? a2.y : a2.x, 0u, (j & 1) ? 0x3232u : 0x1010u);     // (a_sal2, a_sal2) of row j
+      fa[j][0] = hmul2_bits(prmt(unit, 0u, 0x1404u), s2);
+      fa[j][1] = hmul2_bits(prmt(unit, 0u, 0x3424u), s2);
+    }
+    uint2 xr = make_uint2(0, 0);
+    if (kGather) xr = *reinterpret_cast<const uint2*>(xw + k * xw_step);
+    else if (xg) {
+      const uint2 e = __ldg(reinterpret_cast<const uint2*>(rwt + k));
+      const size_t o = (size_t)(e.x >> 3) * kBlock;
+      xr = word_x(xg + o, xg2 ? xg2 + o : nullptr, e.y);
+    }
+    mma16816(acc[0], fa[0][0], fa[1][0], fa[0][1], fa[1][1], xr.x, xr.y);
+    mma16816(acc[1], fa[2][0], fa[3][0], fa[2][1], fa[3][1], xr.x, xr.y);
   }
 }
 
-// The warp's tiles [lo, hi) of phase q: main stream, residual term per span, partial sums out.
+// The warp's run of phase q: chunks of residual words and tiles, partial sums out.
 // kImage: 6:8 from the operand-order image; kStaged: position order with the activations in a plain copy in shared memory
 template <int N, bool kImage, bool kStaged>
-__device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const StackPhase& q, int lo, int hi,
-                                          const uint32_t* ximg, PartSlot* pslot, float* pdata, volatile int* ctl) {
+__device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const StackPhase& q, int* pslot, float* pdata) {
   const StackParams& P = *E.P;
-  const int lane = E.lane, g = E.g, t = E.t, warp = E.warp;
-  const int nb = q.m / kBlock, batch = q.batch;
+  const int lane = E.lane, g = E.g, t = E.t, warp = E.warp, batch = q.batch;
   constexpr uint32_t tb = tile_bytes(N);
-  const uint2* ptab = reinterpret_cast<const uint2*>(E.smem + SSmem::pos) + (N - 4) * kPosTableEntries;
-  // activations of batch row g (this lane group's): in global memory, or staged in shared memory as a plain copy
-  const __half* xg = nullptr;
-  if (g < batch) xg = q.use_image == 2 ? reinterpret_cast<const __half*>(ximg) + (size_t)g * q.m : q.x + (size_t)g * q.ldx;
-  // (with the operand-order image the tiles read the image; the residual term takes its few activations from global
-  // memory unless the input is a formed one)
-  const uint32_t img_row_words = (uint32_t)nb * kImgWordsPerBlock;
-  int R = lo / nb, b_first = lo - R * nb, left = hi - lo, nslot_used = 0;
-  while (left > 0 && !W.failed) {
-    const int seg = left < nb - b_first ? left : nb - b_first, b_end = b_first + seg;
-    const int si = step_of(q, R);
-    const int rt = R - q.tile_start[si];
-    const uint8_t* packed = q.packed[si];
-    const BlockInfo* binfo = reinterpret_cast<const BlockInfo*>(packed + sizeof(Header));
-    const ResidWord* rwt = reinterpret_cast<const ResidWord*>(packed + rwtab_offset(nb));
-    const int ntile = (q.n[si] + kTileRows - 1) / kTileRows;
-    const uint32_t nrw_all = __ldg(&reinterpret_cast<const Header*>(packed)->nrw);
-    const uint8_t* resid_rt = packed + tiles_offset(nb) + (size_t)tb * nb * ntile + (size_t)rt * resid_rt_bytes(nb, nrw_all);
-    float acc[2][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc[a][d] = 0.0f;
-
-    for (int bs = b_first; bs < b_end && !W.failed; bs += kSpan) {
-      const int be = bs + kSpan < b_end ? bs + kSpan : b_end;
-      // the span's records of the residual stream and its piece of the residual word table: one bulk copy each
-      const uint32_t rw0 = __ldg(&binfo[bs].rw_off), rw1 = __ldg(&binfo[be - 1].rw_off) + __ldg(&binfo[be - 1].nrw);
-      const uint32_t rec_bytes = (uint32_t)(be - bs) * kResidA2Bytes + (rw1 - rw0) * kResidWordBytes;
-      const uint32_t tab0 = rw0 & ~1u, tab_bytes = ((rw1 - tab0) * 8u + 15u) & ~15u;       // 16-byte aligned piece of the table
-      __syncwarp();
-      if (lane == 0) {
-        fence_async_smem();
-        mbar_expect_tx(E.bar_stage, rec_bytes + (rw1 > rw0 ? tab_bytes : 0u));
-        if (!P.copies_off) {
-          bulk_g2s(smem_u32(E.stage), resid_rt + resid_block_off(bs, rw0), rec_bytes, E.bar_stage);
-          if (rw1 > rw0) bulk_g2s(smem_u32(E.stage + kStageTab), rwt + tab0, tab_bytes, E.bar_stage);
-        }
-      }
-      const uint32_t stage_parity = W.stage_use & 1u;
-      ++W.stage_use;
-
-      for (int b = bs; b < be; ++b) {
-        const int slot = (int)(W.consumed % kSDepth);
-        if (W.cur_in == 0 && !__all_sync(0xFFFFFFFFu, mbar_wait(E.bar0 + 8u * slot, (W.consumed / kSDepth) & 1u, P.wait_limit))) { W.failed = true; break; }
-        const uint8_t* tile = E.ring + (size_t)slot * kSlotBytes + (size_t)W.cur_in * tb;
-        const bool last_of_chunk = W.cur_in + 1 == (slot == 0 ? W.chunk_cnt0 : W.chunk_cnt1);
-        LaneTile<N> lt;
-        load_lane_tile<N>(tile, lane, lt, kImage);
-        uint32_t fld[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if constexpr (kImage) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) fld[k] = *reinterpret_cast<const uint16_t*>(tile + lane * 16 + 2 * k);
-        }
-        if (last_of_chunk) { __syncwarp(); ring_issue(E, W, slot); W.cur_in = 0; ++W.consumed; }
-        else ++W.cur_in;
-        if constexpr (kImage) tile_sp6(lt, fld, E.smem, ximg + (uint32_t)g * img_row_words + (uint32_t)b * kImgWordsPerBlock + (uint32_t)(t * 24), g < batch, acc);
-        else tile_dense<N, kStaged>(lt, ptab, xg ? xg + (size_t)b * kBlock + t * 8 : nullptr, acc);
-      }
-      if (W.failed) break;
-
-      // residual term of the span's salient columns: four residual words (16 salient slots) per tensor-core step
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(E.bar_stage, stage_parity, P.wait_limit))) { W.failed = true; break; }
-      if (rw1 > rw0) {
-        const uint32_t nstep = (rw1 - rw0 + 3u) >> 2;
-#pragma unroll 1
-        for (uint32_t i = 0; i < nstep; ++i) {
-          const uint32_t wi = rw0 + 4u * i + (uint32_t)t;
-          uint32_t rw = 0x55555555u, cols = 0u, block = (uint32_t)bs;
-          uint2 a2 = make_uint2(0u, 0u);
-          if (wi < rw1) {
-            const uint2 e = *reinterpret_cast<const uint2*>(E.stage + kStageTab + (wi - tab0) * 8u);
-            block = e.x >> 3; cols = e.y;
-            const uint8_t* rec = E.stage + kResidA2Bytes * (block - (uint32_t)bs) + kResidWordBytes * (wi - (e.x & 7u) - rw0);
-            a2 = *reinterpret_cast<const uint2*>(rec + resid_a2_off(g, 0));
-            rw = *reinterpret_cast<const uint32_t*>(rec + resid_code_off(e.x & 7u, g));
-          }
-          // operand registers of the lane's four rows: the two-bit codes pick the high byte of +1, 0 or -1 (one byte
-          // permute per row), two more spread them to fp16 pairs, and one fp16 multiply per register (not on the
-          // busy integer pipe) scales them by the row's a_sal2: exact, the factors are +-1 and 0
-          uint32_t fa[4][2];
-          const uint32_t code_lo = rw & 0x33333333u, code_hi = (rw >> 2) & 0x33333333u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t codes = (j & 2) ? code_hi : code_lo;
-            const uint32_t unit = prmt(0x00BC003Cu, 0u, (j & 1) ? (codes >> 16) : codes);          // high bytes of +1, 0, -1, 0 by code
-            const uint32_t s2 = prmt((j & 2) ? a2.y : a2.x, 0u, (j & 1) ? 0x3232u : 0x1010u);     // (a_sal2, a_sal2) of row j
-            fa[j][0] = hmul2_bits(prmt(unit, 0u, 0x1404u), s2);
-            fa[j][1] = hmul2_bits(prmt(unit, 0u, 0x3424u), s2);
-          }
-          uint2 xr = make_uint2(0, 0);
-          if (kImage && q.x2 != nullptr) {
-            // a formed input exists only in the image: pick the four values out of its operand order
-            if (g < batch) {
-              const uint32_t* ir = ximg + (uint32_t)g * img_row_words;
-              xr.x = image_x(ir, block, cols & 0xFFu) | (image_x(ir, block, (cols >> 8) & 0xFFu) << 16);
-              xr.y = image_x(ir, block, (cols >> 16) & 0xFFu) | (image_x(ir, block, cols >> 24) << 16);
-            }
-          } else if (xg) {
-            const __half* xq = xg + (size_t)block * kBlock;
-            if constexpr (!kStaged) {      // global memory for sure
-              xr.x = ldg_u16_coherent(xq + (cols & 0xFFu)) | (ldg_u16_coherent(xq + ((cols >> 8) & 0xFFu)) << 16);
-              xr.y = ldg_u16_coherent(xq + ((cols >> 16) & 0xFFu)) | (ldg_u16_coherent(xq + (cols >> 24)) << 16);
-            } else {                       // global memory or the plain copy in shared memory
-              xr.x = ld_u16(xq + (cols & 0xFFu)) | (ld_u16(xq + ((cols >> 8) & 0xFFu)) << 16);
-              xr.y = ld_u16(xq + ((cols >> 16) & 0xFFu)) | (ld_u16(xq + (cols >> 24)) << 16);
-            }
-          }
-          mma16816(acc[0], fa[0][0], fa[1][0], fa[0][1], fa[1][1], xr.x, xr.y);
-          mma16816(acc[1], fa[2][0], fa[3][0], fa[2][1], fa[3][1], xr.x, xr.y);
-        }
-      }
-    }
-    if (W.failed) break;
-
-    // ---- the segment [b_first, b_end) of row tile R is summed: a whole row tile goes to y, a piece to shared memory ----
-    if (b_first == 0 && b_end == nb) {
-      const bool f16 = (q.f16_mask >> si) & 1;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-          const int row = rt * kTileRows + g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
-          if (row < q.n[si] && bc < batch) {
-            if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(acc[mt][d]);
-            else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = acc[mt][d];
-          }
-        }
-      if (lane == 0) atomicAdd(const_cast<int*>(&ctl[1]), 1);
-    } else {
-      const int slot = 2 * warp + nslot_used;
-      ++nslot_used;
-      float* pd = pdata + (size_t)slot * P.part_floats;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-          const int r = g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
-          if (bc < batch) pd[r * batch + bc] = acc[mt][d];
-        }
-      if (lane == 0) { pslot[slot].R = R; pslot[slot].lo = b_first; pslot[slot].hi = b_end; }
-    }
-    left -= seg; ++R; b_first = 0;
+  const bool xlive = g < batch;
+  const uint8_t* zero = E.base + SSmem::zero;
+  // The lane's activations: base and bytes per block.  Lanes beyond the batch read zeros.
+  const uint8_t* xbase;
+  uint32_t xstep;
+  if (kImage) {
+    xbase = xlive ? E.smem + P.x_off + (uint32_t)g * ((uint32_t)(q.m / kBlock) * kImgWordsPerBlock * 4u) + (uint32_t)t * 96u : zero;
+    xstep = xlive ? kImgWordsPerBlock * 4u : 0u;
+  } else if (kStaged) {
+    xbase = xlive ? E.smem + P.x_off + (uint32_t)g * (2u * (uint32_t)q.m + kXPad) + (uint32_t)t * 16u : zero;
+    xstep = xlive ? 2u * kBlock : 0u;
+  } else {
+    xbase = xlive ? reinterpret_cast<const uint8_t*>(q.x + (size_t)g * q.ldx + 8 * t) : nullptr;
+    xstep = xlive ? 2u * kBlock : 0u;
   }
+  const uint32_t xw_step = xlive ? 8u * (uint32_t)batch : 0u;
+  const uint8_t* xs = xlive ? E.smem + P.xs_off + (uint32_t)g * 8u : zero;
+  const uint8_t* ptab = kImage ? nullptr : E.smem + P.pos_off[N - 4] + (uint32_t)(lane & (kPosCopies - 1)) * 8u;
+  const uint32_t prow = P.pos_row;
+  float acc[2][4];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int d = 0; d < 4; ++d) acc[a][d] = 0.0f;
+  uint4 c;
+  do {
+    const uint32_t slot = W.slot, bar = E.full + 8u * slot;
+    // all lanes poll; the verdict is made warp-uniform
+    if (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, W.parity)) && !__all_sync(0xFFFFFFFFu, mbar_wait(bar, W.parity, P.wait_limit))) { W.failed = true; return; }
+    c = E.chunk[slot];
+    const uint8_t* tile = E.ring + slot * kSlotBytes;
+    const uint32_t na = (c.x >> 8) & 0xFFu, nw = (c.x >> 16) & 0xFFu;
+    if (nw) {
+      if (q.gather) resid_mul<true>(tile + kSlotTiles, na, nw, g, t, xs + c.z * xw_step, xw_step, nullptr, nullptr, nullptr, acc);
+      else {
+        const ResidWord* rwt = reinterpret_cast<const ResidWord*>(q.packed[step_of(q, (int)c.w)] + rwtab_offset(q.m / kBlock));
+        resid_mul<false>(tile + kSlotTiles, na, nw, g, t, nullptr, 0, rwt + c.z, xlive ? q.x + (size_t)g * q.ldx : nullptr,
+                         q.x2 ? q.x2 + (size_t)g * q.ldx : nullptr, acc);
+      }
+    }
+    const uint8_t* xb = xbase + (size_t)c.y * xstep;
+    const int cnt = (int)(c.x & 3u);
+#pragma unroll 1
+    for (int k = 0; k < cnt; ++k) {
+      // once the slot's last tile is in registers the slot is handed back
+      if constexpr (kImage) {
+        Tile6 d;
+        load_tile(tile, lane, d);
+        if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        tile_mul(d, E.smem, xb, acc);
+      } else {
+        TileD<N> d;
+        load_tile<N>(tile, lane, ptab, prow, d);
+        if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        tile_mul<N, kStaged>(d, xb, acc);
+      }
+      tile += tb;
+      xb += xstep;
+    }
+    W.slot ^= 1u;
+    W.parity ^= slot;
+    if (c.x & kSegEnd) {
+      // the warp's tiles of the row tile are summed: a whole row tile goes to y, a piece to shared memory
+      if (c.x & kSegWhole) {
+        const int si = step_of(q, (int)c.w), rt = (int)c.w - q.tile_start[si];
+        const bool f16 = (q.f16_mask >> si) & 1;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+          for (int d = 0; d < 4; ++d) {
+            const int row = rt * kTileRows + g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
+            if (row < q.n[si] && bc < batch) {
+              if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(acc[mt][d]);
+              else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = acc[mt][d];
+            }
+          }
+      } else {
+        // slot 2 w: the row tile began with another warp (or CTA); slot 2 w + 1: it begins here
+        const int ps = 2 * warp + (c.x & kSegLeads ? 1 : 0);
+        float* pd = pdata + (size_t)ps * P.part_floats;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+          for (int d = 0; d < 4; ++d) {
+            const int r = g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
+            if (bc < batch) pd[r * batch + bc] = acc[mt][d];
+          }
+        if (lane == 0) pslot[ps] = (int)c.w;
+      }
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int d = 0; d < 4; ++d) acc[a][d] = 0.0f;
+    }
+  } while (!(c.x & kRunEnd));
 }
 
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSThreads, 1)
-stack_kernel(const __grid_constant__ StackParams P) {
-  extern __shared__ __align__(128) uint8_t smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cta = (int)blockIdx.x, G = (int)gridDim.x;
-  volatile int* ctl = reinterpret_cast<volatile int*>(smem + SSmem::ctl);      // [0] failed, [1] row tiles finished by this CTA, [2] last CTA out, [3] a packed header does not match
-  PartSlot* pslot = reinterpret_cast<PartSlot*>(smem + SSmem::slots);
-  float* pdata = reinterpret_cast<float*>(smem + SSmem::pdata);
-  uint32_t* ximg = reinterpret_cast<uint32_t*>(smem + SSmem::pdata + 32u * P.part_floats * 4u);
-
-  // Packed headers must match the steps; every CTA reads the same headers and takes the same way out, before it
-  // has touched the workspace.
-  {
-    if (threadIdx.x == 0) ctl[3] = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < P.nphase * kMaxFusedSteps; i += blockDim.x) {
-      const StackPhase& q = P.ph[i / kMaxFusedSteps];
-      const int k = i % kMaxFusedSteps;
-      if (k < q.count && !header_matches(reinterpret_cast<const Header*>(q.packed[k]), q.n[k], q.m, q.N)) ctl[3] = 1;
-    }
-    __syncthreads();
-    if (ctl[3]) {
-      if (threadIdx.x == 0 && cta == 0 && P.dev_status) *P.dev_status = STB_ERR_CORRUPT;
-      return;
-    }
-  }
-
-  // tables, barriers, control words
-  for (int i = threadIdx.x; i < (int)(kMasks6 * kMasks6); i += blockDim.x)
-    reinterpret_cast<uint4*>(smem + SSmem::meta6)[i] = *reinterpret_cast<const uint4*>(g_meta6_joint.v[i]);
-  for (int i = threadIdx.x; i < 3 * kPosTableEntries; i += blockDim.x)
-    reinterpret_cast<uint2*>(smem + SSmem::pos)[i] = g_pos_table.v[4 + i / kPosTableEntries][i % kPosTableEntries];
-  WarpEnv E;
-  E.P = &P; E.smem = smem; E.cta = cta; E.G = G; E.warp = warp; E.lane = lane; E.g = lane >> 2; E.t = lane & 3;
-  E.bar0 = smem_u32(smem + SSmem::bars) + (uint32_t)warp * kSDepth * 8u;
-  E.bar_stage = smem_u32(smem + SSmem::bars) + (uint32_t)(kSWarps * kSDepth + warp) * 8u;
-  E.ring = smem + SSmem::ring + (size_t)warp * kSDepth * kSlotBytes;
-  E.stage = smem + SSmem::stage + (size_t)warp * kStageBytes;
-  if (lane == 0) {
-    for (int i = 0; i < kSDepth; ++i) mbar_init(E.bar0 + 8u * i, 1);
-    mbar_init(E.bar_stage, 1);
+// Checks the packed headers of all steps (every CTA reads the same headers and takes the same way out), notes their
+// residual word counts, and works out this CTA's tile range of every phase.
+__device__ __forceinline__ bool stack_setup(const StackParams& P, uint8_t* base, volatile int* ctl) {
+  if (threadIdx.x == 0) ctl[3] = 0;
+  if (threadIdx.x < kSWarps * kSDepth) {
+    mbar_init(smem_u32(base + SSmem::full) + 8u * threadIdx.x, 1);
+    mbar_init(smem_u32(base + SSmem::empty) + 8u * threadIdx.x, 1);
     fence_async_smem();
   }
-  if (threadIdx.x == 0) { ctl[0] = 0; ctl[1] = 0; ctl[2] = 0; }
-  __syncwarp();
-
-  // ring: the producer walk runs kSDepth chunks ahead of the tiles the warp consumes
-  WarpState W;
-  W.prod.enter(P, 0, cta, G, warp);
-  W.consumed = 0; W.cur_in = 0; W.stage_use = 0; W.failed = false;
-#pragma unroll
-  for (int i = 0; i < kSDepth; ++i) ring_issue(E, W, i);
   __syncthreads();
+  for (int i = threadIdx.x; i < P.nphase * kMaxFusedSteps; i += kSAllThreads) {
+    const StackPhase& q = P.ph[i / kMaxFusedSteps];
+    const int k = i % kMaxFusedSteps;
+    uint32_t nrw = 0;
+    if (k < q.count) {
+      const Header* h = reinterpret_cast<const Header*>(q.packed[k]);
+      nrw = h->nrw;
+      if (!header_matches(h, q.n[k], q.m, q.N)) ctl[3] = 1;
+    }
+    reinterpret_cast<uint32_t*>(base + SSmem::nrw)[i] = nrw;
+  }
+  // from the last thread down: the first ones load headers
+  for (int i = kSAllThreads - 1 - (int)threadIdx.x; i < P.nphase; i += kSAllThreads) {
+    const StackPhase& q = P.ph[i];
+    const int nb = q.m / kBlock, R = q.tile_start[q.count], cta = (int)blockIdx.x, G = (int)gridDim.x;
+    const int Ge = dealt_ctas(R, nb, q.aligned != 0, G);
+    CtaRange r = {0, 0, 0, 0, 0, 1, 0, 1};
+    if (cta < Ge) {
+      cta_range(R, nb, q.aligned != 0, Ge, cta, r.lo, r.hi);
+      r.first = (int)((uint32_t)r.lo / (uint32_t)nb);
+      const int up = (int)(((uint32_t)r.lo + (uint32_t)nb - 1u) / (uint32_t)nb), down = (int)((uint32_t)r.hi / (uint32_t)nb);
+      r.whole = down > up ? down - up : 0;
+      if (!q.aligned) {
+        const long long T = (long long)R * nb;
+        const int last = (int)((uint32_t)(r.hi - 1) / (uint32_t)nb);
+        r.head_cta = owner_of((long long)r.first * nb, T, Ge);
+        r.head_share = owner_of((long long)(r.first + 1) * nb - 1, T, Ge) - r.head_cta + 1;
+        r.tail_cta = owner_of((long long)last * nb, T, Ge);
+        r.tail_share = owner_of((long long)(last + 1) * nb - 1, T, Ge) - r.tail_cta + 1;
+      }
+    }
+    reinterpret_cast<CtaRange*>(base + SSmem::range)[i] = r;
+  }
+  __syncthreads();
+  return ctl[3] == 0;
+}
+
+// The decoding warps: all phases in order.
+__device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* smem, uint8_t* base, volatile int* ctl, int* pslot, float* pdata, int cta) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t* ximg = reinterpret_cast<uint32_t*>(smem + P.x_off);
+  WarpEnv E;
+  E.P = &P; E.smem = smem; E.base = base; E.warp = warp; E.lane = lane; E.g = lane >> 2; E.t = lane & 3;
+  E.ring = smem + P.ring_off + (size_t)warp * kSDepth * kSlotBytes;
+  E.chunk = reinterpret_cast<const uint4*>(base + SSmem::chunks) + kSDepth * warp;
+  E.full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)warp;
+  E.empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)warp;
+  WarpState W;
+  W.slot = 0; W.parity = 0; W.failed = false;
+  const uint32_t epoch = __ldcg(P.sync + 4);          // changed only by the last CTA out
+  // tables, while the first copies are under way
+  if (P.use_meta6)
+    for (int i = threadIdx.x; i < (int)(kMasks6 * kMasks6); i += kSThreads)
+      reinterpret_cast<uint4*>(smem)[i] = *reinterpret_cast<const uint4*>(g_meta6_joint.v[i]);
+#pragma unroll
+  for (int N = 4; N <= 6; ++N)
+    if (P.pos_off[N - 4])
+      for (int i = threadIdx.x; i < kPosTableEntries * (int)kPosCopies; i += kSThreads)
+        reinterpret_cast<uint2*>(smem + P.pos_off[N - 4])[i] = g_pos_table.v[N][i / (int)kPosCopies];
+  if (threadIdx.x < 384 / 4) reinterpret_cast<uint32_t*>(base + SSmem::zero)[threadIdx.x] = 0u;
 
   for (int ph = 0; ph < P.nphase; ++ph) {
     const StackPhase& q = P.ph[ph];
     const int nb = q.m / kBlock, batch = q.batch;
+    const uint32_t* nrw = reinterpret_cast<const uint32_t*>(base + SSmem::nrw) + ph * kMaxFusedSteps;
+    const CtaRange range = reinterpret_cast<const CtaRange*>(base + SSmem::range)[ph];
     int wl, wh;
-    warp_range(q, nb, cta, G, warp, wl, wh);
+    warp_range(range, warp, wl, wh);
 
-    // ---- wait until every earlier phase has finished, then (6:8) lay the activations out in operand order ----
-    if (threadIdx.x == 0 && !ctl[0] && q.done_before > 0) {
-      const long long t0 = clock64();
-      for (;;) {
-        // one load brings the count of finished row tiles (low word) and the abort flag (high word)
-        const unsigned long long v = ld_acquire_u64(P.sync);
-        if ((uint32_t)v >= q.done_before) break;
-        if ((uint32_t)(v >> 32) != 0u) { ctl[0] = 1; break; }
-        if (clock64() - t0 > P.wait_limit) {
-          ctl[0] = 1;
-          atomicExch(P.sync + 1, 1u);
-          if (P.dev_status) *P.dev_status = STB_ERR_TIMEOUT;
-          break;
+    // where the activation of every residual slot will stand in the staged x (in halves, batch row 0): known before the wait
+    uint16_t* cols = reinterpret_cast<uint16_t*>(smem + P.cols_off);
+    uint32_t slots = 0;
+    if (q.gather) {
+#pragma unroll 1
+      for (int k = 0; k < q.count; ++k) {
+        const uint2* rwt = reinterpret_cast<const uint2*>(q.packed[k] + rwtab_offset(nb));
+        const uint32_t cnt = 4u * nrw[k];
+#pragma unroll 1
+        for (uint32_t i = threadIdx.x; i < cnt; i += kSThreads) {
+          const uint2 e = __ldg(rwt + (i >> 2));
+          cols[slots + i] = (uint16_t)staged_index(q.use_image == 1, e.x >> 3, (e.y >> (8u * (i & 3u))) & 0xFFu);
         }
+        slots += cnt;
       }
     }
-    __syncthreads();
-    if (ctl[0]) W.failed = true;
-    if (q.use_image == 1 && !ctl[0]) {
-      // one item = the 8 activations of one group of one batch row: a 16-byte load, six 4-byte stores (see stb_gemv.cu)
-      const uint32_t img_row_words = (uint32_t)nb * kImgWordsPerBlock;
-      const int per_row = nb * 16, items = batch * per_row;
-      for (int base = 0; base < items; base += 4 * kSThreads) {
-        uint4 v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int it = base + k * kSThreads + (int)threadIdx.x;
-          v[k] = make_uint4(0, 0, 0, 0);
-          if (it < items) {
-            const int r = it >= per_row ? 1 : 0, qq = it - r * per_row;       // the image serves one or two batch rows
-            v[k] = staged_x(q.x, q.x2, (size_t)r * q.ldx + (size_t)qq * 8);
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int it = base + k * kSThreads + (int)threadIdx.x;
-          if (it < items) {
-            const int r = it >= per_row ? 1 : 0, qq = it - r * per_row, blk = qq >> 4, Gp = qq & 15;
-            uint32_t* d = ximg + (uint32_t)r * img_row_words + (uint32_t)blk * kImgWordsPerBlock +
-                          (uint32_t)((4 * (Gp & 1) + ((Gp >> 2) & 1)) * 12 + 2 * (Gp >> 3) + ((Gp >> 1) & 1));
-            d[0] = v[k].x; d[4] = v[k].y; d[8] = v[k].z;
-            d[24] = v[k].y; d[28] = v[k].z; d[32] = v[k].w;
+    if (lane < 2) pslot[2 * warp + lane] = -1;
+
+    // ---- wait until every earlier phase has finished, then stage the activations ----
+    if (q.done_before > 0) {
+      if (threadIdx.x == 0 && !ctl[0]) {
+        const long long t0 = clock64();
+        for (;;) {
+          // one load brings the count of finished row tiles (low word) and the abort flag (high word)
+          const unsigned long long v = ld_acquire_u64(P.sync);
+          if ((uint32_t)v >= q.done_before) break;
+          if ((uint32_t)(v >> 32) != 0u) { ctl[0] = 1; break; }
+          if (clock64() - t0 > P.wait_limit) {
+            ctl[0] = 1;
+            atomicExch(P.sync + 1, 1u);
+            if (P.dev_status) *P.dev_status = STB_ERR_TIMEOUT;
+            break;
           }
         }
       }
-    } else if (q.use_image == 2 && !ctl[0]) {
-      // plain fp16 copy [batch][m] of the (formed) activations
+      consumers_sync();
+    }
+    const bool stop = ctl[0] != 0;
+    if (stop) W.failed = true;
+    // The code between two phases runs once per phase, much of it out of a cold instruction cache: it is kept short rather
+    // than unrolled.  An item = eight activations of a batch row; the next item is on its way while one is stored.
+    if (q.use_image && !stop) {
       const int per_row = q.m / 8, items = batch * per_row;
-      for (int it = threadIdx.x; it < items; it += kSThreads) {
-        const int r = it / per_row, qq = it - r * per_row;
-        reinterpret_cast<uint4*>(ximg)[it] = staged_x(q.x, q.x2, (size_t)r * q.ldx + (size_t)qq * 8);
+      uint4 v = make_uint4(0, 0, 0, 0), v2 = v;
+      auto fetch = [&](int it) {
+        const int r = batch == 1 ? 0 : it / per_row;
+        const size_t o = (size_t)r * q.ldx + (size_t)(it - r * per_row) * 8;
+        if (it < items) {
+          v = ldg_v4_coherent(q.x + o);
+          if (q.x2) v2 = ldg_v4_coherent(q.x2 + o);
+        }
+      };
+      int it = threadIdx.x;
+      fetch(it);
+#pragma unroll 1
+      while (it < items) {
+        uint32_t a[4] = {v.x, v.y, v.z, v.w};
+        const uint32_t b[4] = {v2.x, v2.y, v2.z, v2.w};
+        const int cur = it;
+        it += kSThreads;
+        fetch(it);
+        if (q.x2) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) a[k] = silu_mul_bits(a[k], b[k]);
+        }
+        const int r = batch == 1 ? 0 : cur / per_row, qq = cur - r * per_row;
+        if (q.use_image == 1) {
+          // operand order: lanes t = 2 (G & 1) + p read word i + p of group G as chunk i: words 0..2 for p = 0, 1..3 for p = 1
+          uint32_t* d = ximg + (uint32_t)r * ((uint32_t)nb * kImgWordsPerBlock) + image_word((uint32_t)qq >> 4, (uint32_t)qq & 15u);
+          d[0] = a[0]; d[4] = a[1]; d[8] = a[2];
+          d[24] = a[1]; d[28] = a[2]; d[32] = a[3];
+        } else {
+          *reinterpret_cast<uint4*>(smem + P.x_off + (uint32_t)r * (2u * (uint32_t)q.m + kXPad) + (uint32_t)qq * 16u) = make_uint4(a[0], a[1], a[2], a[3]);
+        }
       }
     }
-    if (lane == 0) { pslot[2 * warp].R = -1; pslot[2 * warp + 1].R = -1; }
-    __syncthreads();
+    consumers_sync();
+    if (q.gather && !stop) {
+      // activations of the residual slots: [word of all steps][batch row], four fp16 each
+      uint16_t* xs = reinterpret_cast<uint16_t*>(smem + P.xs_off);
+      const uint32_t pitch = q.use_image == 1 ? (uint32_t)nb * kImgWordsPerBlock * 2u : (uint32_t)q.m + kXPad / 2u;
+#pragma unroll 1
+      for (uint32_t i = threadIdx.x; i < slots; i += kSThreads) {
+        const uint16_t* src = reinterpret_cast<const uint16_t*>(smem + P.x_off) + cols[i];
+        uint16_t* d = xs + (size_t)(i >> 2) * 4u * (uint32_t)batch + (i & 3u);
+#pragma unroll 1
+        for (int r = 0; r < batch; ++r) d[4 * r] = src[r * pitch];
+      }
+      consumers_sync();
+    }
 
     // ---- this warp's tiles ----
     if (!W.failed && wl < wh) {
-      if (q.N == 6 && q.use_image == 1) run_tiles<6, true, false>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
+      if (q.use_image == 1) run_tiles<6, true, false>(E, W, q, pslot, pdata);
       else if (q.use_image == 2) {
-        if (q.N == 6) run_tiles<6, false, true>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
-        else if (q.N == 5) run_tiles<5, false, true>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
-        else run_tiles<4, false, true>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
-      } else if (q.N == 6) run_tiles<6, false, false>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
-      else if (q.N == 5) run_tiles<5, false, false>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
-      else run_tiles<4, false, false>(E, W, q, wl, wh, ximg, pslot, pdata, ctl);
+        if (q.N == 6) run_tiles<6, false, true>(E, W, q, pslot, pdata);
+        else if (q.N == 5) run_tiles<5, false, true>(E, W, q, pslot, pdata);
+        else run_tiles<4, false, true>(E, W, q, pslot, pdata);
+      } else if (q.N == 6) run_tiles<6, false, false>(E, W, q, pslot, pdata);
+      else if (q.N == 5) run_tiles<5, false, false>(E, W, q, pslot, pdata);
+      else run_tiles<4, false, false>(E, W, q, pslot, pdata);
     }
     if (W.failed && lane == 0 && !ctl[0]) {
       // this warp's own wait ran out: tell the CTA and the grid
@@ -663,87 +795,108 @@ stack_kernel(const __grid_constant__ StackParams P) {
       atomicExch(P.sync + 1, 1u);
       if (P.dev_status) *P.dev_status = STB_ERR_TIMEOUT;
     }
-    __syncthreads();
+    consumers_sync();
 
-    // ---- pieces of row tiles, added in tile order.  Slot 2 w (head piece of warp w), 2 w + 1 (tail piece) are in tile
-    // order; a run of slots with the same row tile is one group, handled by the warp that owns its first slot. ----
+    // ---- pieces of row tiles, added in tile order by the warp where the row tile begins (in this CTA) ----
     if (!ctl[0]) {
-      const int Rall = q.tile_start[q.count];
-      // every warp looks at all 32 slot descriptors at once, one per lane
-      const PartSlot mine = pslot[lane];
-      const uint32_t used = __ballot_sync(0xFFFFFFFFu, mine.R >= 0);
+      const int cont = lane < kSWarps ? pslot[2 * lane] : -1;           // the row tile each warp continues
+      const int nval = 32 * batch;                                      // values of a row tile: [row][batch column]
+#pragma unroll 1
       for (int s0 = 2 * warp; s0 < 2 * warp + 2; ++s0) {
-        if (!((used >> s0) & 1u)) continue;
-        const int R = __shfl_sync(0xFFFFFFFFu, mine.R, s0);
-        // the nearest used slot before s0 decides whether s0 starts a group
-        const uint32_t below = used & ((1u << s0) - 1u);
-        if (below != 0u && __shfl_sync(0xFFFFFFFFu, mine.R, 31 - __clz(below)) == R) continue;
-        const uint32_t members = __ballot_sync(0xFFFFFFFFu, mine.R == R);
-        const int lo_b = __shfl_sync(0xFFFFFFFFu, mine.lo, s0), hi_b = __shfl_sync(0xFFFFFFFFu, mine.hi, 31 - __clz(members));
+        const int R = pslot[s0];
+        // slot 2 w leads only where the CTA's range begins inside a row tile and no earlier warp has a piece of it
+        const uint32_t others = __ballot_sync(0xFFFFFFFFu, cont == R);
+        if (R < 0 || (!(s0 & 1) && ((others & ((1u << warp) - 1u)) != 0u || R != range.first || range.lo == R * nb))) continue;
+        const uint32_t members = others & ~((2u << warp) - 1u);        // later warps' pieces, in order
         const int si = step_of(q, R);
         const int rt = R - q.tile_start[si];
         const bool f16 = (q.f16_mask >> si) & 1;
-        const int nval = 32 * batch;                 // values of the row tile: [row][batch column]
-        const bool whole = lo_b == 0 && hi_b == nb;
-        float* gp = nullptr;
-        int share = 1;
-        if (!whole) {
-          const long long T = (long long)Rall * nb;
-          const int Ge = dealt_ctas(Rall, nb, false, G);
-          const int c_first = owner_of((long long)R * nb, T, Ge), c_last = owner_of((long long)(R + 1) * nb - 1, T, Ge);
-          share = c_last - c_first + 1;
-          gp = P.gpart + ((size_t)R * P.max_share + (size_t)(cta - c_first)) * P.part_floats;
-        }
+        const bool whole = range.lo <= R * nb && range.hi >= (R + 1) * nb;
+        // a straddling row tile: the CTA where it begins gathers the others' sums, in CTA order
+        const int c_first = R == range.first ? range.head_cta : range.tail_cta, share = R == range.first ? range.head_share : range.tail_share;
+        uint2* gp = P.gpart + (size_t)R * P.max_share * P.part_floats;
+        const uint32_t tag = ((epoch + 1u) << 6) | (uint32_t)ph;
+        bool lost = false;
         for (int v = lane; v < nval; v += 32) {
-          float sum = 0.0f;
-          for (uint32_t mm = members; mm != 0u; mm &= mm - 1u) sum += pdata[(size_t)(__ffs(mm) - 1) * P.part_floats + v];
-          if (whole) {
-            const int row = rt * kTileRows + v / batch, bc = v % batch;
-            if (row < q.n[si]) {
-              if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(sum);
-              else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = sum;
+          const float* pv = pdata + v;
+          float sum = pv[(size_t)s0 * P.part_floats];
+          for (uint32_t mm = members; mm != 0u;) {
+            // four loads at a time, added in order
+            float x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              x[k] = mm ? pv[(size_t)(2 * (__ffs(mm) - 1)) * P.part_floats] : 0.0f;
+              mm &= mm - 1u;
             }
-          } else {
-            gp[v] = sum;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sum += x[k];
+          }
+          if (!whole && cta != c_first) {
+            st_tagged(gp + (size_t)(cta - c_first) * P.part_floats + v, sum, tag);
+            continue;
+          }
+          if (!whole) {
+            const long long t0 = clock64();
+            for (int k = 1; k < share && !lost; ++k) {
+              uint2 x = ld_tagged(gp + (size_t)k * P.part_floats + v);
+              while (x.y != tag && !lost) {
+                lost = clock64() - t0 > P.wait_limit || *reinterpret_cast<volatile uint32_t*>(P.sync + 1) != 0u;
+                x = ld_tagged(gp + (size_t)k * P.part_floats + v);
+              }
+              sum += __uint_as_float(x.x);
+            }
+          }
+          const int row = rt * kTileRows + (batch == 1 ? v : v / batch), bc = batch == 1 ? 0 : v % batch;
+          if (row < q.n[si]) {
+            if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(sum);
+            else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = sum;
           }
         }
-        if (whole) {
-          if (lane == 0) atomicAdd(const_cast<int*>(&ctl[1]), 1);
-        } else {
-          // the row tile straddles CTAs: whoever arrives last adds the partial tiles in CTA order
-          __syncwarp();
-          uint32_t old = 0;
-          if (lane == 0) { __threadfence(); old = atomicAdd(P.sync + 4 + R, 1u); }
-          old = __shfl_sync(0xFFFFFFFFu, old, 0);
-          if ((int)old == share - 1) {
-            __threadfence();
-            const float* g0 = P.gpart + (size_t)R * P.max_share * P.part_floats;
-            for (int v = lane; v < nval; v += 32) {
-              float sum = 0.0f;
-              for (int k = 0; k < share; ++k) sum += __ldcg(g0 + (size_t)k * P.part_floats + v);
-              const int row = rt * kTileRows + v / batch, bc = v % batch;
-              if (row < q.n[si]) {
-                if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(sum);
-                else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = sum;
-              }
-            }
-            if (lane == 0) { P.sync[4 + R] = 0u; atomicAdd(const_cast<int*>(&ctl[1]), 1); }
-          }
+        if (!whole && cta == c_first && lane == 0) atomicAdd(const_cast<int*>(&ctl[1]), 1);
+        if (__any_sync(0xFFFFFFFFu, lost) && lane == 0) {
+          ctl[0] = 1;
+          atomicExch(P.sync + 1, 1u);
+          if (P.dev_status) *P.dev_status = STB_ERR_TIMEOUT;
         }
       }
     }
-    __syncthreads();
+    consumers_sync();
     if (threadIdx.x == 0) {
-      const int fin = ctl[1];
+      const int fin = range.whole + ctl[1];
       ctl[1] = 0;
       // release at GPU scope: the CTA's stores to y (ordered before this thread by the barrier) are visible to
       // whoever sees the count
       if (fin > 0 && !ctl[0]) red_release_add(P.sync, (uint32_t)fin);
     }
   }
+}
+
+__global__ void __launch_bounds__(kSAllThreads, 1)
+stack_kernel(const __grid_constant__ StackParams P) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int cta = (int)blockIdx.x, G = (int)gridDim.x;
+  uint8_t* base = smem + (P.use_meta6 ? SSmem::meta6_bytes : 0u);
+  volatile int* ctl = reinterpret_cast<volatile int*>(base + SSmem::ctl);      // [0] failed, [1] straddling row tiles this CTA finished, [2] last CTA out, [3] a packed header does not match
+  int* pslot = reinterpret_cast<int*>(base + SSmem::slots);
+  float* pdata = reinterpret_cast<float*>(smem + P.pdata_off);
+
+  if (!stack_setup(P, base, ctl)) {          // before anything was streamed or the workspace touched
+    if (threadIdx.x == 0 && cta == 0 && P.dev_status) *P.dev_status = STB_ERR_CORRUPT;
+    return;
+  }
+  if (threadIdx.x == 0) { ctl[0] = 0; ctl[1] = 0; ctl[2] = 0; }
+  __syncthreads();
+  if (threadIdx.x >= kSThreads) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFeedRegs));
+    if ((threadIdx.x >> 5) == kSWarps) feed_rings(P, smem, base, ctl);
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDecodeRegs));
+    decode_phases(P, smem, base, ctl, pslot, pdata, cta);
+  }
 
   // ---- leaving: let copies in flight land, then the last CTA out restores the workspace ----
-  if (ctl[0] || W.failed) {
+  __syncthreads();
+  if (ctl[0]) {
     const long long t0 = clock64();
     while (clock64() - t0 < 200000) {}
   }
@@ -756,99 +909,67 @@ stack_kernel(const __grid_constant__ StackParams P) {
   __syncthreads();
   if (ctl[2]) {
     __threadfence();
-    const bool aborted = ld_acquire_u32(P.sync + 1) != 0u;
-    if (aborted) {
-      int maxR = 0;
-      for (int ph = 0; ph < P.nphase; ++ph) maxR = max(maxR, P.ph[ph].tile_start[P.ph[ph].count]);
-      for (int i = threadIdx.x; i < maxR; i += blockDim.x) P.sync[4 + i] = 0u;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; __threadfence(); }
+    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; P.sync[4] += 1u; __threadfence(); }
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // stb_layer_stack_checksum: XOR of all 32-bit words of the tiles and residual streams of every step's packed layer
 // (an integrity check for packed layers that were stored or moved).  It walks the layers exactly as stack_kernel
-// does -- same dealing, same per-warp rings and bulk copies, same residual-span copies -- and folds the words
-// instead of decoding them, so its rate is also the rate this way of streaming reaches with no arithmetic behind it.
-__global__ void __launch_bounds__(kSThreads, 1)
+// does -- same dealing, same per-warp rings and bulk copies -- and folds the words instead of decoding them, so its
+// rate is also the rate this way of streaming reaches with no arithmetic behind it.
+__global__ void __launch_bounds__(kSAllThreads, 1)
 checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __restrict__ sums, int first_step) {
   extern __shared__ __align__(128) uint8_t smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cta = (int)blockIdx.x, G = (int)gridDim.x;
-  WarpEnv E;
-  E.P = &P; E.smem = smem; E.cta = cta; E.G = G; E.warp = warp; E.lane = lane; E.g = lane >> 2; E.t = lane & 3;
-  E.bar0 = smem_u32(smem + SSmem::bars) + (uint32_t)warp * kSDepth * 8u;
-  E.bar_stage = smem_u32(smem + SSmem::bars) + (uint32_t)(kSWarps * kSDepth + warp) * 8u;
-  E.ring = smem + SSmem::ring + (size_t)warp * kSDepth * kSlotBytes;
-  E.stage = smem + SSmem::stage + (size_t)warp * kStageBytes;
-  if (lane == 0) {
-    for (int i = 0; i < kSDepth; ++i) mbar_init(E.bar0 + 8u * i, 1);
-    mbar_init(E.bar_stage, 1);
-    fence_async_smem();
+  const int lane = threadIdx.x & 31;
+  uint8_t* base = smem + (P.use_meta6 ? SSmem::meta6_bytes : 0u);
+  volatile int* ctl = reinterpret_cast<volatile int*>(base + SSmem::ctl);
+  if (!stack_setup(P, base, ctl)) {
+    if (threadIdx.x == 0 && blockIdx.x == 0 && P.dev_status) *P.dev_status = STB_ERR_CORRUPT;
+    return;
   }
-  __syncwarp();
-  WarpState W;
-  W.prod.enter(P, 0, cta, G, warp);
-  W.consumed = 0; W.cur_in = 0; W.stage_use = 0; W.failed = false;
-#pragma unroll
-  for (int i = 0; i < kSDepth; ++i) ring_issue(E, W, i);
-
-  int step_base = first_step;                    // index, in the caller's list, of the phase's first step
-  for (int ph = 0; ph < P.nphase && !W.failed; ++ph) {
-    const StackPhase& q = P.ph[ph];
-    const int nb = q.m / kBlock;
-    const uint32_t tb = tile_bytes(q.N);
-    int lo, hi;
-    warp_range(q, nb, cta, G, warp, lo, hi);
-    int R = lo / nb, b_first = lo - R * nb, left = hi - lo;
-    while (left > 0 && !W.failed) {
-      const int seg = left < nb - b_first ? left : nb - b_first, b_end = b_first + seg;
-      const int si = step_of(q, R), rt = R - q.tile_start[si];
-      const uint8_t* packed = q.packed[si];
-      const BlockInfo* binfo = reinterpret_cast<const BlockInfo*>(packed + sizeof(Header));
-      const ResidWord* rwt = reinterpret_cast<const ResidWord*>(packed + rwtab_offset(nb));
-      const int ntile = (q.n[si] + kTileRows - 1) / kTileRows;
-      const uint32_t nrw_all = __ldg(&reinterpret_cast<const Header*>(packed)->nrw);
-      const uint8_t* resid_rt = packed + tiles_offset(nb) + (size_t)tb * nb * ntile + (size_t)rt * resid_rt_bytes(nb, nrw_all);
+  if (threadIdx.x == 0) ctl[0] = 0;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  bool failed = false;
+  if (warp >= kSWarps) { if (warp == kSWarps) feed_rings(P, smem, base, ctl); }
+  else {
+    const uint8_t* ring = smem + P.ring_off + (size_t)warp * kSDepth * kSlotBytes;
+    const uint4* chunk = reinterpret_cast<const uint4*>(base + SSmem::chunks) + kSDepth * warp;
+    const uint32_t full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)warp, empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)warp;
+    uint32_t slot = 0, parity = 0;
+    int step_base = first_step;                    // index, in the caller's list, of the phase's first step
+    for (int ph = 0; ph < P.nphase && !failed; ++ph) {
+      const StackPhase& q = P.ph[ph];
+      const uint32_t tb = tile_bytes(q.N);
+      int lo, hi;
+      warp_range(reinterpret_cast<const CtaRange*>(base + SSmem::range)[ph], warp, lo, hi);
       uint32_t fold = 0;
-      for (int bs = b_first; bs < b_end && !W.failed; bs += kSpan) {
-        const int be = bs + kSpan < b_end ? bs + kSpan : b_end;
-        const uint32_t rw0 = __ldg(&binfo[bs].rw_off), rw1 = __ldg(&binfo[be - 1].rw_off) + __ldg(&binfo[be - 1].nrw);
-        const uint32_t rec_bytes = (uint32_t)(be - bs) * kResidA2Bytes + (rw1 - rw0) * kResidWordBytes;
-        const uint32_t tab0 = rw0 & ~1u, tab_bytes = ((rw1 - tab0) * 8u + 15u) & ~15u;
+      for (bool more = lo < hi; more;) {
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(full + 8u * slot, parity, P.wait_limit))) { failed = true; break; }
+        const uint4 c = chunk[slot];
+        const uint8_t* tile = ring + (size_t)slot * kSlotBytes;
+        const uint32_t cnt = c.x & 3u, rec_b = cnt * kResidA2Bytes + ((c.x >> 16) & 0xFFu) * kResidWordBytes;
+        for (uint32_t o = (uint32_t)lane * 4u; o < cnt * tb; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + o);
+        for (uint32_t o = (uint32_t)lane * 4u; o < rec_b; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + kSlotTiles + o);
         __syncwarp();
-        if (lane == 0) {
-          fence_async_smem();
-          mbar_expect_tx(E.bar_stage, rec_bytes + (rw1 > rw0 ? tab_bytes : 0u));
-          bulk_g2s(smem_u32(E.stage), resid_rt + resid_block_off(bs, rw0), rec_bytes, E.bar_stage);
-          if (rw1 > rw0) bulk_g2s(smem_u32(E.stage + kStageTab), rwt + tab0, tab_bytes, E.bar_stage);
-        }
-        const uint32_t stage_parity = W.stage_use & 1u;
-        ++W.stage_use;
-        for (int b = bs; b < be; ++b) {
-          const int slot = (int)(W.consumed % kSDepth);
-          if (W.cur_in == 0 && !__all_sync(0xFFFFFFFFu, mbar_wait(E.bar0 + 8u * slot, (W.consumed / kSDepth) & 1u, P.wait_limit))) { W.failed = true; break; }
-          const uint8_t* tile = E.ring + (size_t)slot * kSlotBytes + (size_t)W.cur_in * tb;
-          const bool last_of_chunk = W.cur_in + 1 == (slot == 0 ? W.chunk_cnt0 : W.chunk_cnt1);
-          for (uint32_t o = (uint32_t)lane * 4u; o < tb; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + o);
-          if (last_of_chunk) { __syncwarp(); ring_issue(E, W, slot); W.cur_in = 0; ++W.consumed; }
-          else ++W.cur_in;
-        }
-        if (W.failed) break;
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait(E.bar_stage, stage_parity, P.wait_limit))) { W.failed = true; break; }
-        for (uint32_t o = (uint32_t)lane * 4u; o < rec_bytes; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(E.stage + o);
-      }
-      // words of one step only ever meet words of the same step
+        if (lane == 0) mbar_arrive(empty + 8u * slot);
+        parity ^= slot;
+        slot ^= 1u;
+        more = !(c.x & kRunEnd);
+        if (c.x & kSegEnd) {
+          // words of one step only ever meet words of the same step
 #pragma unroll
-      for (int d = 16; d > 0; d >>= 1) fold ^= __shfl_xor_sync(0xFFFFFFFFu, fold, d);
-      if (lane == 0 && !W.failed) atomicXor(sums + step_base + si, (unsigned long long)fold);
-      left -= seg; ++R; b_first = 0;
+          for (int d = 16; d > 0; d >>= 1) fold ^= __shfl_xor_sync(0xFFFFFFFFu, fold, d);
+          if (lane == 0) atomicXor(sums + step_base + step_of(q, (int)c.w), (unsigned long long)fold);
+          fold = 0;
+        }
+      }
+      step_base += q.count;
     }
-    step_base += q.count;
+    if (failed && lane == 0) ctl[0] = 1;
   }
-  if (W.failed) {
+  if (failed) {
     const long long t0 = clock64();
     while (clock64() - t0 < 200000) {}
     if (lane == 0 && P.dev_status) *P.dev_status = STB_ERR_TIMEOUT;
@@ -888,17 +1009,11 @@ static bool deal_aligned(long long R, int G) {
   return (double)R / (double)G >= 0.85 * (double)rounds;
 }
 
-// most CTAs that share one row tile of a phase of R row tiles x nb blocks dealt to G CTAs by equal tile counts
+// at most so many CTAs share one row tile of a phase of R row tiles x nb blocks dealt to G CTAs by equal tile counts
 static uint32_t max_share_of(long long R, int nb, int G) {
-  const long long T = R * nb;
-  const int Ge = dealt_ctas((int)R, nb, false, G);
-  uint32_t best = 1;
-  for (long long r = 0; r < R; ++r) {
-    const int c0 = owner_of(r * nb, T, Ge), c1 = owner_of((r + 1) * nb - 1, T, Ge);
-    const uint32_t s = (uint32_t)(c1 - c0 + 1);
-    if (s > best) best = s;
-  }
-  return best;
+  const long long Ge = dealt_ctas((int)R, nb, false, G);
+  const long long s = (Ge + R - 1) / R + 1;
+  return (uint32_t)(s < Ge ? s : Ge);
 }
 
 static int stack_sm_count(int* out) {
@@ -916,11 +1031,71 @@ static int stack_sm_count(int* out) {
 }
 
 constexpr uint32_t kSmemLimit = 227 * 1024;
+constexpr unsigned long long kGatherMax = 16 * 1024;     // shared memory for the residual words' activations
+
+// Lays out the shared memory of a launch and chooses each phase's staging; returns the number of phases left without.
+static uint32_t up128(uint32_t v) { return (v + 127u) & ~127u; }
+static int plan_smem(StackParams& sp, bool image) {
+  bool any6 = false, dense[3] = {false, false, false};
+  for (int p = 0; p < sp.nphase; ++p) {
+    if (sp.ph[p].N == 6 && image) any6 = true;
+    else dense[sp.ph[p].N - 4] = true;
+  }
+  // 6:8 phases may fall back to position order; their table is then needed as well
+  for (int round = 0;; ++round) {
+    uint32_t o = 0;
+    sp.use_meta6 = any6 ? 1 : 0;
+    if (any6) o = SSmem::meta6_bytes;
+    o += SSmem::bytes;
+    for (int k = 0; k < 3; ++k) {
+      sp.pos_off[k] = 0;
+      if (dense[k]) { o = up128(o); sp.pos_off[k] = o; o += kPosBytes; }
+    }
+    sp.pos_row = kPosCopies * 8;
+    sp.ring_off = up128(o);
+    o = sp.ring_off + kSWarps * kSDepth * kSlotBytes;
+    sp.pdata_off = o;
+    o += 32u * sp.part_floats * 4u;
+    // the residual words' activations: sized for the most words the phase's layers can have
+    sp.xs_off = o;
+    uint32_t xs_max = 0, cols_max = 0;
+    for (int p = 0; p < sp.nphase; ++p) {
+      StackPhase& q = sp.ph[p];
+      const unsigned long long need = 8ull * q.batch * (unsigned long long)kMaxResidWords * (unsigned long long)(q.m / kBlock) * q.count;
+      q.gather = need <= kGatherMax && q.m <= 32768 ? 1 : 0;
+      if (q.gather && need > xs_max) xs_max = (uint32_t)need;
+      if (q.gather && need / q.batch > cols_max) cols_max = (uint32_t)(need / q.batch);
+    }
+    sp.cols_off = up128(o + xs_max);
+    o = up128(sp.cols_off + cols_max);
+    sp.x_off = o;
+    const long long room = (long long)kSmemLimit - (long long)o;
+    if (room < 0) return sp.nphase + 1;
+    int bare = 0;
+    bool again = false;
+    sp.x_bytes = 0;
+    for (int p = 0; p < sp.nphase; ++p) {
+      StackPhase& q = sp.ph[p];
+      const unsigned long long img = 4ull * q.batch * (unsigned long long)(q.m / kBlock) * kImgWordsPerBlock;
+      const unsigned long long plain = (unsigned long long)q.batch * (2ull * (unsigned long long)q.m + kXPad);
+      q.use_image = 0;
+      unsigned long long need = 0;
+      if (q.N == 6 && any6 && (long long)img <= room) { q.use_image = 1; need = img; }
+      else {
+        if (!dense[q.N - 4]) { dense[q.N - 4] = true; again = true; }
+        if ((long long)plain <= room) { q.use_image = 2; need = plain; }
+        else { ++bare; q.gather = 0; }
+      }
+      if (need > sp.x_bytes) sp.x_bytes = (uint32_t)need;
+    }
+    if (!again || round > 2) return bare;
+  }
+}
 
 // Builds the phases of steps [i0, ...) into `sp` (at most kMaxPhases), returns the index of the first step not taken.
 static int build_phases(const stb_step* steps, int count, int i0, int G, StackParams& sp, size_t& sync_need, size_t& gpart_need) {
   sp.nphase = 0;
-  sp.image_bytes = 0; sp.part_floats = 32; sp.max_share = 1;
+  sp.part_floats = 32; sp.max_share = 1;
   uint32_t done = 0;
   long long maxR = 0;
   int i = i0;
@@ -945,7 +1120,7 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
     q.x = static_cast<const __half*>(st.in);
     q.x2 = st.input == STB_IN_SILU_MUL ? static_cast<const __half*>(st.in2) : nullptr;
     q.ldx = (uint32_t)st.ldin; q.m = st.m; q.N = (uint8_t)st.N; q.batch = (uint8_t)st.batch;
-    q.use_image = 0; q.pad[0] = q.pad[1] = 0;
+    q.use_image = 0; q.gather = 0; q.pad = 0;
     q.done_before = done;
     const long long R = q.tile_start[q.count];
     done += (uint32_t)R;
@@ -957,23 +1132,19 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
     ++sp.nphase;
     i = j;
   }
-  // second pass: where each phase takes its activations from.  6:8 with up to two batch rows: the operand-order
-  // image in shared memory if it fits; a formed input (silu(in) * in2) must be staged: image or plain copy.
-  const uint32_t fixed = SSmem::pdata + 32u * sp.part_floats * 4u;
-  for (int p = 0; p < sp.nphase; ++p) {
-    StackPhase& q = sp.ph[p];
-    const uint32_t img = (uint32_t)q.batch * (uint32_t)(q.m / kBlock) * kImgWordsPerBlock * 4u;
-    const uint32_t plain = (uint32_t)q.batch * (uint32_t)q.m * 2u;
-    uint32_t need = 0;
-    if (q.N == 6 && q.batch <= 2 && fixed + img <= kSmemLimit) { q.use_image = 1; need = img; }
-    else if (q.x2) {
-      if (fixed + plain > kSmemLimit) return -1;          // the formed input does not fit shared memory
-      q.use_image = 2; need = plain;
-    }
-    if (need > sp.image_bytes) sp.image_bytes = need;
+  // second pass: where each phase takes its activations from.  6:8: the operand-order image if it fits, else, as for the
+  // others, a plain copy if that fits, else global memory; a formed input (silu(in) * in2) must be staged.  The image
+  // costs the 12 KB of the metadata table for the whole launch: without it if that lets more phases stage.
+  int best = -1, best_bare = 0;
+  for (int form = 0; form < 2; ++form) {
+    const int bare = plan_smem(sp, form == 0);
+    if (best < 0 || bare < best_bare) { best = form; best_bare = bare; }
   }
-  const size_t s_need = (size_t)(4 + maxR) * sizeof(uint32_t);
-  const size_t g_need = (size_t)maxR * sp.max_share * sp.part_floats * sizeof(float);
+  if (best == 0) plan_smem(sp, true);
+  for (int p = 0; p < sp.nphase; ++p)
+    if (sp.ph[p].x2 && sp.ph[p].use_image == 0) return -1;          // the formed input does not fit shared memory
+  const size_t s_need = 8 * sizeof(uint32_t);
+  const size_t g_need = sp.max_share > 1 ? (size_t)maxR * sp.max_share * sp.part_floats * sizeof(uint2) : 0;
   if (s_need > sync_need) sync_need = s_need;
   if (g_need > gpart_need) gpart_need = g_need;
   return i;
@@ -1040,15 +1211,15 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
     i = stb::build_phases(steps, count, i, G, sp, a, b);
     if (i < 0) return STB_ERR_UNSUPPORTED;
     sp.sync = static_cast<uint32_t*>(ws);
-    sp.gpart = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + sync_bytes);
+    sp.gpart = reinterpret_cast<uint2*>(static_cast<uint8_t*>(ws) + sync_bytes);
     sp.dev_status = dev_status;
     sp.wait_limit = selftest ? stb::kSSelftestLimit : stb::kSWaitLimit;
     sp.copies_off = selftest ? 1 : 0;
-    const uint32_t smem = stb::SSmem::pdata + 32u * sp.part_floats * 4u + sp.image_bytes;
+    const uint32_t smem = sp.x_off + sp.x_bytes;
     if (smem > stb::kSmemLimit) return STB_ERR_UNSUPPORTED;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)G, 1, 1);
-    cfg.blockDim = dim3((unsigned)stb::kSThreads, 1, 1);
+    cfg.blockDim = dim3((unsigned)stb::kSAllThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -1112,8 +1283,8 @@ extern "C" int stb_layer_stack_checksum(const stb_step* steps, int count, unsign
     sp.sync = nullptr; sp.gpart = nullptr; sp.dev_status = dev_status;
     sp.wait_limit = stb::kSWaitLimit; sp.copies_off = 0;
     // the same shared-memory footprint as the arithmetic kernel would have for these steps
-    const uint32_t smem = stb::SSmem::pdata + 32u * sp.part_floats * 4u + sp.image_bytes;
-    stb::checksum_kernel<<<(unsigned)G, stb::kSThreads, smem, s>>>(sp, sums, first);
+    const uint32_t smem = sp.x_off + sp.x_bytes;
+    stb::checksum_kernel<<<(unsigned)G, stb::kSAllThreads, smem, s>>>(sp, sums, first);
     if (cudaGetLastError() != cudaSuccess) return STB_ERR_CUDA;
   }
   return STB_OK;

@@ -2,25 +2,24 @@
 // (tcgen05.mma, fp32 accumulators in tensor memory).  The compute-bound prefilling stage of
 // Appendix C.2: N = sequence length x batch tokens against one packed layer.
 //
-// One CTA computes a 128 (rows of W^) x 256 kAcc (tokens) tile of the output, D = A B^T with
+// One CTA computes a tile of the output of 128 rows of W^ x up to 256 kAcc tokens, D = A B^T with
 //   A = 128 x 64 bf16 slice of W^, decoded from the packed tiles into shared memory in the
 //       K-major 128-byte-swizzled layout the tensor core reads,
-//   B = kAcc slices of 256 x 64 bf16 of X, brought in by TMA with the same swizzle; every decoded
-//       A stage is multiplied with all of them (kAcc accumulators of 256 TMEM columns), which
+//   B = kAcc slices of bn x 64 bf16 of X (bn <= 256, a multiple of 16, chosen per call: see gemm_plan), brought in by TMA
+//       with the same swizzle; every decoded A stage is multiplied with all of them (kAcc accumulators), which
 //       divides the decode work per flop by kAcc,
-// in rings over K (kStagesA decoded A stages, kStagesB X stages: the decode warps run ahead of the tensor core).  Warp roles:
-//   warp 0      TMA producer (one lane): X slices
-//   warp 1, 18  MMA issuers (one lane each, on two schedulers): with two accumulators each takes one (4 x tcgen05.mma,
+// in rings over K (kStagesA decoded A stages, up to eight X boxes: the decode warps run ahead of the tensor core).  Warp roles:
+//   warps 0..15 decode: see below
+//   warp 16     TMA producer (one lane): X slices
+//   warp 17, 18 MMA issuers (one lane each, on two schedulers): with two accumulators each takes one (4 x tcgen05.mma,
 //               K = 16, per stage); with one, each takes half of a stage's K into an accumulator of its own and the
-//               epilogue adds the two.  tcgen05.commit frees the boxes and stages; warp 1 allocates / frees TMEM
-//   warps 2..   decode: warp w works on rows 32 (w % 4) .. +31 of the tile = one packed row tile;
-//               four warps share a row tile, each taking one of the four rows a lane owns (the row
-//               index is a run-time value: one copy of the code; one warp alone per scheduler
-//               would be bound by instruction latency); per 128-column block it loads its row's
-//               words (prefetching the next block), converts the four fp16 scales to bf16
-//               (RN-even) and writes the two 64-column halves of the block into two stages;
-//               afterwards the same warps read the accumulator (TMEM lanes 32 (w % 4) ..) and
-//               store Y.
+//               epilogue adds the two.  tcgen05.commit frees the boxes and stages; warp 17 allocates / frees TMEM
+//   decode:     warp w works on rows 32 (w % 4) .. +31 of the tile = one packed row tile; four warps share a row
+//               tile, each taking every fourth block: it loads the block's words with vector loads (its next block ahead),
+//               converts the scales to bf16 (RN-even), decodes 64 columns of its four rows per lane into registers,
+//               waits for the stage and writes them.  (Four warps sharing every block, one row of a lane each, paid the
+//               loads, the waits and the address arithmetic four times: 370 clocks per 32 x 128 tile and SM, now FIGURE_TILE.)
+//               Afterwards the same warps read the accumulator (TMEM lanes 32 (w % 4) ..) and store Y.
 // The residual term of the salient columns (Eq. 4) is more K: a small kernel first gathers the activations of
 // every residual slot (four per residual word, in word order) into Xs[token][slot]; after the blocks of its K
 // range a CTA runs the residual slots of those blocks as further stages, A = +-bf16(a_sal2) or 0 by the two-bit
@@ -44,31 +43,52 @@
 namespace stb {
 
 constexpr int kBM = 128;          // rows of W^ per CTA (UMMA M)
-// Token side of the CTA tile: kAcc accumulators of kBN tokens (UMMA N).  Prefill: 2 x 256 (all 512 TMEM columns; a
-// decoded A stage is used twice).  Up to 64 tokens (a decode batch): 1 x 64, the tensor core then takes an eighth
-// of the time per stage and the kernel runs at the speed of the decode warps.
-template <int kAcc_, int kBN_>
-struct TokCfg {
-  static constexpr int kAcc = kAcc_, kBN = kBN_, kTok = kAcc_ * kBN_;
-  static constexpr uint32_t kStageB = (uint32_t)kBN_ * 64u * 2u;                 // one X box: kBN tokens x 64 of K
-  static constexpr int kStagesB = kBN_ >= 256 ? 5 : 8;                            // ring of X boxes
-};
+// Token side of the CTA tile: kAcc accumulators of bn tokens (UMMA N, a run-time value).  Prefill: 2 x up to 256 (all 512 TMEM
+// columns; a decoded A stage is used twice).  Up to 64 tokens (a decode batch): 1 x up to 64, the tensor core then takes an
+// eighth of the time per stage and the kernel runs at the speed of the decode warps.
+template <int kAcc_, int kMaxBN_>
+struct TokCfg { static constexpr int kAcc = kAcc_, kMaxBN = kMaxBN_, kTok = kAcc_ * kMaxBN_; };
 constexpr int kBK = 64;           // K per stage: one 128-byte swizzle row of bf16
 constexpr int kStagesA = 4;        // ring of decoded A stages (16 KB each)
-// (the ring of X boxes, TokCfg::kStagesB: 256 tokens x 64 of K = 32 KB each in prefill; a stage of K takes kAcc of them:
-// what is in flight from L2 is what hides its latency, so the ring is deep and its slots small)
-constexpr int kGroups = 4;                              // decode warps per 32-row quarter: one per row of a lane
+constexpr int kMaxStagesB = 8;    // ring of X boxes: as many as fit, up to eight (five of 256 tokens x 64 of K = 32 KB): what is in
+                                  // flight from L2 is what hides its latency; a stage of K takes kAcc of them
+constexpr int kGroups = 4;                              // decode warps per 32-row quarter: each takes every fourth block
 constexpr int kIssuers = 2;                             // MMA-issuing lanes (in two warps, on two schedulers)
-constexpr int kIssuerWarpB = 2 + 4 * kGroups;           // the second one's warp: after the decode warps
-constexpr int kGemmThreads = 64 + 128 * kGroups + 32;
+constexpr int kDecodeWarps = 4 * kGroups;               // warps 0 .. 15; then the copies (16) and the issuers (17, 18)
+constexpr int kTmaWarp = kDecodeWarps, kIssuerWarpA = kDecodeWarps + 1, kIssuerWarpB = kDecodeWarps + 2;
+constexpr int kGemmThreads = 32 * kDecodeWarps + 128;
+// registers: 640 x 96 at launch, of which the fifth warpgroup gives some to the decode warps
+constexpr int kGemmDecodeRegs = 104, kGemmIssueRegs = 64;
+static_assert(32 * kDecodeWarps * kGemmDecodeRegs + 128 * kGemmIssueRegs <= kGemmThreads * 96, "register split within the launch's total");
 constexpr uint32_t kStageA = kBM * kBK * 2;      // 16 KB
-constexpr uint32_t kGemmTab = 0;                                   // position table (576 B)
-constexpr uint32_t kGemmBars = 1024;                               // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
-constexpr uint32_t kGemmA = 2048;                                  // 1024-byte aligned stages
-constexpr uint32_t kGemmB = kGemmA + kStagesA * kStageA;
-template <class Cfg> constexpr uint32_t gemm_smem_bytes() { return kGemmB + (uint32_t)Cfg::kStagesB * Cfg::kStageB; }   // prefill: 231424 B
-static_assert(gemm_smem_bytes<TokCfg<2, 256>>() <= 232448 && gemm_smem_bytes<TokCfg<1, 64>>() <= 232448, "one CTA's shared memory");
-static_assert(8 * (2 * kStagesA + 2 * 8 + 1) + 16 <= 1024, "barrier area");
+// "A stage empty" has twice as many barriers as there are stages: a decode warp writes the stages it = 2 w, 2 w + 1 (mod 8),
+// so it meets every phase of the barriers (it - 4) mod 8 that it waits on, one after the other.
+constexpr int kEmptyA = 2 * kStagesA;
+static_assert(kEmptyA == 2 * kGroups, "the warp of a stage is (stage / 2) mod kGroups");
+constexpr uint32_t kGemmBars = 0;                                  // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
+constexpr uint32_t kGemmTab = 512;                                 // position table, 4 bytes per entry and copy
+static_assert(8 * (kStagesA + kEmptyA + 2 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
+constexpr uint32_t kSmemMax = 232448;
+constexpr double kDecodeClocks = 420.0;    // decode of a stage (gemm_plan)
+// What depends on bn: copies of the position table (16, lane-minor: look-ups nearly free of bank conflicts; one where bn = 256
+// leaves no room), where the stages and the boxes lie, and how many boxes there are.
+struct GemmSmem { uint32_t copies, a, b, box, nbox, total; };
+__host__ __device__ inline GemmSmem gemm_smem(int kAcc, int bn) {
+  GemmSmem g;
+  g.box = (uint32_t)bn * kBK * 2;
+  for (g.copies = 16;; g.copies = 1) {
+    g.a = (kGemmTab + 4u * kPosTableEntries * g.copies + 1023u) & ~1023u;
+    g.b = g.a + kStagesA * kStageA;
+    g.nbox = (kSmemMax - g.b) / g.box;
+    if (g.nbox >= 5u || g.copies == 1u) break;
+  }
+  if (g.nbox > (uint32_t)kMaxStagesB) g.nbox = kMaxStagesB;
+  g.total = g.b + g.nbox * g.box;
+  // a 16-bit output tile is staged where the boxes were
+  const uint32_t out = (uint32_t)(kAcc * bn) * kBM * 2u;
+  if (g.total < g.b + out) g.total = g.b + out;
+  return g;
+}
 constexpr long long kGemmWaitLimit = 2000000000ll;
 
 // ---- tcgen05 / TMA wrappers ---------------------------------------------------------------
@@ -126,11 +146,10 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
   d |= (uint64_t)2 << 61;                  // SWIZZLE_128B
   return d;
 }
-// Instruction descriptor: D = f32, A and B both bf16 (format 1) or both fp16 (format 0), both K-major, N = kBN, M = 128.
-template <int kBN, bool kF16>
-struct GemmIdesc {
-  static constexpr uint32_t value = (1u << 4) | ((kF16 ? 0u : 1u) << 7) | ((kF16 ? 0u : 1u) << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-};
+// Instruction descriptor: D = f32, A and B both bf16 (format 1) or both fp16 (format 0), both K-major, N = bn, M = 128.
+__device__ __forceinline__ uint32_t gemm_idesc(bool f16, int bn) {
+  return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+}
 
 // Bounded mbarrier wait with a CTA-wide abort flag (a volatile int in shared memory).  The two
 // single-lane roles back off between polls so that their spinning does not take issue slots from
@@ -151,121 +170,183 @@ __device__ __forceinline__ uint32_t bf16_bits(uint32_t h16) {
   return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((unsigned short)h16))));
 }
 
+// The byte planes of a row's four main scales (A low, B high bytes, fp16) as bf16.
+__device__ __forceinline__ void scales_to_bf16(uint32_t& A, uint32_t& B) {
+  const uint32_t h01 = prmt(A, B, 0x5140u), h23 = prmt(A, B, 0x7362u);
+  const float2 f01 = __half22float2(*reinterpret_cast<const __half2*>(&h01)), f23 = __half22float2(*reinterpret_cast<const __half2*>(&h23));
+  const __nv_bfloat162 b01 = __floats2bfloat162_rn(f01.x, f01.y), b23 = __floats2bfloat162_rn(f23.x, f23.y);
+  const uint32_t u01 = *reinterpret_cast<const uint32_t*>(&b01), u23 = *reinterpret_cast<const uint32_t*>(&b23);
+  A = prmt(u01, u23, 0x6420u);
+  B = prmt(u01, u23, 0x7531u);
+}
+
 // What a decode warp needs to know.
 struct DecodeArgs {
-  const uint8_t* packed; const Header* hdr; uint8_t* smem; volatile int* abort_flag;
-  uint32_t bar_full, bar_empty;      // of the A ring
-  int mt, b0, b1, nblk, ntile, q, lane;
-  uint32_t rw0, rw1;        // residual words of the blocks [b0, b1)
+  const uint8_t* packed; uint8_t* smem; volatile int* abort_flag;
+  const uint32_t* ptab; uint8_t* stages;
+  uint32_t bar_full, bar_empty, copies;      // of the A ring; copies of the position table
+  int mt, b0, b1, nblk, ntile, q, w, lane;   // q: row tile of the CTA's four, w: which of the row tile's four warps
+  uint32_t nrw, rw0, rw1;   // residual words of a row tile, and of the blocks [b0, b1)
   int nres;                 // residual stages (64 slots = 16 words each, the first one starts at word rw0 & ~1)
 };
 
-// Decode role of one warp: row j (of the four rows g + 8 j each lane owns) of packed row tile 4 mt + q, for
-// every block of the CTA's K range, written into the A stages.  j is a run-time value: the four warps of a
-// row tile run the same code.
+// The words of a tile that a lane decodes: load_lane_tile's, with N = 6's pair fields as they are (word 4 mt + s).
+template <int N>
+struct GemmTile { LaneTile<N> lt; uint32_t fld[8]; };
+template <int N>
+__device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, GemmTile<N>& d) {
+  if constexpr (mask_pairs(N)) {
+    load_planes<N>(tile, off_region(N), d.lt.R, lane);
+    load_planes<LaneTile<N>::kFull>(tile, off_sign(N), d.lt.S, lane);
+    d.lt.half = 0;
+    const uint4 s0 = *reinterpret_cast<const uint4*>(tile + scale_off(N, lane >> 2, 0)), s1 = *reinterpret_cast<const uint4*>(tile + scale_off(N, lane >> 2, 2));
+    d.lt.A[0] = s0.x; d.lt.B[0] = s0.y; d.lt.A[1] = s0.z; d.lt.B[1] = s0.w;
+    d.lt.A[2] = s1.x; d.lt.B[2] = s1.y; d.lt.A[3] = s1.z; d.lt.B[3] = s1.w;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d.fld[k] = *reinterpret_cast<const uint16_t*>(tile + pair_field_off(lane >> 2, k >> 2, k & 3, lane & 3));
+  } else {
+    load_lane_tile<N>(tile, lane, d.lt);
+  }
+}
+
+// Decode role of one warp: packed row tile 4 mt + q, every fourth block of the CTA's K range, written into the A stages.
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
 template <int N, bool kF16>
-__device__ __forceinline__ void decode_row(const DecodeArgs& da, const int j) {
-  const uint8_t* packed = da.packed;
-  const Header* hdr = da.hdr;
-  uint8_t* smem = da.smem;
+__device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   volatile int* abort_flag = da.abort_flag;
-  const uint32_t bar_full = da.bar_full, bar_empty = da.bar_empty;
-  const int mt = da.mt, b0 = da.b0, b1 = da.b1, nblk = da.nblk, ntile = da.ntile, q = da.q;
+  const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1;
   // The lane plays the part of packed-layout lane 4 g + t with g = lane % 8, t = lane / 8: the eight
   // lanes of a quarter-warp then hold eight different rows g and their 16-byte stores into the
   // swizzled stage fall on eight different 16-byte bank groups (no conflict); loads of the
   // lane-major planes stay coalesced, they are only permuted inside the warp.
   const int g = da.lane & 7, t = da.lane >> 3;
   const int lane = 4 * g + t;
-  const int rtile = mt * 4 + q;                 // packed row tile
-  const bool live = rtile < ntile;
-  const uint32_t* ptab = reinterpret_cast<const uint32_t*>(smem + kGemmTab);     // low half: columns 0..3, high half: 4..7
-  const uint8_t* rtbase = packed + hdr->tiles_offset + (size_t)rtile * hdr->rt_stride;
-  const uint8_t* resid_rt = packed + hdr->tiles_offset + hdr->rt_stride * (size_t)ntile +
-                            (size_t)rtile * resid_rt_bytes(nblk, hdr->nrw);
+  const int rtile = da.mt * 4 + q;                 // packed row tile
+  const bool live = rtile < da.ntile;
+  const uint32_t* ptab = da.ptab + (uint32_t)da.lane % da.copies;
+  const uint8_t* rtbase = da.packed + tiles_offset(nblk) + (size_t)rtile * tile_bytes(N) * nblk;
+  const uint8_t* resid_rt = da.packed + tiles_offset(nblk) + (size_t)tile_bytes(N) * nblk * da.ntile + (size_t)rtile * resid_rt_bytes(nblk, da.nrw);
   constexpr uint32_t tbytes = tile_bytes(N);
-  // The row's words are loaded three blocks ahead of their use (three sets of registers in rotation): the loads
-  // come straight from HBM, and one block of decode is shorter than their latency.
-  RowWords w0 = {}, w1 = {}, w2 = {};
-  auto fetch = [&](int b, RowWords& w) {
-    if (live && b < b1) load_row_words<N>(rtbase + (size_t)b * tbytes, lane, j, w);
+  // where the lane's two 16-byte chunks (4 sl + t) of its row g go inside a stage's eight rows
+  const uint32_t off0 = (uint32_t)g * 128u + (uint32_t)((t ^ g) << 4), off1 = (uint32_t)g * 128u + (uint32_t)(((4 + t) ^ g) << 4);
+  uint8_t* rows = da.stages + (size_t)(4 * q) * 1024;
+  // wait for stage `it`; the verdict is made warp-uniform: nobody may be left alone at the __syncwarp() below
+  auto stage_wait = [&](int it) {
+    const uint32_t bar = da.bar_empty + 8u * (uint32_t)((it + kEmptyA - kStagesA) % kEmptyA);
+    return it < kStagesA || __all_sync(0xFFFFFFFFu, gemm_wait(bar, (uint32_t)((it - kStagesA) / kEmptyA) & 1u, abort_flag));
   };
-  auto block = [&](int b, const RowWords& cur) -> bool {
-    // bf16 scale bytes of the row (a salient weight gets s1 bf16(a_sal1) here; its residual term comes with the residual stages)
-    uint32_t A16 = 0, B16 = 0;
-    if (live) {
+  auto stage_done = [&](int it) {
+    fence_async_smem();          // generic-proxy writes -> visible to the tensor core
+    __syncwarp();
+    if (lane == 0) mbar_arrive(da.bar_full + 8 * (it % kStagesA));
+  };
+  // Residual stages come after the blocks: 64 residual slots (16 residual words) of K each.  The lane writes the same
+  // two 16-byte chunks of its rows: chunk c holds the words 2 c and 2 c + 1 of the stage, four slots each, as
+  // +-bf16(a_sal2) or 0.  What a stage needs sits behind two dependent loads from global memory (the word's table
+  // entry, then a_sal2 and the codes from the block's record); the entries of the warp's first one are asked for here.
+  const ResidWord* rwt = reinterpret_cast<const ResidWord*>(da.packed + rwtab_offset(nblk));
+  const uint32_t wfirst = da.rw0 & ~1u;
+  const int nmain = 2 * (b1 - b0), nstage = nmain + da.nres;
+  auto mine = [&](int it) { return ((it >> 1) & (kGroups - 1)) == da.w; };
+  auto next_res = [&](int it) { while (it < nstage && !mine(it)) ++it; return it; };
+  auto res_word = [&](int it, int idx) { return wfirst + 16u * (uint32_t)(it - nmain) + 2u * (uint32_t)(4 * (idx >> 1) + t) + (uint32_t)(idx & 1); };
+  uint2 e[4];
+  auto res_entries = [&](int it) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const uint32_t h16 = ((cur.A >> (8 * c)) & 0xFFu) | (((cur.B >> (8 * c)) & 0xFFu) << 8);
-        const uint32_t v = kF16 ? h16 : bf16_bits(h16);
-        A16 |= (v & 0xFFu) << (8 * c);
-        B16 |= (v >> 8) << (8 * c);
-      }
+    for (int idx = 0; idx < 4; ++idx) {
+      const uint32_t w = res_word(it, idx);
+      e[idx] = make_uint2(0xFFFFFFFFu, 0u);
+      if (live && it < nstage && w >= da.rw0 && w < da.rw1) e[idx] = __ldg(reinterpret_cast<const uint2*>(rwt + w));
     }
-    OneRow<N> row;
-    row.init(cur, j, A16, B16);
-    // position selectors of the row's slots of this block, looked up before the stage waits
-    uint32_t P[4];
+  };
+  int rit = next_res(nmain);
+  GemmTile<N> nxt;
+  int b = b0 + da.w;
+  if (live && b < b1) load_gemm_tile<N>(rtbase + (size_t)b * tbytes, lane, nxt);
+  res_entries(rit);
+#pragma unroll 1
+  for (; b < b1; b += kGroups) {
+    uint32_t mask[4] = {0, 0, 0, 0};                   // word j, byte s: keep-mask index of slot (j, s)
+    FastRows<N> fr;
+    uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
+    if (live) {
+      if constexpr (mask_pairs(N)) {
 #pragma unroll
-    for (int sidx = 0; sidx < 4; ++sidx) P[sidx] = live ? ptab[(cur.mask >> (8 * sidx)) & 0xFFu] : 0u;
+        for (int k = 0; k < 8; ++k) {                  // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)
+          const uint32_t J = nxt.fld[k] >> 4, i1 = (J * 2341u) >> 16, i0 = J - kMasks6 * i1;      // (pair_field_index)
+          mask[2 * (k >> 2)] = i0 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2)];
+          mask[2 * (k >> 2) + 1] = i1 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2) + 1];
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mask[j] = nxt.lt.mask[j];
+      }
+      uint32_t A[4], B[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        A[j] = nxt.lt.A[j]; B[j] = nxt.lt.B[j];
+        // (a salient weight gets s1 bf16(a_sal1) here; its residual term comes with the residual stages)
+        if (!kF16) scales_to_bf16(A[j], B[j]);
+      }
+      fr.init(nxt.lt, A, B);
+      if (N == 5) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fr.high(j, 0, XL[j], XH[j]);
+      }
+      if (b + kGroups < b1) load_gemm_tile<N>(rtbase + (size_t)(b + kGroups) * tbytes, lane, nxt);
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int it = 2 * (b - b0) + h, st = it % kStagesA;
-      // the verdict is made warp-uniform: nobody may be left alone at the __syncwarp() below
-      if (!__all_sync(0xFFFFFFFFu, gemm_wait(bar_empty + 8 * st, ((uint32_t)(it / kStagesA) & 1u) ^ 1u, abort_flag))) return false;
-      uint8_t* As = smem + kGemmA + st * kStageA;
-      uint8_t* rowp = As + (size_t)(4 * q + j) * 1024 + g * 128;
-      if (N == 6 && live) row.high(h);
+      const int it = 2 * (b - b0) + h;
+      uint32_t f[4][2][4];
 #pragma unroll
-      for (int sl = 0; sl < 2; ++sl) {
-        const int sidx = 2 * h + sl;                       // slot s of the block, group 4 sidx + t
-        uint32_t f[4] = {0, 0, 0, 0};
-        if (live) row.slot(sidx, P[sidx], P[sidx] >> 16, f);
-        const int chunk = 4 * sl + t;                      // 16-byte chunk of the 128-byte row
-        *reinterpret_cast<uint4*>(rowp + ((chunk ^ g) << 4)) = make_uint4(f[0], f[1], f[2], f[3]);
+      for (int j = 0; j < 4; ++j) {
+        if (N == 6 && live) fr.high(j, h, XL[j], XH[j]);
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl) {
+          const int sidx = 2 * h + sl;                       // slot s of the block, group 4 sidx + t
+          f[j][sl][0] = f[j][sl][1] = f[j][sl][2] = f[j][sl][3] = 0;
+          if (live) {
+            const uint32_t P = ptab[keep_index_of(mask, j, sidx) * da.copies];
+            fr.slot2(j, sidx, P, P >> 16, XL[j], XH[j], f[j][sl]);
+          }
+        }
       }
-      fence_async_smem();          // generic-proxy writes -> visible to the tensor core
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_full + 8 * st);
+      if (!stage_wait(it)) return;
+      uint8_t* st = rows + (size_t)(it % kStagesA) * kStageA;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        *reinterpret_cast<uint4*>(st + 1024 * j + off0) = make_uint4(f[j][0][0], f[j][0][1], f[j][0][2], f[j][0][3]);
+        *reinterpret_cast<uint4*>(st + 1024 * j + off1) = make_uint4(f[j][1][0], f[j][1][1], f[j][1][2], f[j][1][3]);
+      }
+      stage_done(it);
     }
-    return true;
-  };
-  // Residual stages (after the blocks): 64 residual slots (16 residual words) of K each.  The lane writes the same
-  // two 16-byte chunks of its row as above: chunk c holds the words 2 c and 2 c + 1 of the stage, four slots each,
-  // as +-bf16(a_sal2) or 0.  What a stage needs sits behind two dependent loads from global memory (the word's table
-  // entry, then a_sal2 and the codes from the block's record), so both are taken ahead: the entries two stages, the
-  // records one stage before their use, the first ones before the blocks.
-  const ResidWord* rwt = reinterpret_cast<const ResidWord*>(packed + rwtab_offset(nblk));
-  const uint32_t wfirst = da.rw0 & ~1u;
-  auto res_word = [&](int rs, int idx) { return wfirst + 16u * (uint32_t)rs + 2u * (uint32_t)(4 * (idx >> 1) + t) + (uint32_t)(idx & 1); };
-  auto res_entries = [&](int rs, uint2 (&e)[4], uint32_t& valid) {
-    valid = 0;
+  }
+#pragma unroll 1
+  while (rit < nstage) {
+    uint2 a2[4];
+    uint32_t word[4];
 #pragma unroll
     for (int idx = 0; idx < 4; ++idx) {
-      const uint32_t w = res_word(rs, idx);
-      e[idx] = make_uint2(0u, 0u);
-      if (live && rs < da.nres && w >= da.rw0 && w < da.rw1) { e[idx] = __ldg(reinterpret_cast<const uint2*>(rwt + w)); valid |= 1u << idx; }
-    }
-  };
-  auto res_records = [&](int rs, const uint2 (&e)[4], uint32_t valid, uint32_t (&a2)[4], uint32_t (&word)[4]) {
-#pragma unroll
-    for (int idx = 0; idx < 4; ++idx) {
-      a2[idx] = 0; word[idx] = 0;
-      if ((valid >> idx) & 1u) {
-        const uint8_t* rec = resid_rt + resid_block_off((int)(e[idx].x >> 3), res_word(rs, idx) - (e[idx].x & 7u));
-        a2[idx] = __ldg(reinterpret_cast<const uint16_t*>(rec + resid_a2_off(g, j)));
+      a2[idx] = make_uint2(0u, 0u); word[idx] = 0x55555555u;               // "no term"
+      if (e[idx].x != 0xFFFFFFFFu) {
+        const uint8_t* rec = resid_rt + resid_block_off((int)(e[idx].x >> 3), res_word(rit, idx) - (e[idx].x & 7u));
+        a2[idx] = __ldg(reinterpret_cast<const uint2*>(rec + resid_a2_off(g, 0)));
         word[idx] = __ldg(reinterpret_cast<const uint32_t*>(rec + resid_code_off(e[idx].x & 7u, g)));
       }
     }
-  };
-  auto res_stage = [&](int rs, uint32_t valid, const uint32_t (&a2)[4], const uint32_t (&word)[4]) -> bool {
-    const int it = 2 * (b1 - b0) + rs, st = it % kStagesA;
-    uint32_t f[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+    const int it = rit;
+    rit = next_res(it + 1);
+    res_entries(rit);
+    if (!stage_wait(it)) return;
+    uint8_t* st = rows + (size_t)(it % kStagesA) * kStageA;
 #pragma unroll
-    for (int idx = 0; idx < 4; ++idx)
-      if ((valid >> idx) & 1u) {
-        const uint32_t v = kF16 ? a2[idx] : bf16_bits(a2[idx]);
+    for (int j = 0; j < 4; ++j) {
+      uint32_t f[2][4];
+#pragma unroll
+      for (int idx = 0; idx < 4; ++idx) {
+        const uint32_t h16 = (((j & 2) ? a2[idx].y : a2[idx].x) >> (16 * (j & 1))) & 0xFFFFu;
+        const uint32_t v = kF16 ? h16 : bf16_bits(h16);
         const uint32_t L2 = prmt(v, 0u, 0x4040u);                 // (lo, 0, lo, 0)
         const uint32_t H2 = prmt(v, v ^ 0x8000u, 0x2521u);        // (hi, 0, hi ^ 0x80, 0)
         const uint32_t sel = resid_selector(word[idx], j);
@@ -273,39 +354,10 @@ __device__ __forceinline__ void decode_row(const DecodeArgs& da, const int j) {
         f[idx >> 1][2 * (idx & 1)] = prmt(lo4, hi4, 0x5140u);
         f[idx >> 1][2 * (idx & 1) + 1] = prmt(lo4, hi4, 0x7362u);
       }
-    if (!__all_sync(0xFFFFFFFFu, gemm_wait(bar_empty + 8 * st, ((uint32_t)(it / kStagesA) & 1u) ^ 1u, abort_flag))) return false;
-    uint8_t* rowp = smem + kGemmA + st * kStageA + (size_t)(4 * q + j) * 1024 + g * 128;
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl)
-      *reinterpret_cast<uint4*>(rowp + (((4 * sl + t) ^ g) << 4)) = make_uint4(f[sl][0], f[sl][1], f[sl][2], f[sl][3]);
-    fence_async_smem();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar_full + 8 * st);
-    return true;
-  };
-  uint2 eX[4], eY[4];
-  uint32_t veX = 0, veY = 0, vrX = 0, vrY = 0, a2X[4], a2Y[4], wdX[4], wdY[4];
-  res_entries(0, eX, veX);
-  fetch(b0, w0);
-  fetch(b0 + 1, w1);
-  res_records(0, eX, veX, a2X, wdX); vrX = veX;
-  res_entries(1, eY, veY);
-  bool ok = true;
-  for (int b = b0; b < b1 && ok; b += 3) {
-    fetch(b + 2, w2);
-    ok = block(b, w0);
-    if (ok && b + 1 < b1) { fetch(b + 3, w0); ok = block(b + 1, w1); }
-    if (ok && b + 2 < b1) { fetch(b + 4, w1); ok = block(b + 2, w2); }
-  }
-  for (int rs = 0; rs < da.nres && ok; rs += 2) {
-    res_records(rs + 1, eY, veY, a2Y, wdY); vrY = veY;
-    res_entries(rs + 2, eX, veX);
-    ok = res_stage(rs, vrX, a2X, wdX);
-    if (ok && rs + 1 < da.nres) {
-      res_records(rs + 2, eX, veX, a2X, wdX); vrX = veX;
-      res_entries(rs + 3, eY, veY);
-      ok = res_stage(rs + 1, vrY, a2Y, wdY);
+      *reinterpret_cast<uint4*>(st + 1024 * j + off0) = make_uint4(f[0][0], f[0][1], f[0][2], f[0][3]);
+      *reinterpret_cast<uint4*>(st + 1024 * j + off1) = make_uint4(f[1][0], f[1][1], f[1][2], f[1][3]);
     }
+    stage_done(it);
   }
 }
 
@@ -337,24 +389,19 @@ __global__ void gemm_gather_kernel(const uint8_t* __restrict__ packed, int n, in
 }
 
 // ------------------------------------------------------------------------------------------
+// Where a call's output tiles lie (gemm_plan).
+struct GemmShape { int full_tiles, ksplit, bps, ttiles, bn; GemmSmem smem; };
+
 template <int N, class Cfg, bool kF16>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap xsmap, const uint8_t* __restrict__ packed, int n, int m, int T,
-            void* __restrict__ Y, int y_16, size_t ldy, float* __restrict__ ws, int full_tiles, int ksplit, int bps,
-            int ttiles, uint32_t box_bytes, int* dev_status) {
-  constexpr int kAcc = Cfg::kAcc, kBN = Cfg::kBN, kTok = Cfg::kTok, kStagesB = Cfg::kStagesB;
-  constexpr uint32_t kStageB = Cfg::kStageB, kIdesc = GemmIdesc<kBN, kF16>::value;
+            void* __restrict__ Y, int y_16, size_t ldy, float* __restrict__ ws, const __grid_constant__ GemmShape shape, uint32_t box_bytes, int* dev_status) {
+  constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN;
   extern __shared__ __align__(1024) uint8_t smem[];
-  // (the position table's entry of this thread is asked for before the header: two global-memory latencies side by
-  // side instead of one after the other in every CTA's prologue)
-  uint32_t tab_entry = 0;
-  if (threadIdx.x < kPosTableEntries) tab_entry = g_pos_table.v[N][threadIdx.x].x | (g_pos_table.v[N][threadIdx.x].y << 16);
-  const Header* hdr = reinterpret_cast<const Header*>(packed);
-  if (!header_matches(hdr, n, m, N)) {
-    if (threadIdx.x == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
-    return;
-  }
-  const int nblk = m / kBlock, ntile = hdr->ntile;
+  const int full_tiles = shape.full_tiles, ksplit = shape.ksplit, bps = shape.bps, ttiles = shape.ttiles, bn = shape.bn;
+  const GemmSmem& L = shape.smem;
+  const int ktok = kAcc * bn;
+  const int nblk = m / kBlock, ntile = (n + kTileRows - 1) / kTileRows;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // CTAs 0 .. full_tiles - 1 compute one output tile each over the whole K; the rest come in groups of `ksplit`
   // per tile, each with `bps` blocks of K, and leave fp32 partial tiles in the workspace
@@ -364,53 +411,75 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   const int kz = split ? (cta - full_tiles) % ksplit : 0;
   const int tt = tile % ttiles, mt = tile / ttiles;
   const int b0 = split ? kz * bps : 0, b1 = split ? min(nblk, b0 + bps) : nblk;
-  // residual words of the CTA's blocks -> residual stages of 16 words, the first one starting at an even word
+  // Everything the prologue needs from global memory is asked for at once: the table, the header, the word counts, and (into
+  // L2) the first block each decode warp will read.  Where things lie follows from the shape alone; the header is only checked.
+  const Header* hdr = reinterpret_cast<const Header*>(packed);
   const BlockInfo* binfo_k = reinterpret_cast<const BlockInfo*>(packed + sizeof(Header));
+  if (warp < kDecodeWarps) {
+    const int q = warp & 3, b = b0 + (warp >> 2), rtile = mt * 4 + q;
+    if (b < b1 && rtile < ntile && lane * 128 < (int)tile_bytes(N))
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(packed + tiles_offset(nblk) + ((size_t)rtile * nblk + b) * tile_bytes(N) + lane * 128));
+  }
+  const bool fits = header_matches(hdr, n, m, N);
+  const uint32_t nrw = hdr->nrw;
   uint32_t rw0 = 0, rw1 = 0;
-  if (b0 < b1) { rw0 = __ldg(&binfo_k[b0].rw_off); rw1 = b1 < nblk ? __ldg(&binfo_k[b1].rw_off) : hdr->nrw; }
-  const int nres = rw1 > rw0 ? (int)((rw1 - (rw0 & ~1u) + 15u) / 16u) : 0;
-  const int nmain = 2 * max(b1 - b0, 0);               // 64-column stages of the blocks
-  const int nstage = nmain + nres;
+  if (b0 < b1) { rw0 = __ldg(&binfo_k[b0].rw_off); rw1 = b1 < nblk ? __ldg(&binfo_k[b1].rw_off) : nrw; }
 
   const uint32_t sbase = smem_u32(smem);
-  // A ring: full = the 16 decode warps have written the stage, empty = the tensor core has read it;
+  // A ring: full = the four decode warps of the stage's block have written it, empty = the tensor core has read it;
   // B ring: full = the X boxes have landed, empty = the tensor core has read them
   const uint32_t bar_fullA = sbase + kGemmBars, bar_emptyA = bar_fullA + 8 * kStagesA;
-  const uint32_t bar_fullB = bar_emptyA + 8 * kStagesA, bar_emptyB = bar_fullB + 8 * kStagesB, bar_accum = bar_emptyB + 8 * kStagesB;
-  constexpr uint32_t kBarBytes = 8 * (2 * kStagesA + 2 * kStagesB + 1);
+  const uint32_t bar_fullB = bar_emptyA + 8 * kEmptyA, bar_emptyB = bar_fullB + 8 * kMaxStagesB, bar_accum = bar_emptyB + 8 * kMaxStagesB;
+  constexpr uint32_t kBarBytes = 8 * (kStagesA + kEmptyA + 2 * kMaxStagesB + 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kGemmBars + kBarBytes);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kGemmBars + kBarBytes + 8);
 
   if (threadIdx.x == 0) {
     // a stage of A is read by both issuers; an X box by the issuer of its accumulator (by both when there is one box per stage)
-    for (int i = 0; i < kStagesA; ++i) { mbar_init(bar_fullA + 8 * i, 4 * kGroups); mbar_init(bar_emptyA + 8 * i, kIssuers); }
-    for (int i = 0; i < kStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, kAcc == 1 ? kIssuers : 1); }
+    for (int i = 0; i < kStagesA; ++i) mbar_init(bar_fullA + 8 * i, 4);
+    for (int i = 0; i < kEmptyA; ++i) mbar_init(bar_emptyA + 8 * i, kIssuers);
+    for (int i = 0; i < kMaxStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, kAcc == 1 ? kIssuers : 1); }
     mbar_init(bar_accum, kIssuers);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  static_assert(kPosTableEntries <= kGemmThreads, "one table entry per thread");
-  if (threadIdx.x < kPosTableEntries) reinterpret_cast<uint32_t*>(smem + kGemmTab)[threadIdx.x] = tab_entry;   // 4-byte entries: fewer bank conflicts than 8-byte ones
-  constexpr uint32_t kTmemCols = kAcc == 1 ? 2 * kTok : kTok;      // one accumulator: a second one for the other half of K
-  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+  for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads) {
+    const uint2 v = g_pos_table.v[N][i / L.copies];
+    reinterpret_cast<uint32_t*>(smem + kGemmTab)[i] = v.x | (v.y << 16);
+  }
+  constexpr uint32_t kTmemCols = kAcc == 1 ? 2 * kMaxBN : kAcc * kMaxBN;      // one accumulator: a second one for the other half of K
+  if (warp == kIssuerWarpA) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_d = *tmem_slot;
+  if (!fits) {                                         // the same for every thread of the grid
+    __syncthreads();
+    if (warp == kIssuerWarpA) tmem_dealloc(tmem_d, kTmemCols);
+    if (threadIdx.x == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
+    return;
+  }
+  // residual words of the CTA's blocks -> residual stages of 16 words, the first one starting at an even word
+  const int nres = rw1 > rw0 ? (int)((rw1 - (rw0 & ~1u) + 15u) / 16u) : 0;
+  const int nmain = 2 * max(b1 - b0, 0);               // 64-column stages of the blocks
+  const int nstage = nmain + nres;
 
-  if (warp == 0) {
+  if (warp >= kDecodeWarps) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGemmIssueRegs));
+  if (warp == kTmaWarp) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
+      uint32_t s = 0, ps = 0;
       for (int hb = 0; hb < nstage * kAcc; ++hb) {
-        const int it = hb / kAcc, a = hb % kAcc, s = hb % kStagesB;
-        if (!gemm_wait<true>(bar_emptyB + 8 * s, ((uint32_t)(hb / kStagesB) & 1u) ^ 1u, abort_flag)) break;
+        const int it = hb / kAcc, a = hb % kAcc;
+        if (!gemm_wait<true>(bar_emptyB + 8 * s, ps ^ 1u, abort_flag)) break;
         // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
         if (it == nmain && a == 0) grid_dependency_wait();
         mbar_expect_tx(bar_fullB + 8 * s, box_bytes);
-        const uint32_t dst = sbase + kGemmB + s * kStageB;
-        if (it < nmain) tma_load_2d(dst, &xmap, (b0 * 2 + it) * kBK, tt * kTok + a * kBN, bar_fullB + 8 * s);
-        else tma_load_2d(dst, &xsmap, (int)(4u * (rw0 & ~1u)) + (it - nmain) * kBK, tt * kTok + a * kBN, bar_fullB + 8 * s);
+        const uint32_t dst = sbase + L.b + s * L.box;
+        if (it < nmain) tma_load_2d(dst, &xmap, (b0 * 2 + it) * kBK, tt * ktok + a * bn, bar_fullB + 8 * s);
+        else tma_load_2d(dst, &xsmap, (int)(4u * (rw0 & ~1u)) + (it - nmain) * kBK, tt * ktok + a * bn, bar_fullB + 8 * s);
+        if (++s == L.nbox) { s = 0; ps ^= 1u; }
       }
       grid_dependency_wait();  // (every CTA, whether or not it had residual stages)
       if (*abort_flag) {       // let copies in flight land before the CTA gives its shared memory up
@@ -418,67 +487,71 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         while (clock64() - t0 < 200000) {}
       }
     }
-  } else if (warp == 1 || warp == kIssuerWarpB) {
+  } else if (warp == kIssuerWarpA || warp == kIssuerWarpB) {
     // ---------------- MMA issuers ----------------
     if (lane == 0) {
-      const int w = warp == 1 ? 0 : 1;
+      const int w = warp == kIssuerWarpA ? 0 : 1;
       // two accumulators: issuer w takes accumulator w (box w of every stage, all of K);
       // one accumulator:  issuer w takes the K steps 2 w, 2 w + 1 of every stage into accumulator w
       const uint32_t desc_hi = (uint32_t)(umma_desc(0u) >> 32);
-      const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + kGemmA) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
-      const uint32_t b_lo0 = (uint32_t)umma_desc(sbase + kGemmB) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
-      const uint32_t dt = tmem_d + (uint32_t)(w * (kAcc == 1 ? kTok : kBN));
+      const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + L.a) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
+      const uint32_t b_lo0 = (uint32_t)umma_desc(sbase + L.b) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
+      const uint32_t dt = tmem_d + (uint32_t)(w * kMaxBN), idesc = gemm_idesc(kF16, bn), box_lo = L.box >> 4, nbox = L.nbox;
       constexpr int kSteps = kAcc == 1 ? kBK / 32 : kBK / 16;           // MMAs per stage and issuer
-      int sa = 0, sb = kAcc == 1 ? 0 : w;                               // ring slots, advanced without divisions
+      uint32_t sa = 0, ea = 0, sb = kAcc == 1 ? 0u : (uint32_t)w;       // ring slots, advanced without divisions
       uint32_t pa = 0, pb = 0;                                          // their phase parities
       for (int it = 0; it < nstage; ++it) {
         if (!gemm_wait<true>(bar_fullA + 8 * sa, pa, abort_flag)) break;
         if (!gemm_wait<true>(bar_fullB + 8 * sb, pb, abort_flag)) break;
         tc_fence_after();
-        const uint32_t a_lo = a_lo0 + (uint32_t)sa * (kStageA >> 4), b_lo = b_lo0 + (uint32_t)sb * (kStageB >> 4);
-        if (it > 0) umma_16<true>(dt, a_lo, b_lo, desc_hi, kIdesc);
-        else umma_16<false>(dt, a_lo, b_lo, desc_hi, kIdesc);
+        const uint32_t a_lo = a_lo0 + sa * (kStageA >> 4), b_lo = b_lo0 + sb * box_lo;
+        if (it > 0) umma_16<true>(dt, a_lo, b_lo, desc_hi, idesc);
+        else umma_16<false>(dt, a_lo, b_lo, desc_hi, idesc);
 #pragma unroll
-        for (int kk = 1; kk < kSteps; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, kIdesc);
+        for (int kk = 1; kk < kSteps; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, idesc);
         umma_commit(bar_emptyB + 8 * sb);        // the box is free once the MMAs that read it have completed
-        umma_commit(bar_emptyA + 8 * sa);
+        umma_commit(bar_emptyA + 8 * ea);
         if (++sa == kStagesA) { sa = 0; pa ^= 1u; }
-        sb += kAcc == 1 ? 1 : kAcc;
-        if (sb >= kStagesB) { sb -= kStagesB; pb ^= 1u; }
+        if (++ea == kEmptyA) ea = 0;
+        sb += kAcc == 1 ? 1u : (uint32_t)kAcc;
+        if (sb >= nbox) { sb -= nbox; pb ^= 1u; }
       }
       umma_commit(bar_accum);                    // all MMAs this lane issued have completed
     }
-  } else {
+  } else if (warp < kDecodeWarps) {
     // ---------------- decode warps ----------------
-    const int gi = (warp - 2) >> 2;               // decode group: which of the lane's four rows this warp takes
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kGemmDecodeRegs));
+    const int gi = warp >> 2;               // decode group: which of the row tile's four warps this one is
     DecodeArgs da;
-    da.packed = packed; da.hdr = hdr; da.smem = smem; da.abort_flag = abort_flag;
+    da.packed = packed; da.smem = smem; da.abort_flag = abort_flag;
+    da.ptab = reinterpret_cast<const uint32_t*>(smem + kGemmTab); da.stages = smem + L.a; da.copies = L.copies;
     da.bar_full = bar_fullA; da.bar_empty = bar_emptyA;
-    da.mt = mt; da.b0 = b0; da.b1 = b1; da.nblk = nblk; da.ntile = ntile; da.q = warp & 3; da.lane = lane;
-    da.rw0 = rw0; da.rw1 = rw1; da.nres = nres;
-    decode_row<N, kF16>(da, gi);
+    da.mt = mt; da.b0 = b0; da.b1 = max(b1, b0); da.nblk = nblk; da.ntile = ntile; da.q = warp & 3; da.w = gi; da.lane = lane;
+    da.nrw = nrw; da.rw0 = rw0; da.rw1 = rw1; da.nres = nres;
+    decode_tiles<N, kF16>(da);
 
     // ---------------- epilogue: TMEM -> registers -> Y ----------------
     const int q = warp & 3;                        // TMEM lane quarter of this warp
     // A 16-bit output tile goes through shared memory (the X ring: every box has been consumed by then) so that it
     // leaves in 16-byte pieces along the rows: straight from the registers a warp's store is 32 rows x 2 bytes of
     // one token, and the epilogue took a ninth of the CTA's time.  The same for every thread of the CTA:
-    const bool staged = y_16 != 0 && !split && (ldy % 8) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0 &&
-                        (uint32_t)kTok * kBM * 2u <= (uint32_t)kStagesB * kStageB;
-    uint16_t* stage = reinterpret_cast<uint16_t*>(smem + kGemmB);           // [token of the tile][row of the tile]
+    const bool staged = y_16 != 0 && !split && (ldy % 8) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
+    uint16_t* stage = reinterpret_cast<uint16_t*>(smem + L.b);           // [token of the tile][row of the tile]
     const bool have = __all_sync(0xFFFFFFFFu, gemm_wait(bar_accum, 0u, abort_flag)) && nstage > 0;
     if (have) {
       tc_fence_after();
       const int row = mt * kBM + 32 * q + lane;                // output feature (row of W^)
-      float* wsz = split ? ws + ((size_t)(tile - full_tiles) * ksplit + kz) * (size_t)(kBM * kTok) : nullptr;
+      float* wsz = split ? ws + ((size_t)(tile - full_tiles) * ksplit + kz) * (size_t)(kBM * ktok) : nullptr;
+      const int chunks = (bn + 31) >> 5;                        // of 32 tokens, per accumulator
 #pragma unroll 1
-      for (int cc = gi; cc < kTok / 32; cc += kGroups) {       // the groups share the column chunks
+      for (int cc = gi; cc < kAcc * chunks; cc += kGroups) {    // the groups share the column chunks
+        const int acc = kAcc == 1 || cc < chunks ? 0 : 1, c0 = 32 * (cc - acc * chunks), live = bn - c0, tok0 = acc * bn + c0;
         uint32_t r[32];
-        tmem_ld32(tmem_d + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * cc), r);
+        tmem_ld32(tmem_d + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kMaxBN + c0), r);
         if (kAcc == 1) {
           // the other half of K sits in the second accumulator
           uint32_t r2[32];
-          tmem_ld32(tmem_d + ((uint32_t)(32 * q) << 16) + (uint32_t)(kTok + 32 * cc), r2);
+          tmem_ld32(tmem_d + ((uint32_t)(32 * q) << 16) + (uint32_t)(kMaxBN + c0), r2);
 #pragma unroll
           for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(r2[i]));
         }
@@ -486,15 +559,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const float v = __uint_as_float(r[i]);
-            stage[(32 * cc + i) * kBM + 32 * q + lane] = kF16 ? __half_as_ushort(__float2half_rn(v)) : __bfloat16_as_ushort(__float2bfloat16_rn(v));
+            if (i < live) stage[(tok0 + i) * kBM + 32 * q + lane] = kF16 ? __half_as_ushort(__float2half_rn(v)) : __bfloat16_as_ushort(__float2bfloat16_rn(v));
           }
         } else if (row < n) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const int tok = tt * kTok + 32 * cc + i;
-            if (tok < T) {
+            const int tok = tt * ktok + tok0 + i;
+            if (i < live && tok < T) {
               const float v = __uint_as_float(r[i]);
-              if (wsz) wsz[(size_t)(32 * cc + i) * kBM + 32 * q + lane] = v;
+              if (wsz) wsz[(size_t)(tok0 + i) * kBM + 32 * q + lane] = v;
               else if (y_16 && kF16) static_cast<__half*>(Y)[(size_t)tok * ldy + row] = __float2half_rn(v);
               else if (y_16) static_cast<__nv_bfloat16*>(Y)[(size_t)tok * ldy + row] = __float2bfloat16_rn(v);
               else static_cast<float*>(Y)[(size_t)tok * ldy + row] = v;
@@ -507,12 +580,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       // every decode warp takes the barrier, whatever its wait said
       asm volatile("bar.sync 1, %0;" ::"n"(128 * kGroups) : "memory");
       if (have) {
-        const int d = (warp - 2) * 32 + lane;                  // 0 .. 511: 16 threads per token, 8 rows each
+        const int d = warp * 32 + lane;                  // 0 .. 511: 16 threads per token, 8 rows each
         const int piece = d & 15, row0 = mt * kBM + 8 * piece;
         uint16_t* Y16 = static_cast<uint16_t*>(Y);
 #pragma unroll 4
-        for (int tl = d >> 4; tl < kTok; tl += (128 * kGroups) / 16) {
-          const int tok = tt * kTok + tl;
+        for (int tl = d >> 4; tl < ktok; tl += (128 * kGroups) / 16) {
+          const int tok = tt * ktok + tl;
           if (tok >= T) break;
           const uint4 v = *reinterpret_cast<const uint4*>(stage + tl * kBM + 8 * piece);
           uint16_t* dst = Y16 + (size_t)tok * ldy + row0;
@@ -531,10 +604,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   // The MMA thread makes sure the tensor core is done with TMEM before it is freed.  Its commit on bar_accum was
   // issued whether or not the loop above was left early, so this wait ends when the instructions issued so far
   // have completed; it keeps its own bound and ignores the abort flag.
-  if (warp == 1 && lane == 0) mbar_wait(bar_accum, 0u, kGemmWaitLimit);
+  if (warp == kIssuerWarpA && lane == 0) mbar_wait(bar_accum, 0u, kGemmWaitLimit);
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem_d, kTmemCols);
+  if (warp == kIssuerWarpA) tmem_dealloc(tmem_d, kTmemCols);
   if (threadIdx.x == 0 && *abort_flag && dev_status) *dev_status = STB_ERR_TIMEOUT;
 }
 
@@ -577,68 +650,82 @@ __global__ void gemm_reduce_kernel(const float* __restrict__ ws, int first_tile,
   }
 }
 
-// K split: only when the output tiles alone cannot fill the 148 SMs
-static int gemm_ksplit(int n, int m, int T, int ktok) {
-  const int tiles = ((n + kBM - 1) / kBM) * ((T + ktok - 1) / ktok), nblk = m / kBlock;
+// What stb_gemm_workspace[_min] promise for a shape, in tiles of 128 rows x `ktok` tokens: few output tiles are split along K
+// (mandatory), the tiles of a small last wave too (optional).  A call is laid out by gemm_plan below and never needs more.
+struct GemmBytes { size_t mandatory, preferred; };
+static GemmBytes gemm_bytes(int n, int m, int T, int ktok) {
+  const int nblk = m / kBlock, tiles = ((n + kBM - 1) / kBM) * ((T + ktok - 1) / ktok);
+  const size_t per = (size_t)kBM * ktok * sizeof(float);
+  auto parts = [&](int ks) { const int bps = (nblk + ks - 1) / ks; return (nblk + bps - 1) / bps; };
   int ks = 1;
   if (ktok < 512) {
-    // decode batch: a CTA's time is a fixed part (prologue, first loads, epilogue: measured about as long as the decode
-    // of seven blocks) plus the decode of its blocks, and the call takes as many such times as it has waves of 148
-    // CTAs: take the number of parts (at least four blocks each) with the smallest product
     double best = 0.0;
     for (int k = 1; k <= 16 && (k == 1 || nblk / k >= 4); ++k) {
-      const long long ctas = (long long)tiles * k, waves = (ctas + 147) / 148;
-      const double cost = (double)waves * (7.0 + (double)((nblk + k - 1) / k));
+      const double cost = (double)(((long long)tiles * k + 147) / 148) * (7.0 + (double)((nblk + k - 1) / k));
       if (k == 1 || cost < best - 1e-9) { best = cost; ks = k; }
     }
   } else {
     if (tiles < 100) ks = 148 / tiles;
     if (ks > 16) ks = 16;
     while (ks > 1 && nblk / ks < 4) --ks;
-    if (ks < 1) ks = 1;
   }
-  const int bps = (nblk + ks - 1) / ks;          // blocks per split; every split gets at least one
-  return (nblk + bps - 1) / bps;
-}
-
-// How a call is laid out on the 148 SMs (one CTA per SM at a time).
-//   few output tiles:   every tile is split along K (`ksplit` parts) into the workspace: mandatory
-//   many output tiles:  whole waves of 148 tiles run unsplit; a small last wave (at most half the SMs) would leave
-//                       the machine idle for a whole tile time, so its tiles are split along K as well, if the
-//                       caller's workspace holds their partial tiles: optional
-struct GemmPlan {
-  int ttiles, tiles, full_tiles, split_tiles, ksplit, bps;
-  size_t mandatory_bytes, preferred_bytes;
-};
-static GemmPlan gemm_plan(int n, int m, int T, int ktok, size_t ws_bytes, bool have_ws) {
-  GemmPlan p;
-  const int nblk = m / kBlock;
-  p.ttiles = (T + ktok - 1) / ktok;
-  p.tiles = ((n + kBM - 1) / kBM) * p.ttiles;
-  const size_t per = (size_t)kBM * ktok * sizeof(float);
-  const int ks = gemm_ksplit(n, m, T, ktok);
-  p.full_tiles = p.tiles; p.split_tiles = 0; p.ksplit = 1; p.bps = nblk;
-  p.mandatory_bytes = 0; p.preferred_bytes = 0;
-  if (ks > 1) {
-    p.full_tiles = 0; p.split_tiles = p.tiles; p.ksplit = ks; p.bps = (nblk + ks - 1) / ks;
-    p.mandatory_bytes = p.preferred_bytes = (size_t)p.tiles * ks * per;
-    return p;
-  }
-  const int tail = p.tiles % 148;
-  if (p.tiles > 148 && tail > 0 && tail <= 74) {
+  ks = parts(ks);
+  GemmBytes b = {0, 0};
+  if (ks > 1) { b.mandatory = b.preferred = (size_t)tiles * ks * per; return b; }
+  const int tail = tiles % 148;
+  if (tiles > 148 && tail > 0 && tail <= 74) {
     int kt = 148 / tail;
     if (kt > 16) kt = 16;
     while (kt > 1 && nblk / kt < 4) --kt;
-    if (kt > 1) {
-      const int bps = (nblk + kt - 1) / kt;
-      kt = (nblk + bps - 1) / bps;
-      p.preferred_bytes = (size_t)tail * kt * per;
-      if (have_ws && ws_bytes >= p.preferred_bytes) {
-        p.full_tiles = p.tiles - tail; p.split_tiles = tail; p.ksplit = kt; p.bps = bps;
+    if (kt > 1) b.preferred = (size_t)tail * parts(kt) * per;
+  }
+  return b;
+}
+
+// How a call is laid out on the 148 SMs (one CTA per SM at a time): the width of the token tiles (2 x bn or 1 x bn tokens, bn a
+// multiple of 16), and which tiles are split along K into how many parts -- all of them, or those of the last wave -- chosen
+// as the layout whose estimated time is smallest among those whose partial tiles fit `avail` bytes.  In SM clocks:
+//   a stage (64 of K):   the decode of two 32 x 128 tiles' worth of weights per row tile, or the tensor core's time for the
+//                        tile's tokens, whichever is longer (measured: FIGURE_DEC, and 2.25 per token + 30)
+//   a CTA besides:       prologue, first loads, drain (9000) and epilogue (6 per token)
+//   a split:             the second kernel, and its partial tiles written and read (2500 bytes per clock)
+struct GemmPlan {
+  int bn, ttiles, tiles, full_tiles, split_tiles, ksplit, bps;
+  size_t bytes;
+};
+static GemmPlan gemm_plan(int acc, int max_bn, int n, int m, int T, size_t avail) {
+  const int nblk = m / kBlock, rtiles = (n + kBM - 1) / kBM, most = acc * max_bn;
+  GemmPlan best = {};
+  double best_cost = 0.0;
+  for (int tt = (T + most - 1) / most, end = acc == 1 ? tt : tt + 8; tt <= end; ++tt) {
+    int bn = ((T + tt - 1) / tt + acc - 1) / acc;
+    bn = bn < 16 ? 16 : (bn + 15) / 16 * 16;
+    const int ktok = acc * bn;
+    if (bn > max_bn || (tt - 1) * ktok >= T) continue;
+    const long long tiles = (long long)rtiles * tt;
+    const double mma = 2.25 * ktok + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 9000.0 + 6.0 * ktok;
+    const size_t per = (size_t)kBM * ktok * sizeof(float);
+    auto consider = [&](long long full, int ks) {
+      const int bps = (nblk + ks - 1) / ks;
+      ks = (nblk + bps - 1) / bps;
+      const long long rest = tiles - full;
+      const size_t bytes = ks > 1 ? (size_t)rest * ks * per : 0;
+      if (bytes > avail) return;
+      double cost = (double)((full + 147) / 148) * (fixed + nblk * 2.13 * stage) + (double)((rest * ks + 147) / 148) * (fixed + bps * 2.13 * stage);
+      if (ks > 1) cost += 4000.0 + 2.0 * (double)bytes / 2500.0;
+      if (best.tiles == 0 || cost < best_cost * 0.999) {
+        best_cost = cost;
+        best.bn = bn; best.ttiles = tt; best.tiles = (int)tiles; best.full_tiles = (int)(ks > 1 ? full : tiles); best.split_tiles = (int)(ks > 1 ? rest : 0);
+        best.ksplit = ks; best.bps = bps; best.bytes = bytes;
       }
+    };
+    consider(tiles, 1);
+    for (int ks = 2; ks <= 16 && nblk / ks >= 4; ++ks) {
+      if (tiles < 148) consider(0, ks);
+      else if (tiles % 148) consider(tiles - tiles % 148, ks);
     }
   }
-  return p;
+  return best;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -659,22 +746,32 @@ static EncodeTiledFn encode_tiled_fn() {
 // slots a layer can have (32 per block), so that the size depends on the shape alone.
 static size_t gemm_xs_bytes(int m, int T) { return (((size_t)T * (size_t)(m / 4) * 2u) + 255u) & ~(size_t)255u; }
 
+// partial tiles a call of this shape would like room for
+template <class Cfg>
+static size_t gemm_preferred(int n, int m, int T) {
+  const size_t a = gemm_bytes(n, m, T, Cfg::kTok).preferred, b = gemm_plan(Cfg::kAcc, Cfg::kMaxBN, n, m, T, (size_t)-1).bytes;
+  return a > b ? a : b;
+}
+
 // y_16: 0 = fp32 output, 1 = the 16-bit type of the activations (bf16, or fp16 with kF16)
 template <int N, class Cfg, bool kF16>
 static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T, size_t ldx, void* Y, int y_16,
                        size_t ldy, void* ws, size_t ws_bytes, int* dev_status, cudaStream_t s) {
-  constexpr int kBN = Cfg::kBN, kTok = Cfg::kTok;
-  constexpr uint32_t kSmem = gemm_smem_bytes<Cfg>();
+  constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN;
   const size_t xs_bytes = gemm_xs_bytes(m, T);
   if (ws && (reinterpret_cast<uintptr_t>(ws) & 255u)) return STB_ERR_ARG;
   if (!ws || ws_bytes < xs_bytes) return STB_ERR_SIZE;
   float* ws_split = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + xs_bytes);
-  const GemmPlan plan = gemm_plan(n, m, T, kTok, ws_bytes - xs_bytes, true);
-  if (plan.mandatory_bytes > ws_bytes - xs_bytes) return STB_ERR_SIZE;
+  if (ws_bytes - xs_bytes < gemm_bytes(n, m, T, Cfg::kTok).mandatory) return STB_ERR_SIZE;
+  const size_t preferred = gemm_preferred<Cfg>(n, m, T);
+  const GemmPlan plan = gemm_plan(kAcc, kMaxBN, n, m, T, ws_bytes - xs_bytes < preferred ? ws_bytes - xs_bytes : preferred);
+  GemmShape shape;
+  shape.full_tiles = plan.full_tiles; shape.ksplit = plan.ksplit; shape.bps = plan.bps; shape.ttiles = plan.ttiles; shape.bn = plan.bn;
+  shape.smem = gemm_smem(kAcc, plan.bn);
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return STB_ERR_CUDA;
   const CUtensorMapDataType dt = kF16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  const cuuint32_t box_rows = (cuuint32_t)(T < kBN ? T : kBN);
+  const cuuint32_t box_rows = (cuuint32_t)(T < plan.bn ? T : plan.bn);
   const cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   CUtensorMap map, xsmap;
@@ -700,7 +797,7 @@ static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return STB_ERR_CUDA;
   if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-    if (cudaFuncSetAttribute(gemm_kernel<N, Cfg, kF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) != cudaSuccess) return STB_ERR_CUDA;
+    if (cudaFuncSetAttribute(gemm_kernel<N, Cfg, kF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) return STB_ERR_CUDA;
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
   // the gather moves 16-bit values: the same kernel serves bf16 and fp16
@@ -715,15 +812,15 @@ static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(plan.full_tiles + plan.split_tiles * plan.ksplit));
   cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.dynamicSmemBytes = shape.smem.total;
   cfg.stream = s;
   cfg.attrs = pdl; cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, gemm_kernel<N, Cfg, kF16>, map, xsmap, packed, n, m, T, Y, y_16, ldy, ws_split, plan.full_tiles,
-                         plan.ksplit, plan.bps, plan.ttiles, (uint32_t)(box_rows * kBK * 2), dev_status) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, gemm_kernel<N, Cfg, kF16>, map, xsmap, packed, n, m, T, Y, y_16, ldy, ws_split, shape,
+                         (uint32_t)(box_rows * kBK * 2), dev_status) != cudaSuccess)
     return STB_ERR_CUDA;
   if (plan.split_tiles > 0) {
     gemm_reduce_kernel<<<148 * 4, 256, 0, s>>>(ws_split, plan.full_tiles, plan.split_tiles, plan.ksplit,
-                                               plan.ttiles, kTok, n, T, Y, y_16 ? (kF16 ? 2 : 1) : 0, ldy);
+                                               plan.ttiles, kAcc * plan.bn, n, T, Y, y_16 ? (kF16 ? 2 : 1) : 0, ldy);
     if (cudaGetLastError() != cudaSuccess) return STB_ERR_CUDA;
   }
   return STB_OK;
@@ -731,8 +828,6 @@ static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T
 
 using PrefillCfg = TokCfg<2, 256>;
 using BatchCfg = TokCfg<1, 64>;
-// fp16 activations: up to 64 tokens take the small token tile
-static int ktok_f16(int T) { return T <= BatchCfg::kTok ? BatchCfg::kTok : PrefillCfg::kTok; }
 
 template <bool kF16>
 static int launch_gemm_n(int N, const uint8_t* packed, int n, int m, const void* X, int T, size_t ldx, void* Y, int y_16,
@@ -753,18 +848,20 @@ static int launch_gemm_n(int N, const uint8_t* packed, int n, int m, const void*
 
 }  // namespace stb
 
-static int gemm_workspace_impl(int n, int m, int N, int T, int ktok, size_t* bytes, bool minimum) {
+template <class Cfg>
+static int gemm_workspace_impl(int n, int m, int N, int T, size_t* bytes, bool minimum) {
   if (!bytes) return STB_ERR_ARG;
   if (n < 1 || m < stb::kBlock || m % stb::kBlock != 0 || T < 1) return STB_ERR_SHAPE;
   if (N < 1 || N > 8) return STB_ERR_NM;
-  const stb::GemmPlan plan = stb::gemm_plan(n, m, T, ktok, 0, false);
-  *bytes = stb::gemm_xs_bytes(m, T) + (minimum ? plan.mandatory_bytes : plan.preferred_bytes);
+  *bytes = stb::gemm_xs_bytes(m, T) + (minimum ? stb::gemm_bytes(n, m, T, Cfg::kTok).mandatory : stb::gemm_preferred<Cfg>(n, m, T));
   return STB_OK;
 }
 
-extern "C" int stb_gemm_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::PrefillCfg::kTok, bytes, false); }
-extern "C" int stb_gemm_workspace_min(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::PrefillCfg::kTok, bytes, true); }
-extern "C" int stb_gemm_f16_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::ktok_f16(T), bytes, false); }
+extern "C" int stb_gemm_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, false); }
+extern "C" int stb_gemm_workspace_min(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, true); }
+extern "C" int stb_gemm_f16_workspace(int n, int m, int N, int T, size_t* bytes) {
+  return T <= stb::BatchCfg::kTok ? gemm_workspace_impl<stb::BatchCfg>(n, m, N, T, bytes, false) : gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, false);
+}
 
 static int gemm_check_args(const void* packed, int n, int m, int N, const void* X, int T, size_t ldx, void* Y, size_t ldy) {
   if (!packed || !X || !Y) return STB_ERR_ARG;
@@ -813,7 +910,7 @@ extern "C" int stb_gemm_noalloc(const void* packed, int n, int m, int N, const v
   if (ydt != STB_F32 && ydt != STB_BF16) return STB_ERR_UNSUPPORTED;
   if (ldx < (size_t)m || ldy < (size_t)n || (ldx % 8) != 0 || (reinterpret_cast<uintptr_t>(X) & 15u)) return STB_ERR_ARG;
   // this shape needs the caller-workspace entry point if the scratch it cannot do without does not fit
-  if (stb::gemm_xs_bytes(m, T) + stb::gemm_plan(n, m, T, stb::PrefillCfg::kTok, 0, false).mandatory_bytes > stb::kNoAllocScratchBytes) return STB_ERR_SIZE;
+  if (stb::gemm_xs_bytes(m, T) + stb::gemm_bytes(n, m, T, stb::PrefillCfg::kTok).mandatory > stb::kNoAllocScratchBytes) return STB_ERR_SIZE;
   // The array's name is only a host-side handle: ask the runtime for its address on the current
   // device, once per device, and give the kernels that address.
   static float* scratch_of_device[64] = {nullptr};

@@ -12,7 +12,7 @@
 //   warps 0..15 decode: see below
 //   warp 16     TMA producer (one lane): X slices
 //   warp 17, 18 MMA issuers (one lane each, on two schedulers): with two accumulators each takes one (4 x tcgen05.mma,
-//               K = 16, per stage); with one, each takes half of a stage's K into an accumulator of its own and the
+//               K = 16, per stage); with one, each takes every other stage into an accumulator of its own and the
 //               epilogue adds the two.  tcgen05.commit frees the boxes and stages; warp 17 allocates / frees TMEM
 //   decode:     warp w works on rows 32 (w % 4) .. +31 of the tile = one packed row tile; four warps share a row
 //               tile, each taking every fourth block: it loads the block's words with vector loads (its next block ahead),
@@ -64,9 +64,10 @@ constexpr uint32_t kStageA = kBM * kBK * 2;      // 16 KB
 // "A stage empty" has twice as many barriers as there are stages: a decode warp writes the stages it = 2 w, 2 w + 1 (mod 8),
 // so it meets every phase of the barriers (it - 4) mod 8 that it waits on, one after the other.
 constexpr int kEmptyA = 2 * kStagesA;
-static_assert(kEmptyA == 2 * kGroups, "the warp of a stage is (stage / 2) mod kGroups");
+static_assert(kEmptyA == 2 * kGroups && kStagesA == 4, "the warp of a stage is (stage / 2) mod kGroups");
 constexpr uint32_t kGemmBars = 0;                                  // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
-constexpr uint32_t kGemmTab = 512;                                 // position table, 4 bytes per entry and copy
+constexpr uint32_t kGemmTab = 512;                                 // position table, 8 bytes per entry and copy
+static_assert(kMaxStagesB == kEmptyA, "one accumulator: boxes and stages are freed by the same barriers");
 static_assert(8 * (kStagesA + kEmptyA + 2 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
 constexpr uint32_t kSmemMax = 232448;
 constexpr double kDecodeClocks = 420.0;    // decode of a stage (gemm_plan)
@@ -77,12 +78,12 @@ __host__ __device__ inline GemmSmem gemm_smem(int kAcc, int bn) {
   GemmSmem g;
   g.box = (uint32_t)bn * kBK * 2;
   for (g.copies = 16;; g.copies = 1) {
-    g.a = (kGemmTab + 4u * kPosTableEntries * g.copies + 1023u) & ~1023u;
+    g.a = (kGemmTab + 8u * kPosTableEntries * g.copies + 1023u) & ~1023u;
     g.b = g.a + kStagesA * kStageA;
     g.nbox = (kSmemMax - g.b) / g.box;
     if (g.nbox >= 5u || g.copies == 1u) break;
   }
-  if (g.nbox > (uint32_t)kMaxStagesB) g.nbox = kMaxStagesB;
+  if (g.nbox > (uint32_t)kMaxStagesB) g.nbox = kMaxStagesB;      // (one accumulator: always eight, as many as there are "stage empty" barriers)
   g.total = g.b + g.nbox * g.box;
   // a 16-bit output tile is staged where the boxes were
   const uint32_t out = (uint32_t)(kAcc * bn) * kBM * 2u;
@@ -106,9 +107,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // The descriptors come as their low words (start address / 16; the high word is the same for every operand tile of
-// this kernel) and the accumulate flag as a template argument: an issuing lane is ONE thread whose instructions go
-// out one dependent step at a time, and what it runs per stage of K (waits, descriptors, MMAs, commits) was longer
-// than the tensor core needs for the stage.
+// this kernel) and the accumulate flag as a template argument: what an issuing lane runs per stage of K (waits,
+// descriptors, MMAs, commits) must stay shorter than the tensor core needs for the stage.
 template <bool kAccumulate>
 __device__ __forceinline__ void umma_16(uint32_t d_tmem, uint32_t adesc_lo, uint32_t bdesc_lo, uint32_t desc_hi, uint32_t idesc) {
   if (kAccumulate)
@@ -119,6 +119,11 @@ __device__ __forceinline__ void umma_16(uint32_t d_tmem, uint32_t adesc_lo, uint
     asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, 0, 0;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
                  ::"r"(d_tmem), "r"(adesc_lo), "r"(bdesc_lo), "r"(desc_hi), "r"(idesc) : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 r;\n\telect.sync r|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -180,11 +185,20 @@ __device__ __forceinline__ void scales_to_bf16(uint32_t& A, uint32_t& B) {
   B = prmt(u01, u23, 0x7531u);
 }
 
+__device__ __forceinline__ void sts_v4(uint32_t a, const uint32_t (&v)[4]) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ uint2 lds_v2(uint32_t a) {            // (of the position table: written before the roles part, never changed)
+  uint2 v;
+  asm("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+
 // What a decode warp needs to know.
 struct DecodeArgs {
-  const uint8_t* packed; uint8_t* smem; volatile int* abort_flag;
-  const uint32_t* ptab; uint8_t* stages;
-  uint32_t bar_full, bar_empty, copies;      // of the A ring; copies of the position table
+  const uint8_t* packed; volatile int* abort_flag;
+  uint32_t ptab, entry, stages;              // shared-memory addresses of the position table (bytes per entry of it) and the A stages
+  uint32_t bar_full, bar_empty;              // of the A ring
   int mt, b0, b1, nblk, ntile, q, w, lane;   // q: row tile of the CTA's four, w: which of the row tile's four warps
   uint32_t nrw, rw0, rw1;   // residual words of a row tile, and of the blocks [b0, b1)
   int nres;                 // residual stages (64 slots = 16 words each, the first one starts at word rw0 & ~1)
@@ -213,8 +227,7 @@ __device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, Ge
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
 template <int N, bool kF16>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
-  volatile int* abort_flag = da.abort_flag;
-  const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1;
+  const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1, w = da.w;
   // The lane plays the part of packed-layout lane 4 g + t with g = lane % 8, t = lane / 8: the eight
   // lanes of a quarter-warp then hold eight different rows g and their 16-byte stores into the
   // swizzled stage fall on eight different 16-byte bank groups (no conflict); loads of the
@@ -222,104 +235,108 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   const int g = da.lane & 7, t = da.lane >> 3;
   const int lane = 4 * g + t;
   const int rtile = da.mt * 4 + q;                 // packed row tile
-  const bool live = rtile < da.ntile;
-  const uint32_t* ptab = da.ptab + (uint32_t)da.lane % da.copies;
-  const uint8_t* rtbase = da.packed + tiles_offset(nblk) + (size_t)rtile * tile_bytes(N) * nblk;
-  const uint8_t* resid_rt = da.packed + tiles_offset(nblk) + (size_t)tile_bytes(N) * nblk * da.ntile + (size_t)rtile * resid_rt_bytes(nblk, da.nrw);
   constexpr uint32_t tbytes = tile_bytes(N);
-  // where the lane's two 16-byte chunks (4 sl + t) of its row g go inside a stage's eight rows
-  const uint32_t off0 = (uint32_t)g * 128u + (uint32_t)((t ^ g) << 4), off1 = (uint32_t)g * 128u + (uint32_t)(((4 + t) ^ g) << 4);
-  uint8_t* rows = da.stages + (size_t)(4 * q) * 1024;
-  // wait for stage `it`; the verdict is made warp-uniform: nobody may be left alone at the __syncwarp() below
-  auto stage_wait = [&](int it) {
-    const uint32_t bar = da.bar_empty + 8u * (uint32_t)((it + kEmptyA - kStagesA) % kEmptyA);
-    return it < kStagesA || __all_sync(0xFFFFFFFFu, gemm_wait(bar, (uint32_t)((it - kStagesA) / kEmptyA) & 1u, abort_flag));
+  const int nmain = 2 * (b1 - b0), nstage = nmain + da.nres;
+  // Stage `it` belongs to warp (it / 2) mod 4: the stages 2 w + h (mod 8) with h = 0, 1, so that slot, barriers and the place
+  // of the lane's two 16-byte chunks (4 sl + t of its row g) in the slot are the same every time; only the parity changes.
+  const uint32_t row_at = da.stages + (uint32_t)((2 * w) % kStagesA) * kStageA + (uint32_t)q * 4096u + (uint32_t)g * 128u;
+  const uint32_t at0 = row_at + (uint32_t)((t ^ g) << 4), at1 = row_at + (uint32_t)(((4 + t) ^ g) << 4);
+  const uint32_t full = da.bar_full + 8u * (uint32_t)((2 * w) % kStagesA), empty = da.bar_empty + 8u * (uint32_t)((2 * w + kEmptyA - kStagesA) % kEmptyA);
+  // before stage `it` is written, stage it - 4 must have been read: use it / 8 of the slot pair waits for that barrier's phase
+  // it / 8 (w >= 2) or it / 8 - 1 (w < 2: nothing to wait for the first time).  The verdict is made warp-uniform.
+  const uint32_t early = w < 2 ? 1u : 0u;
+  auto stage_wait = [&](uint32_t use, int h) -> bool {
+    if (use < early) return true;
+    const uint32_t parity = (use - early) & 1u;
+    return __all_sync(0xFFFFFFFFu, mbar_try_wait(empty + 8u * h, parity)) || __all_sync(0xFFFFFFFFu, gemm_wait(empty + 8u * h, parity, da.abort_flag));
   };
-  auto stage_done = [&](int it) {
+  auto stage_done = [&](int h) {
     fence_async_smem();          // generic-proxy writes -> visible to the tensor core
     __syncwarp();
-    if (lane == 0) mbar_arrive(da.bar_full + 8 * (it % kStagesA));
+    if (da.lane == 0) mbar_arrive(full + 8u * h);
   };
+  auto next_mine = [&](int it) { while (it < nstage && ((it >> 1) & (kGroups - 1)) != w) ++it; return it; };
+  if (rtile >= da.ntile) {       // no such rows: zeros
+    const uint32_t z[4] = {0, 0, 0, 0};
+#pragma unroll 1
+    for (int it = next_mine(0); it < nstage; it = next_mine(it + 1)) {
+      if (!stage_wait((uint32_t)it / kEmptyA, it & 1)) return;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { sts_v4(at0 + (uint32_t)(it & 1) * kStageA + 1024u * j, z); sts_v4(at1 + (uint32_t)(it & 1) * kStageA + 1024u * j, z); }
+      stage_done(it & 1);
+    }
+    return;
+  }
+  const uint8_t* rtbase = da.packed + tiles_offset(nblk) + (size_t)rtile * tbytes * nblk;
+  const uint8_t* resid_rt = da.packed + tiles_offset(nblk) + (size_t)tbytes * nblk * da.ntile + (size_t)rtile * resid_rt_bytes(nblk, da.nrw);
   // Residual stages come after the blocks: 64 residual slots (16 residual words) of K each.  The lane writes the same
   // two 16-byte chunks of its rows: chunk c holds the words 2 c and 2 c + 1 of the stage, four slots each, as
   // +-bf16(a_sal2) or 0.  What a stage needs sits behind two dependent loads from global memory (the word's table
   // entry, then a_sal2 and the codes from the block's record); the entries of the warp's first one are asked for here.
   const ResidWord* rwt = reinterpret_cast<const ResidWord*>(da.packed + rwtab_offset(nblk));
   const uint32_t wfirst = da.rw0 & ~1u;
-  const int nmain = 2 * (b1 - b0), nstage = nmain + da.nres;
-  auto mine = [&](int it) { return ((it >> 1) & (kGroups - 1)) == da.w; };
-  auto next_res = [&](int it) { while (it < nstage && !mine(it)) ++it; return it; };
   auto res_word = [&](int it, int idx) { return wfirst + 16u * (uint32_t)(it - nmain) + 2u * (uint32_t)(4 * (idx >> 1) + t) + (uint32_t)(idx & 1); };
   uint2 e[4];
   auto res_entries = [&](int it) {
 #pragma unroll
     for (int idx = 0; idx < 4; ++idx) {
-      const uint32_t w = res_word(it, idx);
+      const uint32_t wd = res_word(it, idx);
       e[idx] = make_uint2(0xFFFFFFFFu, 0u);
-      if (live && it < nstage && w >= da.rw0 && w < da.rw1) e[idx] = __ldg(reinterpret_cast<const uint2*>(rwt + w));
+      if (it < nstage && wd >= da.rw0 && wd < da.rw1) e[idx] = __ldg(reinterpret_cast<const uint2*>(rwt + wd));
     }
   };
-  int rit = next_res(nmain);
+  int rit = next_mine(nmain);
   GemmTile<N> nxt;
-  int b = b0 + da.w;
-  if (live && b < b1) load_gemm_tile<N>(rtbase + (size_t)b * tbytes, lane, nxt);
+  if (b0 + w < b1) load_gemm_tile<N>(rtbase + (size_t)(b0 + w) * tbytes, lane, nxt);
   res_entries(rit);
+  uint32_t use = 0;
 #pragma unroll 1
-  for (; b < b1; b += kGroups) {
+  for (int b = b0 + w; b < b1; b += kGroups, ++use) {
     uint32_t mask[4] = {0, 0, 0, 0};                   // word j, byte s: keep-mask index of slot (j, s)
+    if constexpr (mask_pairs(N)) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {                    // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)
+        const uint32_t J = nxt.fld[k] >> 4, i1 = (J * 2341u) >> 16, i0 = J - kMasks6 * i1;      // (pair_field_index)
+        mask[2 * (k >> 2)] = i0 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2)];
+        mask[2 * (k >> 2) + 1] = i1 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2) + 1];
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mask[j] = nxt.lt.mask[j];
+    }
+    uint32_t A[4], B[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      A[j] = nxt.lt.A[j]; B[j] = nxt.lt.B[j];
+      // (a salient weight gets s1 bf16(a_sal1) here; its residual term comes with the residual stages)
+      if (!kF16) scales_to_bf16(A[j], B[j]);
+    }
     FastRows<N> fr;
+    fr.init(nxt.lt, A, B);
+    if (b + kGroups < b1) load_gemm_tile<N>(rtbase + (size_t)(b + kGroups) * tbytes, lane, nxt);
     uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
-    if (live) {
-      if constexpr (mask_pairs(N)) {
+    if (N == 5) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {                  // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)
-          const uint32_t J = nxt.fld[k] >> 4, i1 = (J * 2341u) >> 16, i0 = J - kMasks6 * i1;      // (pair_field_index)
-          mask[2 * (k >> 2)] = i0 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2)];
-          mask[2 * (k >> 2) + 1] = i1 * (1u << (8 * (k & 3))) + mask[2 * (k >> 2) + 1];
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) mask[j] = nxt.lt.mask[j];
-      }
-      uint32_t A[4], B[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        A[j] = nxt.lt.A[j]; B[j] = nxt.lt.B[j];
-        // (a salient weight gets s1 bf16(a_sal1) here; its residual term comes with the residual stages)
-        if (!kF16) scales_to_bf16(A[j], B[j]);
-      }
-      fr.init(nxt.lt, A, B);
-      if (N == 5) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) fr.high(j, 0, XL[j], XH[j]);
-      }
-      if (b + kGroups < b1) load_gemm_tile<N>(rtbase + (size_t)(b + kGroups) * tbytes, lane, nxt);
+      for (int j = 0; j < 4; ++j) fr.high(j, 0, XL[j], XH[j]);
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int it = 2 * (b - b0) + h;
+      uint2 P[4][2];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int sl = 0; sl < 2; ++sl) P[j][sl] = lds_v2(keep_index_of(mask, j, 2 * h + sl) * da.entry + da.ptab);
       uint32_t f[4][2][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (N == 6 && live) fr.high(j, h, XL[j], XH[j]);
+        if (N == 6) fr.high(j, h, XL[j], XH[j]);
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl) {
-          const int sidx = 2 * h + sl;                       // slot s of the block, group 4 sidx + t
-          f[j][sl][0] = f[j][sl][1] = f[j][sl][2] = f[j][sl][3] = 0;
-          if (live) {
-            const uint32_t P = ptab[keep_index_of(mask, j, sidx) * da.copies];
-            fr.slot2(j, sidx, P, P >> 16, XL[j], XH[j], f[j][sl]);
-          }
-        }
+        for (int sl = 0; sl < 2; ++sl) fr.slot2(j, 2 * h + sl, P[j][sl].x, P[j][sl].y, XL[j], XH[j], f[j][sl]);      // group 4 s + t
       }
-      if (!stage_wait(it)) return;
-      uint8_t* st = rows + (size_t)(it % kStagesA) * kStageA;
+      if (!stage_wait(use, h)) return;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        *reinterpret_cast<uint4*>(st + 1024 * j + off0) = make_uint4(f[j][0][0], f[j][0][1], f[j][0][2], f[j][0][3]);
-        *reinterpret_cast<uint4*>(st + 1024 * j + off1) = make_uint4(f[j][1][0], f[j][1][1], f[j][1][2], f[j][1][3]);
-      }
-      stage_done(it);
+      for (int j = 0; j < 4; ++j) { sts_v4(at0 + h * kStageA + 1024u * j, f[j][0]); sts_v4(at1 + h * kStageA + 1024u * j, f[j][1]); }
+      stage_done(h);
     }
   }
 #pragma unroll 1
@@ -336,10 +353,10 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
       }
     }
     const int it = rit;
-    rit = next_res(it + 1);
+    rit = next_mine(it + 1);
     res_entries(rit);
-    if (!stage_wait(it)) return;
-    uint8_t* st = rows + (size_t)(it % kStagesA) * kStageA;
+    if (!stage_wait((uint32_t)it / kEmptyA, it & 1)) return;
+    const uint32_t shift = (uint32_t)(it & 1) * kStageA;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       uint32_t f[2][4];
@@ -354,10 +371,10 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
         f[idx >> 1][2 * (idx & 1)] = prmt(lo4, hi4, 0x5140u);
         f[idx >> 1][2 * (idx & 1) + 1] = prmt(lo4, hi4, 0x7362u);
       }
-      *reinterpret_cast<uint4*>(st + 1024 * j + off0) = make_uint4(f[0][0], f[0][1], f[0][2], f[0][3]);
-      *reinterpret_cast<uint4*>(st + 1024 * j + off1) = make_uint4(f[1][0], f[1][1], f[1][2], f[1][3]);
+      sts_v4(at0 + shift + 1024u * j, f[0]);
+      sts_v4(at1 + shift + 1024u * j, f[1]);
     }
-    stage_done(it);
+    stage_done(it & 1);
   }
 }
 
@@ -435,19 +452,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kGemmBars + kBarBytes + 8);
 
   if (threadIdx.x == 0) {
-    // a stage of A is read by both issuers; an X box by the issuer of its accumulator (by both when there is one box per stage)
+    // a stage of A is read by both issuers (with one accumulator by one of them), an X box by the issuer of its accumulator
     for (int i = 0; i < kStagesA; ++i) mbar_init(bar_fullA + 8 * i, 4);
-    for (int i = 0; i < kEmptyA; ++i) mbar_init(bar_emptyA + 8 * i, kIssuers);
-    for (int i = 0; i < kMaxStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, kAcc == 1 ? kIssuers : 1); }
+    for (int i = 0; i < kEmptyA; ++i) mbar_init(bar_emptyA + 8 * i, kAcc == 1 ? 1 : kIssuers);
+    for (int i = 0; i < kMaxStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, 1); }
     mbar_init(bar_accum, kIssuers);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads) {
-    const uint2 v = g_pos_table.v[N][i / L.copies];
-    reinterpret_cast<uint32_t*>(smem + kGemmTab)[i] = v.x | (v.y << 16);
-  }
+  for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads)
+    reinterpret_cast<uint2*>(smem + kGemmTab)[i] = g_pos_table.v[N][L.copies == 1u ? i : i >> 4];
   constexpr uint32_t kTmemCols = kAcc == 1 ? 2 * kMaxBN : kAcc * kMaxBN;      // one accumulator: a second one for the other half of K
   if (warp == kIssuerWarpA) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   tc_fence_before();
@@ -472,7 +487,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       uint32_t s = 0, ps = 0;
       for (int hb = 0; hb < nstage * kAcc; ++hb) {
         const int it = hb / kAcc, a = hb % kAcc;
-        if (!gemm_wait<true>(bar_emptyB + 8 * s, ps ^ 1u, abort_flag)) break;
+        // (one accumulator: box s goes with the stages s, s + 8, .. and is freed with them)
+        if (!gemm_wait<true>((kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * s, ps ^ 1u, abort_flag)) break;
         // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
         if (it == nmain && a == 0) grid_dependency_wait();
         mbar_expect_tx(bar_fullB + 8 * s, box_bytes);
@@ -489,42 +505,53 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     }
   } else if (warp == kIssuerWarpA || warp == kIssuerWarpB) {
     // ---------------- MMA issuers ----------------
-    if (lane == 0) {
-      const int w = warp == kIssuerWarpA ? 0 : 1;
-      // two accumulators: issuer w takes accumulator w (box w of every stage, all of K);
-      // one accumulator:  issuer w takes the K steps 2 w, 2 w + 1 of every stage into accumulator w
-      const uint32_t desc_hi = (uint32_t)(umma_desc(0u) >> 32);
-      const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + L.a) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
-      const uint32_t b_lo0 = (uint32_t)umma_desc(sbase + L.b) + (kAcc == 1 ? 4u * (uint32_t)w : 0u);
-      const uint32_t dt = tmem_d + (uint32_t)(w * kMaxBN), idesc = gemm_idesc(kF16, bn), box_lo = L.box >> 4, nbox = L.nbox;
-      constexpr int kSteps = kAcc == 1 ? kBK / 32 : kBK / 16;           // MMAs per stage and issuer
-      uint32_t sa = 0, ea = 0, sb = kAcc == 1 ? 0u : (uint32_t)w;       // ring slots, advanced without divisions
-      uint32_t pa = 0, pb = 0;                                          // their phase parities
-      for (int it = 0; it < nstage; ++it) {
-        if (!gemm_wait<true>(bar_fullA + 8 * sa, pa, abort_flag)) break;
-        if (!gemm_wait<true>(bar_fullB + 8 * sb, pb, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t a_lo = a_lo0 + sa * (kStageA >> 4), b_lo = b_lo0 + sb * box_lo;
-        if (it > 0) umma_16<true>(dt, a_lo, b_lo, desc_hi, idesc);
+    // The whole warp runs the loop and one elected lane issues: every operand is then warp-uniform to the compiler and sits in
+    // uniform registers, where tcgen05 instructions take them (under `lane == 0` each was moved there one by one: an
+    // issuer's stage took 850 clocks at 64 tokens, 600 of them its own instructions; now FIGURE_ISSUE).
+    const int w = __shfl_sync(0xFFFFFFFFu, warp == kIssuerWarpA ? 0 : 1, 0);
+    const uint32_t tmem_u = __shfl_sync(0xFFFFFFFFu, tmem_d, 0);
+    const bool leader = elect_one();
+    // two accumulators: issuer w takes accumulator w (box w of every stage);
+    // one accumulator:  issuer w takes the stages 2 i + w into an accumulator of its own
+    constexpr int kStep = kAcc == 1 ? kIssuers : 1;
+    const uint32_t desc_hi = (uint32_t)(umma_desc(0u) >> 32);
+    const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + L.a), b_lo0 = (uint32_t)umma_desc(sbase + L.b);
+    const uint32_t dt = tmem_u + (uint32_t)(w * kMaxBN), idesc = gemm_idesc(kF16, bn), box_lo = L.box >> 4, nbox = L.nbox;
+    uint32_t sa = kAcc == 1 ? (uint32_t)w : 0u, ea = sa, sb = (uint32_t)w;      // ring slots, advanced without divisions
+    uint32_t pa = 0, pb = 0;                                                    // their phase parities
+    for (int it = kAcc == 1 ? w : 0; it < nstage; it += kStep) {
+      const bool ra = mbar_try_wait(bar_fullA + 8 * sa, pa), rb = mbar_try_wait(bar_fullB + 8 * sb, pb);     // both at once
+      bool ok = true;
+      if (!ra) ok = gemm_wait<true>(bar_fullA + 8 * sa, pa, abort_flag);
+      if (!rb && ok) ok = gemm_wait<true>(bar_fullB + 8 * sb, pb, abort_flag);
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      tc_fence_after();
+      const uint32_t a_lo = a_lo0 + sa * (kStageA >> 4), b_lo = b_lo0 + sb * box_lo;
+      if (leader) {
+        if (it >= kStep) umma_16<true>(dt, a_lo, b_lo, desc_hi, idesc);
         else umma_16<false>(dt, a_lo, b_lo, desc_hi, idesc);
 #pragma unroll
-        for (int kk = 1; kk < kSteps; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, idesc);
-        umma_commit(bar_emptyB + 8 * sb);        // the box is free once the MMAs that read it have completed
-        umma_commit(bar_emptyA + 8 * ea);
-        if (++sa == kStagesA) { sa = 0; pa ^= 1u; }
-        if (++ea == kEmptyA) ea = 0;
-        sb += kAcc == 1 ? 1u : (uint32_t)kAcc;
-        if (sb >= nbox) { sb -= nbox; pb ^= 1u; }
+        for (int kk = 1; kk < kBK / 16; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, idesc);
+        if (kAcc > 1) umma_commit(bar_emptyB + 8 * sb);        // the box is free once the MMAs that read it have completed
+        umma_commit(bar_emptyA + 8 * ea);                      // (one accumulator: the box of a stage is freed with it)
       }
-      umma_commit(bar_accum);                    // all MMAs this lane issued have completed
+      __syncwarp();
+      sa += kStep;
+      if (sa >= kStagesA) { sa -= kStagesA; pa ^= 1u; }
+      ea += kStep;
+      if (ea >= kEmptyA) ea -= kEmptyA;
+      sb += kAcc == 1 ? kStep : kAcc;
+      if (sb >= nbox) { sb -= nbox; pb ^= 1u; }
     }
+    if (leader) umma_commit(bar_accum);                        // all MMAs this warp issued have completed
+    __syncwarp();
   } else if (warp < kDecodeWarps) {
     // ---------------- decode warps ----------------
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kGemmDecodeRegs));
     const int gi = warp >> 2;               // decode group: which of the row tile's four warps this one is
     DecodeArgs da;
-    da.packed = packed; da.smem = smem; da.abort_flag = abort_flag;
-    da.ptab = reinterpret_cast<const uint32_t*>(smem + kGemmTab); da.stages = smem + L.a; da.copies = L.copies;
+    da.packed = packed; da.abort_flag = abort_flag;
+    da.entry = 8u * L.copies; da.ptab = sbase + kGemmTab + 8u * ((uint32_t)lane & (L.copies - 1u)); da.stages = sbase + L.a;
     da.bar_full = bar_fullA; da.bar_empty = bar_emptyA;
     da.mt = mt; da.b0 = b0; da.b1 = max(b1, b0); da.nblk = nblk; da.ntile = ntile; da.q = warp & 3; da.w = gi; da.lane = lane;
     da.nrw = nrw; da.rw0 = rw0; da.rw1 = rw1; da.nres = nres;

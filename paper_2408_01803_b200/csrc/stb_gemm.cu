@@ -47,9 +47,13 @@ constexpr int kBM = 128;          // rows of W^ per CTA (UMMA M)
 // columns; a decoded A stage is used twice).  Up to 64 tokens (a decode batch): 1 x up to 64, the tensor core then takes an
 // eighth of the time per stage and the kernel runs at the speed of the decode warps.
 template <int kAcc_, int kMaxBN_>
-struct TokCfg { static constexpr int kAcc = kAcc_, kMaxBN = kMaxBN_, kTok = kAcc_ * kMaxBN_; };
+struct TokCfg {
+  static constexpr int kAcc = kAcc_, kMaxBN = kMaxBN_, kTok = kAcc_ * kMaxBN_;
+  // ring of decoded A stages (16 KB each): four beside the wide X boxes, eight beside the narrow ones (a stage's way round
+  // -- written, multiplied, freed, seen -- takes about 2000 clocks, four decodes of a decode batch's stage)
+  static constexpr int kStagesA = kAcc_ == 1 ? 8 : 4;
+};
 constexpr int kBK = 64;           // K per stage: one 128-byte swizzle row of bf16
-constexpr int kStagesA = 4;        // ring of decoded A stages (16 KB each)
 constexpr int kMaxStagesB = 8;    // ring of X boxes: as many as fit, up to eight (five of 256 tokens x 64 of K = 32 KB): what is in
                                   // flight from L2 is what hides its latency; a stage of K takes kAcc of them
 constexpr int kGroups = 4;                              // decode warps per 32-row quarter: each takes every fourth block
@@ -61,14 +65,14 @@ constexpr int kGemmThreads = 32 * kDecodeWarps + 128;
 constexpr int kGemmDecodeRegs = 104, kGemmIssueRegs = 64;
 static_assert(32 * kDecodeWarps * kGemmDecodeRegs + 128 * kGemmIssueRegs <= kGemmThreads * 96, "register split within the launch's total");
 constexpr uint32_t kStageA = kBM * kBK * 2;      // 16 KB
-// "A stage empty" has twice as many barriers as there are stages: a decode warp writes the stages it = 2 w, 2 w + 1 (mod 8),
-// so it meets every phase of the barriers (it - 4) mod 8 that it waits on, one after the other.
-constexpr int kEmptyA = 2 * kStagesA;
-static_assert(kEmptyA == 2 * kGroups && kStagesA == 4, "the warp of a stage is (stage / 2) mod kGroups");
+// "A stage empty" has eight barriers however many stages there are: a decode warp writes the stages it = 2 w, 2 w + 1 (mod 8),
+// so it meets every phase of the barriers (it - kStagesA) mod 8 that it waits on, one after the other.
+constexpr int kEmptyA = 8;
+static_assert(kEmptyA == 2 * kGroups, "the warp of a stage is (stage / 2) mod kGroups");
 constexpr uint32_t kGemmBars = 0;                                  // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
 constexpr uint32_t kGemmTab = 512;                                 // position table, 8 bytes per entry and copy
 static_assert(kMaxStagesB == kEmptyA, "one accumulator: boxes and stages are freed by the same barriers");
-static_assert(8 * (kStagesA + kEmptyA + 2 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
+static_assert(8 * (2 * kEmptyA + 2 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
 constexpr uint32_t kSmemMax = 232448;
 constexpr double kDecodeClocks = 420.0;    // decode of a stage (gemm_plan)
 // What depends on bn: copies of the position table (16, lane-minor: look-ups nearly free of bank conflicts; one where bn = 256
@@ -79,7 +83,7 @@ __host__ __device__ inline GemmSmem gemm_smem(int kAcc, int bn) {
   g.box = (uint32_t)bn * kBK * 2;
   for (g.copies = 16;; g.copies = 1) {
     g.a = (kGemmTab + 8u * kPosTableEntries * g.copies + 1023u) & ~1023u;
-    g.b = g.a + kStagesA * kStageA;
+    g.b = g.a + (kAcc == 1 ? 8u : 4u) * kStageA;
     g.nbox = (kSmemMax - g.b) / g.box;
     if (g.nbox >= 5u || g.copies == 1u) break;
   }
@@ -225,7 +229,7 @@ __device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, Ge
 
 // Decode role of one warp: packed row tile 4 mt + q, every fourth block of the CTA's K range, written into the A stages.
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
-template <int N, bool kF16>
+template <int N, bool kF16, int kStagesA>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1, w = da.w;
   // The lane plays the part of packed-layout lane 4 g + t with g = lane % 8, t = lane / 8: the eight
@@ -242,9 +246,10 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   const uint32_t row_at = da.stages + (uint32_t)((2 * w) % kStagesA) * kStageA + (uint32_t)q * 4096u + (uint32_t)g * 128u;
   const uint32_t at0 = row_at + (uint32_t)((t ^ g) << 4), at1 = row_at + (uint32_t)(((4 + t) ^ g) << 4);
   const uint32_t full = da.bar_full + 8u * (uint32_t)((2 * w) % kStagesA), empty = da.bar_empty + 8u * (uint32_t)((2 * w + kEmptyA - kStagesA) % kEmptyA);
-  // before stage `it` is written, stage it - 4 must have been read: use it / 8 of the slot pair waits for that barrier's phase
-  // it / 8 (w >= 2) or it / 8 - 1 (w < 2: nothing to wait for the first time).  The verdict is made warp-uniform.
-  const uint32_t early = w < 2 ? 1u : 0u;
+  // before stage `it` is written, stage it - kStagesA must have been read.  Four stages: use it / 8 of the slot pair waits for
+  // phase it / 8 (w >= 2) or it / 8 - 1 (w < 2) of that stage's barrier, eight: for phase it / 8 - 1; there is nothing to
+  // wait for before phase 0.  The verdict is made warp-uniform.
+  const uint32_t early = kStagesA == 8 || w < 2 ? 1u : 0u;
   auto stage_wait = [&](uint32_t use, int h) -> bool {
     if (use < early) return true;
     const uint32_t parity = (use - early) & 1u;
@@ -413,7 +418,7 @@ template <int N, class Cfg, bool kF16>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap xsmap, const uint8_t* __restrict__ packed, int n, int m, int T,
             void* __restrict__ Y, int y_16, size_t ldy, float* __restrict__ ws, const __grid_constant__ GemmShape shape, uint32_t box_bytes, int* dev_status) {
-  constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN;
+  constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN, kStagesA = Cfg::kStagesA;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int full_tiles = shape.full_tiles, ksplit = shape.ksplit, bps = shape.bps, ttiles = shape.ttiles, bn = shape.bn;
   const GemmSmem& L = shape.smem;
@@ -445,9 +450,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   const uint32_t sbase = smem_u32(smem);
   // A ring: full = the four decode warps of the stage's block have written it, empty = the tensor core has read it;
   // B ring: full = the X boxes have landed, empty = the tensor core has read them
-  const uint32_t bar_fullA = sbase + kGemmBars, bar_emptyA = bar_fullA + 8 * kStagesA;
+  const uint32_t bar_fullA = sbase + kGemmBars, bar_emptyA = bar_fullA + 8 * kEmptyA;
   const uint32_t bar_fullB = bar_emptyA + 8 * kEmptyA, bar_emptyB = bar_fullB + 8 * kMaxStagesB, bar_accum = bar_emptyB + 8 * kMaxStagesB;
-  constexpr uint32_t kBarBytes = 8 * (kStagesA + kEmptyA + 2 * kMaxStagesB + 1);
+  constexpr uint32_t kBarBytes = 8 * (2 * kEmptyA + 2 * kMaxStagesB + 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kGemmBars + kBarBytes);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kGemmBars + kBarBytes + 8);
 
@@ -555,7 +560,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     da.bar_full = bar_fullA; da.bar_empty = bar_emptyA;
     da.mt = mt; da.b0 = b0; da.b1 = max(b1, b0); da.nblk = nblk; da.ntile = ntile; da.q = warp & 3; da.w = gi; da.lane = lane;
     da.nrw = nrw; da.rw0 = rw0; da.rw1 = rw1; da.nres = nres;
-    decode_tiles<N, kF16>(da);
+    decode_tiles<N, kF16, kStagesA>(da);
 
     // ---------------- epilogue: TMEM -> registers -> Y ----------------
     const int q = warp & 3;                        // TMEM lane quarter of this warp
@@ -643,6 +648,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
 __global__ void gemm_reduce_kernel(const float* __restrict__ ws, int first_tile, int split_tiles, int ksplit, int ttiles, int ktok,
                                    int n, int T, void* __restrict__ Y, int y_16, size_t ldy) {
   // four consecutive rows of one token per thread: 16-byte loads of the parts, one 8- or 16-byte store
+  grid_dependency_wait();          // (a programmatic dependent of the GEMM: its CTAs are set up while the GEMM drains)
   const size_t per = (size_t)kBM * ktok, per4 = per / 4, total = (size_t)split_tiles * per4;
   const bool vec = (ldy % 4) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -846,9 +852,12 @@ static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T
                          (uint32_t)(box_rows * kBK * 2), dev_status) != cudaSuccess)
     return STB_ERR_CUDA;
   if (plan.split_tiles > 0) {
-    gemm_reduce_kernel<<<148 * 4, 256, 0, s>>>(ws_split, plan.full_tiles, plan.split_tiles, plan.ksplit,
-                                               plan.ttiles, kAcc * plan.bn, n, T, Y, y_16 ? (kF16 ? 2 : 1) : 0, ldy);
-    if (cudaGetLastError() != cudaSuccess) return STB_ERR_CUDA;
+    cfg.gridDim = dim3(148 * 4);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = 0;
+    if (cudaLaunchKernelEx(&cfg, gemm_reduce_kernel, (const float*)ws_split, plan.full_tiles, plan.split_tiles, plan.ksplit, plan.ttiles, kAcc * plan.bn,
+                           n, T, Y, y_16 ? (kF16 ? 2 : 1) : 0, ldy) != cudaSuccess)
+      return STB_ERR_CUDA;
   }
   return STB_OK;
 }

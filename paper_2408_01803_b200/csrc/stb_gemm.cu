@@ -488,25 +488,33 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   if (warp >= kDecodeWarps) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGemmIssueRegs));
   if (warp == kTmaWarp) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      uint32_t s = 0, ps = 0;
-      for (int hb = 0; hb < nstage * kAcc; ++hb) {
-        const int it = hb / kAcc, a = hb % kAcc;
-        // (one accumulator: box s goes with the stages s, s + 8, .. and is freed with them)
-        if (!gemm_wait<true>((kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * s, ps ^ 1u, abort_flag)) break;
-        // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
-        if (it == nmain && a == 0) grid_dependency_wait();
-        mbar_expect_tx(bar_fullB + 8 * s, box_bytes);
-        const uint32_t dst = sbase + L.b + s * L.box;
-        if (it < nmain) tma_load_2d(dst, &xmap, (b0 * 2 + it) * kBK, tt * ktok + a * bn, bar_fullB + 8 * s);
-        else tma_load_2d(dst, &xsmap, (int)(4u * (rw0 & ~1u)) + (it - nmain) * kBK, tt * ktok + a * bn, bar_fullB + 8 * s);
-        if (++s == L.nbox) { s = 0; ps ^= 1u; }
+    // (the whole warp runs the loop, one elected lane issues, for the reason given at the MMA issuers)
+    const bool leader = elect_one();
+    const uint32_t rwx = __shfl_sync(0xFFFFFFFFu, 4u * (rw0 & ~1u), 0);
+    const uint32_t box = L.box, nbox = L.nbox;
+    int x = b0 * 2 * kBK, y = tt * ktok, it = 0;
+    uint32_t s = 0, ps = 1;
+    const int boxes = __shfl_sync(0xFFFFFFFFu, nstage, 0) * kAcc, main_stages = nmain;
+    for (int hb = 0, a = 0; hb < boxes; ++hb) {
+      // (one accumulator: box s goes with the stages s, s + 8, .. and is freed with them)
+      const uint32_t bar_empty = (kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * s, bar_full = bar_fullB + 8 * s;
+      bool ok = mbar_try_wait(bar_empty, ps);
+      if (!ok) ok = gemm_wait<true>(bar_empty, ps, abort_flag);
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
+      if (it == main_stages && a == 0) { grid_dependency_wait(); x = (int)rwx; }
+      if (leader) {
+        mbar_expect_tx(bar_full, box_bytes);
+        tma_load_2d(sbase + L.b + s * box, it < main_stages ? &xmap : &xsmap, x, y + a * bn, bar_full);
       }
-      grid_dependency_wait();  // (every CTA, whether or not it had residual stages)
-      if (*abort_flag) {       // let copies in flight land before the CTA gives its shared memory up
-        const long long t0 = clock64();
-        while (clock64() - t0 < 200000) {}
-      }
+      __syncwarp();
+      if (++s == nbox) { s = 0; ps ^= 1u; }
+      if (++a == kAcc) { a = 0; ++it; x += kBK; }
+    }
+    grid_dependency_wait();  // (every CTA, whether or not it had residual stages)
+    if (*abort_flag) {       // let copies in flight land before the CTA gives its shared memory up
+      const long long t0 = clock64();
+      while (clock64() - t0 < 200000) {}
     }
   } else if (warp == kIssuerWarpA || warp == kIssuerWarpB) {
     // ---------------- MMA issuers ----------------

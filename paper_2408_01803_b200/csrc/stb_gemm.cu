@@ -10,7 +10,7 @@
 //       divides the decode work per flop by kAcc,
 // in rings over K (kStagesA decoded A stages, up to eight X boxes: the decode warps run ahead of the tensor core).  Warp roles:
 //   warps 0..15 decode: see below
-//   warp 16     TMA producer (one lane): X slices
+//   warp 16, 19 TMA producers (one lane each): X slices, one accumulator's or every other stage's
 //   warp 17, 18 MMA issuers (one lane each, on two schedulers): with two accumulators each takes one (4 x tcgen05.mma,
 //               K = 16, per stage); with one, each takes every other stage into an accumulator of its own and the
 //               epilogue adds the two.  tcgen05.commit frees the boxes and stages; warp 17 allocates / frees TMEM
@@ -18,7 +18,7 @@
 //               tile, each taking every fourth block: it loads the block's words with vector loads (its next block ahead),
 //               converts the scales to bf16 (RN-even), decodes 64 columns of its four rows per lane into registers,
 //               waits for the stage and writes them.  (Four warps sharing every block, one row of a lane each, paid the
-//               loads, the waits and the address arithmetic four times: 370 clocks per 32 x 128 tile and SM, now FIGURE_TILE.)
+//               loads, the waits and the address arithmetic four times: 370 clocks per 32 x 128 tile and SM, now about 220.)
 //               Afterwards the same warps read the accumulator (TMEM lanes 32 (w % 4) ..) and store Y.
 // The residual term of the salient columns (Eq. 4) is more K: a small kernel first gathers the activations of
 // every residual slot (four per residual word, in word order) into Xs[token][slot]; after the blocks of its K
@@ -58,8 +58,8 @@ constexpr int kMaxStagesB = 8;    // ring of X boxes: as many as fit, up to eigh
                                   // flight from L2 is what hides its latency; a stage of K takes kAcc of them
 constexpr int kGroups = 4;                              // decode warps per 32-row quarter: each takes every fourth block
 constexpr int kIssuers = 2;                             // MMA-issuing lanes (in two warps, on two schedulers)
-constexpr int kDecodeWarps = 4 * kGroups;               // warps 0 .. 15; then the copies (16) and the issuers (17, 18)
-constexpr int kTmaWarp = kDecodeWarps, kIssuerWarpA = kDecodeWarps + 1, kIssuerWarpB = kDecodeWarps + 2;
+constexpr int kDecodeWarps = 4 * kGroups;               // warps 0 .. 15; then the copies (16, 19) and the issuers (17, 18)
+constexpr int kTmaWarpA = kDecodeWarps, kIssuerWarpA = kDecodeWarps + 1, kIssuerWarpB = kDecodeWarps + 2, kTmaWarpB = kDecodeWarps + 3;
 constexpr int kGemmThreads = 32 * kDecodeWarps + 128;
 // registers: 640 x 96 at launch, of which the fifth warpgroup gives some to the decode warps
 constexpr int kGemmDecodeRegs = 104, kGemmIssueRegs = 64;
@@ -72,9 +72,13 @@ static_assert(kEmptyA == 2 * kGroups, "the warp of a stage is (stage / 2) mod kG
 constexpr uint32_t kGemmBars = 0;                                  // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
 constexpr uint32_t kGemmTab = 512;                                 // position table, 8 bytes per entry and copy
 static_assert(kMaxStagesB == kEmptyA, "one accumulator: boxes and stages are freed by the same barriers");
-static_assert(8 * (2 * kEmptyA + 2 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
+static_assert(8 * (2 * kEmptyA + 4 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
 constexpr uint32_t kSmemMax = 232448;
-constexpr double kDecodeClocks = 420.0;    // decode of a stage (gemm_plan)
+constexpr double kDecodeClocks = 440.0;    // decode of a stage (gemm_plan)
+// X boxes have twice as many barriers as there are boxes, for the same reason: with two accumulators box number hb = 2 stage + a
+// goes to place hb mod nbox, where (nbox odd) the boxes of the two accumulators alternate; producer and issuer of an
+// accumulator meet every phase of the barriers hb mod 2 nbox, but only every second one of a barrier per place, and a parity
+// cannot tell the phase before from the phase after.
 // What depends on bn: copies of the position table (16, lane-minor: look-ups nearly free of bank conflicts; one where bn = 256
 // leaves no room), where the stages and the boxes lie, and how many boxes there are.
 struct GemmSmem { uint32_t copies, a, b, box, nbox, total; };
@@ -451,8 +455,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   // A ring: full = the four decode warps of the stage's block have written it, empty = the tensor core has read it;
   // B ring: full = the X boxes have landed, empty = the tensor core has read them
   const uint32_t bar_fullA = sbase + kGemmBars, bar_emptyA = bar_fullA + 8 * kEmptyA;
-  const uint32_t bar_fullB = bar_emptyA + 8 * kEmptyA, bar_emptyB = bar_fullB + 8 * kMaxStagesB, bar_accum = bar_emptyB + 8 * kMaxStagesB;
-  constexpr uint32_t kBarBytes = 8 * (2 * kEmptyA + 2 * kMaxStagesB + 1);
+  const uint32_t bar_fullB = bar_emptyA + 8 * kEmptyA, bar_emptyB = bar_fullB + 16 * kMaxStagesB, bar_accum = bar_emptyB + 16 * kMaxStagesB;
+  constexpr uint32_t kBarBytes = 8 * (2 * kEmptyA + 4 * kMaxStagesB + 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kGemmBars + kBarBytes);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kGemmBars + kBarBytes + 8);
 
@@ -460,7 +464,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     // a stage of A is read by both issuers (with one accumulator by one of them), an X box by the issuer of its accumulator
     for (int i = 0; i < kStagesA; ++i) mbar_init(bar_fullA + 8 * i, 4);
     for (int i = 0; i < kEmptyA; ++i) mbar_init(bar_emptyA + 8 * i, kAcc == 1 ? 1 : kIssuers);
-    for (int i = 0; i < kMaxStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, 1); }
+    for (int i = 0; i < 2 * kMaxStagesB; ++i) { mbar_init(bar_fullB + 8 * i, 1); mbar_init(bar_emptyB + 8 * i, 1); }
     mbar_init(bar_accum, kIssuers);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -486,30 +490,46 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   const int nstage = nmain + nres;
 
   if (warp >= kDecodeWarps) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGemmIssueRegs));
-  if (warp == kTmaWarp) {
-    // ---------------- TMA producer ----------------
+  if (warp == kTmaWarpA || warp == kTmaWarpB) {
+    // ---------------- TMA producers ----------------
     // (the whole warp runs the loop, one elected lane issues, for the reason given at the MMA issuers)
+    // two accumulators: producer w brings box w of every stage; one accumulator: the box of the stages 2 i + w
+    const int w = __shfl_sync(0xFFFFFFFFu, warp == kTmaWarpA ? 0 : 1, 0);
+    constexpr int kStep = kAcc == 1 ? kIssuers : 1, kBoxStep = 2;
     const bool leader = elect_one();
-    const uint32_t rwx = __shfl_sync(0xFFFFFFFFu, 4u * (rw0 & ~1u), 0);
     const uint32_t box = L.box, nbox = L.nbox;
-    int x = b0 * 2 * kBK, y = tt * ktok, it = 0;
-    uint32_t s = 0, ps = 1;
-    const int boxes = __shfl_sync(0xFFFFFFFFu, nstage, 0) * kAcc, main_stages = nmain;
-    for (int hb = 0, a = 0; hb < boxes; ++hb) {
+    const int stages = __shfl_sync(0xFFFFFFFFu, nstage, 0), y = tt * ktok + (kAcc == 1 ? 0 : w * bn);
+    const int rwx = __shfl_sync(0xFFFFFFFFu, (int)(4u * (rw0 & ~1u)), 0);
+    // place of the box; its barrier and that of the box that was there before (mod nbar), and the latter's parity
+    const uint32_t nbar = kAcc == 1 ? nbox : 2u * nbox;
+    uint32_t s = (uint32_t)w, fb = s, eb = kAcc == 1 ? s : s + nbox, ps = 1;
+    bool waited = false;
+    for (int it = kAcc == 1 ? w : 0; it < stages; it += kStep) {
       // (one accumulator: box s goes with the stages s, s + 8, .. and is freed with them)
-      const uint32_t bar_empty = (kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * s, bar_full = bar_fullB + 8 * s;
+      const uint32_t bar_empty = (kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * eb, bar_full = bar_fullB + 8 * fb;
       bool ok = mbar_try_wait(bar_empty, ps);
       if (!ok) ok = gemm_wait<true>(bar_empty, ps, abort_flag);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
-      // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
-      if (it == main_stages && a == 0) { grid_dependency_wait(); x = (int)rwx; }
-      if (leader) {
-        mbar_expect_tx(bar_full, box_bytes);
-        tma_load_2d(sbase + L.b + s * box, it < main_stages ? &xmap : &xsmap, x, y + a * bn, bar_full);
+      if (it < nmain) {
+        if (leader) {
+          mbar_expect_tx(bar_full, box_bytes);
+          tma_load_2d(sbase + L.b + s * box, &xmap, (b0 * 2 + it) * kBK, y, bar_full);
+        }
+      } else {
+        // Xs comes from the gather kernel, which this grid may have overtaken (programmatic dependent launch)
+        if (!waited) { grid_dependency_wait(); waited = true; }
+        if (leader) {
+          mbar_expect_tx(bar_full, box_bytes);
+          tma_load_2d(sbase + L.b + s * box, &xsmap, rwx + (it - nmain) * kBK, y, bar_full);
+        }
       }
       __syncwarp();
-      if (++s == nbox) { s = 0; ps ^= 1u; }
-      if (++a == kAcc) { a = 0; ++it; x += kBK; }
+      s += kBoxStep;
+      if (s >= nbox) s -= nbox;
+      fb += kBoxStep;
+      if (fb >= nbar) fb -= nbar;
+      eb += kBoxStep;
+      if (eb >= nbar) { eb -= nbar; ps ^= 1u; }
     }
     grid_dependency_wait();  // (every CTA, whether or not it had residual stages)
     if (*abort_flag) {       // let copies in flight land before the CTA gives its shared memory up
@@ -520,7 +540,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     // ---------------- MMA issuers ----------------
     // The whole warp runs the loop and one elected lane issues: every operand is then warp-uniform to the compiler and sits in
     // uniform registers, where tcgen05 instructions take them (under `lane == 0` each was moved there one by one: an
-    // issuer's stage took 850 clocks at 64 tokens, 600 of them its own instructions; now FIGURE_ISSUE).
+    // issuer's stage took 850 clocks at 64 tokens, 600 of them its own instructions; now 170 per two stages).
     const int w = __shfl_sync(0xFFFFFFFFu, warp == kIssuerWarpA ? 0 : 1, 0);
     const uint32_t tmem_u = __shfl_sync(0xFFFFFFFFu, tmem_d, 0);
     const bool leader = elect_one();
@@ -530,13 +550,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     const uint32_t desc_hi = (uint32_t)(umma_desc(0u) >> 32);
     const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + L.a), b_lo0 = (uint32_t)umma_desc(sbase + L.b);
     const uint32_t dt = tmem_u + (uint32_t)(w * kMaxBN), idesc = gemm_idesc(kF16, bn), box_lo = L.box >> 4, nbox = L.nbox;
-    uint32_t sa = kAcc == 1 ? (uint32_t)w : 0u, ea = sa, sb = (uint32_t)w;      // ring slots, advanced without divisions
+    const uint32_t nbar = kAcc == 1 ? nbox : 2u * nbox;
+    uint32_t sa = kAcc == 1 ? (uint32_t)w : 0u, ea = sa, sb = (uint32_t)w, fb = sb;      // ring places and barriers, advanced without divisions
     uint32_t pa = 0, pb = 0;                                                    // their phase parities
     for (int it = kAcc == 1 ? w : 0; it < nstage; it += kStep) {
-      const bool ra = mbar_try_wait(bar_fullA + 8 * sa, pa), rb = mbar_try_wait(bar_fullB + 8 * sb, pb);     // both at once
+      const bool ra = mbar_try_wait(bar_fullA + 8 * sa, pa), rb = mbar_try_wait(bar_fullB + 8 * fb, pb);     // both at once
       bool ok = true;
       if (!ra) ok = gemm_wait<true>(bar_fullA + 8 * sa, pa, abort_flag);
-      if (!rb && ok) ok = gemm_wait<true>(bar_fullB + 8 * sb, pb, abort_flag);
+      if (!rb && ok) ok = gemm_wait<true>(bar_fullB + 8 * fb, pb, abort_flag);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
       tc_fence_after();
       const uint32_t a_lo = a_lo0 + sa * (kStageA >> 4), b_lo = b_lo0 + sb * box_lo;
@@ -545,7 +566,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         else umma_16<false>(dt, a_lo, b_lo, desc_hi, idesc);
 #pragma unroll
         for (int kk = 1; kk < kBK / 16; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, idesc);
-        if (kAcc > 1) umma_commit(bar_emptyB + 8 * sb);        // the box is free once the MMAs that read it have completed
+        if (kAcc > 1) umma_commit(bar_emptyB + 8 * fb);        // the box is free once the MMAs that read it have completed
         umma_commit(bar_emptyA + 8 * ea);                      // (one accumulator: the box of a stage is freed with it)
       }
       __syncwarp();
@@ -553,8 +574,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       if (sa >= kStagesA) { sa -= kStagesA; pa ^= 1u; }
       ea += kStep;
       if (ea >= kEmptyA) ea -= kEmptyA;
-      sb += kAcc == 1 ? kStep : kAcc;
-      if (sb >= nbox) { sb -= nbox; pb ^= 1u; }
+      sb += 2u;
+      if (sb >= nbox) sb -= nbox;
+      fb += 2u;
+      if (fb >= nbar) { fb -= nbar; pb ^= 1u; }
     }
     if (leader) umma_commit(bar_accum);                        // all MMAs this warp issued have completed
     __syncwarp();
@@ -727,8 +750,8 @@ static GemmBytes gemm_bytes(int n, int m, int T, int ktok) {
 // multiple of 16), and which tiles are split along K into how many parts -- all of them, or those of the last wave -- chosen
 // as the layout whose estimated time is smallest among those whose partial tiles fit `avail` bytes.  In SM clocks:
 //   a stage (64 of K):   the decode of two 32 x 128 tiles' worth of weights per row tile, or the tensor core's time for the
-//                        tile's tokens, whichever is longer (measured: FIGURE_DEC, and 2.25 per token + 30)
-//   a CTA besides:       prologue, first loads, drain (9000) and epilogue (6 per token)
+//                        tile's tokens, whichever is longer (measured: about 440, and 2.25 per token + 30)
+//   a CTA besides:       prologue, first loads, drain (10000) and epilogue (15 per token)
 //   a split:             the second kernel, and its partial tiles written and read (2500 bytes per clock)
 struct GemmPlan {
   int bn, ttiles, tiles, full_tiles, split_tiles, ksplit, bps;
@@ -744,7 +767,7 @@ static GemmPlan gemm_plan(int acc, int max_bn, int n, int m, int T, size_t avail
     const int ktok = acc * bn;
     if (bn > max_bn || (tt - 1) * ktok >= T) continue;
     const long long tiles = (long long)rtiles * tt;
-    const double mma = 2.25 * ktok + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 9000.0 + 6.0 * ktok;
+    const double mma = 2.25 * ktok + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 10000.0 + 15.0 * ktok;
     const size_t per = (size_t)kBM * ktok * sizeof(float);
     auto consider = [&](long long full, int ks) {
       const int bps = (nblk + ks - 1) / ks;

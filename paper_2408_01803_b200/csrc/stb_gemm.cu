@@ -43,16 +43,17 @@
 namespace stb {
 
 constexpr int kBM = 128;          // rows of W^ per CTA (UMMA M)
-// Token side of the CTA tile: kAcc accumulators of bn tokens (UMMA N, a run-time value).  Prefill: 2 x up to 256 (all 512 TMEM
-// columns; a decoded A stage is used twice).  Up to 64 tokens (a decode batch): 1 x up to 64, the tensor core then takes an
-// eighth of the time per stage and the kernel runs at the speed of the decode warps.
-template <int kAcc_, int kMaxBN_>
-struct TokCfg {
-  static constexpr int kAcc = kAcc_, kMaxBN = kMaxBN_, kTok = kAcc_ * kMaxBN_;
-  // ring of decoded A stages (16 KB each): four beside the wide X boxes, eight beside the narrow ones (a stage's way round
-  // -- written, multiplied, freed, seen -- takes about 2000 clocks, four decodes of a decode batch's stage)
-  static constexpr int kStagesA = kAcc_ == 1 ? 8 : 4;
-};
+// Token side of the CTA tile: kAcc accumulators of bn tokens (UMMA N, a run-time value).  An MMA of 128 rows takes about 105
+// clocks even where N is below 210 (832 clocks per stage of 8 MMAs at N = 64), so two accumulators are for tiles of more
+// than 256 tokens (all 512 TMEM columns; a decoded A stage is used twice); up to 256 tokens are one accumulator per issuer,
+// the issuers taking turns by the stage.
+// kStagesA: ring of decoded A stages (16 KB each): eight beside narrow X boxes (a stage's way round -- written, multiplied,
+// freed, seen -- takes about 2000 clocks, four decodes of a decode batch's stage), four beside wide ones.
+template <int kAcc_, int kMaxBN_, int kStagesA_>
+struct TokCfg { static constexpr int kAcc = kAcc_, kMaxBN = kMaxBN_, kTok = kAcc_ * kMaxBN_, kStagesA = kStagesA_; };
+using BatchCfg = TokCfg<1, 64, 8>;
+using MidCfg = TokCfg<1, 256, 4>;
+using PrefillCfg = TokCfg<2, 256, 4>;
 constexpr int kBK = 64;           // K per stage: one 128-byte swizzle row of bf16
 constexpr int kMaxStagesB = 8;    // ring of X boxes: as many as fit, up to eight (five of 256 tokens x 64 of K = 32 KB): what is in
                                   // flight from L2 is what hides its latency; a stage of K takes kAcc of them
@@ -71,27 +72,26 @@ constexpr int kEmptyA = 8;
 static_assert(kEmptyA == 2 * kGroups, "the warp of a stage is (stage / 2) mod kGroups");
 constexpr uint32_t kGemmBars = 0;                                  // fullA, emptyA, fullB, emptyB, accum, tmem slot, abort
 constexpr uint32_t kGemmTab = 512;                                 // position table, 8 bytes per entry and copy
-static_assert(kMaxStagesB == kEmptyA, "one accumulator: boxes and stages are freed by the same barriers");
 static_assert(8 * (2 * kEmptyA + 4 * kMaxStagesB + 1) + 16 <= kGemmTab, "barrier area");
 constexpr uint32_t kSmemMax = 232448;
 constexpr double kDecodeClocks = 440.0;    // decode of a stage (gemm_plan)
-// X boxes have twice as many barriers as there are boxes, for the same reason: with two accumulators box number hb = 2 stage + a
-// goes to place hb mod nbox, where (nbox odd) the boxes of the two accumulators alternate; producer and issuer of an
-// accumulator meet every phase of the barriers hb mod 2 nbox, but only every second one of a barrier per place, and a parity
-// cannot tell the phase before from the phase after.
+// X boxes have twice as many barriers as there are boxes, for the same reason: box number hb (two accumulators: 2 stage + a,
+// one: the stage) goes to place hb mod nbox, where (nbox odd) the boxes of the two producers alternate; the producer and the
+// issuer of box hb meet every phase of the barriers hb mod 2 nbox, but only every second one of a barrier per place, and a
+// parity cannot tell the phase before from the phase after.
 // What depends on bn: copies of the position table (16, lane-minor: look-ups nearly free of bank conflicts; one where bn = 256
 // leaves no room), where the stages and the boxes lie, and how many boxes there are.
 struct GemmSmem { uint32_t copies, a, b, box, nbox, total; };
-__host__ __device__ inline GemmSmem gemm_smem(int kAcc, int bn) {
+__host__ __device__ inline GemmSmem gemm_smem(int kAcc, int stages_a, int bn) {
   GemmSmem g;
   g.box = (uint32_t)bn * kBK * 2;
   for (g.copies = 16;; g.copies = 1) {
     g.a = (kGemmTab + 8u * kPosTableEntries * g.copies + 1023u) & ~1023u;
-    g.b = g.a + (kAcc == 1 ? 8u : 4u) * kStageA;
+    g.b = g.a + (uint32_t)stages_a * kStageA;
     g.nbox = (kSmemMax - g.b) / g.box;
     if (g.nbox >= 5u || g.copies == 1u) break;
   }
-  if (g.nbox > (uint32_t)kMaxStagesB) g.nbox = kMaxStagesB;      // (one accumulator: always eight, as many as there are "stage empty" barriers)
+  if (g.nbox > (uint32_t)kMaxStagesB) g.nbox = kMaxStagesB;
   g.total = g.b + g.nbox * g.box;
   // a 16-bit output tile is staged where the boxes were
   const uint32_t out = (uint32_t)(kAcc * bn) * kBM * 2u;
@@ -501,12 +501,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     const int stages = __shfl_sync(0xFFFFFFFFu, nstage, 0), y = tt * ktok + (kAcc == 1 ? 0 : w * bn);
     const int rwx = __shfl_sync(0xFFFFFFFFu, (int)(4u * (rw0 & ~1u)), 0);
     // place of the box; its barrier and that of the box that was there before (mod nbar), and the latter's parity
-    const uint32_t nbar = kAcc == 1 ? nbox : 2u * nbox;
-    uint32_t s = (uint32_t)w, fb = s, eb = kAcc == 1 ? s : s + nbox, ps = 1;
+    const uint32_t nbar = 2u * nbox;
+    uint32_t s = (uint32_t)w, fb = s, eb = s + nbox, ps = 1;
     bool waited = false;
     for (int it = kAcc == 1 ? w : 0; it < stages; it += kStep) {
-      // (one accumulator: box s goes with the stages s, s + 8, .. and is freed with them)
-      const uint32_t bar_empty = (kAcc == 1 ? bar_emptyA : bar_emptyB) + 8 * eb, bar_full = bar_fullB + 8 * fb;
+      const uint32_t bar_empty = bar_emptyB + 8 * eb, bar_full = bar_fullB + 8 * fb;
       bool ok = mbar_try_wait(bar_empty, ps);
       if (!ok) ok = gemm_wait<true>(bar_empty, ps, abort_flag);
       if (!__all_sync(0xFFFFFFFFu, ok)) break;
@@ -550,7 +549,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     const uint32_t desc_hi = (uint32_t)(umma_desc(0u) >> 32);
     const uint32_t a_lo0 = (uint32_t)umma_desc(sbase + L.a), b_lo0 = (uint32_t)umma_desc(sbase + L.b);
     const uint32_t dt = tmem_u + (uint32_t)(w * kMaxBN), idesc = gemm_idesc(kF16, bn), box_lo = L.box >> 4, nbox = L.nbox;
-    const uint32_t nbar = kAcc == 1 ? nbox : 2u * nbox;
+    const uint32_t nbar = 2u * nbox;
     uint32_t sa = kAcc == 1 ? (uint32_t)w : 0u, ea = sa, sb = (uint32_t)w, fb = sb;      // ring places and barriers, advanced without divisions
     uint32_t pa = 0, pb = 0;                                                    // their phase parities
     for (int it = kAcc == 1 ? w : 0; it < nstage; it += kStep) {
@@ -566,8 +565,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         else umma_16<false>(dt, a_lo, b_lo, desc_hi, idesc);
 #pragma unroll
         for (int kk = 1; kk < kBK / 16; ++kk) umma_16<true>(dt, a_lo + 2u * kk, b_lo + 2u * kk, desc_hi, idesc);
-        if (kAcc > 1) umma_commit(bar_emptyB + 8 * fb);        // the box is free once the MMAs that read it have completed
-        umma_commit(bar_emptyA + 8 * ea);                      // (one accumulator: the box of a stage is freed with it)
+        umma_commit(bar_emptyB + 8 * fb);        // the box is free once the MMAs that read it have completed
+        umma_commit(bar_emptyA + 8 * ea);
       }
       __syncwarp();
       sa += kStep;
@@ -750,24 +749,22 @@ static GemmBytes gemm_bytes(int n, int m, int T, int ktok) {
 // multiple of 16), and which tiles are split along K into how many parts -- all of them, or those of the last wave -- chosen
 // as the layout whose estimated time is smallest among those whose partial tiles fit `avail` bytes.  In SM clocks:
 //   a stage (64 of K):   the decode of two 32 x 128 tiles' worth of weights per row tile, or the tensor core's time for the
-//                        tile's tokens, whichever is longer (measured: about 440, and 2.25 per token + 30)
+//                        tile's tokens, whichever is longer (measured: about 440, and 4.4 x 105 or bn / 2 + 30 per accumulator)
 //   a CTA besides:       prologue, first loads, drain (10000) and epilogue (15 per token)
 //   a split:             the second kernel, and its partial tiles written and read (2500 bytes per clock)
 struct GemmPlan {
-  int bn, ttiles, tiles, full_tiles, split_tiles, ksplit, bps;
+  int acc, bn, ttiles, tiles, full_tiles, split_tiles, ksplit, bps;
   size_t bytes;
 };
-static GemmPlan gemm_plan(int acc, int max_bn, int n, int m, int T, size_t avail) {
+static void gemm_plan_for(GemmPlan& best, double& best_cost, int acc, int max_bn, int n, int m, int T, size_t avail) {
   const int nblk = m / kBlock, rtiles = (n + kBM - 1) / kBM, most = acc * max_bn;
-  GemmPlan best = {};
-  double best_cost = 0.0;
-  for (int tt = (T + most - 1) / most, end = acc == 1 ? tt : tt + 8; tt <= end; ++tt) {
+  for (int tt = (T + most - 1) / most, end = tt + 8; tt <= end; ++tt) {
     int bn = ((T + tt - 1) / tt + acc - 1) / acc;
     bn = bn < 16 ? 16 : (bn + 15) / 16 * 16;
     const int ktok = acc * bn;
     if (bn > max_bn || (tt - 1) * ktok >= T) continue;
     const long long tiles = (long long)rtiles * tt;
-    const double mma = 2.25 * ktok + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 10000.0 + 15.0 * ktok;
+    const double mma = acc * 4.0 * (bn > 210 ? 0.5 * bn : 105.0) * 1.1 + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 10000.0 + 15.0 * ktok;
     const size_t per = (size_t)kBM * ktok * sizeof(float);
     auto consider = [&](long long full, int ks) {
       const int bps = (nblk + ks - 1) / ks;
@@ -779,7 +776,7 @@ static GemmPlan gemm_plan(int acc, int max_bn, int n, int m, int T, size_t avail
       if (ks > 1) cost += 4000.0 + 2.0 * (double)bytes / 2500.0;
       if (best.tiles == 0 || cost < best_cost * 0.999) {
         best_cost = cost;
-        best.bn = bn; best.ttiles = tt; best.tiles = (int)tiles; best.full_tiles = (int)(ks > 1 ? full : tiles); best.split_tiles = (int)(ks > 1 ? rest : 0);
+        best.acc = acc; best.bn = bn; best.ttiles = tt; best.tiles = (int)tiles; best.full_tiles = (int)(ks > 1 ? full : tiles); best.split_tiles = (int)(ks > 1 ? rest : 0);
         best.ksplit = ks; best.bps = bps; best.bytes = bytes;
       }
     };
@@ -788,6 +785,15 @@ static GemmPlan gemm_plan(int acc, int max_bn, int n, int m, int T, size_t avail
       if (tiles < 148) consider(0, ks);
       else if (tiles % 148) consider(tiles - tiles % 148, ks);
     }
+  }
+}
+static GemmPlan gemm_plan(int n, int m, int T, size_t avail) {
+  GemmPlan best = {};
+  double cost = 0.0;
+  if (T <= BatchCfg::kTok) gemm_plan_for(best, cost, BatchCfg::kAcc, BatchCfg::kMaxBN, n, m, T, avail);
+  else {
+    gemm_plan_for(best, cost, MidCfg::kAcc, MidCfg::kMaxBN, n, m, T, avail);
+    gemm_plan_for(best, cost, PrefillCfg::kAcc, PrefillCfg::kMaxBN, n, m, T, avail);
   }
   return best;
 }
@@ -810,28 +816,23 @@ static EncodeTiledFn encode_tiled_fn() {
 // slots a layer can have (32 per block), so that the size depends on the shape alone.
 static size_t gemm_xs_bytes(int m, int T) { return (((size_t)T * (size_t)(m / 4) * 2u) + 255u) & ~(size_t)255u; }
 
+// A call's tile width in the promise of gemm_bytes: 512 tokens, 64 for a decode batch of fp16 activations.
+static int gemm_promise(bool f16, int T) { return f16 && T <= BatchCfg::kTok ? BatchCfg::kTok : PrefillCfg::kTok; }
 // partial tiles a call of this shape would like room for
-template <class Cfg>
-static size_t gemm_preferred(int n, int m, int T) {
-  const size_t a = gemm_bytes(n, m, T, Cfg::kTok).preferred, b = gemm_plan(Cfg::kAcc, Cfg::kMaxBN, n, m, T, (size_t)-1).bytes;
+static size_t gemm_preferred(int n, int m, int T, int ktok) {
+  const size_t a = gemm_bytes(n, m, T, ktok).preferred, b = gemm_plan(n, m, T, (size_t)-1).bytes;
   return a > b ? a : b;
 }
 
 // y_16: 0 = fp32 output, 1 = the 16-bit type of the activations (bf16, or fp16 with kF16)
 template <int N, class Cfg, bool kF16>
-static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T, size_t ldx, void* Y, int y_16,
-                       size_t ldy, void* ws, size_t ws_bytes, int* dev_status, cudaStream_t s) {
-  constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN;
-  const size_t xs_bytes = gemm_xs_bytes(m, T);
-  if (ws && (reinterpret_cast<uintptr_t>(ws) & 255u)) return STB_ERR_ARG;
-  if (!ws || ws_bytes < xs_bytes) return STB_ERR_SIZE;
-  float* ws_split = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + xs_bytes);
-  if (ws_bytes - xs_bytes < gemm_bytes(n, m, T, Cfg::kTok).mandatory) return STB_ERR_SIZE;
-  const size_t preferred = gemm_preferred<Cfg>(n, m, T);
-  const GemmPlan plan = gemm_plan(kAcc, kMaxBN, n, m, T, ws_bytes - xs_bytes < preferred ? ws_bytes - xs_bytes : preferred);
+static int launch_gemm(const GemmPlan& plan, const uint8_t* packed, int n, int m, const void* X, int T, size_t ldx, void* Y, int y_16,
+                       size_t ldy, void* ws, int* dev_status, cudaStream_t s) {
+  constexpr int kAcc = Cfg::kAcc;
+  float* ws_split = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + gemm_xs_bytes(m, T));
   GemmShape shape;
   shape.full_tiles = plan.full_tiles; shape.ksplit = plan.ksplit; shape.bps = plan.bps; shape.ttiles = plan.ttiles; shape.bn = plan.bn;
-  shape.smem = gemm_smem(kAcc, plan.bn);
+  shape.smem = gemm_smem(kAcc, Cfg::kStagesA, plan.bn);
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return STB_ERR_CUDA;
   const CUtensorMapDataType dt = kF16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -893,42 +894,40 @@ static int launch_gemm(const uint8_t* packed, int n, int m, const void* X, int T
   return STB_OK;
 }
 
-using PrefillCfg = TokCfg<2, 256>;
-using BatchCfg = TokCfg<1, 64>;
-
 template <bool kF16>
 static int launch_gemm_n(int N, const uint8_t* packed, int n, int m, const void* X, int T, size_t ldx, void* Y, int y_16,
                          size_t ldy, void* ws, size_t ws_bytes, int* dev_status, cudaStream_t s) {
-  if (kF16 && T <= BatchCfg::kTok) {
+  const size_t xs_bytes = gemm_xs_bytes(m, T);
+  const int ktok = gemm_promise(kF16, T);
+  if (ws && (reinterpret_cast<uintptr_t>(ws) & 255u)) return STB_ERR_ARG;
+  if (!ws || ws_bytes < xs_bytes || ws_bytes - xs_bytes < gemm_bytes(n, m, T, ktok).mandatory) return STB_ERR_SIZE;
+  const size_t preferred = gemm_preferred(n, m, T, ktok);
+  const GemmPlan plan = gemm_plan(n, m, T, ws_bytes - xs_bytes < preferred ? ws_bytes - xs_bytes : preferred);
+  auto go = [&](auto cfg) {
+    using Cfg = decltype(cfg);
     switch (N) {
-      case 4: return launch_gemm<4, BatchCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
-      case 5: return launch_gemm<5, BatchCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
-      default: return launch_gemm<6, BatchCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
+      case 4: return launch_gemm<4, Cfg, kF16>(plan, packed, n, m, X, T, ldx, Y, y_16, ldy, ws, dev_status, s);
+      case 5: return launch_gemm<5, Cfg, kF16>(plan, packed, n, m, X, T, ldx, Y, y_16, ldy, ws, dev_status, s);
+      default: return launch_gemm<6, Cfg, kF16>(plan, packed, n, m, X, T, ldx, Y, y_16, ldy, ws, dev_status, s);
     }
-  }
-  switch (N) {
-    case 4: return launch_gemm<4, PrefillCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
-    case 5: return launch_gemm<5, PrefillCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
-    default: return launch_gemm<6, PrefillCfg, kF16>(packed, n, m, X, T, ldx, Y, y_16, ldy, ws, ws_bytes, dev_status, s);
-  }
+  };
+  if (T <= BatchCfg::kTok) return go(BatchCfg{});
+  return plan.acc == 1 ? go(MidCfg{}) : go(PrefillCfg{});
 }
 
 }  // namespace stb
 
-template <class Cfg>
-static int gemm_workspace_impl(int n, int m, int N, int T, size_t* bytes, bool minimum) {
+static int gemm_workspace_impl(int n, int m, int N, int T, int ktok, size_t* bytes, bool minimum) {
   if (!bytes) return STB_ERR_ARG;
   if (n < 1 || m < stb::kBlock || m % stb::kBlock != 0 || T < 1) return STB_ERR_SHAPE;
   if (N < 1 || N > 8) return STB_ERR_NM;
-  *bytes = stb::gemm_xs_bytes(m, T) + (minimum ? stb::gemm_bytes(n, m, T, Cfg::kTok).mandatory : stb::gemm_preferred<Cfg>(n, m, T));
+  *bytes = stb::gemm_xs_bytes(m, T) + (minimum ? stb::gemm_bytes(n, m, T, ktok).mandatory : stb::gemm_preferred(n, m, T, ktok));
   return STB_OK;
 }
 
-extern "C" int stb_gemm_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, false); }
-extern "C" int stb_gemm_workspace_min(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, true); }
-extern "C" int stb_gemm_f16_workspace(int n, int m, int N, int T, size_t* bytes) {
-  return T <= stb::BatchCfg::kTok ? gemm_workspace_impl<stb::BatchCfg>(n, m, N, T, bytes, false) : gemm_workspace_impl<stb::PrefillCfg>(n, m, N, T, bytes, false);
-}
+extern "C" int stb_gemm_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::gemm_promise(false, T), bytes, false); }
+extern "C" int stb_gemm_workspace_min(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::gemm_promise(false, T), bytes, true); }
+extern "C" int stb_gemm_f16_workspace(int n, int m, int N, int T, size_t* bytes) { return gemm_workspace_impl(n, m, N, T, stb::gemm_promise(true, T), bytes, false); }
 
 static int gemm_check_args(const void* packed, int n, int m, int N, const void* X, int T, size_t ldx, void* Y, size_t ldy) {
   if (!packed || !X || !Y) return STB_ERR_ARG;

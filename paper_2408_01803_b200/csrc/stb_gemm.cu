@@ -437,19 +437,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   const int kz = split ? (cta - full_tiles) % ksplit : 0;
   const int tt = tile % ttiles, mt = tile / ttiles;
   const int b0 = split ? kz * bps : 0, b1 = split ? min(nblk, b0 + bps) : nblk;
-  // Everything the prologue needs from global memory is asked for at once: the table, the header, the word counts, and (into
-  // L2) the first block each decode warp will read.  Where things lie follows from the shape alone; the header is only checked.
+  // The header first (a buffer packed for another shape must not be read as this one), then at once what the rest of the
+  // prologue needs: the word counts and, into L2, the first block each decode warp will read.
   const Header* hdr = reinterpret_cast<const Header*>(packed);
   const BlockInfo* binfo_k = reinterpret_cast<const BlockInfo*>(packed + sizeof(Header));
-  if (warp < kDecodeWarps) {
+  const bool fits = header_matches(hdr, n, m, N);
+  if (fits && warp < kDecodeWarps) {
     const int q = warp & 3, b = b0 + (warp >> 2), rtile = mt * 4 + q;
     if (b < b1 && rtile < ntile && lane * 128 < (int)tile_bytes(N))
       asm volatile("prefetch.global.L2 [%0];" ::"l"(packed + tiles_offset(nblk) + ((size_t)rtile * nblk + b) * tile_bytes(N) + lane * 128));
   }
-  const bool fits = header_matches(hdr, n, m, N);
   const uint32_t nrw = hdr->nrw;
   uint32_t rw0 = 0, rw1 = 0;
-  if (b0 < b1) { rw0 = __ldg(&binfo_k[b0].rw_off); rw1 = b1 < nblk ? __ldg(&binfo_k[b1].rw_off) : nrw; }
+  if (fits && b0 < b1) { rw0 = __ldg(&binfo_k[b0].rw_off); rw1 = b1 < nblk ? __ldg(&binfo_k[b1].rw_off) : nrw; }
 
   const uint32_t sbase = smem_u32(smem);
   // A ring: full = the four decode warps of the stage's block have written it, empty = the tensor core has read it;

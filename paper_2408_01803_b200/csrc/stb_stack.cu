@@ -45,10 +45,9 @@
 #include "stb_decode.cuh"
 #include "stb_layout.cuh"
 #include "stb_ptx.cuh"
+#include "stb_tile.cuh"
 
 namespace stb {
-
-__device__ const Meta6Joint g_meta6_joint = make_meta6_joint();
 
 constexpr int kSWarps = 16;
 constexpr int kSThreads = kSWarps * 32;       // the decoding warps; the copies are issued by one warp of a fifth warpgroup,
@@ -63,10 +62,6 @@ constexpr uint32_t kSlotBytes = kSlotTiles + kSChunk * (kResidA2Bytes + kMaxResi
 static_assert(kSlotBytes % 128 == 0, "slots stay 128-byte aligned");
 constexpr long long kSWaitLimit = 2000000000ll;        // about a second of SM clocks
 constexpr long long kSSelftestLimit = 100000ll;
-constexpr uint32_t kImgWordsPerBlock = 96;    // 6:8 operand-order image: words per block and batch row
-constexpr uint32_t kXPad = 64;                // bytes between the rows of the plain copy beyond 2 m: the eight lane groups' loads do not conflict
-constexpr uint32_t kPosCopies = 16;           // copies of a position table, lane-minor: the look-ups of 16 lanes never conflict
-constexpr uint32_t kPosBytes = kPosTableEntries * kPosCopies * 8;
 
 struct StackPhase {
   const uint8_t* packed[kMaxFusedSteps];
@@ -105,14 +100,13 @@ struct StackParams {
 // shared memory: joint 6:8 metadata table first (784 x 16 B, at offset 0: a pair field of a tile is the shared-memory
 // address of its entry), when a phase needs it; then, from `base`:
 struct SSmem {
-  static constexpr uint32_t meta6_bytes = kMasks6 * kMasks6 * 16;
   static constexpr uint32_t full = 0;                                          // ring barriers, 16 warps x 2: copies landed ...
   static constexpr uint32_t empty = full + 8 * kSWarps * kSDepth;              // ... and slot read
   static constexpr uint32_t ctl = empty + 8 * kSWarps * kSDepth;               // control words
   static constexpr uint32_t slots = ctl + 64;                                  // row tiles of the partial slots: 32 x 4 B
   static constexpr uint32_t chunks = slots + 2 * kSWarps * 4;                  // what each ring slot holds: 32 x 16 B
   static constexpr uint32_t zero = chunks + kSWarps * kSDepth * 16;            // 384 bytes of zeros: the activations of lanes beyond the batch
-  static constexpr uint32_t range = zero + 384;                                // this CTA's tiles of every phase
+  static constexpr uint32_t range = zero + kZeroBytes;                                // this CTA's tiles of every phase
   static constexpr uint32_t nrw = range + 32 * kMaxPhases;                     // residual words per row tile of every step
   static constexpr uint32_t bytes = nrw + 4 * kMaxPhases * kMaxFusedSteps;
 };
@@ -138,18 +132,7 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const void* p) {
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-// product of two fp16 pairs given and returned as bit patterns
-__device__ __forceinline__ uint32_t hmul2_bits(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
 // Coherent loads of activations (written by this kernel, so never through the read-only path)
-__device__ __forceinline__ uint4 ldg_v4_coherent(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ uint32_t ldg_u16_coherent(const void* p) {
   unsigned short v;
   asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
@@ -170,15 +153,6 @@ __device__ __forceinline__ uint32_t silu_mul_bits(uint32_t a, uint32_t b) {
   const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&a)), fb = __half22float2(*reinterpret_cast<const __half2*>(&b));
   const __half2 r = __floats2half2_rn(silu_mul(fa.x, fb.x), silu_mul(fa.y, fb.y));
   return *reinterpret_cast<const uint32_t*>(&r);
-}
-// where column c of block b stands in the staged activations of a batch row, in halves: in operand order (6:8), word
-// ((t 2 + sl) 3 + i) 4 + u of a block = operand register u of chunk i of step sl of lane t, or plainly
-__device__ __forceinline__ uint32_t image_word(uint32_t b, uint32_t group) {
-  return b * kImgWordsPerBlock + (4u * (group & 1u) + ((group >> 2) & 1u)) * 12u + 2u * (group >> 3) + ((group >> 1) & 1u);
-}
-__device__ __forceinline__ uint32_t staged_index(bool image, uint32_t b, uint32_t c) {
-  const uint32_t pr = (c >> 1) & 3u;
-  return image ? 2u * (image_word(b, c >> 3) + (pr < 3u ? 4u * pr : 32u)) + (c & 1u) : b * (uint32_t)kBlock + c;
 }
 // the activations of a residual word's four columns (the bytes of `cols`), as two fp16 pairs
 __device__ __forceinline__ uint2 word_x(const __half* x, const __half* x2, uint32_t cols) {
@@ -360,137 +334,22 @@ struct WarpEnv {
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSThreads) : "memory"); }
 
 // ------------------------------------------------------------------------------------------
-// One 32 x 128 tile at 6:8 through the sparse instruction: the weights stay in rank order and the instruction places
-// them (stb_decode.cuh, meta6_nibble).  x: the lane's place in the operand-order image.
-struct Tile6 { LaneTile<6> lt; uint32_t fld[8]; };
-__device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, Tile6& d) {
-  load_lane_tile<6>(tile, lane, d.lt, true);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) d.fld[k] = *reinterpret_cast<const uint16_t*>(tile + lane * 16 + 2 * k);
-}
-__device__ __forceinline__ void tile_mul(const Tile6& d, const uint8_t* smem, const uint8_t* x, float (&acc)[2][4]) {
-  FastRows<6> fr;
-  fr.init(d.lt, d.lt.A, d.lt.B);
-  // Metadata: fld[4 bb + tq] is the pair field (= the address of the joint-table entry) of slot 2 h + bb of lane tq of
-  // the quad, for the two rows whose metadata this lane supplies; word i of the entries, shifted to the lane's
-  // nibble and added (multiply-adds: the integer pipe is the busy one), is the metadata of chunk i.
-  uint32_t E[2][3];
-#pragma unroll
-  for (int bb = 0; bb < 2; ++bb) {
-    uint4 en[4];
-#pragma unroll
-    for (int tq = 0; tq < 4; ++tq) en[tq] = *reinterpret_cast<const uint4*>(smem + d.fld[4 * bb + tq]);
-    E[bb][0] = ((en[3].x * 16u + en[2].x) * 16u + en[1].x) * 16u + en[0].x;
-    E[bb][1] = ((en[3].y * 16u + en[2].y) * 16u + en[1].y) * 16u + en[0].y;
-    E[bb][2] = ((en[3].z * 16u + en[2].z) * 16u + en[1].z) * 16u + en[0].z;
-  }
-  // the activations of the tile's six chunk positions, once for both halves of the rows
-  uint4 bxs[2][3];
-#pragma unroll
-  for (int sl = 0; sl < 2; ++sl)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) bxs[sl][i] = *reinterpret_cast<const uint4*>(x + sl * 48 + 16 * i);
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    uint32_t XLh[2][2], XHh[2][2];
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj)
-#pragma unroll
-      for (int sp = 0; sp < 2; ++sp) fr.high(2 * mt + jj, sp, XLh[jj][sp], XHh[jj][sp]);
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      uint32_t R[2][2][3];
-#pragma unroll
-      for (int jj = 0; jj < 2; ++jj)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) fr.pairs(2 * mt + jj, 2 * h + sl, XLh[jj][h], XHh[jj][h], R[jj][h]);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const uint4 bx = bxs[sl][i];
-        if (mt == 0) mma_sp16832<0>(acc[0], R[0][0][i], R[1][0][i], R[0][1][i], R[1][1][i], bx.x, bx.y, bx.z, bx.w, E[sl][i]);
-        else mma_sp16832<1>(acc[1], R[0][0][i], R[1][0][i], R[0][1][i], R[1][1][i], bx.x, bx.y, bx.z, bx.w, E[sl][i]);
-      }
-    }
-  }
-}
-
-// One tile in position order (N = 4, 5, 6): byte-permute decode into m16n8k16 operands.  The position selectors are looked
-// up by keep-mask index: where a lane's mask bytes are its slots' indices they are loaded one by one (the load pipe has
-// room, the integer pipe has not), and each of 16 lanes has a copy of the table in its own pair of banks.
-template <int N>
-struct TileD { LaneTile<N> lt; uint2 P[16]; };
-template <int N>
-__device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, const uint8_t* ptab, uint32_t prow, TileD<N>& d) {
-  load_lane_tile<N>(tile, lane, d.lt);
-#pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const uint32_t idx = mask_pairs(N) ? keep_index_of(d.lt.mask, u >> 2, u & 3) : (uint32_t)tile[lane * 16 + u];
-    d.P[u] = *reinterpret_cast<const uint2*>(ptab + idx * prow);
-  }
-}
-// x: the lane's activations of the block, in shared memory (kStaged) or global
-template <int N, bool kStaged>
-__device__ __forceinline__ void tile_mul(const TileD<N>& d, const uint8_t* x, float (&acc)[2][4]) {
-  FastRows<N> fr;
-  fr.init(d.lt, d.lt.A, d.lt.B);
-  uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
-  if (N == 5) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) fr.high(j, 0, XL[j], XH[j]);
-  }
-  uint4 xf[4];
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    if (kStaged) xf[s] = *reinterpret_cast<const uint4*>(x + s * 64);
-    else {
-      xf[s] = make_uint4(0, 0, 0, 0);
-      if (x) xf[s] = ldg_v4_coherent(x + s * 64);
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    uint32_t f[4][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (N == 6 && (s & 1) == 0) fr.high(j, s >> 1, XL[j], XH[j]);
-      fr.slot2(j, s, d.P[4 * j + s].x, d.P[4 * j + s].y, XL[j], XH[j], f[j]);
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      mma16816(acc[mt], f[2 * mt][0], f[2 * mt + 1][0], f[2 * mt][1], f[2 * mt + 1][1], xf[s].x, xf[s].y);
-      mma16816(acc[mt], f[2 * mt][2], f[2 * mt + 1][2], f[2 * mt][3], f[2 * mt + 1][3], xf[s].z, xf[s].w);
-    }
-  }
-}
-
 // Residual term of a chunk: its residual words, four (16 salient slots) per tensor-core step, lane t the t-th.  rec: the
 // chunk's records; na / nw: words of its first block / of all; xw: activations of the chunk's first word for the lane's
 // batch row, xw_step bytes per word.  kGather false: they are fetched one by one (word table entry, then x).
 template <bool kGather>
 __device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint32_t nw, int g, int t, const uint8_t* xw, uint32_t xw_step,
-                                          const ResidWord* rwt, const __half* xg, const __half* xg2, float (&acc)[2][4]) {
+                                          const ResidWord* rwt, const __half* xg, const __half* xg2, float (&acc)[2][1][4]) {
 #pragma unroll 1
   for (uint32_t k0 = 0; k0 < nw; k0 += 4u) {
     const uint32_t kk = k0 + (uint32_t)t, k = min(kk, nw - 1u);
     const bool second = k >= na;
     // records: a_sal2 of the 32 rows, then the block's words
     const uint8_t* r = rec + k * kResidWordBytes + (second ? 2u * kResidA2Bytes : kResidA2Bytes);
-    uint32_t rw = *reinterpret_cast<const uint32_t*>(r + 4 * g);
+    uint32_t rw = *reinterpret_cast<const uint32_t*>(r + 4 * g), fa[4][2];
     const uint2 a2 = *reinterpret_cast<const uint2*>(rec + (second ? kResidA2Bytes + na * kResidWordBytes : 0u) + 8 * g);
-    if (kk >= nw) rw = 0x55555555u;
-    // operand registers of the lane's four rows: the two-bit codes pick the high byte of +1, 0 or -1 (one byte
-    // permute per row), two more spread them to fp16 pairs, and one fp16 multiply per register (not on the
-    // busy integer pipe) scales them by the row's a_sal2: exact, the factors are +-1 and 0
-    uint32_t fa[4][2];
-    const uint32_t code_lo = rw & 0x33333333u, code_hi = (rw >> 2) & 0x33333333u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t codes = (j & 2) ? code_hi : code_lo;
-      const uint32_t unit = prmt(0x00BC003Cu, 0u, (j & 1) ? (codes >> 16) : codes);          // high bytes of +1, 0, -1, 0 by code
-      const uint32_t s2 = prmt((j & 2) ? a2.y : a2.x, 0u, (j & 1) ? 0x3232u : 0x1010u);     // (a_sal2, a_sal2) of row j
-      fa[j][0] = hmul2_bits(prmt(unit, 0u, 0x1404u), s2);
-      fa[j][1] = hmul2_bits(prmt(unit, 0u, 0x3424u), s2);
-    }
+    if (kk >= nw) rw = kNoTerms;
+    resid_operands(rw, a2, fa);
     uint2 xr = make_uint2(0, 0);
     if (kGather) xr = *reinterpret_cast<const uint2*>(xw + k * xw_step);
     else if (xg) {
@@ -498,8 +357,8 @@ __device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint3
       const size_t o = (size_t)(e.x >> 3) * kBlock;
       xr = word_x(xg + o, xg2 ? xg2 + o : nullptr, e.y);
     }
-    mma16816(acc[0], fa[0][0], fa[1][0], fa[0][1], fa[1][1], xr.x, xr.y);
-    mma16816(acc[1], fa[2][0], fa[3][0], fa[2][1], fa[3][1], xr.x, xr.y);
+    mma16816(acc[0][0], fa[0][0], fa[1][0], fa[0][1], fa[1][1], xr.x, xr.y);
+    mma16816(acc[1][0], fa[2][0], fa[3][0], fa[2][1], fa[3][1], xr.x, xr.y);
   }
 }
 
@@ -529,11 +388,11 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
   const uint8_t* xs = xlive ? E.smem + P.xs_off + (uint32_t)g * 8u : zero;
   const uint8_t* ptab = kImage ? nullptr : E.smem + P.pos_off[N - 4] + (uint32_t)(lane & (kPosCopies - 1)) * 8u;
   const uint32_t prow = P.pos_row;
-  float acc[2][4];
+  float acc[2][1][4];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int d = 0; d < 4; ++d) acc[a][d] = 0.0f;
+    for (int d = 0; d < 4; ++d) acc[a][0][d] = 0.0f;
   uint4 c;
   do {
     const uint32_t slot = W.slot, bar = E.full + 8u * slot;
@@ -554,17 +413,18 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
     const int cnt = (int)(c.x & 3u);
 #pragma unroll 1
     for (int k = 0; k < cnt; ++k) {
+      const uint8_t* const xp[1] = {xb};
       // once the slot's last tile is in registers the slot is handed back
       if constexpr (kImage) {
         Tile6 d;
         load_tile(tile, lane, d);
         if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
-        tile_mul(d, E.smem, xb, acc);
+        tile_mul<1>(d, E.smem, xp, acc);
       } else {
         TileD<N> d;
         load_tile<N>(tile, lane, ptab, prow, d);
         if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
-        tile_mul<N, kStaged>(d, xb, acc);
+        tile_mul<N, kStaged, 1>(d, xp, acc);
       }
       tile += tb;
       xb += xstep;
@@ -582,8 +442,8 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
           for (int d = 0; d < 4; ++d) {
             const int row = rt * kTileRows + g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
             if (row < q.n[si] && bc < batch) {
-              if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(acc[mt][d]);
-              else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = acc[mt][d];
+              if (f16) static_cast<__half*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = __float2half_rn(acc[mt][0][d]);
+              else static_cast<float*>(q.y[si])[(size_t)bc * q.ldy[si] + row] = acc[mt][0][d];
             }
           }
       } else {
@@ -595,14 +455,14 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
 #pragma unroll
           for (int d = 0; d < 4; ++d) {
             const int r = g + 16 * mt + 8 * (d >> 1), bc = 2 * t + (d & 1);
-            if (bc < batch) pd[r * batch + bc] = acc[mt][d];
+            if (bc < batch) pd[r * batch + bc] = acc[mt][0][d];
           }
         if (lane == 0) pslot[ps] = (int)c.w;
       }
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int d = 0; d < 4; ++d) acc[a][d] = 0.0f;
+        for (int d = 0; d < 4; ++d) acc[a][0][d] = 0.0f;
     }
   } while (!(c.x & kRunEnd));
 }
@@ -754,10 +614,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
         }
         const int r = batch == 1 ? 0 : cur / per_row, qq = cur - r * per_row;
         if (q.use_image == 1) {
-          // operand order: lanes t = 2 (G & 1) + p read word i + p of group G as chunk i: words 0..2 for p = 0, 1..3 for p = 1
-          uint32_t* d = ximg + (uint32_t)r * ((uint32_t)nb * kImgWordsPerBlock) + image_word((uint32_t)qq >> 4, (uint32_t)qq & 15u);
-          d[0] = a[0]; d[4] = a[1]; d[8] = a[2];
-          d[24] = a[1]; d[28] = a[2]; d[32] = a[3];
+          image_store(ximg + (uint32_t)r * ((uint32_t)nb * kImgWordsPerBlock), (uint32_t)qq >> 4, (uint32_t)qq & 15u, a);
         } else {
           *reinterpret_cast<uint4*>(smem + P.x_off + (uint32_t)r * (2u * (uint32_t)q.m + kXPad) + (uint32_t)qq * 16u) = make_uint4(a[0], a[1], a[2], a[3]);
         }
@@ -875,7 +732,7 @@ __global__ void __launch_bounds__(kSAllThreads, 1)
 stack_kernel(const __grid_constant__ StackParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int cta = (int)blockIdx.x, G = (int)gridDim.x;
-  uint8_t* base = smem + (P.use_meta6 ? SSmem::meta6_bytes : 0u);
+  uint8_t* base = smem + (P.use_meta6 ? kMeta6Bytes : 0u);
   volatile int* ctl = reinterpret_cast<volatile int*>(base + SSmem::ctl);      // [0] failed, [1] straddling row tiles this CTA finished, [2] last CTA out, [3] a packed header does not match
   int* pslot = reinterpret_cast<int*>(base + SSmem::slots);
   float* pdata = reinterpret_cast<float*>(smem + P.pdata_off);
@@ -922,7 +779,7 @@ __global__ void __launch_bounds__(kSAllThreads, 1)
 checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __restrict__ sums, int first_step) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31;
-  uint8_t* base = smem + (P.use_meta6 ? SSmem::meta6_bytes : 0u);
+  uint8_t* base = smem + (P.use_meta6 ? kMeta6Bytes : 0u);
   volatile int* ctl = reinterpret_cast<volatile int*>(base + SSmem::ctl);
   if (!stack_setup(P, base, ctl)) {
     if (threadIdx.x == 0 && blockIdx.x == 0 && P.dev_status) *P.dev_status = STB_ERR_CORRUPT;
@@ -1045,7 +902,7 @@ static int plan_smem(StackParams& sp, bool image) {
   for (int round = 0;; ++round) {
     uint32_t o = 0;
     sp.use_meta6 = any6 ? 1 : 0;
-    if (any6) o = SSmem::meta6_bytes;
+    if (any6) o = kMeta6Bytes;
     o += SSmem::bytes;
     for (int k = 0; k < 3; ++k) {
       sp.pos_off[k] = 0;

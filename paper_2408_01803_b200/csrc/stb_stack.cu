@@ -9,10 +9,10 @@
 //     the SM time used) every CTA gets whole row tiles and no sum crosses CTAs; otherwise the ranges are equal
 //     in tiles and a row tile may straddle CTAs.
 //   * Each warp's tiles stream through a private ring in shared memory (two slots of up to two tiles and their
-//     residual records, two 1-D bulk copies each, mbarrier completion, bounded waits).  A seventeenth warp issues the
-//     copies, one lane per ring, and runs ahead into the NEXT phases: packed weights never depend on activations, so the
-//     stream does not stop at a phase boundary.  It also works out where a chunk belongs (row tile, first block, residual
-//     words, end of a run) and leaves that beside the slot, so that the other warps only wait, decode and multiply.
+//     residual records, two 1-D bulk copies each, mbarrier completion, bounded waits).  Four more warps issue the
+//     copies, one lane per ring, and run ahead into the NEXT phases: packed weights never depend on activations, so the
+//     stream does not stop at a phase boundary.  They also work out where a chunk belongs (row tile, first block, residual
+//     words, end of a run) and leave that beside the slot, so that the other warps only wait, decode and multiply.
 //   * Decode and multiply per tile: 6:8 keeps the weights in rank order and lets mma.sp.m16n8k32 place them
 //     (activations from an image of x in operand order in shared memory, built once per phase and CTA); 4:8 and 5:8
 //     (and 6:8 when the image does not fit) decode to position order for mma.m16n8k16 with the activations from a
@@ -50,7 +50,7 @@
 namespace stb {
 
 constexpr int kSWarps = 16;
-constexpr int kSThreads = kSWarps * 32;       // the decoding warps; the copies are issued by one warp of a fifth warpgroup,
+constexpr int kSThreads = kSWarps * 32;       // the decoding warps; the copies are issued by a fifth warpgroup,
 constexpr int kSAllThreads = kSThreads + 128; // which gives registers up to the other four: 640 x 96 at launch, then
 constexpr int kDecodeRegs = 104, kFeedRegs = 64;   // 512 x 104 + 128 x 64 of them
 static_assert(kSThreads * kDecodeRegs + 128 * kFeedRegs <= kSAllThreads * 96, "register split within the launch's total");
@@ -265,10 +265,11 @@ struct TileWalk {
   }
 };
 
-// The copying warp: lane w feeds the ring of warp w.  A slot is refilled when its reader has arrived on its empty barrier;
+// The copying warps, one per scheduler so that none of them loses more issue slots to copying than the others: lane l of
+// the i-th feeds the ring of warp 4 l + i.  A slot is refilled when its reader has arrived on its empty barrier;
 // the wait has no limit of its own (a reader may be waiting for other CTAs) but ends with the CTA's failed flag.
 __device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, uint8_t* base, volatile int* ctl) {
-  const int w = threadIdx.x & 31;
+  const int w = 4 * (int)(threadIdx.x & 31) + (int)((threadIdx.x >> 5) & 3u);
   const CtaRange* range = reinterpret_cast<const CtaRange*>(base + SSmem::range);
   const uint32_t* nrw = reinterpret_cast<const uint32_t*>(base + SSmem::nrw);
   if (w >= kSWarps) return;
@@ -282,7 +283,7 @@ __device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, 
     const uint32_t slot = k % kSDepth;
     if (k >= kSDepth && !mbar_try_wait(empty + 8u * slot, (k / kSDepth - 1u) & 1u)) {
       if (ctl[0]) return;
-      __nanosleep(20);
+      __nanosleep(100);               // (a slot lasts its reader about 3 us)
       continue;
     }
     const StackPhase& q = P.ph[t.phase];
@@ -737,15 +738,17 @@ stack_kernel(const __grid_constant__ StackParams P) {
   int* pslot = reinterpret_cast<int*>(base + SSmem::slots);
   float* pdata = reinterpret_cast<float*>(smem + P.pdata_off);
 
+  grid_dependency_wait();          // a programmatic dependent of whatever ran before (see the launch): nothing in memory is touched until that is done
   if (!stack_setup(P, base, ctl)) {          // before anything was streamed or the workspace touched
     if (threadIdx.x == 0 && cta == 0 && P.dev_status) *P.dev_status = STB_ERR_CORRUPT;
     return;
   }
   if (threadIdx.x == 0) { ctl[0] = 0; ctl[1] = 0; ctl[2] = 0; }
   __syncthreads();
+  grid_launch_dependents();
   if (threadIdx.x >= kSThreads) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFeedRegs));
-    if ((threadIdx.x >> 5) == kSWarps) feed_rings(P, smem, base, ctl);
+    feed_rings(P, smem, base, ctl);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDecodeRegs));
     decode_phases(P, smem, base, ctl, pslot, pdata, cta);
@@ -789,7 +792,7 @@ checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __res
   __syncthreads();
   const int warp = threadIdx.x >> 5;
   bool failed = false;
-  if (warp >= kSWarps) { if (warp == kSWarps) feed_rings(P, smem, base, ctl); }
+  if (warp >= kSWarps) feed_rings(P, smem, base, ctl);
   else {
     const uint8_t* ring = smem + P.ring_off + (size_t)warp * kSDepth * kSlotBytes;
     const uint4* chunk = reinterpret_cast<const uint4*>(base + SSmem::chunks) + kSDepth * warp;
@@ -1079,10 +1082,14 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
     cfg.blockDim = dim3((unsigned)stb::kSAllThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    // programmatic: the launch is prepared while the kernel before it drains, and its CTAs start as that one's leave (each
+    // waits in its first instructions until all of it is complete)
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, stb::stack_kernel, sp) != cudaSuccess) return STB_ERR_CUDA;
   }
   return STB_OK;

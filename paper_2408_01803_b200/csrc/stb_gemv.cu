@@ -9,6 +9,7 @@
 #include "stb_decode.cuh"
 #include "stb_layout.cuh"
 #include "stb_ptx.cuh"
+#include "stb_tile.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -17,7 +18,7 @@ namespace stb {
 __device__ const Meta6Table g_meta6 = make_meta6_table();
 
 // ------------------------------------------------------------------------------------------
-// Tensor-core GEMV, N = 4, 5, 6, batch <= 8 NB (NB = 1, 2, 4, 8).
+// Tensor-core GEMV of small layers and of 9 to 64 batch rows, N = 4, 5, 6, batch <= 8 NB (NB = 1, 2, 4, 8).
 //
 // Grid: one thread-block cluster of `ksplit` CTAs per row tile (32 rows); CTA k of the cluster
 // takes the k-th slice of the 128-column blocks and its warps take contiguous runs of that
@@ -48,10 +49,9 @@ struct GemvSmem {
 // N = 6, up to two batch rows: the CTA's slice of the activations is kept in shared memory in the order the lanes
 // consume it: per block and batch row 96 words, word ((t * 2 + sl) * 3 + i) * 4 + u = operand register u of chunk i
 // of step sl of lane t (two fp16 each).
-constexpr uint32_t kImgWords = 96;
 constexpr uint32_t kImgMaxBytes = 20 * 1024;
 __host__ __device__ inline uint32_t gemv_image_bytes(int N, int NB, int batch, int bpp) {
-  const uint32_t bytes = (uint32_t)batch * (uint32_t)bpp * kImgWords * 4u;
+  const uint32_t bytes = (uint32_t)batch * (uint32_t)bpp * kImgWordsPerBlock * 4u;
   return (N == 6 && NB == 1 && batch <= 2 && bytes <= kImgMaxBytes) ? bytes : 0u;
 }
 __host__ __device__ inline GemvSmem gemv_smem(int N, int warps, int ksplit, int NB, uint32_t image_bytes) {
@@ -157,7 +157,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
   grid_launch_dependents();
   x = after_dependency_wait(x);
   const uint32_t* ximg = reinterpret_cast<const uint32_t*>(smem + L.ximg);
-  const uint32_t img_row_words = (uint32_t)bpp * kImgWords;
+  const uint32_t img_row_words = (uint32_t)bpp * kImgWordsPerBlock;
   if (N == 6 && NB == 1 && image_bytes != 0u) {
     // one item = the 8 activations of one group of one block of one batch row: a 16-byte load, six 4-byte stores
     // (lanes t = 2 (G & 1) + p read word i + p of group G as chunk i: words 0..2 for p = 0, words 1..3 for p = 1)
@@ -179,7 +179,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
         const int it = base + k * (int)blockDim.x + (int)threadIdx.x;
         if (it < items) {
           const int r = it / (nbp * 16), q = it - r * nbp * 16, blk = q >> 4, G = q & 15;
-          uint32_t* d = img + (uint32_t)r * img_row_words + (uint32_t)blk * kImgWords +
+          uint32_t* d = img + (uint32_t)r * img_row_words + (uint32_t)blk * kImgWordsPerBlock +
                         (uint32_t)((4 * (G & 1) + ((G >> 2) & 1)) * 12 + 2 * (G >> 3) + ((G >> 1) & 1));
           d[0] = v[k].x; d[4] = v[k].y; d[8] = v[k].z;
           d[24] = v[k].y; d[28] = v[k].z; d[32] = v[k].w;
@@ -273,7 +273,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
       if (image_bytes != 0u) {
         // activations from the CTA's image in shared memory: two rows of the lane at a time (fewer live registers;
         // the 16-byte operand loads are cheap enough to be issued once per row pair)
-        const uint32_t* xi0 = ximg + (uint32_t)g * img_row_words + (uint32_t)(b - b0) * kImgWords + (uint32_t)(t * 24);
+        const uint32_t* xi0 = ximg + (uint32_t)g * img_row_words + (uint32_t)(b - b0) * kImgWordsPerBlock + (uint32_t)(t * 24);
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
           uint32_t XLh[2][2], XHh[2][2];
@@ -496,6 +496,380 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// The GEMV of larger layers, N = 4, 5, 6, up to 16 batch rows (8 NB).
+//
+// Grid: Q thread-block clusters of `ksplit` CTAs, one CTA of 16 warps per SM.  CTA k of a cluster takes the k-th slice of the
+// 128-column blocks of ALL row tiles of the cluster, so that its slice of the activations is staged in shared memory once and
+// used for every row tile; its 32 x 128 tiles, in (row tile, block) order, are dealt to the warps as equal contiguous runs.
+// gemv_plan takes the split for which the fullest CTA has least to do.
+// Each warp streams its tiles and their residual records from HBM into a private ring (two slots of one or two tiles) with 1-D
+// bulk copies, and decodes and multiplies them on the tensor cores, fp32 accumulators in registers (stb_tile.cuh):
+//   N = 4, 5        position-order decode, m16n8k16, activations from a plain copy in shared memory
+//   N = 6           rank order through the 2:4 sparse instruction, activations from an image in operand order (position order
+//                   where the image does not fit)
+// The residual term of a chunk of tiles goes through the dense instruction with 16 salient slots as K; the columns behind the
+// residual words of the slice are turned into places in the staged activations once per CTA.
+// Sums: a warp writes the rows it begins to shared memory and the piece it continues beside it; the CTA adds them in order, the
+// cluster adds its CTAs' sums through distributed shared memory, in order.
+// What bounds it: the decode (about 175 clocks per tile and SM, integer issue), and a chain of latencies before and after it
+// (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small layers stay with gemv_mma_kernel).
+// Against that kernel, cold L2, microseconds: 28672 x 8192 4:8 batch 1 58.9 -> 48.1, 5120 x 13824 5:8 batch 8 32.6 -> 25.3,
+// 4096 x 11008 6:8 batch 1 20.0 -> 16.4, 11008 x 4096 6:8 batch 16 24.1 -> 20.0, 4096 x 4096 4:8 batch 1 11.3 -> 9.7.
+constexpr int kGWarps = 16, kGThreads = kGWarps * 32;
+__device__ __forceinline__ int layer_of(const GemvLayers& layers, int rt) {
+  int li = 0;
+#pragma unroll
+  for (int i = 1; i < kMaxFused; ++i)
+    if (i < layers.count && rt >= layers.tile_start[i]) li = i;
+  return li;
+}
+
+// Split and shared memory of a launch (byte offsets; the 6:8 metadata table or the position table comes first).
+struct GemvPlan {
+  int ksplit, clusters, bs, chunk, image;             // bs: blocks per slice; chunk: tiles per ring slot
+  uint32_t zero, bars, masks, head, part, roff, wtab, ring, slot, x, xpitch, total;
+};
+constexpr uint32_t kGemvSmem = 227 * 1024;
+static inline uint32_t gemv_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
+static bool gemv_layout(GemvPlan& p, int N, int batch, int rows, int layers, int image, int chunk) {
+  p.image = image; p.chunk = chunk;
+  uint32_t o = image ? kMeta6Bytes : kPosBytes;
+  p.zero = gemv_up(o, 128) + (image ? kImgPad : kXPad); o = gemv_up(p.zero + kZeroBytes, 16);
+  p.bars = o; o += kGWarps * 2 * 8;
+  p.masks = o; o += gemv_up((uint32_t)rows * 4u, 16);                         // per row tile: the warps that continue it
+  p.head = gemv_up(o, 16); o = p.head + (uint32_t)(kGWarps * 32 * batch) * 4u;                       // sums of the row tile a warp continues
+  const unsigned long long part = 128ull * (unsigned long long)rows * batch;   // sums of the CTA's row tiles
+  const unsigned long long roff = 4ull * (unsigned long long)layers * (p.bs + 1), wtab = 64ull * (unsigned long long)layers * p.bs;
+  p.xpitch = image ? (uint32_t)p.bs * kImgWordsPerBlock * 4u + kImgPad : (uint32_t)p.bs * 256u + kXPad;
+  if (part + roff + wtab + (unsigned long long)p.xpitch * batch > kGemvSmem || p.bs * 256 > 65535) return false;
+  p.part = gemv_up(o, 16); o = p.part + (uint32_t)part;
+  p.roff = o; o += (uint32_t)roff;                                             // residual words before every block of the slice, per layer
+  p.wtab = gemv_up(o, 16); o = p.wtab + (uint32_t)wtab;                        // places of the four activations of every residual word
+  p.slot = gemv_up((uint32_t)chunk * (tile_bytes(N) + kResidA2Bytes + kMaxResidWords * kResidWordBytes), 128);
+  p.ring = gemv_up(o, 128); o = p.ring + kGWarps * 2 * p.slot;
+  p.x = o; o += p.xpitch * (uint32_t)batch;
+  p.total = o;
+  return o <= kGemvSmem;
+}
+
+// The tiles of a warp as its copies see them.
+struct GemvWalk {
+  int left, row, blk;             // tiles left; row tile (of the CTA) and block (of the slice) of the next one
+  const uint8_t* tiles;           // of the row tile's slice
+  const uint8_t* recs;            // of the row tile, at the slice's first a_sal2
+  const uint32_t* roff;           // of the row tile's layer
+};
+
+template <int N, int NB, bool kImage>
+__global__ void __launch_bounds__(kGThreads, 1)
+gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_constant__ GemvPlan P, int m, const __half* x, int batch, size_t ldx,
+                   int* dev_status, long long wait_limit, int copies_off, int chained) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3, tid = threadIdx.x;
+  const int nblk = m / kBlock, ksplit = P.ksplit;
+  const int kpart = (int)(blockIdx.x % (unsigned)ksplit), cl = (int)(blockIdx.x / (unsigned)ksplit);
+  const int b0 = kpart * P.bs, nbp = max(min(nblk - b0, P.bs), 0);              // this CTA's slice of the blocks
+  const int R = layers.tile_start[layers.count];
+  const int R0 = (int)((long long)R * cl / P.clusters), rows = (int)((long long)R * (cl + 1) / P.clusters) - R0;   // and the cluster's row tiles
+  constexpr uint32_t tb = tile_bytes(N);
+  // What needs no other memory comes first: the launch is a programmatic dependent of whatever ran before it on the stream.
+  // Within a chain (stb_layer_stack, whose packed layers nobody writes meanwhile) the weights may be read before that is done too.
+  if (kImage) {
+    for (int i = tid; i < (int)(kMasks6 * kMasks6); i += kGThreads) reinterpret_cast<uint4*>(smem)[i] = *reinterpret_cast<const uint4*>(g_meta6_joint.v[i]);
+  } else {
+    for (int i = tid; i < kPosTableEntries * (int)kPosCopies; i += kGThreads) reinterpret_cast<uint2*>(smem)[i] = g_pos_table.v[N][i / (int)kPosCopies];
+  }
+  if (tid < (int)kZeroBytes / 4) reinterpret_cast<uint32_t*>(smem + P.zero)[tid] = 0u;
+  for (int i = tid; i < rows; i += kGThreads) reinterpret_cast<uint32_t*>(smem + P.masks)[i] = 0u;
+  if (!chained) grid_dependency_wait();
+  // a buffer packed for another shape must not be read as this one (every CTA of the grid comes to the same verdict)
+  bool fits = true;
+  uint32_t nrw[kMaxFused];
+#pragma unroll
+  for (int i = 0; i < kMaxFused; ++i)
+    if (i < layers.count) {
+      const Header* h = reinterpret_cast<const Header*>(layers.packed[i]);
+      fits = fits && header_matches(h, layers.n[i], m, N);
+      nrw[i] = h->nrw;
+    }
+  if (!fits) {
+    if (tid == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
+    return;
+  }
+  const uint32_t bar0 = smem_u32(smem + P.bars) + 16u * (uint32_t)warp;
+  const uint32_t ring = smem_u32(smem + P.ring) + (uint32_t)warp * 2u * P.slot;
+  const uint8_t* ringp = smem + P.ring + (size_t)warp * 2u * P.slot;
+  uint32_t* roff_all = reinterpret_cast<uint32_t*>(smem + P.roff);
+  // this warp's run of tiles
+  const int T = rows * nbp, lo = (int)((long long)T * warp / kGWarps), hi = (int)((long long)T * (warp + 1) / kGWarps);
+
+  GemvWalk w;
+  auto enter = [&](int row) {
+    const int rt = R0 + row, li = layer_of(layers, rt), rl = rt - layers.tile_start[li];
+    const int ntile = layers.tile_start[li + 1] - layers.tile_start[li];
+    const uint8_t* base = layers.packed[li] + tiles_offset(nblk);
+    uint32_t words = 0;
+#pragma unroll
+    for (int i = 0; i < kMaxFused; ++i)
+      if (i == li) words = nrw[i];
+    w.tiles = base + ((size_t)rl * nblk + b0) * tb;
+    w.recs = base + (size_t)tb * nblk * ntile + (size_t)rl * resid_rt_bytes(nblk, words) + (size_t)kResidA2Bytes * b0;
+    w.roff = roff_all + li * (P.bs + 1);
+  };
+  auto chunk_of = [&](int left, int blk) { return min(min(P.chunk, left), nbp - blk); };
+  w.left = hi - lo; w.row = nbp > 0 ? lo / nbp : 0; w.blk = lo - w.row * nbp;
+  // The first chunk's tiles at once and its records as soon as its blocks' word counts are here, which the warp asks for itself
+  // (everything later goes by the table below).  A copy may land before its bytes are announced: the barrier's phase cannot
+  // end before that, its one arrival.
+  if (w.left > 0) {
+    enter(w.row);
+    const int c = chunk_of(w.left, w.blk);
+    if (lane == 0) {
+      mbar_init(bar0, 1);
+      mbar_init(bar0 + 8u, 1);
+      fence_async_smem();
+      if (!copies_off) bulk_g2s(ring, w.tiles + (size_t)w.blk * tb, (uint32_t)c * tb, bar0);
+      const BlockInfo* bi = reinterpret_cast<const BlockInfo*>(layers.packed[layer_of(layers, R0 + w.row)] + sizeof(Header)) + b0 + w.blk;
+      const uint32_t w0 = __ldg(&bi[0].rw_off), nw = __ldg(&bi[0].nrw) + (c > 1 ? __ldg(&bi[1].nrw) : 0u), rec_b = (uint32_t)c * kResidA2Bytes + nw * kResidWordBytes;
+      mbar_expect_tx(bar0, (uint32_t)c * tb + rec_b);
+      if (!copies_off) bulk_g2s(ring + (uint32_t)P.chunk * tb, w.recs + (size_t)kResidA2Bytes * w.blk + (size_t)kResidWordBytes * w0, rec_b, bar0);
+    }
+  }
+  for (int i = tid; i < layers.count * (nbp + 1); i += kGThreads) {
+    const int li = i / (nbp + 1), k = i - li * (nbp + 1);
+    const BlockInfo* bi = reinterpret_cast<const BlockInfo*>(layers.packed[li] + sizeof(Header));
+    uint32_t v = 0;
+#pragma unroll
+    for (int q = 0; q < kMaxFused; ++q)
+      if (q == li) v = nrw[q];
+    if (b0 + k < nblk) v = __ldg(&bi[b0 + k].rw_off);
+    roff_all[li * (P.bs + 1) + k] = v;
+  }
+  __syncthreads();
+
+  auto advance = [&](int c) {
+    w.left -= c; w.blk += c;
+    if (w.blk == nbp && w.left > 0) { w.blk = 0; ++w.row; enter(w.row); }
+  };
+  // next chunk of the walk into ring slot `slot`
+  auto issue = [&](uint32_t slot) {
+    if (w.left <= 0) return;
+    const int c = chunk_of(w.left, w.blk);
+    if (lane == 0) {
+      const uint32_t w0 = w.roff[w.blk], nw = w.roff[w.blk + c] - w0;
+      const uint32_t tile_b = (uint32_t)c * tb, rec_b = (uint32_t)c * kResidA2Bytes + nw * kResidWordBytes, bar = bar0 + 8u * slot, dst = ring + slot * P.slot;
+      fence_async_smem();
+      mbar_expect_tx(bar, tile_b + rec_b);
+      // copies off (the wait self-test): the barrier is armed but nothing will ever complete it
+      if (!copies_off) {
+        bulk_g2s(dst, w.tiles + (size_t)w.blk * tb, tile_b, bar);
+        bulk_g2s(dst + (uint32_t)P.chunk * tb, w.recs + (size_t)kResidA2Bytes * w.blk + (size_t)kResidWordBytes * w0, rec_b, bar);
+      }
+    }
+    advance(c);
+  };
+  if (w.left > 0) advance(chunk_of(w.left, w.blk));
+  issue(1u);
+  // where the activations behind the slice's residual words will stand
+  uint2* wtab = reinterpret_cast<uint2*>(smem + P.wtab);
+  for (int li = 0; li < layers.count; ++li) {
+    const uint32_t w0 = roff_all[li * (P.bs + 1)], cnt = roff_all[li * (P.bs + 1) + nbp] - w0;
+    const uint2* rwt = reinterpret_cast<const uint2*>(layers.packed[li] + rwtab_offset(nblk)) + w0;
+    for (uint32_t i = tid; i < cnt; i += kGThreads) {
+      const uint2 e = __ldg(rwt + i);
+      const uint32_t b = (e.x >> 3) - (uint32_t)b0;
+      uint32_t at[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) at[k] = staged_index(kImage, b, (e.y >> (8 * k)) & 0xFFu);
+      wtab[(size_t)li * kMaxResidWords * P.bs + i] = make_uint2(at[0] | (at[1] << 16), at[2] | (at[3] << 16));
+    }
+  }
+
+  // Everything below reads the activations (the previous layer's output) or writes y: wait for the
+  // previous grid of the stream to have completed, then let the next grid start its own prologue.
+  if (chained) grid_dependency_wait();
+  grid_launch_dependents();
+  {
+    const int per_row = nbp * 16, items = batch * per_row;
+#pragma unroll 1
+    for (int first = tid; first < items; first += 4 * kGThreads) {
+      uint4 v[4];
+      uint32_t at[4];                       // batch row and group, for the stores
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int it = first + k * kGThreads, r = batch == 1 ? 0 : it / per_row, q = it - r * per_row;
+        at[k] = ((uint32_t)r << 16) | (uint32_t)q;
+        if (it < items) v[k] = ldg_v4_coherent(x + (size_t)r * ldx + (size_t)b0 * kBlock + (size_t)q * 8);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (first + k * kGThreads < items) {
+          const uint32_t a[4] = {v[k].x, v[k].y, v[k].z, v[k].w}, q = at[k] & 0xFFFFu;
+          uint8_t* row = smem + P.x + (at[k] >> 16) * P.xpitch;
+          if (kImage) image_store(reinterpret_cast<uint32_t*>(row), q >> 4, q & 15u, a);
+          else *reinterpret_cast<uint4*>(row + 16 * q) = v[k];
+        }
+    }
+  }
+  __syncthreads();
+
+  bool failed = false;
+  float* part = reinterpret_cast<float*>(smem + P.part);
+  {
+    const uint8_t* xrow[NB];
+    uint32_t live[NB];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+      live[c] = g + 8 * c < batch ? 0xFFFFFFFFu : 0u;
+      xrow[c] = live[c] ? smem + P.x + (uint32_t)(g + 8 * c) * P.xpitch : smem + P.zero;
+    }
+    const uint32_t xstep = kImage ? kImgWordsPerBlock * 4u : 2u * kBlock, xlane = (uint32_t)t * (kImage ? 96u : 16u);
+    const uint8_t* ptab = smem + (uint32_t)(lane & (kPosCopies - 1)) * 8u;
+    uint32_t slot = 0, parity = 0;
+    int left = hi - lo, row = nbp > 0 ? lo / nbp : 0, blk = lo - row * nbp;
+    while (left > 0 && !failed) {
+      const int first = blk, end = min(nbp, blk + left);
+      const int li = layer_of(layers, R0 + row);
+      const uint32_t* roff = roff_all + li * (P.bs + 1);
+      const uint2* words = wtab + (size_t)li * kMaxResidWords * P.bs;
+      const uint32_t wfirst = roff[0];
+      float acc[2][NB][4];
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = 0; c < NB; ++c)
+#pragma unroll
+          for (int d = 0; d < 4; ++d) acc[a][c][d] = 0.0f;
+      while (blk < end) {
+        const int cnt = chunk_of(left, blk);
+        const uint32_t bar = bar0 + 8u * slot;
+        // all lanes poll; the verdict is made warp-uniform
+        if (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)) && !__all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, wait_limit))) { failed = true; break; }
+        const uint8_t* tile = ringp + slot * P.slot;
+        const uint8_t* rec = tile + (uint32_t)P.chunk * tb;
+        const uint32_t w0 = roff[blk], na = roff[blk + 1] - w0, nw = roff[blk + cnt] - w0;
+        // residual words of the chunk, four (16 salient slots) per tensor-core step, lane t the t-th
+#pragma unroll 1
+        for (uint32_t kk = (uint32_t)t; kk < nw + (uint32_t)t; kk += 4u) {
+          const uint32_t k = min(kk, nw - 1u);
+          const bool second = k >= na;
+          uint32_t rw = *reinterpret_cast<const uint32_t*>(rec + k * kResidWordBytes + (second ? 2u * kResidA2Bytes : kResidA2Bytes) + 4 * g), fa[4][2];
+          const uint2 a2 = *reinterpret_cast<const uint2*>(rec + (second ? kResidA2Bytes + na * kResidWordBytes : 0u) + 8 * g);
+          if (kk >= nw) rw = kNoTerms;
+          resid_operands(rw, a2, fa);
+          const uint2 at = words[w0 - wfirst + k];
+#pragma unroll
+          for (int c = 0; c < NB; ++c) {
+            const uint16_t* xr = reinterpret_cast<const uint16_t*>(xrow[c]);
+            const uint32_t p0 = at.x & live[c], p1 = at.y & live[c];
+            const uint32_t q0 = (uint32_t)xr[p0 & 0xFFFFu] | ((uint32_t)xr[p0 >> 16] << 16), q1 = (uint32_t)xr[p1 & 0xFFFFu] | ((uint32_t)xr[p1 >> 16] << 16);
+            mma16816(acc[0][c], fa[0][0], fa[1][0], fa[0][1], fa[1][1], q0, q1);
+            mma16816(acc[1][c], fa[2][0], fa[3][0], fa[2][1], fa[3][1], q0, q1);
+          }
+        }
+#pragma unroll 1
+        for (int k = 0; k < cnt; ++k) {
+          const uint8_t* xp[NB];
+#pragma unroll
+          for (int c = 0; c < NB; ++c) xp[c] = xrow[c] + xlane + (live[c] & ((uint32_t)(blk + k) * xstep));
+          // once the slot's last tile is in registers the slot is filled again
+          if constexpr (kImage) {
+            Tile6 d;
+            load_tile(tile, lane, d);
+            if (k == cnt - 1) { __syncwarp(); issue(slot); }
+            tile_mul<NB>(d, smem, xp, acc);
+          } else {
+            TileD<N> d;
+            load_tile<N>(tile, lane, ptab, kPosCopies * 8u, d);
+            if (k == cnt - 1) { __syncwarp(); issue(slot); }
+            tile_mul<N, true, NB>(d, xp, acc);
+          }
+          tile += tb;
+        }
+        parity ^= slot;
+        slot ^= 1u;
+        blk += cnt; left -= cnt;
+      }
+      if (failed) break;
+      // the row tile's sums (or the piece of it): beside the CTA's if another warp began it
+      float* dst = first == 0 ? part + (size_t)row * 32 * batch : reinterpret_cast<float*>(smem + P.head) + (size_t)warp * 32 * batch;
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int c = 0; c < NB; ++c)
+#pragma unroll
+          for (int d = 0; d < 4; ++d) {
+            const int r = g + 16 * mt + 8 * (d >> 1), bc = 8 * c + 2 * t + (d & 1);
+            if (bc < batch) dst[r * batch + bc] = acc[mt][c][d];
+          }
+      if (first != 0 && lane == 0) atomicOr(reinterpret_cast<uint32_t*>(smem + P.masks) + row, 1u << warp);
+      ++row; blk = 0;
+    }
+  }
+  if (failed) {
+    // give the copies still in flight time to land before the shared memory is given up
+    const long long t0 = clock64();
+    while (clock64() - t0 < 200000) {}
+    if (lane == 0 && dev_status) *dev_status = STB_ERR_TIMEOUT;
+  }
+  __syncthreads();
+
+  // Sums of the CTA: what the row tile's first warp has, then the pieces of the warps after it; four values of one row tile per
+  // thread and step (values of a row tile: [row][batch row]).
+  const int per4 = 8 * batch, E4 = rows * per4;
+  const uint32_t* masks = reinterpret_cast<const uint32_t*>(smem + P.masks);
+  const float4* head4 = reinterpret_cast<const float4*>(smem + P.head);
+  float4* part4 = reinterpret_cast<float4*>(part);
+  auto add = [](float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; };
+  auto store = [&](int row, int v4, const float4& s) {
+    const int rt = R0 + row, li = layer_of(layers, rt), first = (rt - layers.tile_start[li]) * kTileRows, n = layers.n[li];
+    const size_t ldy = layers.ldy[li];
+    void* y = layers.y[li];
+    const bool f16 = layers.y_f16[li] != 0;
+    const float w[4] = {s.x, s.y, s.z, s.w};
+    int r = batch == 1 ? 4 * v4 : 4 * v4 / batch, bc = 4 * v4 - r * batch;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (first + r < n) {
+        if (f16) static_cast<__half*>(y)[(size_t)bc * ldy + first + r] = __float2half_rn(w[k]);
+        else static_cast<float*>(y)[(size_t)bc * ldy + first + r] = w[k];
+      }
+      if (++bc == batch) { bc = 0; ++r; }
+    }
+  };
+#pragma unroll 1
+  for (int e = tid; e < E4; e += kGThreads) {
+    const int row = e / per4, v = e - row * per4;
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (nbp > 0) s = part4[e];
+#pragma unroll 1
+    for (uint32_t mm = masks[row]; mm != 0u; mm &= mm - 1u) add(s, head4[(__ffs(mm) - 1) * per4 + v]);      // in warp order
+    if (ksplit == 1) store(row, v, s);
+    else part4[e] = s;
+  }
+  if (ksplit == 1) return;
+  // the cluster's CTAs, in order: CTA k finishes the k-th share of the values
+  cluster_arrive();
+  cluster_wait();
+  const int e0 = (int)((long long)E4 * kpart / ksplit), e1 = (int)((long long)E4 * (kpart + 1) / ksplit);
+#pragma unroll 1
+  for (int e = e0 + tid; e < e1; e += kGThreads) {
+    float4 v[8], s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < ksplit) v[k] = *cg::this_cluster().map_shared_rank(part4 + e, k);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < ksplit) add(s, v[k]);
+    const int row = e / per4;
+    store(row, e - row * per4, s);
+  }
+  cluster_arrive();        // nobody leaves while its sums are being read
+  cluster_wait();
+}
+
+// ------------------------------------------------------------------------------------------
 // Launch shape: ksplit CTAs per row tile and warps per CTA.  A warp should get a run of several
 // tiles (its ring then streams while it decodes) and the grid should have at least two CTAs per
 // SM while leaving room on the SM for the next layer's CTAs, which start their own weight
@@ -561,9 +935,118 @@ static cudaError_t launch_mma_n(int N, const GemvLayers& layers, int m, const __
   return launch_mma<6, NB>(layers, m, x, batch, ldx, dev_status, s, chained, selftest);
 }
 
+// Launch of gemv_stream_kernel, batch <= 16: the split of the blocks (1, 2, 4 or 8 slices) for which the fullest CTA is done
+// first, by the clocks of a tile (measured: about 150, 50 more for a second group of eight rows, 60 more for 6:8 in position
+// order), of a warp's tile alone (900), of the launch and the prologue (2500) and of a cluster (1500); the wider ring where it fits.
+// Returns false where no split fits shared memory.
+static bool gemv_plan(int N, int row_tiles, int nblk, int batch, int layers, const int (&most)[4], GemvPlan& best) {
+  double best_cost = 0.0;
+  bool found = false;
+  for (int lg = 0; lg < 4; ++lg) {
+    const int C = 1 << lg;
+    if (most[lg] < 1 || (C > 1 && nblk < 2 * C)) continue;
+    GemvPlan p = {};
+    p.ksplit = C;
+    p.clusters = row_tiles < most[lg] ? row_tiles : most[lg];
+    p.bs = (nblk + C - 1) / C;
+    const int rows = (row_tiles + p.clusters - 1) / p.clusters;
+    bool ok = false;
+    for (int form = 0; form < 4 && !ok; ++form) {
+      const int image = form < 2;
+      if (image && N != 6) continue;
+      ok = gemv_layout(p, N, batch, rows, layers, image, form % 2 == 0 ? 2 : 1);
+    }
+    if (!ok) continue;
+    const double tiles = (double)rows * p.bs, clk = 150.0 + (batch > 8 ? 50.0 : 0.0) + (N == 6 && !p.image ? 60.0 : 0.0);
+    const double busy = tiles * clk, chain = (double)((int)(tiles + kGWarps - 1) / kGWarps) * 900.0;
+    const double cost = (busy > chain ? busy : chain) + 2500.0 + (C > 1 ? 1500.0 : 0.0) + 2.0 * batch * p.bs;
+    if (!found || cost < best_cost) { best = p; best_cost = cost; found = true; }
+  }
+  return found;
+}
+
+template <int N, int NB, bool kImage>
+static cudaError_t launch_stream(const GemvLayers& layers, const GemvPlan& plan, int m, const __half* x, int batch, size_t ldx, int* dev_status, cudaStream_t s,
+                                 bool chained, bool wait_selftest, int dev) {
+  static bool attr_done[kMaxDevices] = {};          // the shared-memory limit of a kernel is a per-device setting
+  if (dev < 0 || dev >= kMaxDevices || !attr_done[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(gemv_stream_kernel<N, NB, kImage>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemvSmem);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < kMaxDevices) attr_done[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(plan.clusters * plan.ksplit), 1, 1);
+  cfg.blockDim = dim3((unsigned)kGThreads, 1, 1);
+  cfg.dynamicSmemBytes = plan.total;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (plan.ksplit > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)plan.ksplit; at[na].val.clusterDim.y = 1; at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
+  cfg.attrs = at; cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, gemv_stream_kernel<N, NB, kImage>, layers, plan, m, x, batch, ldx, dev_status,
+                            wait_selftest ? kSelftestWaitLimit : kWaitLimit, wait_selftest ? 1 : 0, chained ? 1 : 0);
+}
+
+// Clusters of 1, 2, 4 and 8 CTAs (one CTA per SM) that a device holds at once.
+static cudaError_t gemv_clusters(int dev, int (&most)[4]) {
+  static int cached[kMaxDevices][4] = {};
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!cached[dev][0]) {
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(gemv_stream_kernel<4, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemvSmem);
+    if (e != cudaSuccess) return e;
+    int v[4] = {sms, 0, 0, 0};
+    for (int lg = 1; lg < 4; ++lg) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(sms >> lg << lg), 1, 1);
+      cfg.blockDim = dim3((unsigned)kGThreads, 1, 1);
+      cfg.dynamicSmemBytes = kGemvSmem;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.attrs = at; cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&v[lg], gemv_stream_kernel<4, 1, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); v[lg] = 0; }
+    }
+    for (int lg = 3; lg >= 0; --lg) cached[dev][lg] = v[lg];      // [0] last: it marks the entry as filled
+  }
+  for (int lg = 0; lg < 4; ++lg) most[lg] = cached[dev][lg];
+  return cudaSuccess;
+}
+
 // batch -> number of 8-row batch groups (1, 2, 4 or 8)
 static cudaError_t launch_mma_b(int batch, int N, const GemvLayers& layers, int m, const __half* x, size_t ldx,
                                 int* dev_status, cudaStream_t s, bool chained, bool selftest = false) {
+  // gemv_stream_kernel where its longer prologue is repaid: from 4096 tiles (16.8 million weights) on, measured level with
+  // gemv_mma_kernel at 4096 x 4096 and behind it at 5003 x 2816 (11.4 against 9.6 us, L2-resident); with a second batch group
+  // only in the sparse form (in position order 26.4 against 24.4 us at 4096 x 11008 5:8, batch 16) and where the split leaves the
+  // fullest CTA at most a quarter more than its share (11008 x 4096: 20.0 against 24.1 us; 4096 x 11008, a third more: 23.4
+  // against 22.3, L2-resident).
+  const long long tiles = (long long)layers.tile_start[layers.count] * (m / kBlock);
+  if (batch <= 16 && tiles >= 4096 && (batch <= 8 || N == 6)) {
+    int dev = 0, most[4];
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = gemv_clusters(dev, most);
+    if (e != cudaSuccess) return e;
+    GemvPlan plan;
+    if (gemv_plan(N, layers.tile_start[layers.count], m / kBlock, batch, layers.count, most, plan) &&
+        (batch <= 8 || (plan.image && 4ll * most[0] * plan.bs * ((layers.tile_start[layers.count] + plan.clusters - 1) / plan.clusters) <= 5 * tiles))) {
+      if (batch > 8) return launch_stream<6, 2, true>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+      if (N == 4) return launch_stream<4, 1, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+      if (N == 5) return launch_stream<5, 1, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+      if (plan.image) return launch_stream<6, 1, true>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+      return launch_stream<6, 1, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+    }
+  }
   if (batch <= 8) return launch_mma_n<1>(N, layers, m, x, batch, ldx, dev_status, s, chained, selftest);
   if (batch <= 16) return launch_mma_n<2>(N, layers, m, x, batch, ldx, dev_status, s, chained, selftest);
   if (batch <= 32) return launch_mma_n<4>(N, layers, m, x, batch, ldx, dev_status, s, chained, selftest);

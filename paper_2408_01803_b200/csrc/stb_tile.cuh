@@ -17,6 +17,7 @@ constexpr uint32_t kMeta6Bytes = kMasks6 * kMasks6 * 16;   // the joint 6:8 meta
                                                            // tile is the address of its entry
 constexpr uint32_t kImgWordsPerBlock = 96;    // 6:8 operand-order image: words per block and batch row
 constexpr uint32_t kXPad = 64;                // bytes between the rows of the plain copy beyond 2 m: the eight lane groups' loads do not conflict
+constexpr uint32_t kImgPad = 16;              // the same beyond the rows of the image
 constexpr uint32_t kPosCopies = 16;           // copies of a position table, lane-minor: the look-ups of 16 lanes never conflict
 constexpr uint32_t kPosBytes = kPosTableEntries * kPosCopies * 8;
 constexpr uint32_t kZeroBytes = 384;          // zeros for the lanes beyond the batch: a block of the image

@@ -693,3 +693,23 @@ def test_native_host_path_equals_the_python_form(stb, call, dtype, rows):
         fast(layer, wide[:, :m].float())
     with pytest.raises(stb.StbError):
         fast(stb.PackedLayer(n, m, 9, layer.buf, layer.dev_status), wide[:, :m])
+
+
+@pytest.mark.parametrize("N,n,m,batch", [(4, 8192 * 4 - 5, 512, 1), (5, 1030, 16640, 8), (6, 4101, 4096, 1), (6, 8192, 2048 + 128, 7), (6, 11008, 1536, 16),
+                                         (4, 32, 128 * 4099, 2), (6, 700, 25600, 3)])
+def test_gemv_of_larger_layers(stb, N, n, m, batch):
+    """The GEMV kernel that large layers take (4096 tiles and more): ragged rows, one to eight slices of the blocks with a short last
+    one, one row tile, a second batch group, 6:8 with and without room for the image; against the product of the dense
+    matrix of stb_dequant (exact) in float64 on the GPU, for fp32 and fp16 outputs."""
+    import torch
+    layer = stb.pack_numpy(si.logical_layer(n, m, N, 3400 + n % 97, salient_counts=[3, 0, 17, 8, 32]))
+    W = stb.dequant(layer).double()
+    x = torch.from_numpy(si.activations(batch, m, 3401)).cuda()
+    ref = x.double() @ W.t()
+    y = stb.gemv(layer, x)
+    assert int(layer.dev_status.item()) == 0
+    assert float((y.double() - ref).abs().max()) <= TOL * float(ref.abs().max())
+    # fp32 sums of m products in a fixed order: m 2^-24 of the sum of magnitudes bounds their error
+    bound = (x.double().abs() @ W.abs().t()) * (m * 2.0 ** -24)
+    assert bool(((y.double() - ref).abs() <= bound).all())
+    assert torch.equal(stb.gemv(layer, x, out_dtype=torch.float16), y.half())

@@ -391,7 +391,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
 // word w of the layer, and zeros in the 128 columns after the last word (a CTA's last residual stage may reach there).
 __global__ void gemm_gather_kernel(const uint8_t* __restrict__ packed, int n, int m, int N, const __nv_bfloat16* __restrict__ X, int T,
                                    size_t ldx, __nv_bfloat16* __restrict__ Xs, int ldxs) {
-  grid_launch_dependents();        // the GEMM may start; it waits for this grid before it reads Xs
+  begin_after(packed, X);          // (the GEMM may start; it waits for this grid before it reads Xs)
   const Header* hdr = reinterpret_cast<const Header*>(packed);
   if (!header_matches(hdr, n, m, N)) return;
   const int nblk = m / kBlock;
@@ -678,7 +678,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
 __global__ void gemm_reduce_kernel(const float* __restrict__ ws, int first_tile, int split_tiles, int ksplit, int ttiles, int ktok,
                                    int n, int T, void* __restrict__ Y, int y_16, size_t ldy) {
   // four consecutive rows of one token per thread: 16-byte loads of the parts, one 8- or 16-byte store
-  grid_dependency_wait();          // (a programmatic dependent of the GEMM: its CTAs are set up while the GEMM drains)
+  begin_after(ws);                 // (a programmatic dependent of the GEMM: its CTAs are set up while the GEMM drains)
   const size_t per = (size_t)kBM * ktok, per4 = per / 4, total = (size_t)split_tiles * per4;
   const bool vec = (ldy % 4) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -866,9 +866,9 @@ static int launch_gemm(const GemmPlan& plan, const uint8_t* packed, int n, int m
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
   }
   // the gather moves 16-bit values: the same kernel serves bf16 and fp16
-  gemm_gather_kernel<<<148 * 4, 256, 0, s>>>(packed, n, m, N, static_cast<const __nv_bfloat16*>(X), T, ldx,
-                                             static_cast<__nv_bfloat16*>(ws), ldxs);
-  if (cudaGetLastError() != cudaSuccess) return STB_ERR_CUDA;
+  if (launch_after(gemm_gather_kernel, dim3(148 * 4), dim3(256), 0, s, packed, n, m, N, static_cast<const __nv_bfloat16*>(X), T, ldx,
+                   static_cast<__nv_bfloat16*>(ws), ldxs) != cudaSuccess)
+    return STB_ERR_CUDA;
   // The GEMM is a programmatic dependent of the gather: its CTAs may be scheduled while the gather runs (they need
   // Xs only for the residual stages at the end of their K range) and wait (griddepcontrol.wait) before they read it.
   cudaLaunchAttribute pdl[1];

@@ -89,13 +89,16 @@ constexpr int kMaxDevices = 64;
 template <int N, int NB>
 __global__ void __launch_bounds__(kGemvMaxThreads, NB <= 2 ? 4 : 1)
 gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* __restrict__ x, int batch,
-                size_t ldx, int* dev_status, int lg_ksplit, int bpp, long long wait_limit, int copies_off) {
+                size_t ldx, int* dev_status, int lg_ksplit, int bpp, long long wait_limit, int copies_off, int chained) {
+  // A programmatic dependent of whatever ran before it: prepared while that drains.  Only within a chain (stb_layer_stack,
+  // whose packed layers nobody writes meanwhile) may anything be read before that is complete.
+  if (!chained) { grid_dependency_wait(); grid_launch_dependents(); }
   extern __shared__ __align__(128) uint8_t smem[];
   int li = 0, rt_all = (int)(blockIdx.x >> lg_ksplit);
 #pragma unroll
   for (int i = 1; i < kMaxFused; ++i)
     if (i < layers.count && rt_all >= layers.tile_start[i]) li = i;
-  const uint8_t* __restrict__ packed = layers.packed[li];
+  const uint8_t* packed = after_dependency_wait(layers.packed[li]);
   void* __restrict__ y = layers.y[li];
   const size_t ldy = layers.ldy[li];
   const int n = layers.n[li], y_f16 = layers.y_f16[li];
@@ -153,8 +156,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
   // Everything below reads the activations (the previous layer's output) or writes y: wait for the
   // previous grid of the stream to have completed (no-op without a programmatic launch), then let
   // the next grid start its own weight stream.
-  grid_dependency_wait();
-  grid_launch_dependents();
+  if (chained) { grid_dependency_wait(); grid_launch_dependents(); }
   x = after_dependency_wait(x);
   const uint32_t* ximg = reinterpret_cast<const uint32_t*>(smem + L.ximg);
   const uint32_t img_row_words = (uint32_t)bpp * kImgWordsPerBlock;
@@ -582,7 +584,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
   }
   if (tid < (int)kZeroBytes / 4) reinterpret_cast<uint32_t*>(smem + P.zero)[tid] = 0u;
   for (int i = tid; i < rows; i += kGThreads) reinterpret_cast<uint32_t*>(smem + P.masks)[i] = 0u;
-  if (!chained) grid_dependency_wait();
+  if (!chained) { grid_dependency_wait(); grid_launch_dependents(); }
   // a buffer packed for another shape must not be read as this one (every CTA of the grid comes to the same verdict)
   bool fits = true;
   uint32_t nrw[kMaxFused];
@@ -631,7 +633,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
       fence_async_smem();
       if (!copies_off) bulk_g2s(ring, w.tiles + (size_t)w.blk * tb, (uint32_t)c * tb, bar0);
       const BlockInfo* bi = reinterpret_cast<const BlockInfo*>(layers.packed[layer_of(layers, R0 + w.row)] + sizeof(Header)) + b0 + w.blk;
-      const uint32_t w0 = __ldg(&bi[0].rw_off), nw = __ldg(&bi[0].nrw) + (c > 1 ? __ldg(&bi[1].nrw) : 0u), rec_b = (uint32_t)c * kResidA2Bytes + nw * kResidWordBytes;
+      const uint32_t w0 = bi[0].rw_off, nw = bi[0].nrw + (c > 1 ? bi[1].nrw : 0u), rec_b = (uint32_t)c * kResidA2Bytes + nw * kResidWordBytes;
       mbar_expect_tx(bar0, (uint32_t)c * tb + rec_b);
       if (!copies_off) bulk_g2s(ring + (uint32_t)P.chunk * tb, w.recs + (size_t)kResidA2Bytes * w.blk + (size_t)kResidWordBytes * w0, rec_b, bar0);
     }
@@ -643,7 +645,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
 #pragma unroll
     for (int q = 0; q < kMaxFused; ++q)
       if (q == li) v = nrw[q];
-    if (b0 + k < nblk) v = __ldg(&bi[b0 + k].rw_off);
+    if (b0 + k < nblk) v = bi[b0 + k].rw_off;
     roff_all[li * (P.bs + 1) + k] = v;
   }
   __syncthreads();
@@ -677,7 +679,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
     const uint32_t w0 = roff_all[li * (P.bs + 1)], cnt = roff_all[li * (P.bs + 1) + nbp] - w0;
     const uint2* rwt = reinterpret_cast<const uint2*>(layers.packed[li] + rwtab_offset(nblk)) + w0;
     for (uint32_t i = tid; i < cnt; i += kGThreads) {
-      const uint2 e = __ldg(rwt + i);
+      const uint2 e = rwt[i];
       const uint32_t b = (e.x >> 3) - (uint32_t)b0;
       uint32_t at[4];
 #pragma unroll
@@ -688,8 +690,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
 
   // Everything below reads the activations (the previous layer's output) or writes y: wait for the
   // previous grid of the stream to have completed, then let the next grid start its own prologue.
-  if (chained) grid_dependency_wait();
-  grid_launch_dependents();
+  if (chained) { grid_dependency_wait(); grid_launch_dependents(); }
   {
     const int per_row = nbp * 16, items = batch * per_row;
 #pragma unroll 1
@@ -882,8 +883,8 @@ static void gemv_shape(int n, int m, int& ksplit, int& warps) {
   ksplit = ks;
 }
 
-// `chained`: launch as a programmatic dependent of the previous kernel of the stream (only used
-// between the GEMVs of one stb_layer_stack call, whose packed layers nobody writes meanwhile).
+// `chained`: the kernel before it on the stream is another GEMV of the same stb_layer_stack call, so that nobody writes the
+// packed layer meanwhile.
 template <int N, int NB>
 static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, int batch, size_t ldx,
                               int* dev_status, cudaStream_t s, bool chained, bool wait_selftest = false) {
@@ -915,16 +916,14 @@ static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, 
     at[na].val.clusterDim.x = (unsigned)ksplit; at[na].val.clusterDim.y = 1; at[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (chained) {
-    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
+  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
   cfg.attrs = at; cfg.numAttrs = na;
   int lg = 0;
   while ((1 << lg) < ksplit) ++lg;
   const long long limit = wait_selftest ? kSelftestWaitLimit : kWaitLimit;
-  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0, chained ? 1 : 0);
 }
 
 template <int NB>

@@ -72,6 +72,15 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // memory is visible (no-op for an ordinary launch) / allow the dependent grid to be scheduled.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The first statement of a kernel that is launched with launch_after: everything before it on the stream is complete and
+// visible; the kernel after it may be prepared from now on.  The pointers the kernel reads through are passed, so that no load
+// is moved ahead of the wait (a read-only one otherwise may be).
+template <typename... P>
+__device__ __forceinline__ void begin_after(P&... p) {
+  grid_dependency_wait();
+  grid_launch_dependents();
+  ([&] { asm volatile("" : "+l"(p) :: "memory"); }(), ...);
+}
 // a pointer to data of the producer grid: anything computed from the returned value stays behind the wait
 template <typename T>
 __device__ __forceinline__ const T* after_dependency_wait(const T* p) {
@@ -114,6 +123,19 @@ __device__ __forceinline__ uint32_t ldg_nc_u32(const void* p) {
   uint32_t v;
   asm("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
+}
+
+// Launches a kernel that opens with begin_after() as a programmatic dependent of whatever is before it on the stream: it is
+// set up while that drains, which hides the launch (2 to 3 us on a stream) and changes no order.
+template <typename... P, typename... A>
+static cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 }  // namespace stb

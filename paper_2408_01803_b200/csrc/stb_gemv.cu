@@ -18,7 +18,7 @@ namespace stb {
 __device__ const Meta6Table g_meta6 = make_meta6_table();
 
 // ------------------------------------------------------------------------------------------
-// Tensor-core GEMV of small layers and of 9 to 64 batch rows, N = 4, 5, 6, batch <= 8 NB (NB = 1, 2, 4, 8).
+// Tensor-core GEMV of small layers, of chains of small layers and of 17 to 64 batch rows, N = 4, 5, 6, batch <= 8 NB (NB = 1, 2, 4, 8).
 //
 // Grid: one thread-block cluster of `ksplit` CTAs per row tile (32 rows); CTA k of the cluster
 // takes the k-th slice of the 128-column blocks and its warps take contiguous runs of that
@@ -86,19 +86,20 @@ struct GemvLayers {
 // registers, was measured slower: the spills cost more than the extra resident CTA brings).
 constexpr int kGemvMaxThreads = 128;
 constexpr int kMaxDevices = 64;
-template <int N, int NB>
+template <int N, int NB, bool kChained>
 __global__ void __launch_bounds__(kGemvMaxThreads, NB <= 2 ? 4 : 1)
 gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* __restrict__ x, int batch,
-                size_t ldx, int* dev_status, int lg_ksplit, int bpp, long long wait_limit, int copies_off, int chained) {
+                size_t ldx, int* dev_status, int lg_ksplit, int bpp, long long wait_limit, int copies_off) {
   // A programmatic dependent of whatever ran before it: prepared while that drains.  Only within a chain (stb_layer_stack,
   // whose packed layers nobody writes meanwhile) may anything be read before that is complete.
-  if (!chained) { grid_dependency_wait(); grid_launch_dependents(); }
+  if constexpr (!kChained) { grid_dependency_wait(); grid_launch_dependents(); }
   extern __shared__ __align__(128) uint8_t smem[];
   int li = 0, rt_all = (int)(blockIdx.x >> lg_ksplit);
 #pragma unroll
   for (int i = 1; i < kMaxFused; ++i)
     if (i < layers.count && rt_all >= layers.tile_start[i]) li = i;
-  const uint8_t* packed = after_dependency_wait(layers.packed[li]);
+  const uint8_t* __restrict__ packed = layers.packed[li];
+  if constexpr (!kChained) packed = after_dependency_wait(packed);
   void* __restrict__ y = layers.y[li];
   const size_t ldy = layers.ldy[li];
   const int n = layers.n[li], y_f16 = layers.y_f16[li];
@@ -156,7 +157,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
   // Everything below reads the activations (the previous layer's output) or writes y: wait for the
   // previous grid of the stream to have completed (no-op without a programmatic launch), then let
   // the next grid start its own weight stream.
-  if (chained) { grid_dependency_wait(); grid_launch_dependents(); }
+  if constexpr (kChained) { grid_dependency_wait(); grid_launch_dependents(); }
   x = after_dependency_wait(x);
   const uint32_t* ximg = reinterpret_cast<const uint32_t*>(smem + L.ximg);
   const uint32_t img_row_words = (uint32_t)bpp * kImgWordsPerBlock;
@@ -504,7 +505,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
 // Grid: Q thread-block clusters of `ksplit` CTAs, one CTA of 16 warps per SM.  CTA k of a cluster takes the k-th slice of the
 // 128-column blocks of ALL row tiles of the cluster, so that its slice of the activations is staged in shared memory once and
 // used for every row tile; its 32 x 128 tiles, in (row tile, block) order, are dealt to the warps as equal contiguous runs.
-// gemv_plan takes the split for which the fullest CTA has least to do.
+// gemv_plan takes the split (1, 2, 4, 6 or 8) that is done first.
 // Each warp streams its tiles and their residual records from HBM into a private ring (two slots of one or two tiles) with 1-D
 // bulk copies, and decodes and multiplies them on the tensor cores, fp32 accumulators in registers (stb_tile.cuh):
 //   N = 4, 5        position-order decode, m16n8k16, activations from a plain copy in shared memory
@@ -515,9 +516,11 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
 // Sums: a warp writes the rows it begins to shared memory and the piece it continues beside it; the CTA adds them in order, the
 // cluster adds its CTAs' sums through distributed shared memory, in order.
 // What bounds it: the decode (about 175 clocks per tile and SM, integer issue), and a chain of latencies before and after it
-// (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small layers stay with gemv_mma_kernel).
+// (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small layers stay with gemv_mma_kernel;
+// launch_mma_b has the rule).
 // Against that kernel, cold L2, microseconds: 28672 x 8192 4:8 batch 1 58.9 -> 48.1, 5120 x 13824 5:8 batch 8 32.6 -> 25.3,
-// 4096 x 11008 6:8 batch 1 20.0 -> 16.4, 11008 x 4096 6:8 batch 16 24.1 -> 20.0, 4096 x 4096 4:8 batch 1 11.3 -> 9.7.
+// 4096 x 11008 6:8 batch 1 20.0 -> 16.4, 11008 x 4096 6:8 batch 16 24.1 -> 20.0, 4096 x 4096 4:8 batch 1 11.3 -> 9.7; in L2, 16
+// rows: 5120 x 13824 4:8 41.8 -> 31.0, 5:8 48.0 -> 35.0, 6:8 50.4 -> 31.6, 1500 x 5120 6:8 13.0 -> 10.4.
 constexpr int kGWarps = 16, kGThreads = kGWarps * 32;
 __device__ __forceinline__ int layer_of(const GemvLayers& layers, int rt) {
   int li = 0;
@@ -883,11 +886,11 @@ static void gemv_shape(int n, int m, int& ksplit, int& warps) {
   ksplit = ks;
 }
 
-// `chained`: the kernel before it on the stream is another GEMV of the same stb_layer_stack call, so that nobody writes the
-// packed layer meanwhile.
-template <int N, int NB>
+// kChained: nobody writes the packed layer while the kernel before it on the stream runs.  That is another GEMV of the same
+// stb_layer_stack call (`early`: a programmatic dependent of it), or the kernel is launched in stream order.
+template <int N, int NB, bool kChained>
 static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, int batch, size_t ldx,
-                              int* dev_status, cudaStream_t s, bool chained, bool wait_selftest = false) {
+                              int* dev_status, cudaStream_t s, bool early, bool wait_selftest) {
   const int ntile = layers.tile_start[layers.count], nblk = m / kBlock;
   int ksplit, warps;
   gemv_shape(ntile * kTileRows, m, ksplit, warps);
@@ -899,7 +902,7 @@ static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices || !attr_done[dev]) {
-    e = cudaFuncSetAttribute(gemv_mma_kernel<N, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(gemv_mma_kernel<N, NB, kChained>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) attr_done[dev] = true;
   }
@@ -916,37 +919,55 @@ static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, 
     at[na].val.clusterDim.x = (unsigned)ksplit; at[na].val.clusterDim.y = 1; at[na].val.clusterDim.z = 1;
     ++na;
   }
-  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[na].val.programmaticStreamSerializationAllowed = 1;
-  ++na;
+  if (early) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
   cfg.attrs = at; cfg.numAttrs = na;
   int lg = 0;
   while ((1 << lg) < ksplit) ++lg;
   const long long limit = wait_selftest ? kSelftestWaitLimit : kWaitLimit;
-  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0, chained ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB, kChained>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0);
 }
 
 template <int NB>
 static cudaError_t launch_mma_n(int N, const GemvLayers& layers, int m, const __half* x, int batch, size_t ldx,
                                 int* dev_status, cudaStream_t s, bool chained, bool selftest) {
-  if (N == 4) return launch_mma<4, NB>(layers, m, x, batch, ldx, dev_status, s, chained, selftest);
-  if (N == 5) return launch_mma<5, NB>(layers, m, x, batch, ldx, dev_status, s, chained, selftest);
-  return launch_mma<6, NB>(layers, m, x, batch, ldx, dev_status, s, chained, selftest);
+  // On its own a launch is a programmatic dependent as well, which hides 2 to 4 us of launch but keeps the compiler from reading
+  // the weights through the read-only path: with more than eight rows 12% of the time (28672 x 8192 5:8, 16 rows: 99 against
+  // 88 us), so that from 16384 tiles on such a launch keeps the stream's order.
+  const bool plain = !chained && NB > 1 && (long long)layers.tile_start[layers.count] * (m / kBlock) >= 16384;
+  auto* f = N == 4 ? (chained || plain ? launch_mma<4, NB, true> : launch_mma<4, NB, false>)
+          : N == 5 ? (chained || plain ? launch_mma<5, NB, true> : launch_mma<5, NB, false>)
+                   : (chained || plain ? launch_mma<6, NB, true> : launch_mma<6, NB, false>);
+  return f(layers, m, x, batch, ldx, dev_status, s, !plain, selftest);
 }
 
-// Launch of gemv_stream_kernel, batch <= 16: the split of the blocks (1, 2, 4 or 8 slices) for which the fullest CTA is done
-// first, by the clocks of a tile (measured: about 150, 50 more for a second group of eight rows, 60 more for 6:8 in position
-// order), of a warp's tile alone (900), of the launch and the prologue (2500) and of a cluster (1500); the wider ring where it fits.
-// Returns false where no split fits shared memory.
-static bool gemv_plan(int N, int row_tiles, int nblk, int batch, int layers, const int (&most)[4], GemvPlan& best) {
-  double best_cost = 0.0;
+// Clocks that a call of gemv_mma_kernel takes (batch <= 16), from its launch shape: terms fitted to 528 measured calls of all
+// three formats, 32 to 32768 tiles, 1 to 16 rows (6% mean error), times the factor for which the choice between the two kernels by
+// their costs was best (over those calls 0.9% slower on average than always the faster one; gemv_mma_kernel throughout: 9%).
+static double gemv_mma_cost(int N, int row_tiles, int nblk, int batch, int sms) {
+  int ksplit, warps;
+  gemv_shape(row_tiles * kTileRows, nblk * kBlock, ksplit, warps);
+  const int ctas = row_tiles * ksplit, bpp = (nblk + ksplit - 1) / ksplit, per_sm = (ctas + sms - 1) / sms, chain = (bpp + warps - 1) / warps;
+  const double clk = (N == 4 ? 100.0 : N == 5 ? 140.0 : 130.0) + (batch > 8 ? 70.0 : 0.0);
+  const double cost = 4100.0 + clk * per_sm * bpp + 1000.0 * chain + 250.0 * chain * (per_sm + (double)ctas / sms) + (ksplit > 1 ? 3600.0 : 0.0) +
+                      6.0 * batch * bpp + (batch > 8 ? 800.0 : 0.0) + (N == 6 && batch > 2 ? 2100.0 : 0.0);
+  return cost * (N == 6 ? 1.1 : 0.95);
+}
+
+// Launch of gemv_stream_kernel, batch <= 16: the split of the blocks (1, 2, 4, 6 or 8 slices) that is done first, and the wider ring where
+// it fits (clusters of 3, 5 and 7 CTAs measured up to 3 us behind their share of the tiles: an SM of a pair stays idle).  The clocks of a split: the fullest CTA's tiles at their issue rate, its longest warp's tiles at their latency (more
+// with a second group of eight rows or single-tile slots), a cluster's sums, the staging, the epilogue (terms fitted to 1900
+// measured calls of the same range, 3% mean error).  Returns false where no split fits shared memory.
+static bool gemv_plan(int N, int row_tiles, int nblk, int batch, int layers, const int (&most)[9], GemvPlan& best, double& best_cost) {
   bool found = false;
-  for (int lg = 0; lg < 4; ++lg) {
-    const int C = 1 << lg;
-    if (most[lg] < 1 || (C > 1 && nblk < 2 * C)) continue;
+  for (int C = 1; C <= 8; ++C) {
+    if (most[C] < 1 || (C > 1 && (C % 2 || nblk < 2 * C))) continue;
     GemvPlan p = {};
     p.ksplit = C;
-    p.clusters = row_tiles < most[lg] ? row_tiles : most[lg];
+    p.clusters = row_tiles < most[C] ? row_tiles : most[C];
     p.bs = (nblk + C - 1) / C;
     const int rows = (row_tiles + p.clusters - 1) / p.clusters;
     bool ok = false;
@@ -956,9 +977,10 @@ static bool gemv_plan(int N, int row_tiles, int nblk, int batch, int layers, con
       ok = gemv_layout(p, N, batch, rows, layers, image, form % 2 == 0 ? 2 : 1);
     }
     if (!ok) continue;
-    const double tiles = (double)rows * p.bs, clk = 150.0 + (batch > 8 ? 50.0 : 0.0) + (N == 6 && !p.image ? 60.0 : 0.0);
-    const double busy = tiles * clk, chain = (double)((int)(tiles + kGWarps - 1) / kGWarps) * 900.0;
-    const double cost = (busy > chain ? busy : chain) + 2500.0 + (C > 1 ? 1500.0 : 0.0) + 2.0 * batch * p.bs;
+    const int tiles = rows * p.bs, chain = (tiles + kGWarps - 1) / kGWarps;
+    const double clk = N == 5 ? 112.0 : N == 6 && !p.image ? 160.0 : 100.0;
+    const double cost = 10000.0 + clk * tiles + ((batch > 8 ? 2400.0 : 1700.0) + (p.chunk == 1 ? 600.0 : 0.0)) * chain +
+                        (C > 1 ? 3500.0 - 130.0 * C : 0.0) + 11.0 * batch * p.bs + 23.0 * batch * rows;
     if (!found || cost < best_cost) { best = p; best_cost = cost; found = true; }
   }
   return found;
@@ -993,53 +1015,74 @@ static cudaError_t launch_stream(const GemvLayers& layers, const GemvPlan& plan,
                             wait_selftest ? kSelftestWaitLimit : kWaitLimit, wait_selftest ? 1 : 0, chained ? 1 : 0);
 }
 
-// Clusters of 1, 2, 4 and 8 CTAs (one CTA per SM) that a device holds at once.
-static cudaError_t gemv_clusters(int dev, int (&most)[4]) {
-  static int cached[kMaxDevices][4] = {};
+// Clusters of 1 to 8 CTAs (one CTA per SM) that a device holds at once, by their size.
+static cudaError_t gemv_clusters(int dev, int (&most)[9]) {
+  static int cached[kMaxDevices][9] = {};
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (!cached[dev][0]) {
+  if (!cached[dev][1]) {
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(gemv_stream_kernel<4, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemvSmem);
     if (e != cudaSuccess) return e;
-    int v[4] = {sms, 0, 0, 0};
-    for (int lg = 1; lg < 4; ++lg) {
+    int v[9] = {0, sms};
+    for (int C = 2; C <= 8; ++C) {
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(sms >> lg << lg), 1, 1);
+      cfg.gridDim = dim3((unsigned)(sms / C * C), 1, 1);
       cfg.blockDim = dim3((unsigned)kGThreads, 1, 1);
       cfg.dynamicSmemBytes = kGemvSmem;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 1u << lg; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      at[0].val.clusterDim.x = (unsigned)C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
       cfg.attrs = at; cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&v[lg], gemv_stream_kernel<4, 1, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); v[lg] = 0; }
+      if (cudaOccupancyMaxActiveClusters(&v[C], gemv_stream_kernel<4, 1, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); v[C] = 0; }
     }
-    for (int lg = 3; lg >= 0; --lg) cached[dev][lg] = v[lg];      // [0] last: it marks the entry as filled
+    for (int C = 8; C >= 1; --C) cached[dev][C] = v[C];           // [1] last: it marks the entry as filled
   }
-  for (int lg = 0; lg < 4; ++lg) most[lg] = cached[dev][lg];
+  for (int C = 0; C <= 8; ++C) most[C] = cached[dev][C];
   return cudaSuccess;
+}
+
+// Which of the two kernels a launch of up to 16 rows takes.
+enum class GemvForm {
+  cheapest,     // a launch on its own: the one with the lower cost
+  stream,       // gemv_stream_kernel from 1024 tiles on
+  mma           // gemv_mma_kernel
+};
+constexpr long long kStreamTiles = 1024;
+
+// The launches of a chain (stb_layer_stack) mostly take the same kernel: gemv_mma_kernel's CTAs start beside the launch before
+// them, those of gemv_stream_kernel, which fill an SM, do not, and each change from one to the other cost about 4 us.  By the mean
+// tiles of the chain's launches, measured per decoder layer (QKV, O, gate/up, down; microseconds, gemv_mma_kernel against
+// gemv_stream_kernel): mean 832 20.6 / 26.8 (4:8, 2 rows), 25.8 / 33.7 (6:8, 8 rows); 2884 35.5 / 39.6 (4:8), 48.8 / 42.3 (6:8, 8
+// rows), 51.0 / 51.4 (6:8, 16 rows); 4266 47.1 / 49.2 (5:8, 8 rows), 59.7 / 53.5 (6:8, 16 rows); 7498 57.4 / 53.8 (4:8, 2 rows),
+// 61.8 / 58.1 (5:8, 2 rows), 70.6 / 53.1 (6:8, 4 rows); 12352 84.7 / 66.6 (6:8, 2 rows); 19360 115.4 / 100.7 (5:8, 4 rows).
+// `fits`: every launch has a split; `wide`: at least one has double slots (5:8 with a second group of rows needs them: 79.8 / 80.9
+// at mean 7498, 16 rows, without, 76.7 / 73.5 at 12 rows with them).
+static GemvForm chain_form(int N, int batch, long long mean, bool fits, bool wide) {
+  if (!fits || (N == 5 && batch > 8 && !wide)) return GemvForm::mma;
+  return mean >= (N != 6 ? 6000 : batch <= 8 ? 2500 : 4000) ? GemvForm::stream : GemvForm::mma;
 }
 
 // batch -> number of 8-row batch groups (1, 2, 4 or 8)
 static cudaError_t launch_mma_b(int batch, int N, const GemvLayers& layers, int m, const __half* x, size_t ldx,
-                                int* dev_status, cudaStream_t s, bool chained, bool selftest = false) {
-  // gemv_stream_kernel where its longer prologue is repaid: from 4096 tiles (16.8 million weights) on, measured level with
-  // gemv_mma_kernel at 4096 x 4096 and behind it at 5003 x 2816 (11.4 against 9.6 us, L2-resident); with a second batch group
-  // only in the sparse form (in position order 26.4 against 24.4 us at 4096 x 11008 5:8, batch 16) and where the split leaves the
-  // fullest CTA at most a quarter more than its share (11008 x 4096: 20.0 against 24.1 us; 4096 x 11008, a third more: 23.4
-  // against 22.3, L2-resident).
-  const long long tiles = (long long)layers.tile_start[layers.count] * (m / kBlock);
-  if (batch <= 16 && tiles >= 4096 && (batch <= 8 || N == 6)) {
-    int dev = 0, most[4];
+                                int* dev_status, cudaStream_t s, bool chained, bool selftest, GemvForm form) {
+  const int R = layers.tile_start[layers.count], nblk = m / kBlock;
+  if (batch <= 16 && form != GemvForm::mma && (form == GemvForm::cheapest || (long long)R * nblk >= kStreamTiles)) {
+    int dev = 0, most[9];
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = gemv_clusters(dev, most);
     if (e != cudaSuccess) return e;
     GemvPlan plan;
-    if (gemv_plan(N, layers.tile_start[layers.count], m / kBlock, batch, layers.count, most, plan) &&
-        (batch <= 8 || (plan.image && 4ll * most[0] * plan.bs * ((layers.tile_start[layers.count] + plan.clusters - 1) / plan.clusters) <= 5 * tiles))) {
-      if (batch > 8) return launch_stream<6, 2, true>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+    double cost = 0.0;
+    if (gemv_plan(N, R, nblk, batch, layers.count, most, plan, cost) && (form == GemvForm::stream || cost < gemv_mma_cost(N, R, nblk, batch, most[1]))) {
+      if (batch > 8) {
+        if (N == 4) return launch_stream<4, 2, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+        if (N == 5) return launch_stream<5, 2, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+        if (plan.image) return launch_stream<6, 2, true>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+        return launch_stream<6, 2, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
+      }
       if (N == 4) return launch_stream<4, 1, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
       if (N == 5) return launch_stream<5, 1, false>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
       if (plan.image) return launch_stream<6, 1, true>(layers, plan, m, x, batch, ldx, dev_status, s, chained, selftest, dev);
@@ -1180,7 +1223,7 @@ static cudaError_t launch_general(const uint8_t* packed, int n, int m, const __h
 
 static int gemv_impl(const void* packed, int n, int m, int N, const void* x, int batch, size_t ldx,
                      void* y, stb_dtype ydt, size_t ldy, int* dev_status, void* stream, bool chained,
-                     bool wait_selftest = false) {
+                     bool wait_selftest = false, stb::GemvForm form = stb::GemvForm::cheapest) {
   if (!packed || !x || !y) return STB_ERR_ARG;
   if (n < 1 || m < stb::kBlock || m % stb::kBlock != 0) return STB_ERR_SHAPE;
   if (N < 1 || N > 8) return STB_ERR_NM;
@@ -1196,7 +1239,7 @@ static int gemv_impl(const void* packed, int n, int m, int N, const void* x, int
     stb::GemvLayers layers = {};
     layers.packed[0] = p; layers.y[0] = y; layers.ldy[0] = ldy; layers.n[0] = n; layers.y_f16[0] = y_f16;
     layers.tile_start[0] = 0; layers.tile_start[1] = (n + stb::kTileRows - 1) / stb::kTileRows; layers.count = 1;
-    e = stb::launch_mma_b(batch, N, layers, m, xh, ldx, dev_status, s, chained, wait_selftest);
+    e = stb::launch_mma_b(batch, N, layers, m, xh, ldx, dev_status, s, chained, wait_selftest, form);
     return e == cudaSuccess ? STB_OK : STB_ERR_CUDA;
   }
   if (wait_selftest) return STB_ERR_UNSUPPORTED;
@@ -1243,16 +1286,42 @@ extern "C" int stb_layer_stack(const stb_step* steps, int count, int* dev_status
   if (!steps || count < 0) return STB_ERR_ARG;
   for (int k = 0; k < count; ++k)
     if (steps[k].input != STB_IN_PLAIN) return STB_ERR_UNSUPPORTED;      // only the resident kernel forms inputs
+  const auto launch_end = [&](int i) {
+    int j = i + 1;
+    while (j < count && j - i < stb::kMaxFused && can_fuse(steps[i], steps[j])) ++j;
+    return j;
+  };
+  // what chain_form goes by: the tensor-core launches of up to 16 rows
+  long long launches = 0, tiles = 0;
+  bool fits = true, wide = false;
+  int dev = 0, most[9];
+  const bool known = count > 1 && cudaGetDevice(&dev) == cudaSuccess && stb::gemv_clusters(dev, most) == cudaSuccess;
+  for (int i = 0, j; known && i < count; i = j) {
+    j = launch_end(i);
+    const stb_step& st = steps[i];
+    if (st.N < 4 || st.N > 6 || st.batch < 1 || st.batch > 16 || st.m < stb::kBlock) continue;
+    int R = 0;
+    for (int k = i; k < j; ++k) R += (steps[k].n + stb::kTileRows - 1) / stb::kTileRows;
+    const long long t = (long long)R * (st.m / stb::kBlock);
+    ++launches; tiles += t;
+    if (t < stb::kStreamTiles) continue;
+    stb::GemvPlan plan;
+    double cost;
+    if (!stb::gemv_plan(st.N, R, st.m / stb::kBlock, st.batch, j - i, most, plan, cost)) fits = false;
+    else if (plan.chunk == 2) wide = true;
+  }
+  const auto form = [&](const stb_step& st) {
+    return !known || launches <= 1 ? stb::GemvForm::cheapest : stb::chain_form(st.N, st.batch, tiles / launches, fits, wide);
+  };
   int i = 0;
   while (i < count) {
     const stb_step& st = steps[i];
-    int j = i + 1;
-    while (j < count && j - i < stb::kMaxFused && can_fuse(st, steps[j])) ++j;
+    const int j = launch_end(i);
     // steps after the first start their weight stream while the previous step drains
     const bool chained = i > 0;
     if (j - i == 1) {
       int rc = gemv_impl(st.packed, st.n, st.m, st.N, st.in, st.batch, st.ldin, st.out, st.odt, st.ldout,
-                         dev_status, stream, chained);
+                         dev_status, stream, chained, false, form(st));
       if (rc != STB_OK) return rc;
     } else {
       // validate the first step like stb_gemv does; can_fuse has checked what differs in the others
@@ -1273,7 +1342,7 @@ extern "C" int stb_layer_stack(const stb_step* steps, int count, int* dev_status
       }
       cudaStream_t s = static_cast<cudaStream_t>(stream);
       const __half* xh = static_cast<const __half*>(st.in);
-      cudaError_t e = stb::launch_mma_b(st.batch, st.N, layers, st.m, xh, st.ldin, dev_status, s, chained);
+      cudaError_t e = stb::launch_mma_b(st.batch, st.N, layers, st.m, xh, st.ldin, dev_status, s, chained, false, form(st));
       if (e != cudaSuccess) return STB_ERR_CUDA;
     }
     i = j;

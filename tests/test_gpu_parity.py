@@ -696,10 +696,11 @@ def test_native_host_path_equals_the_python_form(stb, call, dtype, rows):
 
 
 @pytest.mark.parametrize("N,n,m,batch", [(4, 8192 * 4 - 5, 512, 1), (5, 1030, 16640, 8), (6, 4101, 4096, 1), (6, 8192, 2048 + 128, 7), (6, 11008, 1536, 16),
-                                         (4, 32, 128 * 4099, 2), (6, 700, 25600, 3)])
+                                         (4, 32, 128 * 4099, 2), (6, 700, 25600, 3), (4, 2090, 2816, 16), (5, 1500, 5120 + 128, 9), (5, 700, 25600, 16),
+                                         (6, 1030, 13824, 16), (6, 95, 3712, 4)])
 def test_gemv_of_larger_layers(stb, N, n, m, batch):
-    """The GEMV kernel that large layers take (4096 tiles and more): ragged rows, one to eight slices of the blocks with a short last
-    one, one row tile, a second batch group, 6:8 with and without room for the image; against the product of the dense
+    """The GEMV kernel that most layers of up to 16 rows take: ragged rows, one to eight slices of the blocks (six among them)
+    with a short last one, one row tile, a second batch group in every format, 6:8 with and without room for the image; against the product of the dense
     matrix of stb_dequant (exact) in float64 on the GPU, for fp32 and fp16 outputs."""
     import torch
     layer = stb.pack_numpy(si.logical_layer(n, m, N, 3400 + n % 97, salient_counts=[3, 0, 17, 8, 32]))
@@ -713,3 +714,27 @@ def test_gemv_of_larger_layers(stb, N, n, m, batch):
     bound = (x.double().abs() @ W.abs().t()) * (m * 2.0 ** -24)
     assert bool(((y.double() - ref).abs() <= bound).all())
     assert torch.equal(stb.gemv(layer, x, out_dtype=torch.float16), y.half())
+
+
+@pytest.mark.parametrize("N,batch,h,f", [(6, 3, 1024, 20000), (6, 16, 1024, 20000), (5, 9, 2048, 25603), (4, 1, 512, 6000)])
+def test_chain_takes_one_gemv_kernel(stb, N, batch, h, f):
+    """stb_layer_stack over layers on both sides of its choice of kernel (means of 2500 tiles at 6:8, 6000 otherwise): two projections of
+    one input in one launch, then one that reads what the chain wrote; each against the float64 product of its own input."""
+    import torch
+    up = [stb.pack_numpy(si.logical_layer(f, h, N, 3500 + k, salient_counts=[3, 0, 17, 8, 32])) for k in range(2)]
+    wide = -(-f // 128) * 128
+    down = stb.pack_numpy(si.logical_layer(h, wide, N, 3502, salient_counts=[3, 0, 17, 8, 32]))
+    x = torch.from_numpy(si.activations(batch, h, 3503)).cuda()
+    mid = [torch.zeros(batch, wide, dtype=torch.float16, device="cuda") for _ in range(2)]
+    out = torch.empty(batch, h, dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stb.layer_stack([(up[0], x, mid[0][:, :f]), (up[1], x, mid[1][:, :f]), (down, mid[0], out)], dev_status=status)
+    assert int(status.item()) == 0
+    for layer, v, y in ((up[0], x, mid[0][:, :f]), (up[1], x, mid[1][:, :f]), (down, mid[0], out)):
+        W = stb.dequant(layer).double()
+        err, m = (y.double() - v.double() @ W.t()).abs(), v.shape[1]
+        # fp32 sums of m products in a fixed order, and the rounding of an fp16 result (2^-11 of it, or half its least subnormal)
+        bound = (v.double().abs() @ W.abs().t()) * (m * 2.0 ** -24)
+        if y.dtype == torch.float16:
+            bound = bound + (y.double().abs() + bound) * 2.0 ** -11 * (1 + 2.0 ** -10) + 2.0 ** -25
+        assert bool((err <= bound).all())

@@ -42,7 +42,7 @@ MLP = ("gate", "up", "down")
 L2_BYTES = 126 * 1024 * 1024
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 MIN_TIMED_S = 0.25
-KERNEL_SOURCES = ("stb_stack.cu", "stb_decode.cuh", "stb_layout.cuh", "stb_ptx.cuh")
+KERNEL_SOURCES = ("stb_stack.cu", "stb_decode.cuh", "stb_layout.cuh", "stb_ptx.cuh", "stb_tile.cuh")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_stack_kernel_llama7b_mlp_6of8_batch1.txt")
 
 

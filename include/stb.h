@@ -170,9 +170,8 @@ int stb_gemm(const void *packed, int n, int m, int N, const void *X, int T, size
 /* The same product for fp16 activations: X fp16 [T][ldx], Y fp32 or fp16 (ydt = STB_F32 / STB_F16); W^ is decoded to
  * fp16 with its scales as stored (no rounding: a kept weight is s a_region exactly, a salient one s1 a_sal1 + s2 a_sal2 as
  * two terms of the sum), so the result is the one stb_gemv defines.  Meant for decode batches beyond what the GEMV
- * kernels do well (Appendix C.2 between its two stages: tens of tokens): for T <= 64 the CTA tile is 128 rows x 64 tokens
- * (one accumulator of 64 TMEM columns per MMA-issuing lane), K is split into the number of parts that makes waves of
- * 148 CTAs x (a CTA's fixed cost + its blocks) smallest, and the kernel runs at the speed of its decode warps; for T > 64 it is stb_gemm's tiling.  The workspace (stb_gemm_f16_workspace bytes, 256-byte
+ * kernels do well (Appendix C.2 between its two stages: tens of tokens), where K is split so that the CTAs of a call fill
+ * the GPU and the kernel runs at the speed of its decode warps.  The workspace (stb_gemm_f16_workspace bytes, 256-byte
  * aligned; the gathered residual activations and the fp32 partial tiles) is required.  Errors as stb_gemm. */
 int stb_gemm_f16_workspace(int n, int m, int N, int T, size_t *bytes);
 int stb_gemm_f16(const void *packed, int n, int m, int N, const void *X, int T, size_t ldx, void *Y,
@@ -261,7 +260,7 @@ int stb_layer_stack_host(const stb_step *steps, int count, const void *in_host, 
  * [m], the column norms of the calibration activations; out: a stb_logical whose n, m, N match and whose six DEVICE
  * arrays (sizes as documented at stb_logical) are WRITTEN here, ready for stb_pack.  float64 throughout; sums that
  * are not exact are taken in the order of the definition, so the result does not depend on the launch shape.
- * ws: DEVICE workspace of stb_quantize_workspace bytes, 256-byte aligned.  About a dozen launches on `stream`. */
+ * ws: DEVICE workspace of stb_quantize_workspace bytes, 256-byte aligned.  A handful of launches on `stream`. */
 int stb_quantize_workspace(int n, int m, size_t *bytes);
 int stb_quantize(const void *W, size_t ldw, const double *xnorm, int n, int m, int N, double lambda,
                  const stb_logical *out, void *ws, size_t ws_bytes, void *stream);

@@ -894,8 +894,9 @@ constexpr uint32_t kSmemLimit = 227 * 1024;
 constexpr unsigned long long kGatherMax = 16 * 1024;     // shared memory for the residual words' activations
 
 // Lays out the shared memory of a launch and chooses each phase's staging; returns the number of phases left without.
+// `gather` false: no room is kept for the residual words' activations.
 static uint32_t up128(uint32_t v) { return (v + 127u) & ~127u; }
-static int plan_smem(StackParams& sp, bool image) {
+static int plan_smem(StackParams& sp, bool image, bool gather) {
   bool any6 = false, dense[3] = {false, false, false};
   for (int p = 0; p < sp.nphase; ++p) {
     if (sp.ph[p].N == 6 && image) any6 = true;
@@ -922,7 +923,7 @@ static int plan_smem(StackParams& sp, bool image) {
     for (int p = 0; p < sp.nphase; ++p) {
       StackPhase& q = sp.ph[p];
       const unsigned long long need = 8ull * q.batch * (unsigned long long)kMaxResidWords * (unsigned long long)(q.m / kBlock) * q.count;
-      q.gather = need <= kGatherMax && q.m <= 32768 ? 1 : 0;
+      q.gather = gather && need <= kGatherMax && q.m <= 32768 ? 1 : 0;
       if (q.gather && need > xs_max) xs_max = (uint32_t)need;
       if (q.gather && need / q.batch > cols_max) cols_max = (uint32_t)(need / q.batch);
     }
@@ -995,14 +996,20 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
   // second pass: where each phase takes its activations from.  6:8: the operand-order image if it fits, else, as for the
   // others, a plain copy if that fits, else global memory; a formed input (silu(in) * in2) must be staged.  The image
   // costs the 12 KB of the metadata table for the whole launch: without it if that lets more phases stage.
-  int best = -1, best_bare = 0;
-  for (int form = 0; form < 2; ++form) {
-    const int bare = plan_smem(sp, form == 0);
-    if (best < 0 || bare < best_bare) { best = form; best_bare = bare; }
+  // Where a formed input does not fit beside the residual words' activations, those are left out.
+  bool staged = false;
+  for (int gather = 1; gather >= 0 && !staged; --gather) {
+    int best = -1, best_bare = 0;
+    for (int form = 0; form < 2; ++form) {
+      const int bare = plan_smem(sp, form == 0, gather != 0);
+      if (best < 0 || bare < best_bare) { best = form; best_bare = bare; }
+    }
+    if (best == 0) plan_smem(sp, true, gather != 0);
+    staged = true;
+    for (int p = 0; p < sp.nphase; ++p)
+      if (sp.ph[p].x2 && sp.ph[p].use_image == 0) staged = false;
   }
-  if (best == 0) plan_smem(sp, true);
-  for (int p = 0; p < sp.nphase; ++p)
-    if (sp.ph[p].x2 && sp.ph[p].use_image == 0) return -1;          // the formed input does not fit shared memory
+  if (!staged) return -1;                                            // the formed input does not fit shared memory
   const size_t s_need = 8 * sizeof(uint32_t);
   const size_t g_need = sp.max_share > 1 ? (size_t)maxR * sp.max_share * sp.part_floats * sizeof(uint2) : 0;
   if (s_need > sync_need) sync_need = s_need;

@@ -193,6 +193,16 @@ def test_gated_activation_is_formed_while_down_stages_its_input(stb, N, batch):
     _check_gated_mlp(stb, torch, dg, du, dd, batch)
 
 
+@pytest.mark.parametrize("N,batch,f", [(4, 1, 35456), (6, 1, 24576), (6, 2, 16640), (5, 8, 2560)])
+def test_gated_activation_that_fills_shared_memory(stb, N, batch, f):
+    """Formed inputs so wide that the activations behind the residual words have no room beside them (the widest, and in between)."""
+    import torch
+    dg = si.logical_layer(f, 128, N, 175, max_salient=9)
+    du = si.logical_layer(f, 128, N, 176, max_salient=9)
+    dd = si.logical_layer(70, f, N, 177, salient_counts=[3, 17, 0, 32])
+    _check_gated_mlp(stb, torch, dg, du, dd, batch)
+
+
 def test_gated_mlp_full_size(stb):
     """The LLaMA-2-7B MLP at 6:8 (quantizer-made) with the gated activation, in a CUDA graph as bench.py runs it."""
     import torch

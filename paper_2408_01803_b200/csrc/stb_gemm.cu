@@ -750,6 +750,8 @@ static GemmBytes gemm_bytes(int n, int m, int T, int ktok) {
 // as the layout whose estimated time is smallest among those whose partial tiles fit `avail` bytes.  In SM clocks:
 //   a stage (64 of K):   the decode of two 32 x 128 tiles' worth of weights per row tile, or the tensor core's time for the
 //                        tile's tokens, whichever is longer (measured: about 440, and 4.4 x 105 or bn / 2 + 30 per accumulator)
+//                        (a GPU full of wide single accumulators ran 1.4 times that, each decoded stage being used once: 8192 x 28672
+//                        at 2048 tokens 1006 us against 888 with two, at 1024 tokens 520 against 439)
 //   a CTA besides:       prologue, first loads, drain (10000) and epilogue (15 per token)
 //   a split:             the second kernel, and its partial tiles written and read (2500 bytes per clock)
 struct GemmPlan {
@@ -764,7 +766,8 @@ static void gemm_plan_for(GemmPlan& best, double& best_cost, int acc, int max_bn
     const int ktok = acc * bn;
     if (bn > max_bn || (tt - 1) * ktok >= T) continue;
     const long long tiles = (long long)rtiles * tt;
-    const double mma = acc * 4.0 * (bn > 210 ? 0.5 * bn : 105.0) * 1.1 + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 10000.0 + 15.0 * ktok;
+    const double wide = acc == 1 && bn > 128 && tiles > 148 ? 1.4 : 1.0;
+    const double mma = acc * 4.0 * (bn > 210 ? 0.5 * bn : 105.0) * 1.1 * wide + 30.0, stage = mma > kDecodeClocks ? mma : kDecodeClocks, fixed = 10000.0 + 15.0 * ktok;
     const size_t per = (size_t)kBM * ktok * sizeof(float);
     auto consider = [&](long long full, int ks) {
       const int bps = (nblk + ks - 1) / ks;

@@ -260,6 +260,8 @@ int stb_layer_stack_host(const stb_step *steps, int count, const void *in_host, 
  * [m], the column norms of the calibration activations; out: a stb_logical whose n, m, N match and whose six DEVICE
  * arrays (sizes as documented at stb_logical) are WRITTEN here, ready for stb_pack.  float64 throughout; sums that
  * are not exact are taken in the order of the definition, so the result does not depend on the launch shape.
+ * A NaN lambda is refused (STB_ERR_ARG).  The norms are not looked at here: a group of columns with a NaN among its scores
+ * keeps more than N, which stb_pack then reports as STB_ERR_CORRUPT.
  * ws: DEVICE workspace of stb_quantize_workspace bytes, 256-byte aligned.  A handful of launches on `stream`. */
 int stb_quantize_workspace(int n, int m, size_t *bytes);
 int stb_quantize(const void *W, size_t ldw, const double *xnorm, int n, int m, int N, double lambda,

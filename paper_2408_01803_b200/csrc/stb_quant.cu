@@ -384,7 +384,10 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __re
   {
     // candidate order: column score (h_jj + lambda) sum_i W_ij^2, ties to the lower column
     const int j = b * kBeta + tid;
-    const double sc = __dmul_rn(__dadd_rn(__dmul_rn(__dmul_rn(2.0, xnorm[j]), xnorm[j]), w.scalars[2]), w.colsq[j]);
+    // (a NaN score comes after all others, so that the ranks are a permutation whatever the norms are: every place of
+    // `order` is filled, with a column)
+    double sc = __dmul_rn(__dadd_rn(__dmul_rn(__dmul_rn(2.0, xnorm[j]), xnorm[j]), w.scalars[2]), w.colsq[j]);
+    if (!(sc == sc)) sc = -INFINITY;
     score[tid] = sc;
     inv[tid + 1] = 1.0 / (double)(tid + 1);
     if (tid == 0) inv[0] = 0.0;
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __re
         const uint32_t h = row[order[i]];
         if (h & 0x8000u) { a1 += abs_of(h & 0x7FFFu); ++k1; }
         const double a0 = at - a1;
-        acc[i] += a1 * a1 * inv[k1] + a0 * a0 * inv[16 * N - k1];
+        acc[i] += a1 * a1 * inv[k1] + a0 * a0 * inv[max(16 * N - k1, 0)];      // (groups of NaN scores keep more than N)
       }
     }
   }
@@ -902,7 +905,7 @@ extern "C" int stb_quantize(const void* W, size_t ldw, const double* xnorm, int 
   if (!W || !xnorm || !out || !ws) return STB_ERR_ARG;
   if (n < 1 || m < 128 || m % 128 != 0) return STB_ERR_SHAPE;
   if (N < 1 || N > 8) return STB_ERR_NM;
-  if (ldw < (size_t)m) return STB_ERR_ARG;
+  if (ldw < (size_t)m || lambda != lambda) return STB_ERR_ARG;
   if (out->n != n || out->m != m || out->N != N) return STB_ERR_ARG;
   if (!out->keep || !out->sign || !out->region || !out->sign2 || !out->salient || !out->scale) return STB_ERR_ARG;
   Ws w;

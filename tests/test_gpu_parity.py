@@ -644,6 +644,32 @@ def test_gpu_quantizer_ties_edges_and_layouts(stb, kind, n, m):
         _same_logical(got, L)
 
 
+@pytest.mark.parametrize("N", [1, 4, 6])
+@pytest.mark.parametrize("bad", [slice(5, 6), slice(0, 128), slice(None)])
+def test_gpu_quantizer_with_nan_norms(stb, N, bad):
+    """Calibration norms with NaN in them (every score of lambda's default is then NaN): no field is taken from memory that
+    nothing wrote (two runs over different leftovers agree), groups without such a column keep N, and stb_pack reports the others."""
+    import torch
+    n, m = 200, 384
+    W = torch.from_numpy(si.dense_weight(n, m, 3150)).cuda()
+    xn = si.calib_norms(m, 3150)
+    xn[bad] = np.nan
+    got = [stb.quantize(W, torch.from_numpy(xn).cuda(), N)]
+    torch.empty(1 << 22, dtype=torch.uint8, device="cuda").fill_(0xA5)
+    stb.quantize(torch.from_numpy(si.dense_weight(n, m, 3151)).cuda(), torch.from_numpy(si.calib_norms(m, 3151)).cuda(), N)
+    got.append(stb.quantize(W, torch.from_numpy(xn).cuda(), N))
+    for k in ("keep", "sign", "region", "sign2", "salient", "scale"):
+        assert torch.equal(got[0][k], got[1][k]), k
+    kept = np.unpackbits(got[0]["keep"].cpu().numpy()[..., None], axis=-1).sum(-1)
+    nan_groups = np.isnan(xn).reshape(-1, 8).any(1)
+    assert (kept[:, ~nan_groups] == N).all() and (kept[:, nan_groups] > N).all()
+    g = got[0]
+    layer = stb.pack(n, m, N, g["keep"], g["sign"], g["region"], g["sign2"], g["salient"], g["scale"])
+    assert int(layer.dev_status.item()) == stb.STB_ERR_CORRUPT
+    with pytest.raises(stb.StbError):
+        stb.quantize(W, torch.from_numpy(si.calib_norms(m, 3150)).cuda(), N, lam=float("nan"))
+
+
 @pytest.mark.parametrize("N", [3, 4, 5, 6])
 def test_dequant_row_stride_and_base(stb, N):
     """stb_dequant into a matrix whose rows or base address do not allow 16-byte stores, and into one that does."""

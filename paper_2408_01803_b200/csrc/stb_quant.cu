@@ -13,8 +13,8 @@
 //   * where the bound leaves one outcome, that is the outcome;
 //   * where it leaves several (ties, or differences near 2^-53 of the value: rare, or blocks of few weights), the
 //     definition's own sequence of roundings is carried out for the candidates that are left.
-// Sums of |w| and w^2 of fp16 values are exact in float64 for weights of ordinary range and may be taken in any order;
-// products and differences whose rounding the definition fixes are never fused into multiply-adds.
+// Sums of |w| of fp16 values, and sums of w^2 over a row's 128 columns of ordinary range, are exact in float64 and may be
+// taken in any order; products and differences whose rounding the definition fixes are never fused into multiply-adds.
 // The layer-wide mean and deviation of Eq. 3 and the regularizer lambda are the exception: their rounding moves every
 // score by the same relative 1e-16, which can change a decision only where two scores tie to that precision (a layer whose
 // |w| are all one value is such a tie everywhere: its deviation is rounding noise, and so is the definition's choice).
@@ -99,8 +99,9 @@ __device__ __forceinline__ bool last_arrival(uint32_t* counter, uint32_t arrival
 }
 
 // ---- Eq. 3: sums of |W| per row and per column, sums of W^2 per column -----------------------------------------------
-// CTA: 256 columns (8 per lane) x kRowsPerCta rows, one row per warp at a time.  All sums are exact: atomics may add
-// them in any order.
+// CTA: 256 columns (8 per lane) x kRowsPerCta rows, one row per warp at a time.  The sums of |w| are exact (40 bits and
+// the row count's): atomics may add them in any order.  Those of w^2 are not (80 bits; an outlier column of 4096 rows
+// needs 55 of them): salient_kernel, which orders columns by them, looks again where that matters.
 constexpr int kRowsPerCta = 64, kInFlight = 4;    // (rows of a warp whose loads are in flight together: the passes are bound by latency)
 template <bool kVec>
 __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, double* __restrict__ rowsum,
@@ -372,6 +373,24 @@ __device__ __noinline__ double salient_exact(const __half* W, size_t ldw, int n,
   }
   return err;
 }
+// A NaN score comes after all others, so that the ranks are a permutation whatever the norms are: every place of the
+// candidates' order is filled, with a column.
+__device__ __forceinline__ double column_score(double xn, double lambda, double squares) {
+  const double sc = __dmul_rn(__dadd_rn(__dmul_rn(__dmul_rn(2.0, xn), xn), lambda), squares);
+  return sc == sc ? sc : -INFINITY;
+}
+// the definition's sum of squares of a column: row by row (a square is exact, the sum is not)
+__device__ __noinline__ double column_squares(const __half* W, size_t ldw, int n, int j) {
+  double q = 0.0;
+  for (int i = 0; i < n; i += 8) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = i + k < n ? w_at(W, ldw, i + k, j) : 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q = __dadd_rn(q, v[k] * v[k]);
+  }
+  return q;
+}
 template <bool kVec>
 __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, int N, const uint8_t* __restrict__ keep,
                                                               const double* __restrict__ xnorm, Ws w, uint64_t* __restrict__ salient) {
@@ -384,14 +403,24 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __re
   {
     // candidate order: column score (h_jj + lambda) sum_i W_ij^2, ties to the lower column
     const int j = b * kBeta + tid;
-    // (a NaN score comes after all others, so that the ranks are a permutation whatever the norms are: every place of
-    // `order` is filled, with a column)
-    double sc = __dmul_rn(__dadd_rn(__dmul_rn(__dmul_rn(2.0, xnorm[j]), xnorm[j]), w.scalars[2]), w.colsq[j]);
-    if (!(sc == sc)) sc = -INFINITY;
+    double sc = column_score(xnorm[j], w.scalars[2], w.colsq[j]);
     score[tid] = sc;
     inv[tid + 1] = 1.0 / (double)(tid + 1);
     if (tid == 0) inv[0] = 0.0;
     __syncthreads();
+    // The sums of squares are rounded, in the order in which sums_kernel's CTAs came by: within n ulp of the exact sum, as is
+    // the definition's row by row.  Two scores further apart than both can move are in the definition's order; the columns
+    // of closer ones (duplicated columns, as a rule) are summed again, row by row.  Two zeros are exact.
+    const double window = (4.0 * n + 64.0) * kUlp;
+    bool close = false;
+    for (int a = 0; a < kBeta; ++a) close = close || (a != tid && (score[a] != 0.0 || sc != 0.0) && !(fabs(score[a] - sc) > window * fmax(score[a], sc)));
+    if (__syncthreads_or(close)) {
+      if (close) {
+        sc = column_score(xnorm[j], w.scalars[2], column_squares(W, ldw, n, j));
+        score[tid] = sc;
+      }
+      __syncthreads();
+    }
     int rank = 0;
     for (int a = 0; a < kBeta; ++a) rank += (score[a] > sc || (score[a] == sc && a < tid)) ? 1 : 0;
     if (rank < kMaxSal) order[rank] = tid;

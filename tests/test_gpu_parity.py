@@ -4,6 +4,8 @@
   * stb_gemv: max|y_gpu - y_ref| <= 5e-3 * max|y_ref| against the float64
     dequantise-then-matmul of the oracle.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -642,6 +644,30 @@ def test_gpu_quantizer_ties_edges_and_layouts(stb, kind, n, m):
         got = stb.quantize(Wd, torch.from_numpy(xn).cuda(), N)
         torch.cuda.synchronize()
         _same_logical(got, L)
+
+
+@pytest.mark.parametrize("n", [4096, 9001])
+def test_gpu_quantizer_duplicated_outlier_columns(stb, n):
+    """Outlier columns in equal pairs whose sums of squares do not fit float64 exactly (sd 0.2, thousands of rows): a pair ties in the
+    definition, and where it is split by the limit of 32 salient columns the lower column is taken, in every run."""
+    import torch
+    m, N = 256, 6
+    g = np.random.default_rng(3161)
+    W = si.dense_weight(n, m, 3160).astype(np.float32)
+    cols = np.concatenate([g.permutation(62)[:24], 64 + g.permutation(62)[:24]]) * 2
+    W[:, cols] = g.standard_normal((n, len(cols))) * 0.2
+    W[:, cols + 1] = W[:, cols]
+    W[:, [126, 254]] = g.standard_normal((n, 2)) * 0.4
+    W = W.astype(np.float16)
+    squares = W[:, cols].astype(np.float64) ** 2
+    assert (squares.sum(0) != np.array([math.fsum(c) for c in squares.T])).any()
+    xn = si.calib_norms(m, 3160)
+    xn[1::2] = xn[::2]
+    L, _, _ = oracle.quantize(W.astype(np.float64), xn, N)
+    flags = np.array([(int(L.salient[c // 128, (c // 64) & 1]) >> (c % 64)) & 1 for c in range(m)])
+    assert (flags[cols] > flags[cols + 1]).any()
+    for _ in range(6):
+        _same_logical(stb.quantize(torch.from_numpy(W).cuda(), torch.from_numpy(xn).cuda(), N), L)
 
 
 @pytest.mark.parametrize("N", [1, 4, 6])

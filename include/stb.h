@@ -258,8 +258,9 @@ int stb_layer_stack_host(const stb_step *steps, int count, const void *in_host, 
  * binarization (Eq. 4) and trisection: the block loop of Algorithm 1 without its Hessian update (column score with
  * the diagonal h_jj = 2 ||X_:,j||^2; lambda < 0 selects 0.01 mean_j h_jj).  W: dense fp16 [n][ldw]; xnorm: float64
  * [m], the column norms of the calibration activations; out: a stb_logical whose n, m, N match and whose six DEVICE
- * arrays (sizes as documented at stb_logical) are WRITTEN here, ready for stb_pack.  float64 throughout; sums that
- * are not exact are taken in the order of the definition, so the result does not depend on the launch shape.
+ * arrays (sizes as documented at stb_logical) are WRITTEN here, ready for stb_pack.  float64 throughout.  The result
+ * is that of the definition's order of sums, whatever the launch shape, with one exception: the layer-wide mean and deviation
+ * of Eq. 3 are rounded otherwise, which can show only where two scores of a group tie to about 1e-16 of their size.
  * A NaN lambda is refused (STB_ERR_ARG).  The norms are not looked at here: a group of columns with a NaN among its scores
  * keeps more than N, which stb_pack then reports as STB_ERR_CORRUPT.
  * ws: DEVICE workspace of stb_quantize_workspace bytes, 256-byte aligned.  A handful of launches on `stream`. */

@@ -15,7 +15,7 @@
 //     definition's own sequence of roundings is carried out for the candidates that are left.
 // Sums of |w| of fp16 values, and sums of w^2 over a row's 128 columns of ordinary range, are exact in float64 and may be
 // taken in any order; products and differences whose rounding the definition fixes are never fused into multiply-adds.
-// The layer-wide mean and deviation of Eq. 3 and the regularizer lambda are the exception: their rounding moves every
+// The layer-wide mean and deviation of Eq. 3 are the exception: their rounding moves every
 // score by the same relative 1e-16, which can change a decision only where two scores tie to that precision (a layer whose
 // |w| are all one value is such a tie everywhere: its deviation is rounding noise, and so is the definition's choice).
 //
@@ -391,9 +391,21 @@ __device__ __noinline__ double column_squares(const __half* W, size_t ldw, int n
   }
   return q;
 }
+// 0.01 mean_j h_jj, h_jj = 2 ||X_:,j||^2, summed in column order
+__device__ __noinline__ double definition_lambda(const double* xnorm, int m) {
+  double h = 0.0;
+  for (int j = 0; j < m; j += 8) {          // (m is a multiple of 128)
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = xnorm[j + k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) h = __dadd_rn(h, __dmul_rn(__dmul_rn(2.0, v[k]), v[k]));
+  }
+  return __ddiv_rn(__dmul_rn(0.01, h), (double)m);
+}
 template <bool kVec>
 __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, int N, const uint8_t* __restrict__ keep,
-                                                              const double* __restrict__ xnorm, Ws w, uint64_t* __restrict__ salient) {
+                                                              const double* __restrict__ xnorm, double lambda_in, Ws w, uint64_t* __restrict__ salient) {
   __shared__ __align__(16) uint32_t tile[kSalThreads * kSalPitch];   // per weight: |w| bits, bit 15 = kept; later the gains
   __shared__ double score[kBeta], inv[kBeta + 1], exact[kMaxSal];
   __shared__ int order[kMaxSal];
@@ -409,14 +421,17 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __re
     if (tid == 0) inv[0] = 0.0;
     __syncthreads();
     // The sums of squares are rounded, in the order in which sums_kernel's CTAs came by: within n ulp of the exact sum, as is
-    // the definition's row by row.  Two scores further apart than both can move are in the definition's order; the columns
-    // of closer ones (duplicated columns, as a rule) are summed again, row by row.  Two zeros are exact.
-    const double window = (4.0 * n + 64.0) * kUlp;
+    // the definition's row by row; the sum behind a default lambda likewise within m ulp.  Two scores further apart than both
+    // can move are in the definition's order; the columns of closer ones (duplicated columns, as a rule) are summed again,
+    // row by row, and lambda column by column.  Two zeros are exact.
+    const double window = (4.0 * ((double)n + m) + 64.0) * kUlp;
     bool close = false;
     for (int a = 0; a < kBeta; ++a) close = close || (a != tid && (score[a] != 0.0 || sc != 0.0) && !(fabs(score[a] - sc) > window * fmax(score[a], sc)));
     if (__syncthreads_or(close)) {
+      if (tid == 0) exact[0] = lambda_in < 0.0 ? definition_lambda(xnorm, m) : lambda_in;
+      __syncthreads();
       if (close) {
-        sc = column_score(xnorm[j], w.scalars[2], column_squares(W, ldw, n, j));
+        sc = column_score(xnorm[j], exact[0], column_squares(W, ldw, n, j));
         score[tid] = sc;
       }
       __syncthreads();
@@ -899,7 +914,7 @@ static cudaError_t launch(const __half* W, size_t ldw, const double* xnorm, int 
   const int passes = (n + kSalThreads - 1) / kSalThreads;
   int per_block = (148 * 6 + nblk - 1) / nblk;
   if (per_block > passes) per_block = passes;
-  salient_kernel<kVec><<<dim3((unsigned)nblk, (unsigned)per_block), kSalThreads, 0, s>>>(W, ldw, n, m, N, keep, xnorm, w, const_cast<uint64_t*>(out->salient));
+  salient_kernel<kVec><<<dim3((unsigned)nblk, (unsigned)per_block), kSalThreads, 0, s>>>(W, ldw, n, m, N, keep, xnorm, lambda, w, const_cast<uint64_t*>(out->salient));
   // break_kernel: one CTA per SM; the number of CTAs per block that makes waves x (rounds of 32 rows per warp + a CTA's
   // prologue, worth about half a round) smallest
   const int groups = (n + 31) / 32;

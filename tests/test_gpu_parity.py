@@ -670,6 +670,42 @@ def test_gpu_quantizer_duplicated_outlier_columns(stb, n):
         _same_logical(stb.quantize(torch.from_numpy(W).cuda(), torch.from_numpy(xn).cuda(), N), L)
 
 
+def test_gpu_quantizer_takes_lambda_in_column_order(stb):
+    """Two columns that compete for the last of 32 salient places, their scores so close that the last bits of lambda decide: the
+    sum of 4096 norms in the definition's order gives one of them, an exactly rounded sum the other."""
+    import torch
+    n, m, N, seed = 64, 4096, 6, 3170
+    g = np.random.default_rng(seed)
+    W = si.dense_weight(n, m, seed).astype(np.float32)
+    W[:, :31] = g.standard_normal((n, 31)) * 0.5
+    W[:, 32] = g.standard_normal(n) * 0.4
+    W = W.astype(np.float16)
+    W[:, 40] = np.roll(W[:, 32], 1) * np.float16(2)
+    q = (W.astype(np.float64) ** 2).sum(0)                 # 64 squares: exact
+    xn = si.calib_norms(m, seed)
+    xn[:31], xn[32], xn[40] = 1000.0, 1.0, 0.0
+
+    def lambdas():
+        total = 0.0
+        for x in xn.tolist():
+            total += 2.0 * x * x
+        return 0.01 * total / m, 0.01 * math.fsum((2.0 * xn * xn).tolist()) / m
+
+    first = lambda lam: (2.0 * xn[32] * xn[32] + lam) * q[32] > (2.0 * xn[40] * xn[40] + lam) * q[40]  # noqa: E731
+    for _ in range(4):                                     # the norm of column 32 at which the scores meet ...
+        xn[32] = math.sqrt(lambdas()[0] * (q[40] / q[32] - 1.0) / 2.0)
+    base, differ = xn[32], False
+    for k in range(-60, 61):                               # ... and beside it one where the two sums disagree
+        xn[32] = base + k * np.spacing(base)
+        differ = first(lambdas()[0]) != first(lambdas()[1])
+        if differ:
+            break
+    assert differ
+    L, _, _ = oracle.quantize(W.astype(np.float64), xn, N)
+    assert ((int(L.salient[0, 0]) >> 32) & 1) != ((int(L.salient[0, 0]) >> 40) & 1)
+    _same_logical(stb.quantize(torch.from_numpy(W).cuda(), torch.from_numpy(xn).cuda(), N), L)
+
+
 @pytest.mark.parametrize("N", [1, 4, 6])
 @pytest.mark.parametrize("bad", [slice(5, 6), slice(0, 128), slice(None)])
 def test_gpu_quantizer_with_nan_norms(stb, N, bad):

@@ -103,6 +103,20 @@ __device__ __forceinline__ bool last_arrival(uint32_t* counter, uint32_t arrival
 // the row count's): atomics may add them in any order.  Those of w^2 are not (80 bits; an outlier column of 4096 rows
 // needs 55 of them): salient_kernel, which orders columns by them, looks again where that matters.
 constexpr int kRowsPerCta = 64, kInFlight = 4;    // (rows of a warp whose loads are in flight together: the passes are bound by latency)
+// abs_of reads the codes of infinities and NaN as numbers.  Where a lane's weights have such a code, the sums they belong to are
+// made infinite or NaN here, as the definition's are: with an infinite one mean and deviation are then NaN, so that every group is
+// selected by select_exact; and the sums of squares of their blocks are not finite, so that no candidate of a search is filtered out.
+__device__ __noinline__ void add_non_finite(const __half* W, size_t ldw, int r0, int r1, int j0, double* rowsum, double* colsum, double* colsq) {
+  for (int r = r0; r < r1; r += 8)
+    for (int c = 0; c < 8; ++c) {
+      const double x = fabs(w_at(W, ldw, r, j0 + c));
+      if (!(x < INFINITY)) { atomicAdd(rowsum + r, x); atomicAdd(colsum + j0 + c, x); atomicAdd(colsq + j0 + c, x); }
+    }
+}
+__device__ __forceinline__ uint32_t largest_code(const uint4& v, uint32_t so_far) {      // of both halves of a word
+  return __vmaxu2(__vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu)), so_far);
+}
+__device__ __forceinline__ bool non_finite(uint32_t codes) { return max(codes & 0xFFFFu, codes >> 16) >= 0x7C00u; }
 template <bool kVec>
 __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, double* __restrict__ rowsum,
                                                    double* __restrict__ colsum, double* __restrict__ colsq) {
@@ -112,6 +126,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
   const bool live = j0 < m;
   const int r1 = min(n, (int)(blockIdx.y + 1) * kRowsPerCta);
   double a[8], q[8];
+  uint32_t codes = 0;
 #pragma unroll
   for (int c = 0; c < 8; ++c) a[c] = q[c] = 0.0;
   for (int r = blockIdx.y * kRowsPerCta + warp; r < r1; r += 8 * kInFlight) {
@@ -121,6 +136,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
     double s[kInFlight];
 #pragma unroll
     for (int k = 0; k < kInFlight; ++k) {
+      codes = largest_code(v[k], codes);
       s[k] = 0.0;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
@@ -134,6 +150,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
       if (lane == 0 && r + 8 * k < r1) atomicAdd(rowsum + r + 8 * k, s[k]);
     }
   }
+  if (non_finite(codes)) add_non_finite(W, ldw, blockIdx.y * kRowsPerCta + warp, r1, j0, rowsum, colsum, colsq);
 #pragma unroll
   for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll
@@ -158,6 +175,7 @@ __global__ void __launch_bounds__(256) scalars_kernel(int n, int m, const double
     const double v = i < n ? w.rowsum[i] : w.colsum[i - n];
     const double inv = v > 0.0 ? 1.0 / v : 0.0;
     if (v > 0.0) cnt += 1.0;
+    if (v == INFINITY) cnt = NAN;              // (an infinite weight over its own sum; a NaN sum counts as none)
     if (i < n) w.rinv[i] = inv;
     else { w.cinv[i - n] = inv; h += 2.0 * xnorm[i - n] * xnorm[i - n]; }
   }
@@ -774,6 +792,45 @@ __global__ void __launch_bounds__(kBrkThreads, 1) break_kernel(const __half* __r
 }
 
 // ---- Trisection, Res_Approx and the logical arrays: one thread per (row, block), loops in column order ----------------
+// A row of a block with an infinite or NaN weight: the definition's own comparisons and sums.
+__device__ __noinline__ void emit_non_finite(const __half* wr, const uint8_t* kr, const uint8_t* sal, double p1, double p2, uint8_t* sign, uint16_t* region,
+                                             uint32_t* sign2, uint16_t* scale) {
+  double a[4] = {0, 0, 0, 0}, alpha[5], ar = 0.0;
+  int k[4] = {0, 0, 0, 0}, ts = 0;
+  uint32_t s2 = 0;
+  auto region_of = [&](int c, double aw) { return sal[c] ? 3 : (aw > p2 ? 2 : (aw > p1 ? 1 : 0)); };
+  for (int c = 0; c < kBeta; ++c)
+    if ((kr[c >> 3] >> (c & 7)) & 1u) {
+      const double aw = fabs((double)__half2float(wr[c]));
+      const int reg = region_of(c, aw);
+      for (int g = 0; g < 4; ++g)
+        if (g == reg) { a[g] = __dadd_rn(a[g], aw); ++k[g]; }
+    }
+  for (int g = 0; g < 4; ++g) alpha[g] = k[g] ? __ddiv_rn(a[g], (double)k[g]) : 0.0;
+  for (int c = 0; c < kBeta; ++c) {
+    if (!sal[c]) continue;
+    if ((kr[c >> 3] >> (c & 7)) & 1u) {
+      const double w = (double)__half2float(wr[c]), d = __dsub_rn(w, __dmul_rn(alpha[3], w >= 0.0 ? 1.0 : -1.0));
+      ar = __dadd_rn(ar, fabs(d));
+      if (d >= 0.0) s2 |= 1u << ts;
+    }
+    ++ts;
+  }
+  alpha[4] = k[3] ? __ddiv_rn(ar, (double)k[3]) : 0.0;
+  for (int q = 0; q < 5; ++q) scale[q] = __half_as_ushort(__double2half(alpha[q]));
+  *sign2 = s2;
+  for (int g = 0; g < 16; ++g) {
+    uint32_t rank = 0, sv = 0, rv = 0;
+    for (int c = 8 * g; c < 8 * g + 8; ++c)
+      if ((kr[g] >> (c & 7)) & 1u) {
+        const double w = (double)__half2float(wr[c]);
+        sv |= (w >= 0.0 ? 1u : 0u) << rank;
+        rv |= (uint32_t)region_of(c, fabs(w)) << (2u * rank);
+        ++rank;
+      }
+    sign[g] = (uint8_t)sv; region[g] = (uint16_t)rv;
+  }
+}
 template <bool kVec>
 __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, const uint8_t* __restrict__ keep, Ws w,
                                                    uint8_t* __restrict__ sign, uint16_t* __restrict__ region, uint32_t* __restrict__ sign2,
@@ -791,9 +848,11 @@ __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W,
   const uint8_t* kr = keep + (size_t)r * ngrp + b * 16;
   double above2 = 0.0, above1 = 0.0, all = 0.0, asal = 0.0;      // exact sums: above the second threshold, the first, all, salient
   int k2 = 0, k1 = 0, k0 = 0, ks = 0;
+  uint32_t codes = 0;
 #pragma unroll 2
   for (int g = 0; g < 16; ++g) {
     const uint4 v = load8<kVec>(wr + 8 * g);
+    codes = largest_code(v, codes);
     const uint32_t sb = (salw[g >> 2] >> (8 * (g & 3))) & 0xFFu, kb = kr[g];
     uint32_t m1 = 0, m2 = 0;
 #pragma unroll
@@ -810,6 +869,12 @@ __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W,
       }
     }
     k2 += __popc(m2); k1 += __popc(m1); k0 += __popc(kb & ~sb); ks += __popc(kb & sb);
+  }
+  const size_t rb = (size_t)r * nblk + b;
+  if (non_finite(codes)) {
+    emit_non_finite(wr, kr, w.salflag + b * kBeta, w.bp[2 * b], w.bp[2 * b + 1], sign + (size_t)r * ngrp + b * 16, region + (size_t)r * ngrp + b * 16, sign2 + rb,
+                    scale + rb * 5);
+    return;
   }
   double alpha[5];
   const double set[4] = {all - above1, above1 - above2, above2, asal};
@@ -832,7 +897,6 @@ __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W,
       if (neg ? d <= 0.0 : d >= 0.0) s2 |= 1u << ts;
     }
   alpha[4] = ks ? __ddiv_rn(ar, (double)ks) : 0.0;
-  const size_t rb = (size_t)r * nblk + b;
 #pragma unroll
   for (int q = 0; q < 5; ++q) scale[rb * 5 + q] = __half_as_ushort(__double2half(alpha[q]));
   sign2[rb] = s2;

@@ -670,6 +670,33 @@ def test_gpu_quantizer_duplicated_outlier_columns(stb, n):
         _same_logical(stb.quantize(torch.from_numpy(W).cuda(), torch.from_numpy(xn).cuda(), N), L)
 
 
+@pytest.mark.parametrize("N", [4, 5, 6])
+@pytest.mark.parametrize("values", [[np.inf], [-np.inf, np.inf], [np.nan], [np.nan, -np.inf, np.inf, -np.nan]])
+def test_gpu_quantizer_with_infinite_and_nan_weights(stb, N, values):
+    """Weights that overflowed: every field is the definition's (the scales of their rows and blocks are infinite or NaN where such
+    a weight is kept, and the rest of the layer is what it makes of them), on aligned rows and on others.  NaN scales are compared as NaN."""
+    import torch
+    n, m = 140, 512
+    W, xn = si.dense_weight(n, m, 3155), si.calib_norms(m, 3155)
+    g = np.random.default_rng(3156)
+    for k in range(12):                                  # in blocks 0 and 2
+        v = values[k % len(values)]
+        grp = 32 * (k & 1) + int(g.integers(0, 16))
+        W[int(g.integers(0, n)), 8 * grp + (0 if np.isnan(v) else int(g.integers(0, 8)))] = v
+        if np.isnan(v):                                  # all scores of the group are equal: its first columns are kept
+            xn[8 * grp:8 * grp + 8] = 0.0
+    L, _, _ = oracle.quantize(W.astype(np.float64), xn, N)
+    wide = torch.zeros(n, m + 3, dtype=torch.float16, device="cuda")
+    wide[:, 1:m + 1] = torch.from_numpy(W).cuda()
+    nan = lambda s: np.isnan(np.ascontiguousarray(s).view(np.float16))  # noqa: E731
+    for Wd in (torch.from_numpy(W).cuda(), wide[:, 1:m + 1]):
+        got = stb.quantize(Wd, torch.from_numpy(xn).cuda(), N)
+        scale = got["scale"].cpu().numpy().view(np.uint16)
+        assert np.array_equal(nan(scale), nan(L.scale)) and nan(L.scale).any() == np.isnan(values).any()
+        got["scale"] = torch.from_numpy(np.where(nan(scale), L.scale, scale).view(np.int16))
+        _same_logical(got, L)
+
+
 def test_gpu_quantizer_takes_lambda_in_column_order(stb):
     """Two columns that compete for the last of 32 salient places, their scores so close that the last bits of lambda decide: the
     sum of 4096 norms in the definition's order gives one of them, an exactly rounded sum the other."""

@@ -481,6 +481,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   if (!fits) {                                         // the same for every thread of the grid
     __syncthreads();
     if (warp == kIssuerWarpA) tmem_dealloc(tmem_d, kTmemCols);
+    grid_dependency_wait();                            // (what follows on the stream waits for this grid alone)
     if (threadIdx.x == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
     return;
   }

@@ -106,6 +106,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
   const Header* hdr = reinterpret_cast<const Header*>(packed);
   // every CTA of a cluster takes the same branch here (the header is the same for all)
   if (!header_matches(hdr, n, m, N)) {
+    if constexpr (kChained) grid_dependency_wait();     // (what follows on the stream waits for this grid alone)
     if (threadIdx.x == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
     return;
   }
@@ -599,6 +600,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
       nrw[i] = h->nrw;
     }
   if (!fits) {
+    if (chained) grid_dependency_wait();                // (what follows on the stream waits for this grid alone)
     if (tid == 0 && dev_status) *dev_status = STB_ERR_CORRUPT;
     return;
   }

@@ -853,3 +853,40 @@ def test_chain_takes_one_gemv_kernel(stb, N, batch, h, f):
         if y.dtype == torch.float16:
             bound = bound + (y.double().abs() + bound) * 2.0 ** -11 * (1 + 2.0 ** -10) + 2.0 ** -25
         assert bool((err <= bound).all())
+
+
+@pytest.mark.parametrize("batch,n_bad", [(1, 64), (1, 8192), (9, 64), (9, 8192)])
+def test_calls_after_a_refused_layer_keep_the_stream_order(stb, batch, n_bad):
+    """A chain of a long step and one whose packed buffer does not match (found by the kernel, for either GEMV kernel), then a call
+    on the same stream that reads the long step's output: the refused launch leaves early, the call after it must not."""
+    import torch
+    N, h, f = 4, 4096, 28672
+    long_layer = stb.pack_numpy(si.logical_layer(f, h, N, 3600))
+    next_layer = stb.pack_numpy(si.logical_layer(64, f, N, 3601))
+    other = stb.pack_numpy(si.logical_layer(n_bad + 32, h, N, 3602))
+    bad = stb.PackedLayer(n_bad, h, N, other.buf, other.dev_status)
+    x = torch.from_numpy(si.activations(batch, h, 3603)).cuda()
+    mid = torch.zeros(batch, f, dtype=torch.float16, device="cuda")
+    out = torch.zeros(batch, n_bad, dtype=torch.float16, device="cuda")
+    steps = stb.make_steps([(long_layer, x, mid), (bad, x.clone(), out)])
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    X = torch.from_numpy(si.activations(64, h, 3604)).cuda()
+
+    def chain():
+        stb.layer_stack(None, dev_status=status, marshalled=steps)
+
+    def alone():
+        stb.gemv(long_layer, x, out=mid)
+        stb.gemm_f16(bad, X)
+
+    for call in (chain, alone):
+        call()
+        torch.cuda.synchronize()
+        want_mid = mid.clone()
+        want = stb.gemv(next_layer, want_mid)
+        for _ in range(10):
+            mid.zero_()
+            call()
+            got = stb.gemv(next_layer, mid)
+            assert torch.equal(mid, want_mid) and torch.equal(got, want)
+    assert int(status.item()) == stb.STB_ERR_CORRUPT and int(other.dev_status.item()) == stb.STB_ERR_CORRUPT

@@ -138,15 +138,15 @@ __device__ __forceinline__ uint32_t ldg_u16_coherent(const void* p) {
   asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
   return v;
 }
-// silu(a) b = a b / (1 + exp(-a)) in fp32: one reciprocal and one correction of the quotient (Markstein's: the remainder
-// by a fused multiply-add), within an ulp of the divided form without its slow path.  exp is held below 2^116: there
-// the quotient is far below the smallest fp16 value anyway.
+// silu(a) b = a b / (1 + exp(-a)) in fp32: one reciprocal and one correction of the quotient (Markstein's: the remainder by a
+// fused multiply-add), within an ulp of the divided form without its slow path.  Where the quotient or the divisor is infinite
+// the remainder is NaN and the product with the reciprocal is already what the division gives.
 __device__ __forceinline__ float silu_mul(float a, float b) {
-  const float d = 1.0f + __expf(fminf(-a, 80.0f));
+  const float d = 1.0f + __expf(-a);
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
-  const float q = a * r;
-  return fmaf(fmaf(-d, q, a), r, q) * b;
+  const float q = a * r, e = fmaf(-d, q, a);
+  return (e == e ? fmaf(e, r, q) : q) * b;
 }
 // fp16 pair (bits) of silu(a) * b per half, in fp32, rounded to nearest even
 __device__ __forceinline__ uint32_t silu_mul_bits(uint32_t a, uint32_t b) {

@@ -203,6 +203,57 @@ def test_gated_activation_that_fills_shared_memory(stb, N, batch, f):
     _check_gated_mlp(stb, torch, dg, du, dd, batch)
 
 
+def _picking_layer(m):
+    """A 4:8 layer whose row r is 1 in column r and 0 elsewhere: its output is its staged input."""
+    c = np.arange(m)
+    keep = np.full((m, m // 8), 0x0F, dtype=np.uint8)
+    keep[c, c // 8] = np.where(c % 8 < 4, 0x0F, 0xF0)
+    region = np.full((m, m // 8), 0x55, dtype=np.uint16)
+    region[c, c // 8] = 0x55 & ~(1 << (2 * (c % 4)))
+    scale = np.zeros((m, m // 128, 5), dtype=np.float16)
+    scale[..., 0] = 1.0
+    return dict(n=m, m=m, N=4, keep=keep, sign=np.full((m, m // 8), 0x0F, dtype=np.uint8), region=region, sign2=np.zeros((m, m // 128), dtype=np.uint32),
+                salient=np.zeros((m // 128, 2), dtype=np.uint64), scale=scale.view(np.uint16))
+
+
+def _formed(stb, torch, gate, up):
+    """fp16(silu(gate) * up) as the resident kernel stages it, for arrays of rows of up to 8 x m values."""
+    rows, m = gate.shape
+    layer, y = stb.pack_numpy(_picking_layer(m)), torch.zeros(rows, m, device="cuda")
+    _run(stb, torch, [(layer, (torch.from_numpy(gate).cuda(), torch.from_numpy(up).cuda()), y)])
+    return y.cpu().numpy()
+
+
+@pytest.mark.parametrize("up", [1.0, -0.4375])
+def test_gated_activation_of_every_finite_gate(stb, up):
+    """All finite fp16 gates against float64: fp32 arithmetic (__expf: 2 + 1.173 |a| ulp; sum, quotient and product another 4), one
+    rounding to fp16."""
+    import torch
+    codes = np.arange(65536, dtype=np.uint16).view(np.float16)
+    codes = np.where(np.isfinite(codes), codes, np.float16(0)).reshape(4, 8, 2048)
+    for gate in codes:
+        got = _formed(stb, torch, gate, np.full_like(gate, up)).astype(np.float64)
+        a = gate.astype(np.float64)
+        with np.errstate(over="ignore"):
+            want = a / (1.0 + np.exp(-a)) * up
+        bound = np.abs(want) * (2.0 ** -11 + (6.0 + 1.173 * np.abs(a)) * 2.0 ** -23) * (1 + 2.0 ** -9) + 2.0 ** -25
+        assert (np.abs(got - want) <= bound).all()
+
+
+@pytest.mark.parametrize("a", [np.inf, -np.inf, np.nan, 65504.0, -65504.0, -100.0, -88.0])
+@pytest.mark.parametrize("b", [2.0, -0.5, 0.0, np.inf])
+def test_gated_activation_of_infinite_and_largest_gates(stb, a, b):
+    """What fp32 a / (1 + exp(-a)) * b gives, where a linear before it overflowed."""
+    import torch
+    gate, up = np.zeros((1, 128), dtype=np.float16), np.ones((1, 128), dtype=np.float16)
+    gate[0, 37], up[0, 37] = a, b
+    with np.errstate(all="ignore"):
+        f = np.float32
+        want = float((f(a) / (f(1) + np.exp(f(-a))) * f(b)).astype(np.float16))
+    got = float(_formed(stb, torch, gate, up)[0, 37])
+    assert got == want or (np.isnan(got) and np.isnan(want)), (got, want)
+
+
 def test_gated_mlp_full_size(stb):
     """The LLaMA-2-7B MLP at 6:8 (quantizer-made) with the gated activation, in a CUDA graph as bench.py runs it."""
     import torch

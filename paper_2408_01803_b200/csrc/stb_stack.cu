@@ -24,9 +24,9 @@
 //     word of the phase are gathered into shared memory while x is staged.
 //   * Partial sums: a warp that covers a whole row tile writes y itself; the others leave their head / tail
 //     pieces in shared memory and the CTA adds them in tile order at the end of the phase; of a row tile that
-//     straddles CTAs the later ones hand their sums to the first through the caller's workspace, every value beside a tag
-//     of the launch and phase (one 8-byte store, no fence, no counter), and the first adds them in CTA order.  Every
-//     sum has a fixed order: results are reproducible.
+//     straddles CTAs the later ones hand their sums to the first through the caller's workspace, every value beside the
+//     number of its phase (one 8-byte store, no fence, no counter), and the first adds them in CTA order and empties their
+//     places, so that no value outlives its phase.  Every sum has a fixed order: results are reproducible.
 //   * A phase may read what an earlier phase wrote: a CTA starts a phase's arithmetic only when the count of
 //     finished row tiles (one counter in the workspace, bumped once per CTA and phase) has reached the total
 //     of all earlier phases.  The poll is bounded; when it or an mbarrier wait runs out, an abort flag makes
@@ -90,8 +90,9 @@ struct StackParams {
   uint32_t pos_row;                           // bytes from one entry of a position table to the next
   uint32_t part_floats;                       // floats per partial slot: 32 rows x largest batch
   uint32_t max_share;                         // most CTAs that share one row tile
-  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left, [4] launches so far
-  uint2* gpart;                               // sums handed on for row tiles that straddle CTAs: { value, tag }
+  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left
+  uint2* gpart;                               // sums handed on for row tiles that straddle CTAs: { value, tag }, empty ({ 0, 0 }) between launches
+  uint32_t gpart_slots;
   int* dev_status;
   long long wait_limit;
   int32_t copies_off;
@@ -528,7 +529,6 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
   E.empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)warp;
   WarpState W;
   W.slot = 0; W.parity = 0; W.failed = false;
-  const uint32_t epoch = __ldcg(P.sync + 4);          // changed only by the last CTA out
   // tables, while the first copies are under way
   if (P.use_meta6)
     for (int i = threadIdx.x; i < (int)(kMasks6 * kMasks6); i += kSThreads)
@@ -673,7 +673,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
         // a straddling row tile: the CTA where it begins gathers the others' sums, in CTA order
         const int c_first = R == range.first ? range.head_cta : range.tail_cta, share = R == range.first ? range.head_share : range.tail_share;
         uint2* gp = P.gpart + (size_t)R * P.max_share * P.part_floats;
-        const uint32_t tag = ((epoch + 1u) << 6) | (uint32_t)ph;
+        const uint32_t tag = (uint32_t)ph + 1u;
         bool lost = false;
         for (int v = lane; v < nval; v += 32) {
           const float* pv = pdata + v;
@@ -702,6 +702,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
                 x = ld_tagged(gp + (size_t)k * P.part_floats + v);
               }
               sum += __uint_as_float(x.x);
+              st_tagged(gp + (size_t)k * P.part_floats + v, 0.0f, 0u);      // empty for whoever uses it next
             }
           }
           const int row = rt * kTileRows + (batch == 1 ? v : v / batch), bc = batch == 1 ? 0 : v % batch;
@@ -769,7 +770,11 @@ stack_kernel(const __grid_constant__ StackParams P) {
   __syncthreads();
   if (ctl[2]) {
     __threadfence();
-    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; P.sync[4] += 1u; __threadfence(); }
+    // a launch that was given up leaves sums that nobody took
+    if (*reinterpret_cast<volatile uint32_t*>(P.sync + 1) != 0u)
+      for (uint32_t i = threadIdx.x; i < P.gpart_slots; i += kSAllThreads) P.gpart[i] = make_uint2(0u, 0u);
+    __syncthreads();
+    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; __threadfence(); }
   }
 }
 
@@ -956,7 +961,7 @@ static int plan_smem(StackParams& sp, bool image, bool gather) {
 // Builds the phases of steps [i0, ...) into `sp` (at most kMaxPhases), returns the index of the first step not taken.
 static int build_phases(const stb_step* steps, int count, int i0, int G, StackParams& sp, size_t& sync_need, size_t& gpart_need) {
   sp.nphase = 0;
-  sp.part_floats = 32; sp.max_share = 1;
+  sp.part_floats = 32; sp.max_share = 1; sp.gpart_slots = 0;
   uint32_t done = 0;
   long long maxR = 0;
   int i = i0;
@@ -1011,7 +1016,8 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
   }
   if (!staged) return -1;                                            // the formed input does not fit shared memory
   const size_t s_need = 8 * sizeof(uint32_t);
-  const size_t g_need = sp.max_share > 1 ? (size_t)maxR * sp.max_share * sp.part_floats * sizeof(uint2) : 0;
+  if (sp.max_share > 1) sp.gpart_slots = (uint32_t)maxR * sp.max_share * sp.part_floats;
+  const size_t g_need = (size_t)sp.gpart_slots * sizeof(uint2);
   if (s_need > sync_need) sync_need = s_need;
   if (g_need > gpart_need) gpart_need = g_need;
   return i;

@@ -117,6 +117,29 @@ def test_more_groups_than_one_launch_holds(stb):
     _check_layers(triples, [Ls[k % 4] for k in range(70)])
 
 
+def test_nothing_stays_in_the_workspace(stb):
+    """Row tiles that straddle CTAs hand sums on through the workspace: after every call it is zero as a whole, so that no sum of
+    an earlier launch can ever be taken for this one's, however many launches lie between."""
+    import torch
+    small, wide = si.logical_layer(320, 4096, 6, 94), si.logical_layer(1000, 2048, 5, 95)
+    ls, lw = stb.pack_numpy(small), stb.pack_numpy(wide)
+    xs = torch.from_numpy(si.activations(2, 4096, 96)).cuda()
+    ys, yw = torch.zeros(2, 320, device="cuda"), torch.zeros(2, 1000, device="cuda")
+    lists = [[(ls, xs, ys)], [(lw, xs[:, :2048], yw), (ls, xs, ys)]]
+    steps = [stb.make_steps(t) for t in lists]
+    ws = torch.zeros(max(stb.resident_workspace(s).numel() for s in steps), dtype=torch.uint8, device="cuda")
+    assert ws.numel() > 1024
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for k in range(4):
+        stb.layer_stack_resident(None, ws, dev_status=status, marshalled=steps[k % 2])
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and int(ws.max().item()) == 0
+        _check_layers(lists[k % 2], [oracle.Logical(**d) for d in ((small,), (wide, small))[k % 2]])
+    stb.layer_stack_resident(None, ws, dev_status=status, marshalled=steps[1], selftest=True)
+    torch.cuda.synchronize()
+    assert int(status.item()) == stb.STB_ERR_TIMEOUT and int(ws.max().item()) == 0
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_workspace_is_zero_again(stb):
     import torch
     d1, d2 = si.logical_layer(512, 1024, 6, 91), si.logical_layer(256, 512, 5, 92)

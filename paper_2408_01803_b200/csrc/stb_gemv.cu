@@ -5,6 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <mutex>
+
 #include "../../include/stb.h"
 #include "stb_decode.cuh"
 #include "stb_layout.cuh"
@@ -1017,11 +1020,17 @@ static cudaError_t launch_stream(const GemvLayers& layers, const GemvPlan& plan,
                             wait_selftest ? kSelftestWaitLimit : kWaitLimit, wait_selftest ? 1 : 0, chained ? 1 : 0);
 }
 
-// Clusters of 1 to 8 CTAs (one CTA per SM) that a device holds at once, by their size.
+// Clusters of 1 to 8 CTAs (one CTA per SM) that a device holds at once, by their size.  Asked for once per device; several host
+// threads may come here at the same time, and all must get the whole answer (the choice of kernel, and with it the order of
+// the sums, depends on it).
 static cudaError_t gemv_clusters(int dev, int (&most)[9]) {
   static int cached[kMaxDevices][9] = {};
+  static std::atomic<bool> filled[kMaxDevices] = {};
+  static std::mutex filling;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (!cached[dev][1]) {
+  std::unique_lock<std::mutex> lock(filling, std::defer_lock);
+  if (!filled[dev].load(std::memory_order_acquire)) lock.lock();
+  if (lock.owns_lock() && !filled[dev].load(std::memory_order_relaxed)) {
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -1039,7 +1048,8 @@ static cudaError_t gemv_clusters(int dev, int (&most)[9]) {
       cfg.attrs = at; cfg.numAttrs = 1;
       if (cudaOccupancyMaxActiveClusters(&v[C], gemv_stream_kernel<4, 1, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); v[C] = 0; }
     }
-    for (int C = 8; C >= 1; --C) cached[dev][C] = v[C];           // [1] last: it marks the entry as filled
+    for (int C = 1; C <= 8; ++C) cached[dev][C] = v[C];
+    filled[dev].store(true, std::memory_order_release);
   }
   for (int C = 0; C <= 8; ++C) most[C] = cached[dev][C];
   return cudaSuccess;

@@ -890,3 +890,41 @@ def test_calls_after_a_refused_layer_keep_the_stream_order(stb, batch, n_bad):
             got = stb.gemv(next_layer, mid)
             assert torch.equal(mid, want_mid) and torch.equal(got, want)
     assert int(status.item()) == stb.STB_ERR_CORRUPT and int(other.dev_status.item()) == stb.STB_ERR_CORRUPT
+
+
+FIRST_CALLS = """
+import sys, threading
+sys.path.insert(0, sys.argv[1])
+import torch
+import paper_2408_01803_b200 as stb
+import stb_inputs as si
+shapes = [(4096, 4096, 4, 1), (1500, 5120, 6, 9), (2048, 2816, 5, 16), (8192, 2176, 6, 7), (1024, 8192, 4, 1), (5003, 2816, 5, 3)]
+work = []
+for n, m, N, batch in shapes:
+    work.append((stb.pack_numpy(si.logical_layer(n, m, N, 3700)), torch.from_numpy(si.activations(batch, m, 3701)).cuda()))
+torch.cuda.synchronize()
+got, go = {}, threading.Barrier(len(work))
+def one(k):
+    s = torch.cuda.Stream()
+    go.wait()
+    got[k] = stb.gemv(*work[k], stream=s)
+    s.synchronize()
+threads = [threading.Thread(target=one, args=(k,)) for k in range(len(work))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert len(got) == len(work)
+for k, w in enumerate(work):
+    assert torch.equal(got[k], stb.gemv(*w)), shapes[k]
+print("same")
+"""
+
+
+def test_first_calls_from_several_threads():
+    """A process whose first GEMV calls come from six threads at once: each gets the kernel, and so the order of sums, of any later call."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", FIRST_CALLS, root], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]

@@ -112,6 +112,11 @@ PyObject* wrap(const at::Tensor& t) { return THPVariable_Wrap(t); }
 // what the Python forms are called with where the plain case does not hold
 PyObject* slow[5];
 PyObject* pass_on(int which, PyObject* const* args, Py_ssize_t n) { return PyObject_Vectorcall(slow[which], args, (size_t)n, nullptr); }
+// where torch threw (no device, no memory, a tensor without storage; nothing was launched): the Python form raises what it raises
+PyObject* threw(int which, PyObject* const* args, Py_ssize_t n) {
+  PyErr_Clear();
+  return pass_on(which, args, n);
+}
 
 // gemv(layer, x, out, out_dtype, stream): 17.0 us of host time per call through ctypes, 6.6 us here (1024 x 8192), of which the launch is the larger part
 PyObject* bind_gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -134,7 +139,7 @@ PyObject* bind_gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[2] != Py_None) { Py_INCREF(a[2]); return a[2]; }
     return wrap(y);
   } catch (const std::exception&) {
-    return pass_on(0, a, n);              // (nothing was launched: only the allocation can throw)
+    return threw(0, a, n);
   }
 }
 
@@ -167,7 +172,7 @@ PyObject* bind_gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[2] != Py_None) { Py_INCREF(a[2]); return a[2]; }
     return wrap(y);
   } catch (const std::exception&) {
-    return pass_on(which, a, n);
+    return threw(which, a, n);
   }
 }
 
@@ -178,36 +183,53 @@ bool status_of(PyObject* o, int*& p) {
   p = static_cast<int*>(THPVariable_Unpack(o).data_ptr());
   return true;
 }
+// The marshalled steps of a list call (a ctypes array of stb_step).
+struct Steps {
+  Py_buffer b;
+  const stb_step* data = nullptr;
+  int count = 0;
+  explicit Steps(PyObject* o) {
+    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) { PyErr_Clear(); return; }
+    if (b.len % sizeof(stb_step)) { PyBuffer_Release(&b); return; }
+    data = static_cast<const stb_step*>(b.buf);
+    count = (int)(b.len / sizeof(stb_step));
+    held = true;
+  }
+  ~Steps() { if (held) PyBuffer_Release(&b); }
+  bool held = false;
+};
 // layer_stack(steps, dev_status, stream, marshalled)
 PyObject* bind_layer_stack(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void* s;
   int* st;
-  Py_buffer b;
-  if (n != 4 || a[3] == Py_None || !stream_of(a[2], s) || !status_of(a[1], st)) return pass_on(3, a, n);
-  if (PyObject_GetBuffer(a[3], &b, PyBUF_SIMPLE) != 0) { PyErr_Clear(); return pass_on(3, a, n); }
-  const int rc = b.len % sizeof(stb_step) ? -1 : unlocked([&] { return f_layer_stack(static_cast<const stb_step*>(b.buf), (int)(b.len / sizeof(stb_step)), st, s); });
-  PyBuffer_Release(&b);
-  if (rc == -1) return pass_on(3, a, n);
-  if (rc != STB_OK) return failed(rc, "stb_layer_stack");
-  Py_RETURN_NONE;
+  try {
+    if (n != 4 || a[3] == Py_None || !stream_of(a[2], s) || !status_of(a[1], st)) return pass_on(3, a, n);
+    const Steps steps(a[3]);
+    if (!steps.held) return pass_on(3, a, n);
+    const int rc = unlocked([&] { return f_layer_stack(steps.data, steps.count, st, s); });
+    if (rc != STB_OK) return failed(rc, "stb_layer_stack");
+    Py_RETURN_NONE;
+  } catch (const std::exception&) {
+    return threw(3, a, n);
+  }
 }
 // layer_stack_resident(steps, ws, dev_status, stream, marshalled, selftest)
 PyObject* bind_layer_stack_resident(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void* s;
   int* st;
-  Py_buffer b;
-  if (n != 6 || a[4] == Py_None || a[5] != Py_False || !THPVariable_Check(a[1]) || !stream_of(a[3], s) || !status_of(a[2], st)) return pass_on(4, a, n);
-  const at::Tensor& ws = THPVariable_Unpack(a[1]);
-  if (PyObject_GetBuffer(a[4], &b, PyBUF_SIMPLE) != 0) { PyErr_Clear(); return pass_on(4, a, n); }
-  void* wp = ws.data_ptr();
-  const size_t wb = (size_t)ws.numel();
-  const int rc = b.len % sizeof(stb_step) ? -1 : unlocked([&] {
-    return f_layer_stack_resident(static_cast<const stb_step*>(b.buf), (int)(b.len / sizeof(stb_step)), wp, wb, st, s);
-  });
-  PyBuffer_Release(&b);
-  if (rc == -1) return pass_on(4, a, n);
-  if (rc != STB_OK) return failed(rc, "stb_layer_stack_resident");
-  Py_RETURN_NONE;
+  try {
+    if (n != 6 || a[4] == Py_None || a[5] != Py_False || !THPVariable_Check(a[1]) || !stream_of(a[3], s) || !status_of(a[2], st)) return pass_on(4, a, n);
+    const at::Tensor& ws = THPVariable_Unpack(a[1]);
+    void* wp = ws.data_ptr();
+    const size_t wb = (size_t)ws.numel();
+    const Steps steps(a[4]);
+    if (!steps.held) return pass_on(4, a, n);
+    const int rc = unlocked([&] { return f_layer_stack_resident(steps.data, steps.count, wp, wb, st, s); });
+    if (rc != STB_OK) return failed(rc, "stb_layer_stack_resident");
+    Py_RETURN_NONE;
+  } catch (const std::exception&) {
+    return threw(4, a, n);
+  }
 }
 
 // start(addresses of the seven entry points in the order above, on_error, the five Python forms)

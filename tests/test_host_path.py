@@ -1,0 +1,33 @@
+"""The native host path of the calls (csrc/stb_bind.cpp) on a machine without a GPU: what torch throws inside it reaches Python."""
+import os
+import subprocess
+import sys
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+NO_DEVICE = """
+import sys
+sys.path.insert(0, sys.argv[1])
+import torch
+import paper_2408_01803_b200 as stb
+buf, status = torch.zeros(4096, dtype=torch.uint8), torch.zeros(1, dtype=torch.int32)
+layer = stb.PackedLayer(32, 128, 4, buf, status)
+x, y = torch.zeros(1, 128, dtype=torch.float16), torch.zeros(1, 32)
+steps = stb.make_steps([(layer, x, y)])
+calls = [lambda: stb.layer_stack(None, dev_status=status, marshalled=steps),
+         lambda: stb.layer_stack_resident(None, buf, dev_status=status, marshalled=steps),
+         lambda: stb.layer_stack([(layer, x, y)]),
+         lambda: stb.gemv(layer, x), lambda: stb.gemm_f16(layer, x), lambda: stb.gemm(layer, x.bfloat16())]
+for call in calls:
+    try:
+        call()
+    except (RuntimeError, AssertionError) as e:
+        print("raised", type(e).__name__)
+"""
+
+
+def test_calls_without_a_device_raise():
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")
+    r = subprocess.run([sys.executable, "-c", NO_DEVICE, ROOT], capture_output=True, text=True, timeout=600, env=env)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.count("raised") == 6, r.stdout

@@ -139,6 +139,24 @@ def _stream(stream=None):
     return C.c_void_p(s.cuda_stream)
 
 
+def _on(stream):
+    """The context in which a call allocates what it makes itself: memory belongs to the stream it is first written on, and goes
+    back to that stream's pool, so nothing else is given it while the call still runs."""
+    import contextlib
+    import torch
+    if stream is None:
+        return contextlib.nullcontext()
+    return torch.cuda.stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream))
+
+
+def _result(stream, *tensors):
+    """Tensors made under _on(stream) that the caller gets: read, as a rule, on the current stream (whose reads they then outlive)."""
+    import torch
+    if stream is not None:
+        for t in tensors:
+            t.record_stream(torch.cuda.current_stream(t.device))
+
+
 def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
 
@@ -172,9 +190,11 @@ def pack(n, m, N, keep, sign, region, sign2, salient, scale, stream=None, buf=No
     dev = keep.device
     for t in (keep, sign, region, sign2, salient, scale):
         assert t.is_cuda and t.is_contiguous()
-    if buf is None:
-        buf = torch.empty(pack_size(n, m, N), dtype=torch.uint8, device=dev)
-    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    with _on(stream):
+        made = torch.empty(pack_size(n, m, N), dtype=torch.uint8, device=dev) if buf is None else None
+        status = torch.zeros(1, dtype=torch.int32, device=dev)
+    buf = made if buf is None else buf
+    _result(stream, status, *([made] if made is not None else []))
     L = _Logical(n, m, N, keep.data_ptr(), sign.data_ptr(), region.data_ptr(), sign2.data_ptr(),
                  salient.data_ptr(), scale.data_ptr())
     _check(_lib.stb_pack(C.byref(L), _ptr(buf), buf.numel(), _ptr(status), _stream(stream)), "stb_pack")
@@ -188,9 +208,10 @@ def pack_numpy(d: dict, device="cuda", stream=None) -> PackedLayer:
     import torch
     def up(a, view):
         return torch.from_numpy(np.ascontiguousarray(a).view(view)).to(device)
-    return pack(int(d["n"]), int(d["m"]), int(d["N"]), up(d["keep"], np.uint8), up(d["sign"], np.uint8),
-                up(d["region"], np.int16), up(d["sign2"], np.int32), up(d["salient"], np.int64),
-                up(d["scale"], np.int16), stream=stream)
+    with _on(stream):
+        fields = [up(d["keep"], np.uint8), up(d["sign"], np.uint8), up(d["region"], np.int16), up(d["sign2"], np.int32),
+                  up(d["salient"], np.int64), up(d["scale"], np.int16)]
+    return pack(int(d["n"]), int(d["m"]), int(d["N"]), *fields, stream=stream)
 
 
 def dequant(layer: PackedLayer, dtype=None, out=None, stream=None):
@@ -198,7 +219,9 @@ def dequant(layer: PackedLayer, dtype=None, out=None, stream=None):
     dtype = dtype or torch.float32
     dt = {torch.float32: STB_F32, torch.float16: STB_F16, torch.bfloat16: STB_BF16}[dtype]
     if out is None:
-        out = torch.empty((layer.n, layer.m), dtype=dtype, device=layer.buf.device)
+        with _on(stream):
+            out = torch.empty((layer.n, layer.m), dtype=dtype, device=layer.buf.device)
+        _result(stream, out)
     assert out.dtype == dtype and out.stride(1) == 1
     _check(_lib.stb_dequant(_ptr(layer.buf), layer.n, layer.m, layer.N, _ptr(out), dt, out.stride(0),
                             _stream(stream)), "stb_dequant")
@@ -216,7 +239,9 @@ def _gemv_py(layer: PackedLayer, x, out=None, out_dtype=None, stream=None):
     assert x2.dtype == torch.float16 and x2.is_cuda and x2.stride(1) == 1
     batch = x2.shape[0]
     if out is None:
-        out = torch.empty((batch, layer.n), dtype=out_dtype or torch.float32, device=x.device)
+        with _on(stream):
+            out = torch.empty((batch, layer.n), dtype=out_dtype or torch.float32, device=x.device)
+        _result(stream, out)
     ydt = {torch.float32: STB_F32, torch.float16: STB_F16}[out.dtype]
     _check(_lib.stb_gemv(_ptr(layer.buf), layer.n, layer.m, layer.N, _ptr(x2), batch, x2.stride(0),
                          _ptr(out), ydt, out.stride(0), _ptr(layer.dev_status), _stream(stream)), "stb_gemv")
@@ -250,11 +275,14 @@ def _gemm_py(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, stream=No
     assert X.dtype == torch.bfloat16 and X.is_cuda and X.dim() == 2 and X.stride(1) == 1
     T = X.shape[0]
     if out is None:
-        out = torch.empty((T, layer.n), dtype=out_dtype or torch.float32, device=X.device)
+        with _on(stream):
+            out = torch.empty((T, layer.n), dtype=out_dtype or torch.float32, device=X.device)
+        _result(stream, out)
     ydt = {torch.float32: STB_F32, torch.bfloat16: STB_BF16}[out.dtype]
     need = gemm_workspace(layer.n, layer.m, layer.N, T)
     if need and (ws is None or ws.numel() * ws.element_size() < need):
-        ws = torch.empty(need, dtype=torch.uint8, device=X.device)
+        with _on(stream):
+            ws = torch.empty(need, dtype=torch.uint8, device=X.device)
     _check(_lib.stb_gemm(_ptr(layer.buf), layer.n, layer.m, layer.N, _ptr(X), T, X.stride(0), _ptr(out),
                          ydt, out.stride(0), _ptr(ws), (ws.numel() * ws.element_size()) if ws is not None else 0,
                          _ptr(layer.dev_status), _stream(stream)), "stb_gemm")
@@ -277,11 +305,14 @@ def _gemm_f16_py(layer: PackedLayer, X, out=None, out_dtype=None, ws=None, strea
     assert X.dtype == torch.float16 and X.is_cuda and X.dim() == 2 and X.stride(1) == 1
     T = X.shape[0]
     if out is None:
-        out = torch.empty((T, layer.n), dtype=out_dtype or torch.float32, device=X.device)
+        with _on(stream):
+            out = torch.empty((T, layer.n), dtype=out_dtype or torch.float32, device=X.device)
+        _result(stream, out)
     ydt = {torch.float32: STB_F32, torch.float16: STB_F16}[out.dtype]
     need = gemm_f16_workspace(layer.n, layer.m, layer.N, T)
     if ws is None or ws.numel() * ws.element_size() < need:
-        ws = torch.empty(max(need, 256), dtype=torch.uint8, device=X.device)
+        with _on(stream):
+            ws = torch.empty(max(need, 256), dtype=torch.uint8, device=X.device)
     _check(_lib.stb_gemm_f16(_ptr(layer.buf), layer.n, layer.m, layer.N, _ptr(X), T, X.stride(0), _ptr(out),
                              ydt, out.stride(0), _ptr(ws), ws.numel() * ws.element_size(),
                              _ptr(layer.dev_status), _stream(stream)), "stb_gemm_f16")
@@ -377,7 +408,9 @@ def layer_stack_checksum(marshalled, sums=None, dev_status=None, stream=None):
     """stb_layer_stack_checksum: XOR of the streamed words of every step's packed layer -> torch.int64[count]."""
     import torch
     if sums is None:
-        sums = torch.zeros(len(marshalled), dtype=torch.int64, device="cuda")
+        with _on(stream):
+            sums = torch.zeros(len(marshalled), dtype=torch.int64, device="cuda")
+        _result(stream, sums)
     _check(_lib.stb_layer_stack_checksum(marshalled, len(marshalled), _ptr(sums), _ptr(dev_status), _stream(stream)),
            "stb_layer_stack_checksum")
     return sums
@@ -387,12 +420,13 @@ def allocate_nm(weights, r_target, stream=None):
     """Layer-wise N:M assignment (stb_weight_sumsq per layer, then stb_allocate_nm): `weights` is a list of dense fp16
     CUDA matrices; returns the list of N."""
     import torch
-    sums = torch.zeros(len(weights), dtype=torch.float64, device=weights[0].device)
-    for k, W in enumerate(weights):
-        assert W.dtype == torch.float16 and W.dim() == 2 and W.stride(1) == 1
-        _check(_lib.stb_weight_sumsq(_ptr(W), W.shape[0], W.shape[1], W.stride(0), C.c_void_p(sums.data_ptr() + 8 * k),
-                                     _stream(stream)), "stb_weight_sumsq")
-    host = sums.cpu().numpy()
+    with _on(stream):
+        sums = torch.zeros(len(weights), dtype=torch.float64, device=weights[0].device)
+        for k, W in enumerate(weights):
+            assert W.dtype == torch.float16 and W.dim() == 2 and W.stride(1) == 1
+            _check(_lib.stb_weight_sumsq(_ptr(W), W.shape[0], W.shape[1], W.stride(0), C.c_void_p(sums.data_ptr() + 8 * k),
+                                         _stream(stream)), "stb_weight_sumsq")
+        host = sums.cpu().numpy()
     arr = (C.c_double * len(weights))(*[float(vv) for vv in host])
     out = (C.c_int * len(weights))()
     _check(_lib.stb_allocate_nm(arr, len(weights), float(r_target), out), "stb_allocate_nm")
@@ -407,12 +441,14 @@ def quantize(W, xnorm, N, lam=-1.0, stream=None):
     assert xnorm.dtype == torch.float64 and xnorm.is_cuda and xnorm.is_contiguous()
     n, m = W.shape
     dev = W.device
-    out = {"keep": torch.empty((n, m // 8), dtype=torch.uint8, device=dev), "sign": torch.empty((n, m // 8), dtype=torch.uint8, device=dev),
-           "region": torch.empty((n, m // 8), dtype=torch.int16, device=dev), "sign2": torch.empty((n, m // 128), dtype=torch.int32, device=dev),
-           "salient": torch.empty((m // 128, 2), dtype=torch.int64, device=dev), "scale": torch.empty((n, m // 128, 5), dtype=torch.int16, device=dev)}
     need = C.c_size_t()
     _check(_lib.stb_quantize_workspace(n, m, C.byref(need)), "stb_quantize_workspace")
-    ws = torch.empty(need.value, dtype=torch.uint8, device=dev)
+    with _on(stream):
+        out = {"keep": torch.empty((n, m // 8), dtype=torch.uint8, device=dev), "sign": torch.empty((n, m // 8), dtype=torch.uint8, device=dev),
+               "region": torch.empty((n, m // 8), dtype=torch.int16, device=dev), "sign2": torch.empty((n, m // 128), dtype=torch.int32, device=dev),
+               "salient": torch.empty((m // 128, 2), dtype=torch.int64, device=dev), "scale": torch.empty((n, m // 128, 5), dtype=torch.int16, device=dev)}
+        ws = torch.empty(need.value, dtype=torch.uint8, device=dev)
+    _result(stream, *out.values())
     L = _Logical(n, m, N, out["keep"].data_ptr(), out["sign"].data_ptr(), out["region"].data_ptr(), out["sign2"].data_ptr(),
                  out["salient"].data_ptr(), out["scale"].data_ptr())
     _check(_lib.stb_quantize(_ptr(W), W.stride(0), _ptr(xnorm), n, m, N, float(lam), C.byref(L), _ptr(ws), ws.numel(), _stream(stream)),

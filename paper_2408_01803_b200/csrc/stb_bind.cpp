@@ -8,6 +8,8 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -74,8 +76,19 @@ bool rows_of(PyObject* o, at::ScalarType t, bool vector_too, at::Tensor& x) {
   x = THPVariable_Unpack(o);
   return x.scalar_type() == t && x.is_cuda() && ((x.dim() == 2 && x.stride(1) == 1) || (vector_too && x.dim() == 1 && x.stride(0) == 1));
 }
+// A tensor that the call makes for itself, on the launch stream: its memory belongs to that stream's pool, so that nothing else is
+// given it while the call still runs.  `kept`: one that the caller gets, and reads as a rule on the current stream.
+at::Tensor make(at::IntArrayRef size, const at::TensorOptions& options, void* s, bool kept) {
+  const c10::DeviceIndex dev = options.device().index();
+  const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream(dev);
+  if (current.stream() == static_cast<cudaStream_t>(s)) return at::empty(size, options);
+  const c10::cuda::CUDAStreamGuard guard(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(s), dev));
+  at::Tensor t = at::empty(size, options);
+  if (kept) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), current);
+  return t;
+}
 // output: the given tensor (two-dimensional, of type 32 or 16), or a new one of the asked type
-bool output_of(PyObject* out, PyObject* out_dtype, at::ScalarType t16, int64_t rows, int64_t n, const at::Tensor& like, at::Tensor& y) {
+bool output_of(PyObject* out, PyObject* out_dtype, at::ScalarType t16, int64_t rows, int64_t n, const at::Tensor& like, void* s, at::Tensor& y) {
   if (out != Py_None) {
     if (!THPVariable_Check(out)) return false;
     y = THPVariable_Unpack(out);
@@ -87,7 +100,7 @@ bool output_of(PyObject* out, PyObject* out_dtype, at::ScalarType t16, int64_t r
     t = reinterpret_cast<THPDtype*>(out_dtype)->scalar_type;
     if (t != at::kFloat && t != t16) return false;
   }
-  y = at::empty({rows, n}, like.options().dtype(t));
+  y = make({rows, n}, like.options().dtype(t), s, true);
   return true;
 }
 stb_dtype dtype_code(at::ScalarType t) { return t == at::kFloat ? STB_F32 : (t == at::kHalf ? STB_F16 : STB_BF16); }
@@ -128,7 +141,7 @@ PyObject* bind_gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!layer_of(a[0], l) || !rows_of(a[1], at::kHalf, true, x)) return pass_on(0, a, n);
     const bool vec = x.dim() == 1;
     const int64_t batch = vec ? 1 : x.size(0);
-    if (!stream_of(a[4], s) || !output_of(a[2], a[3], at::kHalf, batch, l.n, x, y)) return pass_on(0, a, n);
+    if (!stream_of(a[4], s) || !output_of(a[2], a[3], at::kHalf, batch, l.n, x, s, y)) return pass_on(0, a, n);
     const void* xp = x.data_ptr();
     void* yp = y.data_ptr();
     const size_t ldx = (size_t)(vec ? x.size(0) : x.stride(0)), ldy = (size_t)y.stride(0);
@@ -161,8 +174,8 @@ PyObject* bind_gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
       if (!THPVariable_Check(a[4])) return pass_on(which, a, n);
       ws = THPVariable_Unpack(a[4]);
     }
-    if (!output_of(a[2], a[3], t16, T, l.n, x, y)) return pass_on(which, a, n);
-    if (!ws.defined() || (size_t)ws.nbytes() < need) ws = at::empty({(int64_t)(need < 256 ? 256 : need)}, x.options().dtype(at::kByte));
+    if (!output_of(a[2], a[3], t16, T, l.n, x, s, y)) return pass_on(which, a, n);
+    if (!ws.defined() || (size_t)ws.nbytes() < need) ws = make({(int64_t)(need < 256 ? 256 : need)}, x.options().dtype(at::kByte), s, false);
     const void* xp = x.data_ptr();
     void *yp = y.data_ptr(), *wp = ws.data_ptr();
     const size_t ldx = (size_t)x.stride(0), ldy = (size_t)y.stride(0), wb = (size_t)ws.nbytes();

@@ -928,3 +928,31 @@ def test_first_calls_from_several_threads():
     for _ in range(2):
         r = subprocess.run([sys.executable, "-c", FIRST_CALLS, root], capture_output=True, text=True, timeout=300)
         assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("form", ["gemm", "gemm_f16", "_gemm_py", "_gemm_f16_py"])
+def test_memory_a_call_makes_belongs_to_its_stream(stb, form):
+    """A GEMM on another stream than the current one, with the workspace left to the call: what the current stream is given
+    and overwrites meanwhile is never that workspace, nor a result that was let go before it was finished."""
+    import torch
+    n, m, N, T = 4096, 4096, 5, 1024
+    layer = stb.pack_numpy(si.logical_layer(n, m, N, 3800, salient_counts=[32, 9, 20]))
+    t16 = torch.float16 if "f16" in form else torch.bfloat16
+    x = torch.from_numpy(si.activations(T, m, 3801).astype(np.float32)).to(t16).cuda()
+    call = getattr(stb, form)
+    want = call(layer, x, out_dtype=t16)
+    need = stb.gemm_f16_workspace(n, m, N, T) if "f16" in form else stb.gemm_workspace(n, m, N, T)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    for _ in range(8):
+        call(layer, x, out_dtype=t16, stream=side)                     # its result goes at once
+        got = call(layer, x, out_dtype=t16, stream=side)
+        others = []
+        for _ in range(40):
+            others += [torch.empty(need, dtype=torch.uint8, device="cuda").fill_(0x7F), torch.empty(n * T * 2, dtype=torch.uint8, device="cuda").fill_(0x7F)]
+            del others[:-6]
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+        assert all(bool((o == 0x7F).all()) for o in others)
+        del got, others

@@ -105,21 +105,34 @@ _lib = _LazyLib()
 _bind = None
 
 
+class _PythonForms:
+    """The same calls through ctypes, where the native host path cannot be loaded."""
+
+    def __init__(self):
+        self.gemv, self.gemm, self.gemm_f16 = _gemv_py, _gemm_py, _gemm_f16_py
+        self.layer_stack, self.layer_stack_resident = _layer_stack_py, _layer_stack_resident_py
+
+
 def _fast():
     """The native host path of the calls that a decode or prefill loop makes (csrc/stb_bind.cpp).  It takes the plain cases
-    and hands everything else to the `_..._py` form of the call below."""
+    and hands everything else to the `_..._py` form of the call below.  Without it (not built, or built against another
+    torch) those forms take every call, with a warning: the kernels are the same, a call costs more host time."""
     global _bind
     if _bind is None:
         import torch  # noqa: F401  (its libraries first)
         from importlib.machinery import ExtensionFileLoader
         from importlib.util import module_from_spec, spec_from_loader
-        if not os.path.exists(BIND_PATH):
-            raise ImportError("_stb_bind.so is not built (%s): run `python -m paper_2408_01803_b200.build`" % BIND_PATH)
-        mod = module_from_spec(spec_from_loader("_stb_bind", ExtensionFileLoader("_stb_bind", BIND_PATH)))
-        mod.__loader__.exec_module(mod)
         names = ("stb_gemv", "stb_gemm_workspace", "stb_gemm", "stb_gemm_f16_workspace", "stb_gemm_f16", "stb_layer_stack", "stb_layer_stack_resident")
-        mod.start(*[C.cast(getattr(_lib, nm), C.c_void_p).value for nm in names], _check, _gemv_py, _gemm_py, _gemm_f16_py, _layer_stack_py,
-                  _layer_stack_resident_py)
+        entries = [C.cast(getattr(_lib, nm), C.c_void_p).value for nm in names]
+        try:
+            mod = module_from_spec(spec_from_loader("_stb_bind", ExtensionFileLoader("_stb_bind", BIND_PATH)))
+            mod.__loader__.exec_module(mod)
+        except ImportError as e:
+            import warnings
+            warnings.warn("the native host path is not available (%s): run `python -m paper_2408_01803_b200.build`" % e)
+            mod = _PythonForms()
+        else:
+            mod.start(*entries, _check, _gemv_py, _gemm_py, _gemm_f16_py, _layer_stack_py, _layer_stack_resident_py)
         _bind = mod
     return _bind
 

@@ -31,3 +31,18 @@ def test_calls_without_a_device_raise():
     r = subprocess.run([sys.executable, "-c", NO_DEVICE, ROOT], capture_output=True, text=True, timeout=600, env=env)
     assert r.returncode == 0, r.stderr[-2000:]
     assert r.stdout.count("raised") == 6, r.stdout
+
+
+def test_without_the_native_module_the_python_forms_take_every_call(monkeypatch, tmp_path):
+    import pytest
+    import paper_2408_01803_b200 as stb
+    broken = tmp_path / "broken.so"
+    broken.write_bytes(b"not a shared object")
+    for path in (tmp_path / "missing.so", broken):
+        monkeypatch.setattr(stb, "BIND_PATH", str(path))
+        monkeypatch.setattr(stb, "_bind", None)
+        with pytest.warns(UserWarning, match="native host path"):
+            forms = stb._fast()
+        for name in ("gemv", "gemm", "gemm_f16", "layer_stack", "layer_stack_resident"):
+            assert getattr(forms, name) is getattr(stb, "_%s_py" % name)
+        assert stb._fast() is forms

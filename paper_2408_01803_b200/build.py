@@ -3,8 +3,10 @@ with g++ against the installed torch, in-tree."""
 from __future__ import annotations
 
 import os
+import re
 import shutil
 import subprocess
+import sys
 import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
@@ -13,6 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstb.so")
 BIND = os.path.join(HERE, "_stb_bind.so")
+BIND_FOR = os.path.join(OBJ, "stb_bind.for")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
          "-Xcompiler", "-fPIC"]
 
@@ -40,23 +43,39 @@ def _torch_dir() -> str:
     return os.path.dirname(find_spec("torch").origin)
 
 
+def _bind_target(torch_dir: str) -> str:
+    """What _stb_bind.so is built for: the installed torch and this interpreter's extension ABI."""
+    with open(os.path.join(torch_dir, "version.py")) as f:
+        version = re.search(r"__version__\s*=\s*['\"]([^'\"]+)", f.read()).group(1)
+    return "torch %s %s" % (version, sysconfig.get_config_var("EXT_SUFFIX"))
+
+
 def build_bind(force: bool = False) -> str:
-    """Compile csrc/stb_bind.cpp into _stb_bind.so."""
+    """Compile csrc/stb_bind.cpp into _stb_bind.so, unless the one there is newer than its sources and for the same torch."""
     src = os.path.join(CSRC, "stb_bind.cpp")
     newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(HERE, "..", "include", "stb.h")))
-    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= newest:
-        return BIND
     torch_dir = _torch_dir()
+    target = _bind_target(torch_dir)
+    built_for = ""
+    if os.path.exists(BIND_FOR):
+        with open(BIND_FOR) as f:
+            built_for = f.read()
+    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= newest and built_for == target:
+        return BIND
+    abi = subprocess.run([sys.executable, "-c", "import torch; print(int(torch._C._GLIBCXX_USE_CXX11_ABI))"], capture_output=True, text=True, check=True)
     inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
     tmp = BIND + ".tmp%d" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", tmp, src, "-I" + sysconfig.get_paths()["include"], "-I" + inc,
-           "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), "-I" + cuda, "-D_GLIBCXX_USE_CXX11_ABI=1",
+           "-I" + os.path.join(inc, "torch", "csrc", "api", "include"), "-I" + cuda, "-D_GLIBCXX_USE_CXX11_ABI=" + abi.stdout.split()[-1],
            "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("g++ failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
     os.replace(tmp, BIND)
+    os.makedirs(OBJ, exist_ok=True)
+    with open(BIND_FOR, "w") as f:
+        f.write(target)
     return BIND
 
 
@@ -96,5 +115,4 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 if __name__ == "__main__":
-    import sys
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))

@@ -46,3 +46,29 @@ def test_without_the_native_module_the_python_forms_take_every_call(monkeypatch,
         for name in ("gemv", "gemm", "gemm_f16", "layer_stack", "layer_stack_resident"):
             assert getattr(forms, name) is getattr(stb, "_%s_py" % name)
         assert stb._fast() is forms
+
+
+def test_the_native_module_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
+    from paper_2408_01803_b200 import build
+    import pytest
+    if not os.path.exists(build.BIND):
+        pytest.skip("not built")
+    ran = []
+
+    def run(cmd, **kw):
+        ran.append(cmd)
+        if cmd[0] == "g++":
+            open(cmd[cmd.index("-o") + 1], "w").close()
+        return subprocess.CompletedProcess(cmd, 0, "1\n", "")
+
+    monkeypatch.setattr(build.subprocess, "run", run)
+    monkeypatch.setattr(build, "BIND", str(tmp_path / "b.so"))
+    monkeypatch.setattr(build, "BIND_FOR", str(tmp_path / "b.for"))
+    monkeypatch.setattr(build, "OBJ", str(tmp_path))
+    build.build_bind()
+    compiled = sum(c[0] == "g++" for c in ran)
+    build.build_bind()                                      # nothing changed
+    assert compiled == 1 and sum(c[0] == "g++" for c in ran) == 1
+    monkeypatch.setattr(build, "_bind_target", lambda d: "another torch")
+    build.build_bind()
+    assert sum(c[0] == "g++" for c in ran) == 2

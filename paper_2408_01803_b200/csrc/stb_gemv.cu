@@ -70,8 +70,6 @@ __host__ __device__ inline GemvSmem gemv_smem(int N, int warps, int ksplit, int 
   return s;
 }
 
-__device__ __forceinline__ int ilog2(int v) { return 31 - __clz(v); }
-
 // Up to kMaxFused layers that read the same activations (q / k / v, gate / up) run as one grid:
 // row tiles [tile_start[i], tile_start[i + 1]) of the grid belong to layer i.
 constexpr int kMaxFused = 4;
@@ -1108,7 +1106,7 @@ static cudaError_t launch_mma_b(int batch, int N, const GemvLayers& layers, int 
 }
 
 // ------------------------------------------------------------------------------------------
-// General kernel: any N in 1..8, batch <= BT.  One CTA per row tile (32 rows), 8 warps split
+// General kernel: N = 1, 2, 3, 7, 8, batch <= BT.  One CTA per row tile (32 rows), 8 warps split
 // the blocks, lane = (g, t); plain position-order decode and fp32 multiply-adds, x read
 // through L1.  The four lanes that share a row combine with shuffles, the 8 warps through
 // shared memory in a fixed order, so the result is deterministic.
@@ -1265,9 +1263,6 @@ static int gemv_impl(const void* packed, int n, int m, int N, const void* x, int
       case 1: e = stb::launch_general<1>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
       case 2: e = stb::launch_general<2>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
       case 3: e = stb::launch_general<3>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
-      case 4: e = stb::launch_general<4>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
-      case 5: e = stb::launch_general<5>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
-      case 6: e = stb::launch_general<6>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
       case 7: e = stb::launch_general<7>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
       case 8: e = stb::launch_general<8>(p, n, m, xc, bt, ldx, yc, y_f16, ldy, dev_status, s); break;
     }

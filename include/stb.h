@@ -214,8 +214,8 @@ int stb_layer_stack(const stb_step *steps, int count, int *dev_status, void *str
  * run as several launches.
  * ws: caller-owned DEVICE workspace of stb_layer_stack_resident_workspace bytes, 256-byte
  * aligned, ZEROED by the caller before its first use; every call leaves its counters zero
- * again (also after a wait that ran out), and the rest of it as well, so the same workspace serves call after call without
- * being cleared.  It belongs to the kernel between calls too: do not write anything but zeros to it.
+ * again (also after a wait that ran out) and no partial sum in the rest of it, so the same workspace serves call after call
+ * without being cleared.  It belongs to the kernel between calls too (a count of the calls stays in it): do not write to it.
  * Calls that share a workspace must not overlap on the GPU.
  * The launch is cooperative: it fails with STB_ERR_CUDA when the GPU cannot hold one 512-thread
  * CTA per SM at once. */

@@ -16,27 +16,29 @@
 //   * Decode and multiply per tile: 6:8 keeps the weights in rank order and lets mma.sp.m16n8k32 place them
 //     (activations from an image of x in operand order in shared memory, built once per phase and CTA); 4:8 and 5:8
 //     (and 6:8 when the image does not fit) decode to position order for mma.m16n8k16 with the activations from a
-//     plain copy in shared memory, or through L1 when that does not fit either.
+//     plain copy in shared memory, or through L1 where that does not fit or is not read often enough to pay.
 //   * A step may take x = silu(in) * in2 (the gated activation between gate / up and down of an MLP): the CTA forms
 //     it while it stages the activations.
 //   * The residual term of the salient columns (Eq. 4): a block's record of the residual stream comes with its tile,
 //     four residual words (16 salient slots) of a chunk per tensor-core step; the activations behind every residual
-//     word of the phase are gathered into shared memory while x is staged.
+//     word of the phase are gathered into shared memory once x is staged, or, where they are too many, read by their places.
 //   * Partial sums: a warp that covers a whole row tile writes y itself; the others leave their head / tail
 //     pieces in shared memory and the CTA adds them in tile order at the end of the phase; of a row tile that
-//     straddles CTAs the later ones hand their sums to the first through the caller's workspace, every value beside the
-//     number of its phase (one 8-byte store, no fence, no counter), and the first adds them in CTA order and empties their
-//     places, so that no value outlives its phase.  Every sum has a fixed order: results are reproducible.
+//     straddles CTAs the later ones hand their sums to the first through the caller's workspace, every value beside a tag
+//     of the launch and phase (one 8-byte store, no fence, no counter), and the first adds them in CTA order and empties
+//     their places, so that no value outlives its phase.  Every sum has a fixed order: results are reproducible.
 //   * A phase may read what an earlier phase wrote: a CTA starts a phase's arithmetic only when the count of
 //     finished row tiles (one counter in the workspace, bumped once per CTA and phase) has reached the total
 //     of all earlier phases.  The poll is bounded; when it or an mbarrier wait runs out, an abort flag makes
 //     every CTA leave, STB_ERR_TIMEOUT is reported and the last CTA out restores the workspace to zero.
 //
-// What bounds it: in the tile loop instruction issue, the integer ALU first (2 warp-instructions per clock and SM; the decode
+// What bounds it.  In the tile loop instruction issue, the integer ALU first (2 warp-instructions per clock and SM; the decode
 // alone takes 126 / 145 / 118 clocks per tile and SM at N = 6 / 5 / 4, with the waits, residual words and copies 180 / 193 /
-// 170); between phases, latencies: the spread of the warps' ends, the sums, one trip through L2 for the count of finished row
-// tiles and one for the activations.  13B block at 5:8, batch 1: 106.4 -> 92.5 us, 7B MLP at 6:8: 44.5 -> 42.3 us, 32 7B
-// layers: 2040 -> 1905 us against one copy per five-block span issued by the decoding warps themselves.
+// 170).  Between phases, latencies, about 7 us each: the spread of the warps' ends, the sums, one trip through L2 for the count of
+// finished row tiles and one for the activations.  And about 9 us per call (launch, set-up, leaving).  Of a 7B MLP at 6:8 and
+// one row (44.6 us) these are 20, 14 and 9 us, of 32 7B layers (1900 us) 980 and 900 and little.
+// Against one copy per five-block span issued by the decoding warps themselves: 7B MLP 45.6 -> 44.6 us, 13B block at 5:8
+// 108.4 -> 95.3, 32 7B layers 2046 -> 1900, at 2 / 4 / 8 rows 2206 / 2477 / 2908 -> 2105 / 2280 / 2775.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -57,9 +59,13 @@ static_assert(kSThreads * kDecodeRegs + 128 * kFeedRegs <= kSAllThreads * 96, "r
 constexpr int kMaxPhases = 64;                // per launch; longer lists run as several launches
 constexpr int kMaxFusedSteps = 4;
 constexpr int kSDepth = 2, kSChunk = 2;       // ring: slots per warp, tiles per slot
-constexpr uint32_t kSlotTiles = kSChunk * 1920;                    // tiles (at most 1920 bytes each) ...
-constexpr uint32_t kSlotBytes = kSlotTiles + kSChunk * (kResidA2Bytes + kMaxResidWords * kResidWordBytes);   // ... and records
-static_assert(kSlotBytes % 128 == 0, "slots stay 128-byte aligned");
+// A slot holds the tiles of a chunk (of the launch's largest N) and their records: of any two blocks, or, where shared memory is
+// short, of two blocks with at most kFewWords residual words together (blocks with more then come one by one).
+constexpr uint32_t kFewWords = 8;
+constexpr uint32_t slot_tiles(int N) { return kSChunk * tile_bytes(N); }
+constexpr uint32_t slot_records(bool few) { return kSChunk * kResidA2Bytes + (few ? kFewWords : kSChunk * kMaxResidWords) * kResidWordBytes; }
+static_assert(kFewWords >= kMaxResidWords && slot_tiles(4) % 128 == 0 && slot_tiles(5) % 128 == 0 && slot_tiles(6) % 128 == 0 &&
+              slot_records(true) % 128 == 0 && slot_records(false) % 128 == 0, "a block's records fit; slots stay 128-byte aligned");
 constexpr long long kSWaitLimit = 2000000000ll;        // about a second of SM clocks
 constexpr long long kSSelftestLimit = 100000ll;
 
@@ -76,7 +82,8 @@ struct StackPhase {
   uint8_t N, batch, count, f16_mask;          // f16_mask bit i: step i writes fp16
   uint8_t use_image, aligned, gather, pad;    // use_image: 0 activations from global memory, 1 operand-order image (6:8),
                                               // 2 plain fp16 copy in shared memory; aligned: CTA ranges are whole row tiles;
-                                              // gather: the residual words' activations fit shared memory
+                                              // gather: 2 the residual words' activations are gathered in shared memory, 1 their
+                                              // places are there, 0 neither
   uint32_t done_before;                       // row tiles finished by all earlier phases of this launch
 };
 
@@ -87,15 +94,17 @@ struct StackParams {
   uint32_t pos_off[3];                        // position tables of N = 4, 5, 6, 0 where no phase needs one
   uint32_t use_meta6;
   uint32_t ring_off, pdata_off, xs_off, cols_off, x_off, x_bytes;
+  uint32_t slot_tiles, slot_bytes, slot_words;     // a ring slot: where its records begin, its size, the residual words it takes
   uint32_t pos_row;                           // bytes from one entry of a position table to the next
   uint32_t part_floats;                       // floats per partial slot: 32 rows x largest batch
   uint32_t max_share;                         // most CTAs that share one row tile
-  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left
+  uint32_t* sync;                             // [0] finished row tiles, [1] abort flag, [2] CTAs that left, [4] launches so far
   uint2* gpart;                               // sums handed on for row tiles that straddle CTAs: { value, tag }, empty ({ 0, 0 }) between launches
   uint32_t gpart_slots;
   int* dev_status;
   long long wait_limit;
   int32_t copies_off;
+  int32_t places;                             // phases that do not gather go by places
 };
 
 // shared memory: joint 6:8 metadata table first (784 x 16 B, at offset 0: a pair field of a tile is the shared-memory
@@ -277,7 +286,7 @@ __device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, 
   TileWalk t;
   t.enter(P, range, nrw, 0, w);
   const uint32_t full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)w, empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)w;
-  const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)w * kSDepth * kSlotBytes;
+  const uint32_t ring = smem_u32(smem + P.ring_off) + (uint32_t)w * kSDepth * P.slot_bytes;
   uint4* chunk = reinterpret_cast<uint4*>(base + SSmem::chunks) + kSDepth * w;
   uint32_t k = 0;                                     // chunks issued
   while (t.phase < P.nphase) {
@@ -288,8 +297,11 @@ __device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, 
       continue;
     }
     const StackPhase& q = P.ph[t.phase];
-    const int nb = q.m / kBlock, cnt = t.count(nb);
-    const uint32_t na = t.ba.z, nw = na + t.bb.z;
+    const int nb = q.m / kBlock;
+    const uint32_t na = t.ba.z;
+    uint32_t nw = na + t.bb.z;
+    int cnt = t.count(nb);
+    if (nw > P.slot_words) { cnt = 1; nw = na; }
     const bool seg_end = t.blk + cnt == nb || t.left == cnt;
     uint4 c;
     c.x = (uint32_t)cnt | (na << 8) | (nw << 16);
@@ -298,12 +310,12 @@ __device__ __forceinline__ void feed_rings(const StackParams& P, uint8_t* smem, 
     c.y = (uint32_t)t.blk; c.z = t.words + t.ba.y; c.w = (uint32_t)t.R;
     chunk[slot] = c;                                  // (seen by the reader through the full barrier)
     const uint32_t tile_b = (uint32_t)cnt * t.tb, rec_b = (uint32_t)cnt * kResidA2Bytes + nw * kResidWordBytes;
-    const uint32_t bar = full + 8u * slot, dst = ring + slot * kSlotBytes;
+    const uint32_t bar = full + 8u * slot, dst = ring + slot * P.slot_bytes;
     mbar_expect_tx(bar, tile_b + rec_b);
     // copies off (the wait self-test): the barrier is armed but nothing will ever complete it
     if (!P.copies_off) {
       bulk_g2s(dst, t.src, tile_b, bar);
-      bulk_g2s(dst + kSlotTiles, t.rec, rec_b, bar);
+      bulk_g2s(dst + P.slot_tiles, t.rec, rec_b, bar);
     }
     ++k;
     t.left -= cnt; t.blk += cnt;
@@ -336,12 +348,23 @@ struct WarpEnv {
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSThreads) : "memory"); }
 
 // ------------------------------------------------------------------------------------------
+// Where the residual term finds the activations of a chunk's words:
+//   kGathered  gathered for the whole phase in shared memory ([word][batch row], four fp16 each)
+//   kPlaced    in the lane's row of activations, staged or in global memory, at places kept in shared memory (four per word)
+//   kListed    in global memory, in the columns that the layer's word table names: two trips, for words too many for the others
+enum class ResidForm { kGathered, kPlaced, kListed };
+struct ResidX {
+  const uint8_t* xw;            // kGathered: of the lane's batch row, at the chunk's first word ...
+  uint32_t xw_step;             // ... and bytes per word
+  const uint2* places;          // kPlaced: of the chunk's first word
+  const uint8_t* row;           // kPlaced: the lane's row of activations, null beyond the batch
+  const ResidWord* words;       // kListed: the chunk's first word
+  const __half *xg, *xg2;       // kListed: the lane's row of the input (null beyond the batch), and of the second one
+};
 // Residual term of a chunk: its residual words, four (16 salient slots) per tensor-core step, lane t the t-th.  rec: the
-// chunk's records; na / nw: words of its first block / of all; xw: activations of the chunk's first word for the lane's
-// batch row, xw_step bytes per word.  kGather false: they are fetched one by one (word table entry, then x).
-template <bool kGather>
-__device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint32_t nw, int g, int t, const uint8_t* xw, uint32_t xw_step,
-                                          const ResidWord* rwt, const __half* xg, const __half* xg2, float (&acc)[2][1][4]) {
+// chunk's records; na / nw: words of its first block / of all.  kShared: kPlaced from staged activations.
+template <ResidForm kForm, bool kShared>
+__device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint32_t nw, int g, int t, const ResidX& X, float (&acc)[2][1][4]) {
 #pragma unroll 1
   for (uint32_t k0 = 0; k0 < nw; k0 += 4u) {
     const uint32_t kk = k0 + (uint32_t)t, k = min(kk, nw - 1u);
@@ -353,11 +376,23 @@ __device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint3
     if (kk >= nw) rw = kNoTerms;
     resid_operands(rw, a2, fa);
     uint2 xr = make_uint2(0, 0);
-    if (kGather) xr = *reinterpret_cast<const uint2*>(xw + k * xw_step);
-    else if (xg) {
-      const uint2 e = __ldg(reinterpret_cast<const uint2*>(rwt + k));
+    if constexpr (kForm == ResidForm::kGathered) xr = *reinterpret_cast<const uint2*>(X.xw + k * X.xw_step);
+    else if constexpr (kForm == ResidForm::kPlaced) {
+      if (X.row) {
+        const uint2 at = X.places[k];
+        const uint16_t* x = reinterpret_cast<const uint16_t*>(X.row);
+        if (kShared) {
+          xr.x = (uint32_t)x[at.x & 0xFFFFu] | ((uint32_t)x[at.x >> 16] << 16);
+          xr.y = (uint32_t)x[at.y & 0xFFFFu] | ((uint32_t)x[at.y >> 16] << 16);
+        } else {
+          xr.x = ldg_u16_coherent(x + (at.x & 0xFFFFu)) | (ldg_u16_coherent(x + (at.x >> 16)) << 16);
+          xr.y = ldg_u16_coherent(x + (at.y & 0xFFFFu)) | (ldg_u16_coherent(x + (at.y >> 16)) << 16);
+        }
+      }
+    } else if (X.xg) {
+      const uint2 e = __ldg(reinterpret_cast<const uint2*>(X.words + k));
       const size_t o = (size_t)(e.x >> 3) * kBlock;
-      xr = word_x(xg + o, xg2 ? xg2 + o : nullptr, e.y);
+      xr = word_x(X.xg + o, X.xg2 ? X.xg2 + o : nullptr, e.y);
     }
     mma16816(acc[0][0], fa[0][0], fa[1][0], fa[0][1], fa[1][1], xr.x, xr.y);
     mma16816(acc[1][0], fa[2][0], fa[3][0], fa[2][1], fa[3][1], xr.x, xr.y);
@@ -366,7 +401,8 @@ __device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint3
 
 // The warp's run of phase q: chunks of residual words and tiles, partial sums out.
 // kImage: 6:8 from the operand-order image; kStaged: position order with the activations in a plain copy in shared memory
-template <int N, bool kImage, bool kStaged>
+// kPlaces: residual activations that are not gathered are found by their places (otherwise by the layer's word table)
+template <int N, bool kImage, bool kStaged, bool kPlaces>
 __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const StackPhase& q, int* pslot, float* pdata) {
   const StackParams& P = *E.P;
   const int lane = E.lane, g = E.g, t = E.t, warp = E.warp, batch = q.batch;
@@ -401,16 +437,30 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
     // all lanes poll; the verdict is made warp-uniform
     if (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, W.parity)) && !__all_sync(0xFFFFFFFFu, mbar_wait(bar, W.parity, P.wait_limit))) { W.failed = true; return; }
     c = E.chunk[slot];
-    const uint8_t* tile = E.ring + slot * kSlotBytes;
+    const uint8_t* tile = E.ring + slot * P.slot_bytes;
     const uint32_t na = (c.x >> 8) & 0xFFu, nw = (c.x >> 16) & 0xFFu;
-    if (nw) {
-      if (q.gather) resid_mul<true>(tile + kSlotTiles, na, nw, g, t, xs + c.z * xw_step, xw_step, nullptr, nullptr, nullptr, acc);
-      else {
-        const ResidWord* rwt = reinterpret_cast<const ResidWord*>(q.packed[step_of(q, (int)c.w)] + rwtab_offset(q.m / kBlock));
-        resid_mul<false>(tile + kSlotTiles, na, nw, g, t, nullptr, 0, rwt + c.z, xlive ? q.x + (size_t)g * q.ldx : nullptr,
-                         q.x2 ? q.x2 + (size_t)g * q.ldx : nullptr, acc);
+    const uint8_t* records = tile + P.slot_tiles;
+    auto residual = [&] {
+      if (nw == 0u) return;
+      ResidX X;
+      if (q.gather == 2) {
+        X.xw = xs + c.z * xw_step; X.xw_step = xw_step;
+        resid_mul<ResidForm::kGathered, true>(records, na, nw, g, t, X, acc);
+      } else if constexpr (kPlaces) {
+        X.places = reinterpret_cast<const uint2*>(E.smem + P.cols_off) + c.z;
+        X.row = xlive ? xbase - (uint32_t)t * (kImage ? 96u : 16u) : nullptr;
+        resid_mul<ResidForm::kPlaced, kImage || kStaged>(records, na, nw, g, t, X, acc);
+      } else {
+        X.words = reinterpret_cast<const ResidWord*>(q.packed[step_of(q, (int)c.w)] + rwtab_offset(q.m / kBlock)) + c.z;
+        X.xg = xlive ? q.x + (size_t)g * q.ldx : nullptr;
+        X.xg2 = q.x2 ? q.x2 + (size_t)g * q.ldx : nullptr;
+        resid_mul<ResidForm::kListed, false>(records, na, nw, g, t, X, acc);
       }
-    }
+    };
+    // In global memory the words' activations lie in the lines that the chunk's tiles read as well: after the tiles the loads of two
+    // bytes find them in L1 (before them, 2 % slower at two rows, 4 to 8 % at eight).  The slot is kept until then.
+    constexpr bool kLate = kPlaces && !kImage && !kStaged;
+    if (!kLate) residual();
     const uint8_t* xb = xbase + (size_t)c.y * xstep;
     const int cnt = (int)(c.x & 3u);
 #pragma unroll 1
@@ -420,17 +470,18 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
       if constexpr (kImage) {
         Tile6 d;
         load_tile(tile, lane, d);
-        if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        if (!kLate && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
         tile_mul<1>(d, E.smem, xp, acc);
       } else {
         TileD<N> d;
         load_tile<N>(tile, lane, ptab, prow, d);
-        if (k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        if (!kLate && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
         tile_mul<N, kStaged, 1>(d, xp, acc);
       }
       tile += tb;
       xb += xstep;
     }
+    if (kLate) { residual(); __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
     W.slot ^= 1u;
     W.parity ^= slot;
     if (c.x & kSegEnd) {
@@ -518,17 +569,19 @@ __device__ __forceinline__ bool stack_setup(const StackParams& P, uint8_t* base,
 }
 
 // The decoding warps: all phases in order.
+template <bool kPlaces>
 __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* smem, uint8_t* base, volatile int* ctl, int* pslot, float* pdata, int cta) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* ximg = reinterpret_cast<uint32_t*>(smem + P.x_off);
   WarpEnv E;
   E.P = &P; E.smem = smem; E.base = base; E.warp = warp; E.lane = lane; E.g = lane >> 2; E.t = lane & 3;
-  E.ring = smem + P.ring_off + (size_t)warp * kSDepth * kSlotBytes;
+  E.ring = smem + P.ring_off + warp * kSDepth * P.slot_bytes;
   E.chunk = reinterpret_cast<const uint4*>(base + SSmem::chunks) + kSDepth * warp;
   E.full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)warp;
   E.empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)warp;
   WarpState W;
   W.slot = 0; W.parity = 0; W.failed = false;
+  const uint32_t epoch = __ldcg(P.sync + 4);          // changed only by the last CTA out
   // tables, while the first copies are under way
   if (P.use_meta6)
     for (int i = threadIdx.x; i < (int)(kMasks6 * kMasks6); i += kSThreads)
@@ -622,7 +675,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
       }
     }
     consumers_sync();
-    if (q.gather && !stop) {
+    if (q.gather == 2 && !stop) {
       // activations of the residual slots: [word of all steps][batch row], four fp16 each
       uint16_t* xs = reinterpret_cast<uint16_t*>(smem + P.xs_off);
       const uint32_t pitch = q.use_image == 1 ? (uint32_t)nb * kImgWordsPerBlock * 2u : (uint32_t)q.m + kXPad / 2u;
@@ -638,14 +691,14 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
 
     // ---- this warp's tiles ----
     if (!W.failed && wl < wh) {
-      if (q.use_image == 1) run_tiles<6, true, false>(E, W, q, pslot, pdata);
+      if (q.use_image == 1) run_tiles<6, true, false, kPlaces>(E, W, q, pslot, pdata);
       else if (q.use_image == 2) {
-        if (q.N == 6) run_tiles<6, false, true>(E, W, q, pslot, pdata);
-        else if (q.N == 5) run_tiles<5, false, true>(E, W, q, pslot, pdata);
-        else run_tiles<4, false, true>(E, W, q, pslot, pdata);
-      } else if (q.N == 6) run_tiles<6, false, false>(E, W, q, pslot, pdata);
-      else if (q.N == 5) run_tiles<5, false, false>(E, W, q, pslot, pdata);
-      else run_tiles<4, false, false>(E, W, q, pslot, pdata);
+        if (q.N == 6) run_tiles<6, false, true, kPlaces>(E, W, q, pslot, pdata);
+        else if (q.N == 5) run_tiles<5, false, true, kPlaces>(E, W, q, pslot, pdata);
+        else run_tiles<4, false, true, kPlaces>(E, W, q, pslot, pdata);
+      } else if (q.N == 6) run_tiles<6, false, false, kPlaces>(E, W, q, pslot, pdata);
+      else if (q.N == 5) run_tiles<5, false, false, kPlaces>(E, W, q, pslot, pdata);
+      else run_tiles<4, false, false, kPlaces>(E, W, q, pslot, pdata);
     }
     if (W.failed && lane == 0 && !ctl[0]) {
       // this warp's own wait ran out: tell the CTA and the grid
@@ -673,7 +726,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
         // a straddling row tile: the CTA where it begins gathers the others' sums, in CTA order
         const int c_first = R == range.first ? range.head_cta : range.tail_cta, share = R == range.first ? range.head_share : range.tail_share;
         uint2* gp = P.gpart + (size_t)R * P.max_share * P.part_floats;
-        const uint32_t tag = (uint32_t)ph + 1u;
+        const uint32_t tag = ((epoch + 1u) << 6) | (uint32_t)ph;
         bool lost = false;
         for (int v = lane; v < nval; v += 32) {
           const float* pv = pdata + v;
@@ -730,6 +783,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
   }
 }
 
+template <bool kPlaces>
 __global__ void __launch_bounds__(kSAllThreads, 1)
 stack_kernel(const __grid_constant__ StackParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -752,7 +806,7 @@ stack_kernel(const __grid_constant__ StackParams P) {
     feed_rings(P, smem, base, ctl);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDecodeRegs));
-    decode_phases(P, smem, base, ctl, pslot, pdata, cta);
+    decode_phases<kPlaces>(P, smem, base, ctl, pslot, pdata, cta);
   }
 
   // ---- leaving: let copies in flight land, then the last CTA out restores the workspace ----
@@ -774,7 +828,7 @@ stack_kernel(const __grid_constant__ StackParams P) {
     if (*reinterpret_cast<volatile uint32_t*>(P.sync + 1) != 0u)
       for (uint32_t i = threadIdx.x; i < P.gpart_slots; i += kSAllThreads) P.gpart[i] = make_uint2(0u, 0u);
     __syncthreads();
-    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; __threadfence(); }
+    if (threadIdx.x == 0) { P.sync[0] = 0u; P.sync[1] = 0u; P.sync[2] = 0u; P.sync[4] += 1u; __threadfence(); }
   }
 }
 
@@ -799,7 +853,7 @@ checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __res
   bool failed = false;
   if (warp >= kSWarps) feed_rings(P, smem, base, ctl);
   else {
-    const uint8_t* ring = smem + P.ring_off + (size_t)warp * kSDepth * kSlotBytes;
+    const uint8_t* ring = smem + P.ring_off + warp * kSDepth * P.slot_bytes;
     const uint4* chunk = reinterpret_cast<const uint4*>(base + SSmem::chunks) + kSDepth * warp;
     const uint32_t full = smem_u32(base + SSmem::full) + 8u * kSDepth * (uint32_t)warp, empty = smem_u32(base + SSmem::empty) + 8u * kSDepth * (uint32_t)warp;
     uint32_t slot = 0, parity = 0;
@@ -813,10 +867,10 @@ checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __res
       for (bool more = lo < hi; more;) {
         if (!__all_sync(0xFFFFFFFFu, mbar_wait(full + 8u * slot, parity, P.wait_limit))) { failed = true; break; }
         const uint4 c = chunk[slot];
-        const uint8_t* tile = ring + (size_t)slot * kSlotBytes;
+        const uint8_t* tile = ring + slot * P.slot_bytes;
         const uint32_t cnt = c.x & 3u, rec_b = cnt * kResidA2Bytes + ((c.x >> 16) & 0xFFu) * kResidWordBytes;
         for (uint32_t o = (uint32_t)lane * 4u; o < cnt * tb; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + o);
-        for (uint32_t o = (uint32_t)lane * 4u; o < rec_b; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + kSlotTiles + o);
+        for (uint32_t o = (uint32_t)lane * 4u; o < rec_b; o += 128u) fold ^= *reinterpret_cast<const uint32_t*>(tile + P.slot_tiles + o);
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + 8u * slot);
         parity ^= slot;
@@ -843,10 +897,6 @@ checksum_kernel(const __grid_constant__ StackParams P, unsigned long long* __res
 
 // ------------------------------------------------------------------------------------------
 // Host side: steps -> phases -> launches.
-struct StackPlan {
-  size_t sync_bytes, gpart_bytes;
-};
-
 static bool same_input(const stb_step& a, const stb_step& b) {
   return a.in == b.in && a.in2 == b.in2 && a.input == b.input && a.ldin == b.ldin && a.batch == b.batch && a.m == b.m &&
          a.N == b.N && b.out != a.in && b.out != a.in2;
@@ -896,18 +946,26 @@ static int stack_sm_count(int* out) {
 }
 
 constexpr uint32_t kSmemLimit = 227 * 1024;
-constexpr unsigned long long kGatherMax = 16 * 1024;     // shared memory for the residual words' activations
+constexpr unsigned long long kGatherMax = 16 * 1024;     // shared memory for the residual words' activations, and for their places
 
-// Lays out the shared memory of a launch and chooses each phase's staging; returns the number of phases left without.
-// `gather` false: no room is kept for the residual words' activations.
+// Lays out the shared memory of a launch and chooses each phase's staging; false where not even the rest fits.  image: 6:8 phases may
+// take the operand-order image.  gather: the residual words' activations are gathered where they fit (2), or read by their places
+// (1), or found by the layer's word table (0).  few: ring slots for few residual words.
 static uint32_t up128(uint32_t v) { return (v + 127u) & ~127u; }
-static int plan_smem(StackParams& sp, bool image, bool gather) {
-  bool any6 = false, dense[3] = {false, false, false};
+struct SmemForm { bool image; int gather; bool few; };
+static bool plan_smem(StackParams& sp, const SmemForm& form, int ctas) {
+  bool any6 = false, dense[3] = {false, false, false}, bare_phase[kMaxPhases] = {};
+  int most_N = 4;
   for (int p = 0; p < sp.nphase; ++p) {
-    if (sp.ph[p].N == 6 && image) any6 = true;
+    if (sp.ph[p].N > most_N) most_N = sp.ph[p].N;
+    if (sp.ph[p].N == 6 && form.image) any6 = true;
     else dense[sp.ph[p].N - 4] = true;
   }
-  // 6:8 phases may fall back to position order; their table is then needed as well
+  sp.slot_tiles = slot_tiles(most_N);
+  sp.slot_bytes = sp.slot_tiles + slot_records(form.few);
+  sp.slot_words = form.few ? kFewWords : kSChunk * kMaxResidWords;
+  // 6:8 phases may fall back to position order; their table is then needed as well.  A phase that stays without staged
+  // activations has none to gather either.
   for (int round = 0;; ++round) {
     uint32_t o = 0;
     sp.use_meta6 = any6 ? 1 : 0;
@@ -919,27 +977,27 @@ static int plan_smem(StackParams& sp, bool image, bool gather) {
     }
     sp.pos_row = kPosCopies * 8;
     sp.ring_off = up128(o);
-    o = sp.ring_off + kSWarps * kSDepth * kSlotBytes;
+    o = sp.ring_off + kSWarps * kSDepth * sp.slot_bytes;
     sp.pdata_off = o;
     o += 32u * sp.part_floats * 4u;
-    // the residual words' activations: sized for the most words the phase's layers can have
+    // the residual words' places and activations: sized for the most words the phase's layers can have
     sp.xs_off = o;
     uint32_t xs_max = 0, cols_max = 0;
     for (int p = 0; p < sp.nphase; ++p) {
       StackPhase& q = sp.ph[p];
-      const unsigned long long need = 8ull * q.batch * (unsigned long long)kMaxResidWords * (unsigned long long)(q.m / kBlock) * q.count;
-      q.gather = gather && need <= kGatherMax && q.m <= 32768 ? 1 : 0;
-      if (q.gather && need > xs_max) xs_max = (uint32_t)need;
-      if (q.gather && need / q.batch > cols_max) cols_max = (uint32_t)(need / q.batch);
+      const unsigned long long need = 8ull * (unsigned long long)kMaxResidWords * (unsigned long long)(q.m / kBlock) * q.count;
+      q.gather = form.gather > 0 && need <= kGatherMax && q.m <= 32768 ? 1 : 0;
+      if (form.gather == 2 && q.gather && !bare_phase[p] && need * q.batch <= kGatherMax) q.gather = 2;
+      if (q.gather == 2 && need * q.batch > xs_max) xs_max = (uint32_t)(need * q.batch);
+      if (q.gather && need > cols_max) cols_max = (uint32_t)need;
     }
     sp.cols_off = up128(o + xs_max);
     o = up128(sp.cols_off + cols_max);
     sp.x_off = o;
-    const long long room = (long long)kSmemLimit - (long long)o;
-    if (room < 0) return sp.nphase + 1;
-    int bare = 0;
-    bool again = false;
     sp.x_bytes = 0;
+    const long long room = (long long)kSmemLimit - (long long)o;
+    if (room < 0) return false;
+    bool again = false;
     for (int p = 0; p < sp.nphase; ++p) {
       StackPhase& q = sp.ph[p];
       const unsigned long long img = 4ull * q.batch * (unsigned long long)(q.m / kBlock) * kImgWordsPerBlock;
@@ -949,12 +1007,16 @@ static int plan_smem(StackParams& sp, bool image, bool gather) {
       if (q.N == 6 && any6 && (long long)img <= room) { q.use_image = 1; need = img; }
       else {
         if (!dense[q.N - 4]) { dense[q.N - 4] = true; again = true; }
-        if ((long long)plain <= room) { q.use_image = 2; need = plain; }
-        else { ++bare; q.gather = 0; }
+        // Staging costs a trip to L2 for all of x before the first tile, and pays where the CTA's row tiles read it again: with
+        // several rows from 1.5 row tiles per CTA and row on (three 4:8 layers of 4096, 4 rows: 213 us against 226 with every
+        // phase staged that fits; 7B gate and up, 4.6 row tiles per CTA, 2 rows: MLP 47.4 against 49.4 without).
+        const bool stage = q.x2 || q.batch == 1 || 2 * q.tile_start[q.count] >= 3 * q.batch * ctas;
+        if (stage && (long long)plain <= room) { q.use_image = 2; need = plain; }
+        else if (q.gather == 2) { bare_phase[p] = true; again = true; }
       }
       if (need > sp.x_bytes) sp.x_bytes = (uint32_t)need;
     }
-    if (!again || round > 2) return bare;
+    if (!again || round > kMaxPhases) return true;
   }
 }
 
@@ -999,22 +1061,31 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
     i = j;
   }
   // second pass: where each phase takes its activations from.  6:8: the operand-order image if it fits, else, as for the
-  // others, a plain copy if that fits, else global memory; a formed input (silu(in) * in2) must be staged.  The image
-  // costs the 12 KB of the metadata table for the whole launch: without it if that lets more phases stage.
-  // Where a formed input does not fit beside the residual words' activations, those are left out.
-  bool staged = false;
-  for (int gather = 1; gather >= 0 && !staged; --gather) {
-    int best = -1, best_bare = 0;
-    for (int form = 0; form < 2; ++form) {
-      const int bare = plan_smem(sp, form == 0, gather != 0);
-      if (best < 0 || bare < best_bare) { best = form; best_bare = bare; }
-    }
-    if (best == 0) plan_smem(sp, true, gather != 0);
-    staged = true;
+  // others, a plain copy or global memory; a formed input (silu(in) * in2) must be staged.  The image costs the 12 KB of the
+  // metadata table for the whole launch, gathering and full slots their room: the first form that fits, has a use for the table and
+  // stages what must be.  (Ranked by measurement: 6:8 in position order takes 160 clocks a tile against 100, few words per
+  // slot 1 %, places instead of gathering 1 to 3 %.)
+  static const SmemForm forms[] = {{true, 2, false}, {true, 2, true}, {true, 1, true}, {false, 2, false}, {false, 2, true}, {false, 1, true}, {true, 0, true}, {false, 0, true}};
+  bool found = false;
+  for (int k = 0; k < (int)(sizeof(forms) / sizeof(forms[0])) && !found; ++k) {
+    found = plan_smem(sp, forms[k], G);
     for (int p = 0; p < sp.nphase; ++p)
-      if (sp.ph[p].x2 && sp.ph[p].use_image == 0) staged = false;
+      if (sp.ph[p].x2 && sp.ph[p].use_image == 0) found = false;
+    if (found && forms[k].image) {                                 // no phase takes the image: without its table
+      found = false;
+      for (int p = 0; p < sp.nphase; ++p) found = found || sp.ph[p].use_image == 1;
+    }
   }
-  if (!staged) return -1;                                            // the formed input does not fit shared memory
+  if (!found) return -1;                                           // a formed input does not fit shared memory
+  bool listed = false, gathered = true;
+  for (int p = 0; p < sp.nphase; ++p) {
+    listed = listed || sp.ph[p].gather == 0;
+    gathered = gathered && sp.ph[p].gather == 2;
+  }
+  sp.places = !listed && !gathered ? 1 : 0;
+  if (listed)                                                      // (one kernel for both would be slower than either)
+    for (int p = 0; p < sp.nphase; ++p)
+      if (sp.ph[p].gather == 1) sp.ph[p].gather = 0;
   const size_t s_need = 8 * sizeof(uint32_t);
   if (sp.max_share > 1) sp.gpart_slots = (uint32_t)maxR * sp.max_share * sp.part_floats;
   const size_t g_need = (size_t)sp.gpart_slots * sizeof(uint2);
@@ -1075,7 +1146,8 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return STB_ERR_CUDA;
   if (!attr_done[dev]) {
-    if (cudaFuncSetAttribute(stb::stack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stb::kSmemLimit) != cudaSuccess) return STB_ERR_CUDA;
+    for (auto* kernel : {stb::stack_kernel<false>, stb::stack_kernel<true>})
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stb::kSmemLimit) != cudaSuccess) return STB_ERR_CUDA;
     attr_done[dev] = true;
   }
   int i = 0;
@@ -1103,7 +1175,7 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, stb::stack_kernel, sp) != cudaSuccess) return STB_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, sp.places ? stb::stack_kernel<true> : stb::stack_kernel<false>, sp) != cudaSuccess) return STB_ERR_CUDA;
   }
   return STB_OK;
 }

@@ -117,9 +117,36 @@ def test_more_groups_than_one_launch_holds(stb):
     _check_layers(triples, [Ls[k % 4] for k in range(70)])
 
 
+@pytest.mark.parametrize("N,batch,m,rows,steps,counts", [
+    (6, 2, 4224, 40, 4, [32, 9, 0, 20]),        # operand-order image, words by their places
+    (5, 2, 4224, 3600, 4, [5, 32, 0]),          # plain copy (row tiles read it often enough), words by their places
+    (4, 2, 512, 14300, 1, [3, 17]),             # plain copy, words gathered
+    (4, 8, 4096, 70, 3, [32, 9, 0, 20]),        # activations through L1, words by their places
+    (5, 3, 1408, 5000, 2, [7]),
+    (6, 5, 5504, 333, 1, [32]),
+    (4, 2, 33024, 64, 1, [2, 0, 32]),           # words too many for their places: by the layer's table
+    (5, 1, 12288, 96, 3, [9]),
+    (6, 8, 13824, 40, 3, [4]),
+])
+def test_activations_and_residual_words_in_every_form(stb, N, batch, m, rows, steps, counts):
+    """Several layers of one input, and a layer that reads the first one's output: where the activations stand (operand-order
+    image, plain copy, global memory) times how the residual words find theirs (gathered, by places, by the layer's table)."""
+    import torch
+    ds = [si.logical_layer(rows + k, m, N, 1100 + k, salient_counts=counts) for k in range(steps)]
+    back = 128 * (rows // 128)
+    if back:
+        ds.append(si.logical_layer(200, back, 4 + (N - 3) % 3, 1150, salient_counts=[9, 0]))
+    layers = [stb.pack_numpy(d) for d in ds]
+    x = torch.from_numpy(si.activations(batch, m, 1160)).cuda()
+    outs = [torch.zeros(batch, -(-d["n"] // 8) * 8, dtype=torch.float16, device="cuda") for d in ds]
+    triples = [(layers[k], x if k < steps else outs[0][:, :back], outs[k][:, :ds[k]["n"]]) for k in range(len(ds))]
+    _run(stb, torch, triples)
+    _check_layers(triples, [oracle.Logical(**d) for d in ds])
+
+
 def test_nothing_stays_in_the_workspace(stb):
-    """Row tiles that straddle CTAs hand sums on through the workspace: after every call it is zero as a whole, so that no sum of
-    an earlier launch can ever be taken for this one's, however many launches lie between."""
+    """Row tiles that straddle CTAs hand sums on through the workspace: after every call it holds none (nothing but the count of
+    launches at its head), so that no sum of an earlier launch can be taken for this one's, however many lie between."""
     import torch
     small, wide = si.logical_layer(320, 4096, 6, 94), si.logical_layer(1000, 2048, 5, 95)
     ls, lw = stb.pack_numpy(small), stb.pack_numpy(wide)
@@ -133,11 +160,11 @@ def test_nothing_stays_in_the_workspace(stb):
     for k in range(4):
         stb.layer_stack_resident(None, ws, dev_status=status, marshalled=steps[k % 2])
         torch.cuda.synchronize()
-        assert int(status.item()) == 0 and int(ws.max().item()) == 0
+        assert int(status.item()) == 0 and int(ws[:16].max().item()) == 0 and int(ws[256:].max().item()) == 0
         _check_layers(lists[k % 2], [oracle.Logical(**d) for d in ((small,), (wide, small))[k % 2]])
     stb.layer_stack_resident(None, ws, dev_status=status, marshalled=steps[1], selftest=True)
     torch.cuda.synchronize()
-    assert int(status.item()) == stb.STB_ERR_TIMEOUT and int(ws.max().item()) == 0
+    assert int(status.item()) == stb.STB_ERR_TIMEOUT and int(ws[:16].max().item()) == 0 and int(ws[256:].max().item()) == 0
 
 
 def test_a_wait_that_runs_out_is_reported_and_the_workspace_is_zero_again(stb):

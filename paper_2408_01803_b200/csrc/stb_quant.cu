@@ -103,7 +103,7 @@ __device__ __forceinline__ bool last_arrival(uint32_t* counter, uint32_t arrival
 // the row count's): atomics may add them in any order.  Those of w^2 are not (80 bits; an outlier column of 4096 rows
 // needs 55 of them): salient_kernel, which orders columns by them, looks again where that matters.
 constexpr int kRowsPerCta = 64, kInFlight = 4;    // (rows of a warp whose loads are in flight together: the passes are bound by latency)
-// abs_of reads the codes of infinities and NaN as numbers.  Where a lane's weights have such a code, the sums they belong to are
+// abs_of reads the codes of infinities and NaN as numbers.  Where a lane's weights may have such a code, the sums they belong to are
 // made infinite or NaN here, as the definition's are: with an infinite one mean and deviation are then NaN, so that every group is
 // selected by select_exact; and the sums of squares of their blocks are not finite, so that no candidate of a search is filtered out.
 __device__ __noinline__ void add_non_finite(const __half* W, size_t ldw, int r0, int r1, int j0, double* rowsum, double* colsum, double* colsq) {
@@ -113,10 +113,7 @@ __device__ __noinline__ void add_non_finite(const __half* W, size_t ldw, int r0,
       if (!(x < INFINITY)) { atomicAdd(rowsum + r, x); atomicAdd(colsum + j0 + c, x); atomicAdd(colsq + j0 + c, x); }
     }
 }
-__device__ __forceinline__ uint32_t largest_code(const uint4& v, uint32_t so_far) {      // of both halves of a word
-  return __vmaxu2(__vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu), __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu)), so_far);
-}
-__device__ __forceinline__ bool non_finite(uint32_t codes) { return max(codes & 0xFFFFu, codes >> 16) >= 0x7C00u; }
+constexpr double kInfiniteCode = 65536.0;         // what abs_of makes of an infinity (of NaN, more): no smaller sum holds one
 template <bool kVec>
 __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, double* __restrict__ rowsum,
                                                    double* __restrict__ colsum, double* __restrict__ colsq) {
@@ -126,7 +123,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
   const bool live = j0 < m;
   const int r1 = min(n, (int)(blockIdx.y + 1) * kRowsPerCta);
   double a[8], q[8];
-  uint32_t codes = 0;
+  bool large = false;
 #pragma unroll
   for (int c = 0; c < 8; ++c) a[c] = q[c] = 0.0;
   for (int r = blockIdx.y * kRowsPerCta + warp; r < r1; r += 8 * kInFlight) {
@@ -136,13 +133,13 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
     double s[kInFlight];
 #pragma unroll
     for (int k = 0; k < kInFlight; ++k) {
-      codes = largest_code(v[k], codes);
       s[k] = 0.0;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const double w = abs_of(half_bits(v[k], c) & 0x7FFFu);
         a[c] += w; q[c] += w * w; s[k] += w;
       }
+      large = large || s[k] >= kInfiniteCode;
     }
 #pragma unroll
     for (int k = 0; k < kInFlight; ++k) {
@@ -150,7 +147,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const __half* __restrict__ W,
       if (lane == 0 && r + 8 * k < r1) atomicAdd(rowsum + r + 8 * k, s[k]);
     }
   }
-  if (non_finite(codes)) add_non_finite(W, ldw, blockIdx.y * kRowsPerCta + warp, r1, j0, rowsum, colsum, colsq);
+  if (large) add_non_finite(W, ldw, blockIdx.y * kRowsPerCta + warp, r1, j0, rowsum, colsum, colsq);
 #pragma unroll
   for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll
@@ -421,11 +418,16 @@ __device__ __noinline__ double definition_lambda(const double* xnorm, int m) {
   }
   return __ddiv_rn(__dmul_rn(0.01, h), (double)m);
 }
+__device__ __noinline__ int rank_among(const double* score, int c) {
+  int rank = 0;
+  for (int a = 0; a < kBeta; ++a) rank += (score[a] > score[c] || (score[a] == score[c] && a < c)) ? 1 : 0;
+  return rank;
+}
 template <bool kVec>
 __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __restrict__ W, size_t ldw, int n, int m, int N, const uint8_t* __restrict__ keep,
                                                               const double* __restrict__ xnorm, double lambda_in, Ws w, uint64_t* __restrict__ salient) {
   __shared__ __align__(16) uint32_t tile[kSalThreads * kSalPitch];   // per weight: |w| bits, bit 15 = kept; later the gains
-  __shared__ double score[kBeta], inv[kBeta + 1], exact[kMaxSal];
+  __shared__ double score[kBeta], ranked[kBeta], inv[kBeta + 1], exact[kMaxSal];
   __shared__ int order[kMaxSal];
   __shared__ uint32_t flag, maybe;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -443,19 +445,20 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __half* __re
     // can move are in the definition's order; the columns of closer ones (duplicated columns, as a rule) are summed again,
     // row by row, and lambda column by column.  Two zeros are exact.
     const double window = (4.0 * ((double)n + m) + 64.0) * kUlp;
-    bool close = false;
-    for (int a = 0; a < kBeta; ++a) close = close || (a != tid && (score[a] != 0.0 || sc != 0.0) && !(fabs(score[a] - sc) > window * fmax(score[a], sc)));
+    int rank = 0;
+    for (int a = 0; a < kBeta; ++a) rank += (score[a] > sc || (score[a] == sc && a < tid)) ? 1 : 0;
+    ranked[rank] = sc;
+    __syncthreads();
+    // (of scores within rounding of one another, those next to each other in rank are)
+    auto near = [&](double hi, double lo) { return hi != 0.0 && !(hi - lo > window * hi); };
+    const bool close = (rank > 0 && near(ranked[rank - 1], sc)) || (rank < kBeta - 1 && near(sc, ranked[rank + 1]));
     if (__syncthreads_or(close)) {
       if (tid == 0) exact[0] = lambda_in < 0.0 ? definition_lambda(xnorm, m) : lambda_in;
       __syncthreads();
-      if (close) {
-        sc = column_score(xnorm[j], exact[0], column_squares(W, ldw, n, j));
-        score[tid] = sc;
-      }
+      if (close) score[tid] = column_score(xnorm[j], exact[0], column_squares(W, ldw, n, j));
       __syncthreads();
+      rank = rank_among(score, tid);
     }
-    int rank = 0;
-    for (int a = 0; a < kBeta; ++a) rank += (score[a] > sc || (score[a] == sc && a < tid)) ? 1 : 0;
     if (rank < kMaxSal) order[rank] = tid;
   }
   double acc[kMaxSal];
@@ -792,7 +795,7 @@ __global__ void __launch_bounds__(kBrkThreads, 1) break_kernel(const __half* __r
 }
 
 // ---- Trisection, Res_Approx and the logical arrays: one thread per (row, block), loops in column order ----------------
-// A row of a block with an infinite or NaN weight: the definition's own comparisons and sums.
+// A row of a block that may keep an infinite or NaN weight: the definition's own comparisons and sums.
 __device__ __noinline__ void emit_non_finite(const __half* wr, const uint8_t* kr, const uint8_t* sal, double p1, double p2, uint8_t* sign, uint16_t* region,
                                              uint32_t* sign2, uint16_t* scale) {
   double a[4] = {0, 0, 0, 0}, alpha[5], ar = 0.0;
@@ -848,11 +851,9 @@ __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W,
   const uint8_t* kr = keep + (size_t)r * ngrp + b * 16;
   double above2 = 0.0, above1 = 0.0, all = 0.0, asal = 0.0;      // exact sums: above the second threshold, the first, all, salient
   int k2 = 0, k1 = 0, k0 = 0, ks = 0;
-  uint32_t codes = 0;
 #pragma unroll 2
   for (int g = 0; g < 16; ++g) {
     const uint4 v = load8<kVec>(wr + 8 * g);
-    codes = largest_code(v, codes);
     const uint32_t sb = (salw[g >> 2] >> (8 * (g & 3))) & 0xFFu, kb = kr[g];
     uint32_t m1 = 0, m2 = 0;
 #pragma unroll
@@ -871,7 +872,7 @@ __global__ void __launch_bounds__(128) emit_kernel(const __half* __restrict__ W,
     k2 += __popc(m2); k1 += __popc(m1); k0 += __popc(kb & ~sb); ks += __popc(kb & sb);
   }
   const size_t rb = (size_t)r * nblk + b;
-  if (non_finite(codes)) {
+  if (all + asal >= kInfiniteCode) {
     emit_non_finite(wr, kr, w.salflag + b * kBeta, w.bp[2 * b], w.bp[2 * b + 1], sign + (size_t)r * ngrp + b * 16, region + (size_t)r * ngrp + b * 16, sign2 + rb,
                     scale + rb * 5);
     return;

@@ -128,13 +128,14 @@ struct CtaRange { int32_t lo, hi, whole, first, head_cta, head_share, tail_cta, 
 __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// a value and its tag in one 8-byte access: whoever sees the tag sees the value
+// a value and its tag in one 8-byte access (a scalar one: of a vector access the elements may be seen one by one): whoever sees
+// the tag sees the value
 __device__ __forceinline__ void st_tagged(uint2* p, float v, uint32_t tag) {
-  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(__float_as_uint(v)), "r"(tag) : "memory");
+  asm volatile("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tst.relaxed.gpu.global.u64 [%0], t;\n\t}" ::"l"(p), "r"(__float_as_uint(v)), "r"(tag) : "memory");
 }
 __device__ __forceinline__ uint2 ld_tagged(const uint2* p) {
   uint2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  asm volatile("{\n\t.reg .b64 t;\n\tld.relaxed.gpu.global.u64 t, [%2];\n\tmov.b64 {%0, %1}, t;\n\t}" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const void* p) {

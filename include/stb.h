@@ -217,7 +217,7 @@ int stb_layer_stack(const stb_step *steps, int count, int *dev_status, void *str
  * again (also after a wait that ran out) and no partial sum in the rest of it, so the same workspace serves call after call
  * without being cleared.  It belongs to the kernel between calls too (a count of the calls stays in it): do not write to it.
  * Calls that share a workspace must not overlap on the GPU.
- * The launch is cooperative: it fails with STB_ERR_CUDA when the GPU cannot hold one 512-thread
+ * The launch is cooperative: it fails with STB_ERR_CUDA when the GPU cannot hold one 640-thread
  * CTA per SM at once. */
 int stb_layer_stack_resident_workspace(const stb_step *steps, int count, size_t *bytes);
 int stb_layer_stack_resident(const stb_step *steps, int count, void *ws, size_t ws_bytes,

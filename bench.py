@@ -709,7 +709,7 @@ def cuda_arm(args):
                    "l2": "cold: %d distinct packed copies of each layer (%.0f MB per rotation, L2 is 126 MB)" % (
                        copies, copies * wl.bytes_step / 1e6),
                    "launch": ("one stb_layer_stack_resident call of %d passes (3 linears each) captured in a CUDA graph and replayed: one "
-                              "cooperative launch of one 512-thread CTA per SM for the whole list" % copies) if wl.resident else
+                              "cooperative launch of one 640-thread CTA per SM for the whole list" % copies) if wl.resident else
                              ("one stb_layer_stack call of %d passes (3 linears each) captured in a CUDA graph and replayed; 2 launches "
                               "per pass (gate+up as one grid, down), chained by programmatic dependent launch" % copies),
                    "multi_gpu": "replicas only" if world > 1 else "single GPU"},

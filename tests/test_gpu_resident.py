@@ -253,6 +253,17 @@ def test_gated_activation_that_fills_shared_memory(stb, N, batch, f):
     _check_gated_mlp(stb, torch, dg, du, dd, batch)
 
 
+@pytest.mark.parametrize("N,batch,f", [(4, 4, 11264), (5, 8, 3840), (6, 4, 8192), (6, 2, 18688), (5, 2, 21760), (4, 1, 40960)])
+def test_gated_activation_beside_slots_for_few_residual_words(stb, N, batch, f):
+    """Formed inputs that fit only where ring slots hold eight residual words at most: blocks of 32 salient columns then come one
+    by one, others in pairs."""
+    import torch
+    dg = si.logical_layer(f, 128, N, 178, max_salient=9)
+    du = si.logical_layer(f, 128, N, 179, max_salient=9)
+    dd = si.logical_layer(70, f, N, 180, salient_counts=[32, 32, 3, 17, 0, 9])
+    _check_gated_mlp(stb, torch, dg, du, dd, batch)
+
+
 def _picking_layer(m):
     """A 4:8 layer whose row r is 1 in column r and 0 elsewhere: its output is its staged input."""
     c = np.arange(m)

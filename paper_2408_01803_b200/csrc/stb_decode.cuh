@@ -35,6 +35,28 @@ STB_HD uint32_t prmt(uint32_t a, uint32_t b, uint32_t s) {
 #endif
 }
 
+// Halves and bytes of a word by the integer dot product, which runs on the multiply-add pipe: the integer ALU, busy with byte permutes
+// (2 warp-instructions per clock and SM), is what bounds the decode in position order.
+template <bool kUpper>
+STB_HD uint32_t pick_half(uint32_t w, uint32_t add) {        // a half of w, plus `add`
+#if defined(__CUDA_ARCH__)
+  uint32_t d;
+  asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(kUpper ? 1u << 8 : 1u), "r"(add));
+  return d;
+#else
+  return (kUpper ? w >> 16 : w & 0xFFFFu) + add;
+#endif
+}
+STB_HD uint32_t pick_byte(uint32_t w, int k) {               // byte k of w; k is known to the compiler
+#if defined(__CUDA_ARCH__)
+  uint32_t d;
+  asm("dp4a.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(1u << (8 * k)), "r"(0u));
+  return d;
+#else
+  return (w >> (8 * k)) & 0xFFu;
+#endif
+}
+
 // ------------------------------------------------------------------------------------------
 template <int N>
 struct LaneTile {
@@ -179,8 +201,13 @@ STB_HD void plain_slot(const LaneTile<N>& t, int u, uint32_t (&out_code)[8], uin
 // the rank of the column among the kept ones, or 7 = a zero byte) that spreads the rank-ordered
 // bytes to the 8 column positions; two more permutes per pair of registers re-interleave low
 // and high bytes into 16-bit values.
-template <int N>
+// kDot: halves and bytes by dot products.  Which form is faster depends on the kernel around it, beyond the clocks of a tile alone
+// (5:8: 152 with shifts, 139 with products): the launches per layer take products at 5:8 (28672 x 8192, one row: 54.6 -> 52.6 us), the
+// resident kernel and the prefill GEMM shifts throughout (4096-wide layers at 6:8 there 193 us with shifts, 208 with products).
+template <int N, bool kDot = false>
 struct FastRows {
+  STB_HD static uint32_t upper(uint32_t w) { return kDot ? pick_half<true>(w, 0u) : w >> 16; }
+  STB_HD static uint32_t byte_at(uint32_t w, int k) { return kDot ? pick_byte(w, k) : prmt(w, 0u, 0x4440u + (uint32_t)k); }
   static_assert(N >= 4 && N <= 6, "fast decode covers N = 4, 5, 6");
   uint32_t A[4], Bp[4], Bn[4];
   uint32_t e[4], o[4];
@@ -213,9 +240,8 @@ struct FastRows {
   // rank-ordered bytes of ranks 4.. : N = 6 one call per (row j, step pair sp), N = 5 one call
   // per row j (sp ignored)
   STB_HD void high(int j, int sp, uint32_t& XL, uint32_t& XH) const {
-    uint32_t sel;
-    if (N == 6) sel = ((j & 1) ? oh[j >> 1] : eh[j >> 1]) >> (16 * sp);
-    else sel = ((j & 2) ? oh[0] : eh[0]) >> (16 * (j & 1));
+    uint32_t sel = N == 6 ? ((j & 1) ? oh[j >> 1] : eh[j >> 1]) : ((j & 2) ? oh[0] : eh[0]);
+    if (N == 6 ? sp : j & 1) sel = upper(sel);
     XL = prmt(A[j], A[j], sel);
     XH = prmt(Bp[j], Bn[j], sel);
   }
@@ -227,15 +253,15 @@ struct FastRows {
   }
   // same, with the selectors of columns 0..3 (P0) and 4..7 (P1) in separate words
   STB_HD void slot2(int j, int s, uint32_t P0, uint32_t P1, uint32_t XL, uint32_t XH, uint32_t (&f)[4]) const {
-    const uint32_t sel = ((s & 2) ? o[j] : e[j]) >> (16 * (s & 1));
+    const uint32_t sels = (s & 2) ? o[j] : e[j], sel = (s & 1) ? upper(sels) : sels;
     const uint32_t lo0 = prmt(A[j], A[j], sel), hi0 = prmt(Bp[j], Bn[j], sel);
     uint32_t lo1 = 0, hi1 = 0;
     if (N == 6) {
-      lo1 = (s & 1) ? (XL >> 16) : (XL & 0xFFFFu);
-      hi1 = (s & 1) ? (XH >> 16) : (XH & 0xFFFFu);
+      lo1 = (s & 1) ? upper(XL) : (XL & 0xFFFFu);
+      hi1 = (s & 1) ? upper(XH) : (XH & 0xFFFFu);
     } else if (N == 5) {
-      lo1 = prmt(XL, 0u, 0x4440u + (uint32_t)s);
-      hi1 = prmt(XH, 0u, 0x4440u + (uint32_t)s);
+      lo1 = byte_at(XL, s);
+      hi1 = byte_at(XH, s);
     }
     const uint32_t pl0 = prmt(lo0, lo1, P0), pl1 = prmt(lo0, lo1, P1);
     const uint32_t ph0 = prmt(hi0, hi1, P0), ph1 = prmt(hi0, hi1, P1);
@@ -248,7 +274,7 @@ struct FastRows {
   // lower rank); XL / XH from high(j, s >> 1).  Nothing is moved to column positions: the sparse
   // tensor-core instruction does that with the metadata of meta6_nibble.
   STB_HD void pairs(int j, int s, uint32_t XL, uint32_t XH, uint32_t (&r)[3]) const {
-    const uint32_t sel = ((s & 2) ? o[j] : e[j]) >> (16 * (s & 1));
+    const uint32_t sels = (s & 2) ? o[j] : e[j], sel = (s & 1) ? upper(sels) : sels;
     const uint32_t lo0 = prmt(A[j], A[j], sel), hi0 = prmt(Bp[j], Bn[j], sel);
     r[0] = prmt(lo0, hi0, 0x5140u);
     r[1] = prmt(lo0, hi0, 0x7362u);
@@ -294,6 +320,26 @@ constexpr Meta6Joint make_meta6_joint() {
       t.v[i0 + kMasks6 * i1][3] = 0;
     }
   return t;
+}
+// The same entries as two words, the form kept in shared memory: 8 bytes cost half the wavefronts of 16 in look-ups that meet in the
+// banks at random, and two more permutes put the metadata together.  Word 0: the nibbles of chunks 0 and 1 for i0 in bytes 0 and 1, for
+// i1 in bytes 2 and 3; word 1: those of chunk 2, at bits 0 and 16.
+struct Meta6Pairs { uint32_t v[kMasks6 * kMasks6][2]; };
+constexpr Meta6Pairs make_meta6_pairs() {
+  Meta6Pairs t{};
+  const Meta6Joint j = make_meta6_joint();
+  for (uint32_t e = 0; e < kMasks6 * kMasks6; ++e) {
+    t.v[e][0] = j.v[e][0] | (j.v[e][1] << 8);
+    t.v[e][1] = j.v[e][2];
+  }
+  return t;
+}
+// metadata words of the three chunks from the entries of the quad's four lanes (multiply-adds, for the sake of the integer ALU)
+STB_HD void meta6_pairs_words(const uint32_t (&en)[4][2], uint32_t (&E)[3]) {
+  const uint32_t z01 = en[1][0] * 16u + en[0][0], z23 = en[3][0] * 16u + en[2][0];
+  E[0] = prmt(z01, z23, 0x6240u);
+  E[1] = prmt(z01, z23, 0x7351u);
+  E[2] = ((en[3][1] * 16u + en[2][1]) * 16u + en[1][1]) * 16u + en[0][1];
 }
 // The six metadata words of a lane from the table entries en[rp][tq] (row g + 16 mt + 8 rp, lane tq of the quad)
 // of one of its two slots: word i has the nibble of lane tq at bit 4 tq (row rp = 0) and 16 + 4 tq (rp = 1).

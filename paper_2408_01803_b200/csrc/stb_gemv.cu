@@ -361,7 +361,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
     LaneTile<N> lt;
     load_lane_tile<N>(tile, lane, lt);
     refill();
-    FastRows<N> fr;
+    FastRows<N, N == 5 && NB == 1> fr;
     fr.init(lt, lt.A, lt.B);
     uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
     if (N == 5) {
@@ -583,7 +583,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
   // What needs no other memory comes first: the launch is a programmatic dependent of whatever ran before it on the stream.
   // Within a chain (stb_layer_stack, whose packed layers nobody writes meanwhile) the weights may be read before that is done too.
   if (kImage) {
-    for (int i = tid; i < (int)(kMasks6 * kMasks6); i += kGThreads) reinterpret_cast<uint4*>(smem)[i] = *reinterpret_cast<const uint4*>(g_meta6_joint.v[i]);
+    fill_meta6(smem, tid, kGThreads);
   } else {
     for (int i = tid; i < kPosTableEntries * (int)kPosCopies; i += kGThreads) reinterpret_cast<uint2*>(smem)[i] = g_pos_table.v[N][i / (int)kPosCopies];
   }
@@ -790,7 +790,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
             TileD<N> d;
             load_tile<N>(tile, lane, ptab, kPosCopies * 8u, d);
             if (k == cnt - 1) { __syncwarp(); issue(slot); }
-            tile_mul<N, true, NB>(d, xp, acc);
+            tile_mul<N, true, NB, N == 5>(d, xp, acc);
           }
           tile += tb;
         }

@@ -584,9 +584,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
   W.slot = 0; W.parity = 0; W.failed = false;
   const uint32_t epoch = __ldcg(P.sync + 4);          // changed only by the last CTA out
   // tables, while the first copies are under way
-  if (P.use_meta6)
-    for (int i = threadIdx.x; i < (int)(kMasks6 * kMasks6); i += kSThreads)
-      reinterpret_cast<uint4*>(smem)[i] = *reinterpret_cast<const uint4*>(g_meta6_joint.v[i]);
+  if (P.use_meta6) fill_meta6(smem, (int)threadIdx.x, kSThreads);
 #pragma unroll
   for (int N = 4; N <= 6; ++N)
     if (P.pos_off[N - 4])

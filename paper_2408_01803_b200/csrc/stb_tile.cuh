@@ -11,10 +11,17 @@
 
 namespace stb {
 
-static __device__ const Meta6Joint g_meta6_joint = make_meta6_joint();
+static __device__ const Meta6Pairs g_meta6_pairs = make_meta6_pairs();
 
-constexpr uint32_t kMeta6Bytes = kMasks6 * kMasks6 * 16;   // the joint 6:8 metadata table; kept at shared-memory offset 0: a pair field of a
-                                                           // tile is the address of its entry
+// The joint 6:8 metadata table, kept at shared-memory offset 0: two copies of every entry side by side, for even and for odd lanes, so
+// that a pair field of a tile (16 times its entry's number) is the address of the entry.
+constexpr uint32_t kMeta6Bytes = kMasks6 * kMasks6 * 16;
+__device__ __forceinline__ void fill_meta6(uint8_t* smem, int thread, int threads) {
+  for (int i = thread; i < (int)(kMasks6 * kMasks6); i += threads) {
+    const uint2 e = *reinterpret_cast<const uint2*>(g_meta6_pairs.v[i]);
+    reinterpret_cast<uint4*>(smem)[i] = make_uint4(e.x, e.y, e.x, e.y);
+  }
+}
 constexpr uint32_t kImgWordsPerBlock = 96;    // 6:8 operand-order image: words per block and batch row
 constexpr uint32_t kXPad = 64;                // bytes between the rows of the plain copy beyond 2 m: the eight lane groups' loads do not conflict
 constexpr uint32_t kImgPad = 16;              // the same beyond the rows of the image
@@ -48,28 +55,35 @@ __device__ __forceinline__ uint32_t hmul2_bits(uint32_t a, uint32_t b) {
 
 // 6:8 through the sparse instruction: the weights stay in rank order and the instruction places them (stb_decode.cuh,
 // meta6_nibble).  x: the lane's place in the operand-order image (t 96 bytes into the block's 384).
+//
+// What bounds it: shared memory and the integer ALU alike.  With 16-byte table entries and the fields loaded one by one a tile took 130
+// wavefronts (82 of the look-ups, 32 of the fields) and as many clocks; now about 93 of both, 149 integer instructions among them.
 struct Tile6 { LaneTile<6> lt; uint32_t fld[8]; };
 __device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, Tile6& d) {
   load_lane_tile<6>(tile, lane, d.lt, true);
+  const uint32_t copy = 8u * ((uint32_t)lane & 1u);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) d.fld[k] = *reinterpret_cast<const uint16_t*>(tile + lane * 16 + 2 * k);
+  for (int k = 0; k < 4; ++k) {
+    d.fld[2 * k] = pick_half<false>(d.lt.mask[k], copy);
+    d.fld[2 * k + 1] = pick_half<true>(d.lt.mask[k], copy);
+  }
 }
 template <int NB>
 __device__ __forceinline__ void tile_mul(const Tile6& d, const uint8_t* smem, const uint8_t* const (&x)[NB], float (&acc)[2][NB][4]) {
   FastRows<6> fr;
   fr.init(d.lt, d.lt.A, d.lt.B);
-  // Metadata: fld[4 bb + tq] is the pair field (= the address of the joint-table entry) of slot 2 h + bb of lane tq of
-  // the quad, for the two rows whose metadata this lane supplies; word i of the entries, shifted to the lane's
-  // nibble and added (multiply-adds: the integer pipe is the busy one), is the metadata of chunk i.
+  // Metadata: fld[4 bb + tq] is the address of the table entry of slot 2 h + bb of lane tq of the quad, for the two rows whose
+  // metadata this lane supplies.
   uint32_t E[2][3];
 #pragma unroll
   for (int bb = 0; bb < 2; ++bb) {
-    uint4 en[4];
+    uint32_t en[4][2];
 #pragma unroll
-    for (int tq = 0; tq < 4; ++tq) en[tq] = *reinterpret_cast<const uint4*>(smem + d.fld[4 * bb + tq]);
-    E[bb][0] = ((en[3].x * 16u + en[2].x) * 16u + en[1].x) * 16u + en[0].x;
-    E[bb][1] = ((en[3].y * 16u + en[2].y) * 16u + en[1].y) * 16u + en[0].y;
-    E[bb][2] = ((en[3].z * 16u + en[2].z) * 16u + en[1].z) * 16u + en[0].z;
+    for (int tq = 0; tq < 4; ++tq) {
+      const uint2 v = *reinterpret_cast<const uint2*>(smem + d.fld[4 * bb + tq]);
+      en[tq][0] = v.x; en[tq][1] = v.y;
+    }
+    meta6_pairs_words(en, E[bb]);
   }
   // the activations of the tile's six chunk positions, once for both halves of the rows (one batch group; of more, as they come)
   uint4 bxs[2][3];
@@ -125,9 +139,9 @@ __device__ __forceinline__ uint4 ldg_v4_coherent(const void* p) {
   return v;
 }
 // x: the lane's activations of the block (8 t columns in), in shared memory (kStaged) or global
-template <int N, bool kStaged, int NB>
+template <int N, bool kStaged, int NB, bool kDot = false>
 __device__ __forceinline__ void tile_mul(const TileD<N>& d, const uint8_t* const (&x)[NB], float (&acc)[2][NB][4]) {
-  FastRows<N> fr;
+  FastRows<N, kDot> fr;
   fr.init(d.lt, d.lt.A, d.lt.B);
   uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
   if (N == 5) {

@@ -32,13 +32,13 @@
 //     of all earlier phases.  The poll is bounded; when it or an mbarrier wait runs out, an abort flag makes
 //     every CTA leave, STB_ERR_TIMEOUT is reported and the last CTA out restores the workspace to zero.
 //
-// What bounds it.  In the tile loop instruction issue, the integer ALU first (2 warp-instructions per clock and SM; the decode
-// alone takes 126 / 145 / 118 clocks per tile and SM at N = 6 / 5 / 4, with the waits, residual words and copies 180 / 193 /
-// 170).  Between phases, latencies, about 7 us each: the spread of the warps' ends, the sums, one trip through L2 for the count of
-// finished row tiles and one for the activations.  And about 9 us per call (launch, set-up, leaving).  Of a 7B MLP at 6:8 and
-// one row (44.6 us) these are 20, 14 and 9 us, of 32 7B layers (1900 us) 980 and 900 and little.
-// Against one copy per five-block span issued by the decoding warps themselves: 7B MLP 45.6 -> 44.6 us, 13B block at 5:8
-// 108.4 -> 95.3, 32 7B layers 2046 -> 1900, at 2 / 4 / 8 rows 2206 / 2477 / 2908 -> 2105 / 2280 / 2775.
+// What bounds it.  In the tile loop the integer ALU at 4:8 and 5:8 (2 warp-instructions per clock and SM) and shared memory and the ALU
+// alike at 6:8: 130 / 155 / 107 clocks per tile and SM at N = 4 / 5 / 6 for decode and product with the tiles on their way from HBM,
+// and about 180 / 200 / 157 with residual words, waits and copies.  Between phases, latencies, 6.5 to 7.5 thousand clocks: the spread of
+// the warps' ends, the sums, a release (1,050), the count of finished row tiles and the activations (a trip through L2 each).  And
+// about 9 us per call (launch, set-up, leaving).
+// At one row: 7B MLP at 6:8 44.8 -> 36.9 us, 13B block at 5:8 95.8 -> 89.4, 32 7B layers 1905 -> 1744 against 16-byte metadata entries,
+// sums of pieces four at a time and one kernel for everything; eight 7B layers at eight rows 692 -> 634.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -104,7 +104,7 @@ struct StackParams {
   int* dev_status;
   long long wait_limit;
   int32_t copies_off;
-  int32_t places;                             // phases that do not gather go by places
+  int32_t form, only5;                        // the kernel: ResidForm, and whether every phase is 5:8
 };
 
 // shared memory: joint 6:8 metadata table first (784 x 16 B, at offset 0: a pair field of a tile is the shared-memory
@@ -402,9 +402,10 @@ __device__ __forceinline__ void resid_mul(const uint8_t* rec, uint32_t na, uint3
 
 // The warp's run of phase q: chunks of residual words and tiles, partial sums out.
 // kImage: 6:8 from the operand-order image; kStaged: position order with the activations in a plain copy in shared memory
-// kPlaces: residual activations that are not gathered are found by their places (otherwise by the layer's word table)
-template <int N, bool kImage, bool kStaged, bool kPlaces>
+// kForm: the residual activations are gathered throughout the launch, or, where a phase's are not, found by places / the layer's word table
+template <int N, bool kImage, bool kStaged, ResidForm kForm, bool kDot = false>
 __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const StackPhase& q, int* pslot, float* pdata) {
+  constexpr bool kPlaces = kForm == ResidForm::kPlaced;
   const StackParams& P = *E.P;
   const int lane = E.lane, g = E.g, t = E.t, warp = E.warp, batch = q.batch;
   constexpr uint32_t tb = tile_bytes(N);
@@ -444,7 +445,7 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
     auto residual = [&] {
       if (nw == 0u) return;
       ResidX X;
-      if (q.gather == 2) {
+      if (kForm == ResidForm::kGathered || q.gather == 2) {
         X.xw = xs + c.z * xw_step; X.xw_step = xw_step;
         resid_mul<ResidForm::kGathered, true>(records, na, nw, g, t, X, acc);
       } else if constexpr (kPlaces) {
@@ -458,9 +459,11 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
         resid_mul<ResidForm::kListed, false>(records, na, nw, g, t, X, acc);
       }
     };
-    // In global memory the words' activations lie in the lines that the chunk's tiles read as well: after the tiles the loads of two
-    // bytes find them in L1 (before them, 2 % slower at two rows, 4 to 8 % at eight).  The slot is kept until then.
-    constexpr bool kLate = kPlaces && !kImage && !kStaged;
+    // Before or after the tiles of their chunk?  In global memory the words' activations lie in the lines that the chunk's tiles read as
+    // well: after the tiles the loads of two bytes find them in L1 (before them, 2 % slower at two rows, 4 to 8 % at eight).  Gathered
+    // in shared memory, after them at 4:8 and 5:8 (7B MLP at 4:8, one row, 44.7 -> 43.1 us), before them at 6:8 (four layers of 5120 at one row 255 us, after them 259).
+    // The slot is kept until then.
+    constexpr bool kLate = kForm == ResidForm::kGathered ? !kImage : kPlaces && !kImage && !kStaged;
     if (!kLate) residual();
     const uint8_t* xb = xbase + (size_t)c.y * xstep;
     const int cnt = (int)(c.x & 3u);
@@ -477,7 +480,7 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
         TileD<N> d;
         load_tile<N>(tile, lane, ptab, prow, d);
         if (!kLate && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
-        tile_mul<N, kStaged, 1>(d, xp, acc);
+        tile_mul<N, kStaged, 1, kDot>(d, xp, acc);
       }
       tile += tb;
       xb += xstep;
@@ -570,7 +573,7 @@ __device__ __forceinline__ bool stack_setup(const StackParams& P, uint8_t* base,
 }
 
 // The decoding warps: all phases in order.
-template <bool kPlaces>
+template <ResidForm kForm, bool kOnly5>
 __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* smem, uint8_t* base, volatile int* ctl, int* pslot, float* pdata, int cta) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* ximg = reinterpret_cast<uint32_t*>(smem + P.x_off);
@@ -640,36 +643,39 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
     const bool stop = ctl[0] != 0;
     if (stop) W.failed = true;
     // The code between two phases runs once per phase, much of it out of a cold instruction cache: it is kept short rather
-    // than unrolled.  An item = eight activations of a batch row; the next item is on its way while one is stored.
+    // than unrolled.  An item = eight activations of a batch row; three at a time are on their way.
     if (q.use_image && !stop) {
       const int per_row = q.m / 8, items = batch * per_row;
-      uint4 v = make_uint4(0, 0, 0, 0), v2 = v;
-      auto fetch = [&](int it) {
-        const int r = batch == 1 ? 0 : it / per_row;
-        const size_t o = (size_t)r * q.ldx + (size_t)(it - r * per_row) * 8;
-        if (it < items) {
-          v = ldg_v4_coherent(q.x + o);
-          if (q.x2) v2 = ldg_v4_coherent(q.x2 + o);
-        }
-      };
-      int it = threadIdx.x;
-      fetch(it);
+      constexpr int kAhead = 3;
 #pragma unroll 1
-      while (it < items) {
-        uint32_t a[4] = {v.x, v.y, v.z, v.w};
-        const uint32_t b[4] = {v2.x, v2.y, v2.z, v2.w};
-        const int cur = it;
-        it += kSThreads;
-        fetch(it);
-        if (q.x2) {
+      for (int first = threadIdx.x; first < items; first += kAhead * kSThreads) {
+        uint4 v[kAhead], v2[kAhead];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) a[k] = silu_mul_bits(a[k], b[k]);
+        for (int k = 0; k < kAhead; ++k) {
+          const int it = first + k * kSThreads, r = batch == 1 ? 0 : it / per_row;
+          const size_t o = (size_t)r * q.ldx + (size_t)(it - r * per_row) * 8;
+          v[k] = v2[k] = make_uint4(0, 0, 0, 0);
+          if (it < items) {
+            v[k] = ldg_v4_coherent(q.x + o);
+            if (q.x2) v2[k] = ldg_v4_coherent(q.x2 + o);
+          }
         }
-        const int r = batch == 1 ? 0 : cur / per_row, qq = cur - r * per_row;
-        if (q.use_image == 1) {
-          image_store(ximg + (uint32_t)r * ((uint32_t)nb * kImgWordsPerBlock), (uint32_t)qq >> 4, (uint32_t)qq & 15u, a);
-        } else {
-          *reinterpret_cast<uint4*>(smem + P.x_off + (uint32_t)r * (2u * (uint32_t)q.m + kXPad) + (uint32_t)qq * 16u) = make_uint4(a[0], a[1], a[2], a[3]);
+#pragma unroll 1
+        for (int cur = first, k = 0; k < kAhead && cur < items; ++k, cur += kSThreads) {
+          uint32_t a[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+          const uint32_t b[4] = {v2[0].x, v2[0].y, v2[0].z, v2[0].w};
+#pragma unroll
+          for (int u = 0; u + 1 < kAhead; ++u) { v[u] = v[u + 1]; v2[u] = v2[u + 1]; }
+          if (q.x2) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[u] = silu_mul_bits(a[u], b[u]);
+          }
+          const int r = batch == 1 ? 0 : cur / per_row, qq = cur - r * per_row;
+          if (q.use_image == 1) {
+            image_store(ximg + (uint32_t)r * ((uint32_t)nb * kImgWordsPerBlock), (uint32_t)qq >> 4, (uint32_t)qq & 15u, a);
+          } else {
+            *reinterpret_cast<uint4*>(smem + P.x_off + (uint32_t)r * (2u * (uint32_t)q.m + kXPad) + (uint32_t)qq * 16u) = make_uint4(a[0], a[1], a[2], a[3]);
+          }
         }
       }
     }
@@ -690,14 +696,18 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
 
     // ---- this warp's tiles ----
     if (!W.failed && wl < wh) {
-      if (q.use_image == 1) run_tiles<6, true, false, kPlaces>(E, W, q, pslot, pdata);
-      else if (q.use_image == 2) {
-        if (q.N == 6) run_tiles<6, false, true, kPlaces>(E, W, q, pslot, pdata);
-        else if (q.N == 5) run_tiles<5, false, true, kPlaces>(E, W, q, pslot, pdata);
-        else run_tiles<4, false, true, kPlaces>(E, W, q, pslot, pdata);
-      } else if (q.N == 6) run_tiles<6, false, false, kPlaces>(E, W, q, pslot, pdata);
-      else if (q.N == 5) run_tiles<5, false, false, kPlaces>(E, W, q, pslot, pdata);
-      else run_tiles<4, false, false, kPlaces>(E, W, q, pslot, pdata);
+      if constexpr (kOnly5) run_tiles<5, false, true, kForm, true>(E, W, q, pslot, pdata);
+      else if (q.use_image == 1) run_tiles<6, true, false, kForm>(E, W, q, pslot, pdata);
+      else if (kForm == ResidForm::kGathered) {
+        if (q.N == 5) run_tiles<5, false, true, kForm>(E, W, q, pslot, pdata);
+        else run_tiles<4, false, true, kForm>(E, W, q, pslot, pdata);
+      } else if (q.use_image == 2) {
+        if (q.N == 6) run_tiles<6, false, true, kForm>(E, W, q, pslot, pdata);
+        else if (q.N == 5) run_tiles<5, false, true, kForm>(E, W, q, pslot, pdata);
+        else run_tiles<4, false, true, kForm>(E, W, q, pslot, pdata);
+      } else if (q.N == 6) run_tiles<6, false, false, kForm>(E, W, q, pslot, pdata);
+      else if (q.N == 5) run_tiles<5, false, false, kForm>(E, W, q, pslot, pdata);
+      else run_tiles<4, false, false, kForm>(E, W, q, pslot, pdata);
     }
     if (W.failed && lane == 0 && !ctl[0]) {
       // this warp's own wait ran out: tell the CTA and the grid
@@ -729,18 +739,12 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
         bool lost = false;
         for (int v = lane; v < nval; v += 32) {
           const float* pv = pdata + v;
-          float sum = pv[(size_t)s0 * P.part_floats];
-          for (uint32_t mm = members; mm != 0u;) {
-            // four loads at a time, added in order
-            float x[4];
+          float sum = pv[(size_t)s0 * P.part_floats], x[kSWarps];
+          // all loads before the additions, which go in order
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              x[k] = mm ? pv[(size_t)(2 * (__ffs(mm) - 1)) * P.part_floats] : 0.0f;
-              mm &= mm - 1u;
-            }
+          for (int w = 1; w < kSWarps; ++w) x[w] = (members >> w) & 1u ? pv[(uint32_t)(2 * w) * P.part_floats] : 0.0f;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) sum += x[k];
-          }
+          for (int w = 1; w < kSWarps; ++w) sum += x[w];
           if (!whole && cta != c_first) {
             st_tagged(gp + (size_t)(cta - c_first) * P.part_floats + v, sum, tag);
             continue;
@@ -782,7 +786,7 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
   }
 }
 
-template <bool kPlaces>
+template <ResidForm kForm, bool kOnly5>
 __global__ void __launch_bounds__(kSAllThreads, 1)
 stack_kernel(const __grid_constant__ StackParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -805,7 +809,7 @@ stack_kernel(const __grid_constant__ StackParams P) {
     feed_rings(P, smem, base, ctl);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDecodeRegs));
-    decode_phases<kPlaces>(P, smem, base, ctl, pslot, pdata, cta);
+    decode_phases<kForm, kOnly5>(P, smem, base, ctl, pslot, pdata, cta);
   }
 
   // ---- leaving: let copies in flight land, then the last CTA out restores the workspace ----
@@ -1076,13 +1080,19 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
     }
   }
   if (!found) return -1;                                           // a formed input does not fit shared memory
+  // The kernel: gathered throughout (every phase is staged then, 6:8 as an image), by places where not all are gathered, or by the word
+  // tables where one phase has neither; phases that are gathered stay so, but places and tables do not go together.  (One kernel with
+  // all seven loops has 165 KB of code, the first of these 84: 9 % of its warps' time went to fetching instructions.)
   bool listed = false, gathered = true;
   for (int p = 0; p < sp.nphase; ++p) {
     listed = listed || sp.ph[p].gather == 0;
-    gathered = gathered && sp.ph[p].gather == 2;
+    gathered = gathered && sp.ph[p].gather == 2 && (sp.ph[p].use_image == 1 || (sp.ph[p].use_image == 2 && sp.ph[p].N < 6));
   }
-  sp.places = !listed && !gathered ? 1 : 0;
-  if (listed)                                                      // (one kernel for both would be slower than either)
+  sp.only5 = 1;
+  for (int p = 0; p < sp.nphase; ++p)
+    if (sp.ph[p].N != 5) sp.only5 = 0;
+  sp.form = (int)(listed ? ResidForm::kListed : gathered ? ResidForm::kGathered : ResidForm::kPlaced);
+  if (listed)
     for (int p = 0; p < sp.nphase; ++p)
       if (sp.ph[p].gather == 1) sp.ph[p].gather = 0;
   const size_t s_need = 8 * sizeof(uint32_t);
@@ -1091,6 +1101,15 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
   if (s_need > sync_need) sync_need = s_need;
   if (g_need > gpart_need) gpart_need = g_need;
   return i;
+}
+
+// Gathered throughout, lists of 5:8 layers alone have a kernel of their own, with halves and bytes picked by dot products (13B block at one
+// row 95.8 -> 89.7 us).  Beside other formats that form costs those more than it brings (6:8 4 to 5 %), and kernels for 4:8 or 6:8 alone
+// were slower than the one for all three (235 against 231 us for four 7B layers at 4:8, 191 against 188 at 6:8).
+static auto kernel_of(ResidForm form, bool only5) {
+  if (form == ResidForm::kPlaced) return stack_kernel<ResidForm::kPlaced, false>;
+  if (form == ResidForm::kListed) return stack_kernel<ResidForm::kListed, false>;
+  return only5 ? stack_kernel<ResidForm::kGathered, true> : stack_kernel<ResidForm::kGathered, false>;
 }
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -1145,7 +1164,8 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return STB_ERR_CUDA;
   if (!attr_done[dev]) {
-    for (auto* kernel : {stb::stack_kernel<false>, stb::stack_kernel<true>})
+    for (auto* kernel : {stb::kernel_of(stb::ResidForm::kGathered, false), stb::kernel_of(stb::ResidForm::kGathered, true),
+                         stb::kernel_of(stb::ResidForm::kPlaced, false), stb::kernel_of(stb::ResidForm::kListed, false)})
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stb::kSmemLimit) != cudaSuccess) return STB_ERR_CUDA;
     attr_done[dev] = true;
   }
@@ -1174,7 +1194,8 @@ static int stack_resident_impl(const stb_step* steps, int count, void* ws, size_
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, sp.places ? stb::stack_kernel<true> : stb::stack_kernel<false>, sp) != cudaSuccess) return STB_ERR_CUDA;
+    auto* kernel = stb::kernel_of((stb::ResidForm)sp.form, sp.only5 != 0);
+    if (cudaLaunchKernelEx(&cfg, kernel, sp) != cudaSuccess) return STB_ERR_CUDA;
   }
   return STB_OK;
 }

@@ -517,7 +517,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
 // residual words of the slice are turned into places in the staged activations once per CTA.
 // Sums: a warp writes the rows it begins to shared memory and the piece it continues beside it; the CTA adds them in order, the
 // cluster adds its CTAs' sums through distributed shared memory, in order.
-// What bounds it: the decode (about 175 clocks per tile and SM, integer issue), and a chain of latencies before and after it
+// What bounds it: the decode with its residual words (about 185 / 195 / 155 clocks per tile and SM at N = 4 / 5 / 6, the integer ALU), and a chain of latencies before and after it
 // (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small layers stay with gemv_mma_kernel;
 // launch_mma_b has the rule).
 // Against that kernel, cold L2, microseconds: 28672 x 8192 4:8 batch 1 58.9 -> 48.1, 5120 x 13824 5:8 batch 8 32.6 -> 25.3,
@@ -733,6 +733,9 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
     }
     const uint32_t xstep = kImage ? kImgWordsPerBlock * 4u : 2u * kBlock, xlane = (uint32_t)t * (kImage ? 96u : 16u);
     const uint8_t* ptab = smem + (uint32_t)(lane & (kPosCopies - 1)) * 8u;
+    // The residual words of a chunk before or after its tiles?  At 4:8 and 5:8 after them (28672 x 8192, one row: 49.3 -> 47.2 us and
+    // 52.6 -> 50.7; 4096 x 11008 at 5:8, eight rows, 18.6 -> 17.3), at 6:8 before them (39.8 against 40.7).  The slot is kept until then.
+    constexpr bool kLate = N != 6;
     uint32_t slot = 0, parity = 0;
     int left = hi - lo, row = nbp > 0 ? lo / nbp : 0, blk = lo - row * nbp;
     while (left > 0 && !failed) {
@@ -757,6 +760,7 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
         const uint8_t* rec = tile + (uint32_t)P.chunk * tb;
         const uint32_t w0 = roff[blk], na = roff[blk + 1] - w0, nw = roff[blk + cnt] - w0;
         // residual words of the chunk, four (16 salient slots) per tensor-core step, lane t the t-th
+        auto residual = [&] {
 #pragma unroll 1
         for (uint32_t kk = (uint32_t)t; kk < nw + (uint32_t)t; kk += 4u) {
           const uint32_t k = min(kk, nw - 1u);
@@ -775,6 +779,8 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
             mma16816(acc[1][c], fa[2][0], fa[3][0], fa[2][1], fa[3][1], q0, q1);
           }
         }
+        };
+        if (!kLate) residual();
 #pragma unroll 1
         for (int k = 0; k < cnt; ++k) {
           const uint8_t* xp[NB];
@@ -784,16 +790,17 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
           if constexpr (kImage) {
             Tile6 d;
             load_tile(tile, lane, d);
-            if (k == cnt - 1) { __syncwarp(); issue(slot); }
+            if (!kLate && k == cnt - 1) { __syncwarp(); issue(slot); }
             tile_mul<NB>(d, smem, xp, acc);
           } else {
             TileD<N> d;
             load_tile<N>(tile, lane, ptab, kPosCopies * 8u, d);
-            if (k == cnt - 1) { __syncwarp(); issue(slot); }
+            if (!kLate && k == cnt - 1) { __syncwarp(); issue(slot); }
             tile_mul<N, true, NB, N == 5>(d, xp, acc);
           }
           tile += tb;
         }
+        if (kLate) { residual(); __syncwarp(); issue(slot); }
         parity ^= slot;
         slot ^= 1u;
         blk += cnt; left -= cnt;

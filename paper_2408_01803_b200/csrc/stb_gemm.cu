@@ -81,12 +81,14 @@ constexpr double kDecodeClocks = 440.0;    // decode of a stage (gemm_plan)
 // parity cannot tell the phase before from the phase after.
 // What depends on bn: copies of the position table (16, lane-minor: look-ups nearly free of bank conflicts; one where bn = 256
 // leaves no room), where the stages and the boxes lie, and how many boxes there are.
+// `pairs`: the table is the joint one of 6:8 (decode_tiles).
+constexpr uint32_t kPairTabBytes = kMasks6 * kMasks6 * 16;
 struct GemmSmem { uint32_t copies, a, b, box, nbox, total; };
-__host__ __device__ inline GemmSmem gemm_smem(int kAcc, int stages_a, int bn) {
+__host__ __device__ inline GemmSmem gemm_smem(int kAcc, int stages_a, int bn, bool pairs) {
   GemmSmem g;
   g.box = (uint32_t)bn * kBK * 2;
   for (g.copies = 16;; g.copies = 1) {
-    g.a = (kGemmTab + 8u * kPosTableEntries * g.copies + 1023u) & ~1023u;
+    g.a = (kGemmTab + (pairs ? kPairTabBytes : 8u * kPosTableEntries * g.copies) + 1023u) & ~1023u;
     g.b = g.a + (uint32_t)stages_a * kStageA;
     g.nbox = (kSmemMax - g.b) / g.box;
     if (g.nbox >= 5u || g.copies == 1u) break;
@@ -233,7 +235,11 @@ __device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, Ge
 
 // Decode role of one warp: packed row tile 4 mt + q, every fourth block of the CTA's K range, written into the A stages.
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
-template <int N, bool kF16, int kStagesA>
+// kPairs (6:8): the position selectors of two rows by one look-up with the tile's pair field, which is the address of their entry: 32 bits
+// of selectors per row, two copies of every entry for even and odd lanes.  Splitting the field into two mask indices and looking
+// each up took 60 of the 760 instructions of a tile (28672 x 8192 at 64 tokens 96.8 -> 94.1 us, 11008 x 4096 27.6 -> 27.2).  For
+// calls of up to 64 tokens, where the decode is what takes the time and the boxes leave room for the table's 12 KB.
+template <int N, bool kF16, int kStagesA, bool kPairs>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1, w = da.w;
   // The lane plays the part of packed-layout lane 4 g + t with g = lane % 8, t = lane / 8: the eight
@@ -302,7 +308,11 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
 #pragma unroll 1
   for (int b = b0 + w; b < b1; b += kGroups, ++use) {
     uint32_t mask[4] = {0, 0, 0, 0};                   // word j, byte s: keep-mask index of slot (j, s)
-    if constexpr (mask_pairs(N)) {
+    uint32_t fld[8];
+    if constexpr (kPairs) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) fld[k] = nxt.fld[k];
+    } else if constexpr (mask_pairs(N)) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) {                    // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)
         const uint32_t J = nxt.fld[k] >> 4, i1 = (J * 2341u) >> 16, i0 = J - kMasks6 * i1;      // (pair_field_index)
@@ -334,7 +344,14 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl) P[j][sl] = lds_v2(keep_index_of(mask, j, 2 * h + sl) * da.entry + da.ptab);
+        for (int sl = 0; sl < 2; ++sl) {
+          if constexpr (!kPairs) P[j][sl] = lds_v2(keep_index_of(mask, j, 2 * h + sl) * da.entry + da.ptab);
+          else if ((j & 1) == 0) {
+            const uint2 e = lds_v2(fld[2 * j + 2 * h + sl] + da.ptab);
+            P[j][sl] = make_uint2(e.x, pick_half<true>(e.x, 0u));
+            P[j + 1][sl] = make_uint2(e.y, pick_half<true>(e.y, 0u));
+          }
+        }
       uint32_t f[4][2][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -418,11 +435,16 @@ __global__ void gemm_gather_kernel(const uint8_t* __restrict__ packed, int n, in
 // Where a call's output tiles lie (gemm_plan).
 struct GemmShape { int full_tiles, ksplit, bps, ttiles, bn; GemmSmem smem; };
 
+// whether the position table is the joint one
+template <class Cfg>
+STB_HD constexpr bool pair_table(int N) { return mask_pairs(N) && Cfg::kMaxBN == BatchCfg::kMaxBN; }
+
 template <int N, class Cfg, bool kF16>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap xsmap, const uint8_t* __restrict__ packed, int n, int m, int T,
             void* __restrict__ Y, int y_16, size_t ldy, float* __restrict__ ws, const __grid_constant__ GemmShape shape, uint32_t box_bytes, int* dev_status) {
   constexpr int kAcc = Cfg::kAcc, kMaxBN = Cfg::kMaxBN, kStagesA = Cfg::kStagesA;
+  constexpr bool kPairs = pair_table<Cfg>(N);
   extern __shared__ __align__(1024) uint8_t smem[];
   const int full_tiles = shape.full_tiles, ksplit = shape.ksplit, bps = shape.bps, ttiles = shape.ttiles, bn = shape.bn;
   const GemmSmem& L = shape.smem;
@@ -470,8 +492,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads)
-    reinterpret_cast<uint2*>(smem + kGemmTab)[i] = g_pos_table.v[N][L.copies == 1u ? i : i >> 4];
+  if constexpr (kPairs) {
+    for (uint32_t i = threadIdx.x; i < kMasks6 * kMasks6; i += kGemmThreads) {
+      const uint2 e0 = g_pos_table.v[N][i % kMasks6], e1 = g_pos_table.v[N][i / kMasks6];
+      const uint32_t r0 = e0.x | (e0.y << 16), r1 = e1.x | (e1.y << 16);
+      reinterpret_cast<uint4*>(smem + kGemmTab)[i] = make_uint4(r0, r1, r0, r1);
+    }
+  } else {
+    for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads)
+      reinterpret_cast<uint2*>(smem + kGemmTab)[i] = g_pos_table.v[N][L.copies == 1u ? i : i >> 4];
+  }
   constexpr uint32_t kTmemCols = kAcc == 1 ? 2 * kMaxBN : kAcc * kMaxBN;      // one accumulator: a second one for the other half of K
   if (warp == kIssuerWarpA) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
   tc_fence_before();
@@ -587,11 +617,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     const int gi = warp >> 2;               // decode group: which of the row tile's four warps this one is
     DecodeArgs da;
     da.packed = packed; da.abort_flag = abort_flag;
-    da.entry = 8u * L.copies; da.ptab = sbase + kGemmTab + 8u * ((uint32_t)lane & (L.copies - 1u)); da.stages = sbase + L.a;
+    da.entry = 8u * L.copies; da.ptab = sbase + kGemmTab + 8u * ((uint32_t)lane & (kPairs ? 1u : L.copies - 1u)); da.stages = sbase + L.a;
     da.bar_full = bar_fullA; da.bar_empty = bar_emptyA;
     da.mt = mt; da.b0 = b0; da.b1 = max(b1, b0); da.nblk = nblk; da.ntile = ntile; da.q = warp & 3; da.w = gi; da.lane = lane;
     da.nrw = nrw; da.rw0 = rw0; da.rw1 = rw1; da.nres = nres;
-    decode_tiles<N, kF16, kStagesA>(da);
+    decode_tiles<N, kF16, kStagesA, kPairs>(da);
 
     // ---------------- epilogue: TMEM -> registers -> Y ----------------
     const int q = warp & 3;                        // TMEM lane quarter of this warp
@@ -836,7 +866,7 @@ static int launch_gemm(const GemmPlan& plan, const uint8_t* packed, int n, int m
   float* ws_split = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + gemm_xs_bytes(m, T));
   GemmShape shape;
   shape.full_tiles = plan.full_tiles; shape.ksplit = plan.ksplit; shape.bps = plan.bps; shape.ttiles = plan.ttiles; shape.bn = plan.bn;
-  shape.smem = gemm_smem(kAcc, Cfg::kStagesA, plan.bn);
+  shape.smem = gemm_smem(kAcc, Cfg::kStagesA, plan.bn, pair_table<Cfg>(N));
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return STB_ERR_CUDA;
   const CUtensorMapDataType dt = kF16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;

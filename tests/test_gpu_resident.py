@@ -81,6 +81,22 @@ def test_chain_with_per_layer_N(stb, batch):
     assert (hg.cpu().numpy()[:, 200:] == 0).all()                            # columns past n untouched
 
 
+@pytest.mark.parametrize("formats", [(5,), (4, 5, 6)])
+@pytest.mark.parametrize("blocks", [1, 15, 17, 33])
+def test_row_tiles_of_one_to_sixteen_pieces(stb, blocks, formats):
+    """About one row tile per SM, whose tiles are dealt to one warp, to fifteen, and to all sixteen with unequal runs; one row (gathered
+    throughout: lists of 5:8 alone have a kernel of their own) and three (the kernel with all forms)."""
+    import torch
+    n, m = 32 * torch.cuda.get_device_properties(0).multi_processor_count - 5, 128 * blocks
+    ds = [si.logical_layer(n, m, N, 1300 + N, max_salient=9) for N in formats]
+    layers, Ls = [stb.pack_numpy(d) for d in ds], [oracle.Logical(**d) for d in ds]
+    for batch in (1, 3):
+        x = torch.from_numpy(si.activations(batch, m, 1310)).cuda()
+        triples = [(layer, x, torch.zeros(batch, n, dtype=torch.float32, device="cuda")) for layer in layers]
+        _run(stb, torch, triples)
+        _check_layers(triples, Ls, rows_of=lambda n, k: np.r_[0:64, n // 2:n // 2 + 32, n - 40:n])
+
+
 def test_results_are_reproducible_and_close_to_the_per_layer_launches(stb):
     import torch
     d1, d2 = si.logical_layer(700, 1024, 6, 81, max_salient=12), si.logical_layer(300, 768, 4, 82, max_salient=12)

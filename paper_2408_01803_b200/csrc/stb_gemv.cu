@@ -733,9 +733,9 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
     }
     const uint32_t xstep = kImage ? kImgWordsPerBlock * 4u : 2u * kBlock, xlane = (uint32_t)t * (kImage ? 96u : 16u);
     const uint8_t* ptab = smem + (uint32_t)(lane & (kPosCopies - 1)) * 8u;
-    // The residual words of a chunk before or after its tiles?  At 4:8 and 5:8 after them (28672 x 8192, one row: 49.3 -> 47.2 us and
-    // 52.6 -> 50.7; 4096 x 11008 at 5:8, eight rows, 18.6 -> 17.3), at 6:8 before them (39.8 against 40.7).  The slot is kept until then.
-    constexpr bool kLate = N != 6;
+    // When a slot is filled again: once its last tile is in registers, in position order after the products (in between, the loads of the
+    // activations stay behind it: 28672 x 8192, one row, 49.3 -> 46.3 us at 4:8, 52.5 -> 49.4 at 5:8).
+    constexpr bool kBack = !kImage;
     uint32_t slot = 0, parity = 0;
     int left = hi - lo, row = nbp > 0 ? lo / nbp : 0, blk = lo - row * nbp;
     while (left > 0 && !failed) {
@@ -759,8 +759,8 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
         const uint8_t* tile = ringp + slot * P.slot;
         const uint8_t* rec = tile + (uint32_t)P.chunk * tb;
         const uint32_t w0 = roff[blk], na = roff[blk + 1] - w0, nw = roff[blk + cnt] - w0;
-        // residual words of the chunk, four (16 salient slots) per tensor-core step, lane t the t-th
-        auto residual = [&] {
+        // residual words of the chunk, four (16 salient slots) per tensor-core step, lane t the t-th; before its tiles, whose sum is larger
+        // (with them after the tiles 4:8 lost 0.8 % and 5:8 2.2 % of their accuracy against float64)
 #pragma unroll 1
         for (uint32_t kk = (uint32_t)t; kk < nw + (uint32_t)t; kk += 4u) {
           const uint32_t k = min(kk, nw - 1u);
@@ -779,28 +779,25 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
             mma16816(acc[1][c], fa[2][0], fa[3][0], fa[2][1], fa[3][1], q0, q1);
           }
         }
-        };
-        if (!kLate) residual();
 #pragma unroll 1
         for (int k = 0; k < cnt; ++k) {
           const uint8_t* xp[NB];
 #pragma unroll
           for (int c = 0; c < NB; ++c) xp[c] = xrow[c] + xlane + (live[c] & ((uint32_t)(blk + k) * xstep));
-          // once the slot's last tile is in registers the slot is filled again
           if constexpr (kImage) {
             Tile6 d;
             load_tile(tile, lane, d);
-            if (!kLate && k == cnt - 1) { __syncwarp(); issue(slot); }
+            if (!kBack && k == cnt - 1) { __syncwarp(); issue(slot); }
             tile_mul<NB>(d, smem, xp, acc);
           } else {
             TileD<N> d;
             load_tile<N>(tile, lane, ptab, kPosCopies * 8u, d);
-            if (!kLate && k == cnt - 1) { __syncwarp(); issue(slot); }
+            if (!kBack && k == cnt - 1) { __syncwarp(); issue(slot); }
             tile_mul<N, true, NB, N == 5>(d, xp, acc);
           }
           tile += tb;
         }
-        if (kLate) { residual(); __syncwarp(); issue(slot); }
+        if (kBack) { __syncwarp(); issue(slot); }
         parity ^= slot;
         slot ^= 1u;
         blk += cnt; left -= cnt;

@@ -459,33 +459,37 @@ __device__ __forceinline__ void run_tiles(const WarpEnv& E, WarpState& W, const 
         resid_mul<ResidForm::kListed, false>(records, na, nw, g, t, X, acc);
       }
     };
-    // Before or after the tiles of their chunk?  In global memory the words' activations lie in the lines that the chunk's tiles read as
-    // well: after the tiles the loads of two bytes find them in L1 (before them, 2 % slower at two rows, 4 to 8 % at eight).  Gathered
-    // in shared memory, after them at 4:8 and 5:8 (7B MLP at 4:8, one row, 44.7 -> 43.1 us), before them at 6:8 (four layers of 5120 at one row 255 us, after them 259).
-    // The slot is kept until then.
-    constexpr bool kLate = kForm == ResidForm::kGathered ? !kImage : kPlaces && !kImage && !kStaged;
+    // The words come before the tiles of their chunk: the tensor core cuts off what it adds to a large sum, so that words added to the
+    // sum of one more chunk lose more (drawn 4:8 and 5:8 layers, one row, against float64: 0.4 % more error with them after the tiles).
+    // Words whose activations are in global memory come after the tiles, whose lines they find in L1 (before them, 2 % slower at two
+    // rows, 4 to 8 % at eight).
+    constexpr bool kLate = kPlaces && !kImage && !kStaged;
+    // When the slot is handed back: once its last tile is in registers, or, gathered in position order, after the products (handing it
+    // back in between keeps the loads of the activations behind it: four 7B layers at 4:8 238 -> 221 us, at 5:8 246 -> 230; at 6:8
+    // 189.4 against 197.8).
+    constexpr bool kBack = kLate || (kForm == ResidForm::kGathered && !kImage);
     if (!kLate) residual();
     const uint8_t* xb = xbase + (size_t)c.y * xstep;
     const int cnt = (int)(c.x & 3u);
 #pragma unroll 1
     for (int k = 0; k < cnt; ++k) {
       const uint8_t* const xp[1] = {xb};
-      // once the slot's last tile is in registers the slot is handed back
       if constexpr (kImage) {
         Tile6 d;
         load_tile(tile, lane, d);
-        if (!kLate && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        if (!kBack && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
         tile_mul<1>(d, E.smem, xp, acc);
       } else {
         TileD<N> d;
         load_tile<N>(tile, lane, ptab, prow, d);
-        if (!kLate && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+        if (!kBack && k == cnt - 1) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
         tile_mul<N, kStaged, 1, kDot>(d, xp, acc);
       }
       tile += tb;
       xb += xstep;
     }
-    if (kLate) { residual(); __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
+    if (kLate) residual();
+    if (kBack) { __syncwarp(); if (lane == 0) mbar_arrive(E.empty + 8u * slot); }
     W.slot ^= 1u;
     W.parity ^= slot;
     if (c.x & kSegEnd) {

@@ -97,6 +97,40 @@ def test_row_tiles_of_one_to_sixteen_pieces(stb, blocks, formats):
         _check_layers(triples, Ls, rows_of=lambda n, k: np.r_[0:64, n // 2:n // 2 + 32, n - 40:n])
 
 
+@pytest.mark.parametrize("N,batch", [(4, 1), (5, 1), (5, 8), (6, 1)])
+def test_residual_words_are_added_before_the_tiles_of_their_chunk(stb, N, batch):
+    """The residual terms of a block, two steps of sixteen with a sum of 1 each, beside one weight's 2^24, where an fp32 sum takes nothing
+    less than 2: added to each other first they come through, added to the weight's product they are cut off one after the other."""
+    import torch
+    n, m = 4096, 11008                                        # a size for gemv_stream_kernel at these rows
+    x = np.zeros((batch, m), dtype=np.float16)
+    cols = np.arange(0, 128, 8)
+    x[:, cols], x[:, cols + 1], x[:, 2] = 1 / 16, 1 / 16, 4096.0
+    ngrp, nblk = m // 8, m // 128
+    d = {"n": n, "m": m, "N": N, "keep": np.full((n, ngrp), (1 << N) - 1, np.uint8), "sign": np.full((n, ngrp), (1 << N) - 1, np.uint8),
+         "region": np.zeros((n, ngrp), np.uint16), "sign2": np.zeros((n, nblk), np.uint32), "salient": np.zeros((nblk, 2), np.uint64),
+         "scale": np.empty((n, nblk, 5), np.float16)}
+    d["region"][:, :16] = 0xF                                 # block 0: columns 8 g and 8 g + 1 of every group are salient
+    d["sign2"][:, 0] = 0xFFFFFFFF
+    d["salient"][0] = 0x0303030303030303
+    d["scale"][:] = [4096.0, 4096.0, 4096.0, 0.0, 1.0]        # the salient weights are their residual term alone
+    d["scale"] = d["scale"].view(np.uint16)
+    layer, want = stb.pack_numpy(d), float(2 ** 24 + 2)
+    assert layer.info()["status"] == 0
+    xd = torch.from_numpy(x).cuda()
+    got = {"gemv": stb.gemv(layer, xd)}
+    if batch == 1:
+        for formats in ((N,), (4, 5, 6)):                     # alone and beside other formats
+            other = [stb.pack_numpy(si.logical_layer(64, 128, k, 1400 + k)) for k in formats if k != N]
+            small = torch.zeros(1, 128, dtype=torch.float16, device="cuda")
+            y = torch.zeros(1, n, dtype=torch.float32, device="cuda")
+            _run(stb, torch, [(layer, xd, y)] + [(o, small, torch.zeros(1, 64, dtype=torch.float32, device="cuda")) for o in other])
+            got["resident %d formats" % len(formats)] = y
+    torch.cuda.synchronize()
+    for call, y in got.items():
+        assert (y == want).all(), (call, y.unique().tolist())
+
+
 def test_results_are_reproducible_and_close_to_the_per_layer_launches(stb):
     import torch
     d1, d2 = si.logical_layer(700, 1024, 6, 81, max_salient=12), si.logical_layer(300, 768, 4, 82, max_salient=12)

@@ -324,7 +324,7 @@ constexpr Meta6Joint make_meta6_joint() {
 // The same entries as two words, the form kept in shared memory: 8 bytes cost half the wavefronts of 16 in look-ups that meet in the
 // banks at random, and two more permutes put the metadata together.  Word 0: the nibbles of chunks 0 and 1 for i0 in bytes 0 and 1, for
 // i1 in bytes 2 and 3; word 1: those of chunk 2, at bits 0 and 16.
-struct Meta6Pairs { uint32_t v[kMasks6 * kMasks6][2]; };
+struct alignas(8) Meta6Pairs { uint32_t v[kMasks6 * kMasks6][2]; };      // (an entry is read as eight bytes)
 constexpr Meta6Pairs make_meta6_pairs() {
   Meta6Pairs t{};
   const Meta6Joint j = make_meta6_joint();

@@ -18,6 +18,8 @@
 
 using namespace stb;
 
+static_assert(alignof(Meta6Pairs) >= alignof(uint2) && sizeof(Meta6Pairs::v[0]) == sizeof(uint2), "an entry of the metadata table is read as eight bytes");
+
 static uint64_t rng_state = 0x9E3779B97F4A7C15ull;
 static uint32_t rnd() {
   rng_state ^= rng_state << 13; rng_state ^= rng_state >> 7; rng_state ^= rng_state << 17;

@@ -83,6 +83,7 @@ constexpr double kDecodeClocks = 440.0;    // decode of a stage (gemm_plan)
 // leaves no room), where the stages and the boxes lie, and how many boxes there are.
 // `pairs`: the table is the joint one of 6:8 (decode_tiles).
 constexpr uint32_t kPairTabBytes = kMasks6 * kMasks6 * 16;
+static_assert(8u * kStageA >= 0x10000u, "whatever a pair field says, its look-up ends in the eight A stages behind the table at the latest");
 struct GemmSmem { uint32_t copies, a, b, box, nbox, total; };
 __host__ __device__ inline GemmSmem gemm_smem(int kAcc, int stages_a, int bn, bool pairs) {
   GemmSmem g;
@@ -235,9 +236,9 @@ __device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, Ge
 
 // Decode role of one warp: packed row tile 4 mt + q, every fourth block of the CTA's K range, written into the A stages.
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
-// kPairs (6:8): the position selectors of two rows by one look-up with the tile's pair field, which is the address of their entry: 32 bits
+// kPairs (6:8): the position selectors of two rows by one look-up with the tile's pair field, whose upper twelve bits are the address of their entry: 32 bits
 // of selectors per row, two copies of every entry for even and odd lanes.  Splitting the field into two mask indices and looking
-// each up took 60 of the 760 instructions of a tile (28672 x 8192 at 64 tokens 96.8 -> 94.1 us, 11008 x 4096 27.6 -> 27.2).  For
+// each up took 60 of the 760 instructions of a tile (28672 x 8192 at 64 tokens 96.5 -> 94.1 us, 11008 x 4096 27.6 -> 27.1).  For
 // calls of up to 64 tokens, where the decode is what takes the time and the boxes leave room for the table's 12 KB.
 template <int N, bool kF16, int kStagesA, bool kPairs>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
@@ -311,7 +312,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
     uint32_t fld[8];
     if constexpr (kPairs) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) fld[k] = nxt.fld[k];
+      for (int k = 0; k < 8; ++k) fld[k] = nxt.fld[k] & 0xFFF0u;        // (a multiple of 16 in any packed layer; in one altered since, a wrong entry and no misaligned load)
     } else if constexpr (mask_pairs(N)) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) {                    // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)

@@ -380,6 +380,25 @@ def test_gemm_f16_salient_extremes(stb, max_salient):
     _check_gemm_f16(stb, layer, L, 48, 19)
 
 
+def test_gemm_does_not_address_by_unused_bits_of_a_layer(stb):
+    """6:8: the four bits below a pair field are zero when packed and name nothing; a layer in which something set them is the same layer."""
+    import torch
+    n, m, T = 300, 1024, 33
+    layer = stb.pack_numpy(si.logical_layer(n, m, 6, 540, max_salient=9))
+    x = torch.from_numpy(si.activations(T, m, 541)).cuda()
+    calls = (lambda: stb.gemm_f16(layer, x), lambda: stb.gemm(layer, x.to(torch.bfloat16)))
+    want = [c() for c in calls]
+    nblk, ntile, tile = m // 128, (n + 31) // 32, 512 + 192 * 6 + 256
+    start = -(-(64 + 64 * nblk + 64 * nblk) // 256) * 256                    # header, block and residual word tables
+    fields = layer.buf[start:start + ntile * nblk * tile].view(ntile * nblk, tile)[:, :512].view(torch.int16)
+    assert (fields & 15).eq(0).all()
+    bits = torch.randint(0, 16, fields.shape, dtype=torch.int16, device="cuda", generator=torch.Generator("cuda").manual_seed(542))
+    fields |= bits
+    for c, w in zip(calls, want):
+        assert torch.equal(c(), w)
+    assert int(layer.dev_status.item()) == 0
+
+
 @pytest.mark.parametrize("name", ["gate", "down"])
 def test_gemm_f16_full_size_decode_batch(stb, name):
     """A decode batch of 64 on the LLaMA-2-7B MLP layers at 6:8 from the oracle's quantizer, sampled rows."""

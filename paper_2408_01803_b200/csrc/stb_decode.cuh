@@ -451,6 +451,10 @@ STB_HD uint32_t position_selector(uint32_t keep_byte) {
   }
   return p;
 }
+// The joint entry of two rows (N = 6) from their entries { selector of columns 0..3, of columns 4..7 } of the position table: a row's
+// two selectors are the halves of a word, the lower one read as it is (what stands above it does not matter to a byte permute).
+STB_HD uint2 pair_selectors(uint2 e0, uint2 e1) { return make_uint2(e0.x | (e0.y << 16), e1.x | (e1.y << 16)); }
+STB_HD uint2 selectors_of(uint32_t word) { return make_uint2(word, pick_half<true>(word, 0u)); }
 // keep-mask index of slot (j, s)
 STB_HD uint32_t keep_index_of(const uint32_t (&mask)[4], int j, int s) {
   return prmt(mask[j], 0u, 0x4440u + (uint32_t)s);

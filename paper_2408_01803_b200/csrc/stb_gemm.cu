@@ -349,8 +349,8 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
           if constexpr (!kPairs) P[j][sl] = lds_v2(keep_index_of(mask, j, 2 * h + sl) * da.entry + da.ptab);
           else if ((j & 1) == 0) {
             const uint2 e = lds_v2(fld[2 * j + 2 * h + sl] + da.ptab);
-            P[j][sl] = make_uint2(e.x, pick_half<true>(e.x, 0u));
-            P[j + 1][sl] = make_uint2(e.y, pick_half<true>(e.y, 0u));
+            P[j][sl] = selectors_of(e.x);
+            P[j + 1][sl] = selectors_of(e.y);
           }
         }
       uint32_t f[4][2][4];
@@ -495,9 +495,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   }
   if constexpr (kPairs) {
     for (uint32_t i = threadIdx.x; i < kMasks6 * kMasks6; i += kGemmThreads) {
-      const uint2 e0 = g_pos_table.v[N][i % kMasks6], e1 = g_pos_table.v[N][i / kMasks6];
-      const uint32_t r0 = e0.x | (e0.y << 16), r1 = e1.x | (e1.y << 16);
-      reinterpret_cast<uint4*>(smem + kGemmTab)[i] = make_uint4(r0, r1, r0, r1);
+      const uint2 e = pair_selectors(g_pos_table.v[N][i % kMasks6], g_pos_table.v[N][i / kMasks6]);
+      reinterpret_cast<uint4*>(smem + kGemmTab)[i] = make_uint4(e.x, e.y, e.x, e.y);
     }
   } else {
     for (uint32_t i = threadIdx.x; i < kPosTableEntries * L.copies; i += kGemmThreads)

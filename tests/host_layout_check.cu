@@ -4,8 +4,10 @@
 //   * plain_slot returns every kept weight's region code and sign at the right column,
 //   * FastRows::slot (N = 4, 5, 6) returns, for every column, the 16-bit pattern of the signed
 //     scale of the weight's region, or zero for a dropped column,
-//   * for N = 6 the rank-order operand pairs and the metadata table of the sparse tensor-core path
-//     rebuild the same 16-bit patterns, and the pair fields return the keep-mask indices,
+//   * FastRows picking halves and bytes by dot products returns what it returns with shifts,
+//   * for N = 6 the rank-order operand pairs and the metadata tables of the sparse tensor-core path
+//     rebuild the same 16-bit patterns, the pair fields return the keep-mask indices, and the joint
+//     position selectors of two rows are each row's own,
 //   * the residual selectors return the stored two-bit codes.
 // Expected values come from the logical fields directly (the definition of the format), not
 // from any packed-side code.
@@ -15,6 +17,7 @@
 #include <vector>
 
 #include "../paper_2408_01803_b200/csrc/stb_decode.cuh"
+#include "../paper_2408_01803_b200/csrc/stb_ptx.cuh"
 
 using namespace stb;
 
@@ -184,8 +187,9 @@ static int check(int trials, int spb) {
         LaneTile<N> raw;
         load_lane_tile<N>(tile.data(), lane, raw, true);
         static const Meta6Joint joint = make_meta6_joint();
+        static const Meta6Pairs pairs = make_meta6_pairs();
         for (int bb = 0; bb < 2; ++bb) {
-          uint32_t en[2][4], E[3], EJ[3] = {0, 0, 0};
+          uint32_t en[2][4], E[3], EJ[3] = {0, 0, 0}, ep[4][2] = {}, EP[3];
           for (int tq = 0; tq < 4; ++tq) {
             // the pair field of lane tq's slot: two keep-mask indices (one way), or the joint-table entry (the other)
             const uint32_t f = (raw.mask[2 * bb + (tq >> 1)] >> (16 * (tq & 1))) & 0xFFFFu;
@@ -193,10 +197,13 @@ static int check(int trials, int spb) {
             en[0][tq] = meta.v[pair_field_index(f, 0)];
             en[1][tq] = meta.v[pair_field_index(f, 1)];
             for (int i = 0; i < 3; ++i) EJ[i] += joint.v[f / 16][i] << (4 * tq);
+            for (int i = 0; i < 2; ++i) ep[tq][i] = pairs.v[f / 16][i];
           }
           meta6_words(en, E);
+          meta6_pairs_words(ep, EP);
           for (int i = 0; i < 3; ++i) {
             if (E[i] != EJ[i]) { if (++errors < 10) std::printf("joint metadata word N=%d\n", N); }
+            if (E[i] != EP[i]) { if (++errors < 10) std::printf("metadata word of the 8-byte entries N=%d\n", N); }
             for (int tq = 0; tq < 4; ++tq)
               for (int rp = 0; rp < 2; ++rp) {
                 const int r = g + 16 * (t >> 1) + 8 * rp, grp = 4 * (2 * (t & 1) + bb) + tq;
@@ -218,6 +225,21 @@ static int check(int trials, int spb) {
             if (kb != keep[r][grp]) { if (++errors < 10) std::printf("keep byte N=%d\n", N); }
             uint32_t f[4];
             fr.slot(j, s, position_selector(kb), XL, XH, f);
+            {   // halves and bytes by dot products: the same registers
+              FastRows<N, true> dot;
+              dot.init(lt, lt.A, lt.B);
+              uint32_t DL = 0, DH = 0, fd[4];
+              if (N == 5) dot.high(j, 0, DL, DH);
+              if (N == 6) dot.high(j, s >> 1, DL, DH);
+              dot.slot(j, s, position_selector(kb), DL, DH, fd);
+              if (std::memcmp(fd, f, sizeof f) != 0) { if (++errors < 10) std::printf("dot products N=%d lane %d j %d s %d\n", N, lane, j, s); }
+              if constexpr (N == 6) {   // and rank order, whose registers are checked above
+                uint32_t r0[3], r1[3];
+                fr.pairs(j, s, XL, XH, r0);
+                dot.pairs(j, s, DL, DH, r1);
+                if (std::memcmp(r0, r1, sizeof r0) != 0) { if (++errors < 10) std::printf("dot products in rank order lane %d j %d s %d\n", lane, j, s); }
+              }
+            }
             {   // the one-row form with a run-time row index must give the same registers
               RowWords rw;
               load_row_words<N>(tile.data(), lane, j, rw);
@@ -280,6 +302,17 @@ int main() {
       else if (nib != 7u) ++e;
     }
   }
+  // joint selectors of two rows (N = 6), as a look-up hands them to slot2: byte permutes read the low 16 bits
+  static const PosTable pos = make_pos_table();
+  for (uint32_t i1 = 0; i1 < kMasks6; ++i1)
+    for (uint32_t i0 = 0; i0 < kMasks6; ++i0) {
+      const uint2 joint = pair_selectors(pos.v[6][i0], pos.v[6][i1]), a = selectors_of(joint.x), b = selectors_of(joint.y);
+      const uint32_t want0 = position_selector(mask_from_index(6, i0)), want1 = position_selector(mask_from_index(6, i1));
+      if ((a.x & 0xFFFFu) != (want0 & 0xFFFFu) || a.y != want0 >> 16 || (b.x & 0xFFFFu) != (want1 & 0xFFFFu) || b.y != want1 >> 16) ++e;
+    }
+  for (uint32_t k = 0; k < 4; ++k)
+    if (pick_half<false>(0x89ABCDEFu, k) != 0xCDEFu + k || pick_half<true>(0x89ABCDEFu, k) != 0x89ABu + k ||
+        pick_byte(0x89ABCDEFu, (int)k) != ((0x89ABCDEFu >> (8 * k)) & 0xFFu)) ++e;
   std::printf("%s: %d errors\n", e ? "FAIL" : "OK", e);
   return e ? 1 : 0;
 }

@@ -744,9 +744,6 @@ __device__ __forceinline__ void decode_phases(const StackParams& P, uint8_t* sme
         for (int v = lane; v < nval; v += 32) {
           const float* pv = pdata + v;
           float sum = pv[(size_t)s0 * P.part_floats];
-#ifndef US
-#define US 8
-#endif
           // The pieces are loaded all at once and added in order; by four where the kernel has more forms of the tile loop to hold registers
           // for (all at once, it spilled: 13B block at 5:8, two rows, 106.2 us against 103.8).
           if constexpr (kForm == ResidForm::kGathered) {

@@ -761,24 +761,27 @@ gemv_stream_kernel(const __grid_constant__ GemvLayers layers, const __grid_const
         const uint32_t w0 = roff[blk], na = roff[blk + 1] - w0, nw = roff[blk + cnt] - w0;
         // residual words of the chunk, four (16 salient slots) per tensor-core step, lane t the t-th; before its tiles, whose sum is larger
         // (with them after the tiles 4:8 lost 0.8 % and 5:8 2.2 % of their accuracy against float64)
+        auto residual = [&] {
 #pragma unroll 1
-        for (uint32_t kk = (uint32_t)t; kk < nw + (uint32_t)t; kk += 4u) {
-          const uint32_t k = min(kk, nw - 1u);
-          const bool second = k >= na;
-          uint32_t rw = *reinterpret_cast<const uint32_t*>(rec + k * kResidWordBytes + (second ? 2u * kResidA2Bytes : kResidA2Bytes) + 4 * g), fa[4][2];
-          const uint2 a2 = *reinterpret_cast<const uint2*>(rec + (second ? kResidA2Bytes + na * kResidWordBytes : 0u) + 8 * g);
-          if (kk >= nw) rw = kNoTerms;
-          resid_operands(rw, a2, fa);
-          const uint2 at = words[w0 - wfirst + k];
+          for (uint32_t kk = (uint32_t)t; kk < nw + (uint32_t)t; kk += 4u) {
+            const uint32_t k = min(kk, nw - 1u);
+            const bool second = k >= na;
+            uint32_t rw = *reinterpret_cast<const uint32_t*>(rec + k * kResidWordBytes + (second ? 2u * kResidA2Bytes : kResidA2Bytes) + 4 * g), fa[4][2];
+            const uint2 a2 = *reinterpret_cast<const uint2*>(rec + (second ? kResidA2Bytes + na * kResidWordBytes : 0u) + 8 * g);
+            if (kk >= nw) rw = kNoTerms;
+            resid_operands(rw, a2, fa);
+            const uint2 at = words[w0 - wfirst + k];
 #pragma unroll
-          for (int c = 0; c < NB; ++c) {
-            const uint16_t* xr = reinterpret_cast<const uint16_t*>(xrow[c]);
-            const uint32_t p0 = at.x & live[c], p1 = at.y & live[c];
-            const uint32_t q0 = (uint32_t)xr[p0 & 0xFFFFu] | ((uint32_t)xr[p0 >> 16] << 16), q1 = (uint32_t)xr[p1 & 0xFFFFu] | ((uint32_t)xr[p1 >> 16] << 16);
-            mma16816(acc[0][c], fa[0][0], fa[1][0], fa[0][1], fa[1][1], q0, q1);
-            mma16816(acc[1][c], fa[2][0], fa[3][0], fa[2][1], fa[3][1], q0, q1);
+            for (int c = 0; c < NB; ++c) {
+              const uint16_t* xr = reinterpret_cast<const uint16_t*>(xrow[c]);
+              const uint32_t p0 = at.x & live[c], p1 = at.y & live[c];
+              const uint32_t q0 = (uint32_t)xr[p0 & 0xFFFFu] | ((uint32_t)xr[p0 >> 16] << 16), q1 = (uint32_t)xr[p1 & 0xFFFFu] | ((uint32_t)xr[p1 >> 16] << 16);
+              mma16816(acc[0][c], fa[0][0], fa[1][0], fa[0][1], fa[1][1], q0, q1);
+              mma16816(acc[1][c], fa[2][0], fa[3][0], fa[2][1], fa[3][1], q0, q1);
+            }
           }
-        }
+        };
+        residual();
 #pragma unroll 1
         for (int k = 0; k < cnt; ++k) {
           const uint8_t* xp[NB];

@@ -113,7 +113,10 @@ int stb_pack_size(int n, int m, int N, size_t *bytes);
  * no bits beyond their fields, that region 3 marks exactly the kept weights of salient
  * columns and that no block has more than 32 salient columns; a violation stores
  * STB_ERR_CORRUPT in *dev_status and in the packed header (the packed data is then not to be
- * used).  Two small launches on `stream`. */
+ * used).  Two small launches on `stream`.
+ * What stb_pack wrote is trusted: the calls that read a packed layer check its header (shape, N,
+ * status), not its tiles and tables.  Bytes altered afterwards are not noticed there and may make
+ * a kernel read at a wrong address; stb_layer_stack_checksum finds them. */
 int stb_pack(const stb_logical *L, void *packed, size_t packed_bytes, int *dev_status,
              void *stream);
 

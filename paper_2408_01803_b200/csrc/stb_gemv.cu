@@ -517,12 +517,12 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
 // residual words of the slice are turned into places in the staged activations once per CTA.
 // Sums: a warp writes the rows it begins to shared memory and the piece it continues beside it; the CTA adds them in order, the
 // cluster adds its CTAs' sums through distributed shared memory, in order.
-// What bounds it: the decode with its residual words (about 185 / 195 / 155 clocks per tile and SM at N = 4 / 5 / 6, the integer ALU), and a chain of latencies before and after it
-// (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small layers stay with gemv_mma_kernel;
-// launch_mma_b has the rule).
-// Against that kernel, cold L2, microseconds: 28672 x 8192 4:8 batch 1 58.9 -> 48.1, 5120 x 13824 5:8 batch 8 32.6 -> 25.3,
-// 4096 x 11008 6:8 batch 1 20.0 -> 16.4, 11008 x 4096 6:8 batch 16 24.1 -> 20.0, 4096 x 4096 4:8 batch 1 11.3 -> 9.7; in L2, 16
-// rows: 5120 x 13824 4:8 41.8 -> 31.0, 5:8 48.0 -> 35.0, 6:8 50.4 -> 31.6, 1500 x 5120 6:8 13.0 -> 10.4.
+// What bounds it: the decode with its residual words (about 180 / 190 / 155 clocks per tile and SM at N = 4 / 5 / 6, the integer ALU),
+// and a chain of latencies before and after it (header - first tile - staging - sums - cluster: about 10,000 clocks, which is why small
+// layers stay with gemv_mma_kernel; launch_mma_b has the rule).
+// Against that kernel, three layers in turn, microseconds: 28672 x 8192 4:8 batch 1 56.3 -> 46.5, 5120 x 13824 5:8 batch 8 38.3 -> 22.7,
+// 4096 x 11008 6:8 batch 1 17.1 -> 13.1, 11008 x 4096 6:8 batch 16 28.9 -> 18.1, 4096 x 4096 4:8 batch 1 8.9 -> 8.7; 16 rows:
+// 5120 x 13824 4:8 34.6 -> 29.0, 5:8 41.4 -> 30.7, 6:8 43.7 -> 28.4; 1500 x 5120 6:8 13 rows 12.8 -> 10.7.
 constexpr int kGWarps = 16, kGThreads = kGWarps * 32;
 __device__ __forceinline__ int layer_of(const GemvLayers& layers, int rt) {
   int li = 0;
@@ -956,7 +956,9 @@ static cudaError_t launch_mma_n(int N, const GemvLayers& layers, int m, const __
 
 // Clocks that a call of gemv_mma_kernel takes (batch <= 16), from its launch shape: terms fitted to 528 measured calls of all
 // three formats, 32 to 32768 tiles, 1 to 16 rows (6% mean error), times the factor for which the choice between the two kernels by
-// their costs was best (over those calls 0.9% slower on average than always the faster one; gemv_mma_kernel throughout: 9%).
+// their costs was best (over those calls 0.9% slower on average than always the faster one).  gemv_stream_kernel has become 3 to 19 %
+// faster since, most at 6:8: over 119 calls drawn from the same range the choice is 1.8 % behind the faster kernel (gemv_mma_kernel
+// throughout: 18 %; at 6:8 gemv_stream_kernel throughout: 0.2 %).
 static double gemv_mma_cost(int N, int row_tiles, int nblk, int batch, int sms) {
   int ksplit, warps;
   gemv_shape(row_tiles * kTileRows, nblk * kBlock, ksplit, warps);
@@ -969,8 +971,8 @@ static double gemv_mma_cost(int N, int row_tiles, int nblk, int batch, int sms) 
 
 // Launch of gemv_stream_kernel, batch <= 16: the split of the blocks (1, 2, 4, 6 or 8 slices) that is done first, and the wider ring where
 // it fits (clusters of 3, 5 and 7 CTAs measured up to 3 us behind their share of the tiles: an SM of a pair stays idle).  The clocks of a split: the fullest CTA's tiles at their issue rate, its longest warp's tiles at their latency (more
-// with a second group of eight rows or single-tile slots), a cluster's sums, the staging, the epilogue (terms fitted to 1900
-// measured calls of the same range, 3% mean error).  Returns false where no split fits shared memory.
+// with a second group of eight rows or single-tile slots), a cluster's sums, the staging, the epilogue (terms fitted to 1900 measured
+// calls of the same range, 3% mean error, before the kernel's tiles took 3 to 19 % less).  Returns false where no split fits shared memory.
 static bool gemv_plan(int N, int row_tiles, int nblk, int batch, int layers, const int (&most)[9], GemvPlan& best, double& best_cost) {
   bool found = false;
   for (int C = 1; C <= 8; ++C) {
@@ -1071,7 +1073,7 @@ constexpr long long kStreamTiles = 1024;
 // The launches of a chain (stb_layer_stack) mostly take the same kernel: gemv_mma_kernel's CTAs start beside the launch before
 // them, those of gemv_stream_kernel, which fill an SM, do not, and each change from one to the other cost about 4 us.  By the mean
 // tiles of the chain's launches, measured per decoder layer (QKV, O, gate/up, down; microseconds, gemv_mma_kernel against
-// gemv_stream_kernel): mean 832 20.6 / 26.8 (4:8, 2 rows), 25.8 / 33.7 (6:8, 8 rows); 2884 35.5 / 39.6 (4:8), 48.8 / 42.3 (6:8, 8
+// gemv_stream_kernel before its tiles took 3 to 19 % less): mean 832 20.6 / 26.8 (4:8, 2 rows), 25.8 / 33.7 (6:8, 8 rows); 2884 35.5 / 39.6 (4:8), 48.8 / 42.3 (6:8, 8
 // rows), 51.0 / 51.4 (6:8, 16 rows); 4266 47.1 / 49.2 (5:8, 8 rows), 59.7 / 53.5 (6:8, 16 rows); 7498 57.4 / 53.8 (4:8, 2 rows),
 // 61.8 / 58.1 (5:8, 2 rows), 70.6 / 53.1 (6:8, 4 rows); 12352 84.7 / 66.6 (6:8, 2 rows); 19360 115.4 / 100.7 (5:8, 4 rows).
 // `fits`: every launch has a split; `wide`: at least one has double slots (5:8 with a second group of rows needs them: 79.8 / 80.9

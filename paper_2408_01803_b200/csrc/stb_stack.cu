@@ -32,13 +32,14 @@
 //     of all earlier phases.  The poll is bounded; when it or an mbarrier wait runs out, an abort flag makes
 //     every CTA leave, STB_ERR_TIMEOUT is reported and the last CTA out restores the workspace to zero.
 //
-// What bounds it.  In the tile loop the integer ALU at 4:8 and 5:8 (2 warp-instructions per clock and SM) and shared memory and the ALU
-// alike at 6:8: 130 / 155 / 107 clocks per tile and SM at N = 4 / 5 / 6 for decode and product with the tiles on their way from HBM,
-// and about 180 / 200 / 157 with residual words, waits and copies.  Between phases, latencies, 6.5 to 7.5 thousand clocks: the spread of
-// the warps' ends, the sums, a release (1,050), the count of finished row tiles and the activations (a trip through L2 each).  And
+// What bounds it.  In the tile loop the integer ALU (2 warp-instructions per clock and SM; at 6:8 it is busy for about 122 of a tile's 157
+// clocks, shared memory for 112): about 165 / 185 / 157 clocks per tile and SM at N = 4 / 5 / 6 with residual words, waits and copies.
+// Between the last tile of a phase and the first of the next, latencies, 6.5 to 7.5 thousand clocks: the sums, a release (1,050), the
+// count of finished row tiles and the activations (a trip through L2 each); before that the warps' ends are spread by 1.5 thousand.  And
 // about 9 us per call (launch, set-up, leaving).
-// At one row: 7B MLP at 6:8 44.8 -> 36.9 us, 13B block at 5:8 95.8 -> 89.4, 32 7B layers 1905 -> 1744 against 16-byte metadata entries,
-// sums of pieces four at a time and one kernel for everything; eight 7B layers at eight rows 692 -> 634.
+// At one row: 7B MLP at 6:8 44.8 -> 36.9 us, 13B block at 5:8 96.1 -> 87.4, 32 7B layers 1905 -> 1683 against 16-byte metadata entries,
+// sums of pieces four at a time, one kernel for everything and slots of 4:8 and 5:8 handed back before the product; eight 7B layers at
+// eight rows 692 -> 637.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -1099,9 +1100,11 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
     }
   }
   if (!found) return -1;                                           // a formed input does not fit shared memory
-  // The kernel: gathered throughout (every phase is staged then, 6:8 as an image), by places where not all are gathered, or by the word
-  // tables where one phase has neither; phases that are gathered stay so, but places and tables do not go together.  (One kernel with
-  // all seven loops has 165 KB of code, the first of these 84: 9 % of its warps' time went to fetching instructions.)
+  // The kernel: gathered throughout (every phase is staged then) with 6:8 as an image, by places where not all are gathered or a 6:8 phase
+  // is in position order, or by the word tables where one phase has neither; phases that are gathered stay so, but places and tables do
+  // not go together.  (One kernel with all seven loops has 165 KB of code, the first of these 84: 9 % of its warps' time went to fetching
+  // instructions.  6:8 in position order, gathered, had a place in the first until its loops were thinned out; such lists are faster
+  // all the same: 7B MLP at two rows 51.7 -> 47.1 us, MLPs of 6144 x 18432 and 8192 x 20480 at one row 85.8 -> 75.7 and 121.7 -> 107.9.)
   bool listed = false, gathered = true;
   for (int p = 0; p < sp.nphase; ++p) {
     listed = listed || sp.ph[p].gather == 0;
@@ -1123,7 +1126,7 @@ static int build_phases(const stb_step* steps, int count, int i0, int G, StackPa
 }
 
 // Gathered throughout, lists of 5:8 layers alone have a kernel of their own, with halves and bytes picked by dot products (13B block at one
-// row 95.8 -> 89.7 us).  Beside other formats that form costs those more than it brings (6:8 4 to 5 %), and kernels for 4:8 or 6:8 alone
+// row 96.1 -> 87.4 us).  Beside other formats that form costs those more than it brings (6:8 4 to 5 %), and kernels for 4:8 or 6:8 alone
 // were slower than the one for all three (235 against 231 us for four 7B layers at 4:8, 191 against 188 at 6:8).
 static auto kernel_of(ResidForm form, bool only5) {
   if (form == ResidForm::kPlaced) return stack_kernel<ResidForm::kPlaced, false>;

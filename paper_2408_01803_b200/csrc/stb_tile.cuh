@@ -56,8 +56,8 @@ __device__ __forceinline__ uint32_t hmul2_bits(uint32_t a, uint32_t b) {
 // 6:8 through the sparse instruction: the weights stay in rank order and the instruction places them (stb_decode.cuh,
 // meta6_nibble).  x: the lane's place in the operand-order image (t 96 bytes into the block's 384).
 //
-// What bounds it: shared memory and the integer ALU alike.  With 16-byte table entries and the fields loaded one by one a tile took 130
-// wavefronts (82 of the look-ups, 32 of the fields) and as many clocks; now about 93 of both, 149 integer instructions among them.
+// What bounds it: shared memory, about 93 wavefronts a tile, and 96 clocks (its 149 integer instructions take 75).  With 16-byte table
+// entries and the fields loaded one by one a tile took 130 wavefronts (82 of the look-ups, 32 of the fields) and as many clocks.
 struct Tile6 { LaneTile<6> lt; uint32_t fld[8]; };
 __device__ __forceinline__ void load_tile(const uint8_t* tile, int lane, Tile6& d) {
   load_lane_tile<6>(tile, lane, d.lt, true);

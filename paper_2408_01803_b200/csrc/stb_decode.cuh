@@ -203,8 +203,8 @@ STB_HD void plain_slot(const LaneTile<N>& t, int u, uint32_t (&out_code)[8], uin
 // and high bytes into 16-bit values.
 // kDot: halves and bytes by dot products.  Which form is faster depends on the kernel around it, beyond the clocks of a tile alone
 // (5:8: 152 with shifts, 139 with products).  Products: 5:8 in gemv_stream_kernel (28672 x 8192, one row: 54.6 -> 52.6 us), in
-// gemv_mma_kernel with up to eight rows (4096 x 4096, one row: 10.2 -> 9.1 us, 28672 x 8192 63.0 -> 59.1; with more rows level or mixed),
-// and in the resident kernel of lists of 5:8 alone (stb_stack.cu, kernel_of).  Shifts everywhere else: the resident kernel of several
+// gemv_mma_kernel with up to eight rows (4096 x 4096, one row: 10.2 -> 9.1 us, 28672 x 8192 63.0 -> 59.1; with more rows level or mixed;
+// short_second_wave has an exception), and in the resident kernel of lists of 5:8 alone (stb_stack.cu, kernel_of).  Shifts everywhere else: the resident kernel of several
 // formats (four 4096-wide layers at 6:8 193 us, with products 208) and the GEMM.
 template <int N, bool kDot = false>
 struct FastRows {

@@ -87,8 +87,9 @@ struct GemvLayers {
 // registers, was measured slower: the spills cost more than the extra resident CTA brings).
 constexpr int kGemvMaxThreads = 128;
 constexpr int kMaxDevices = 64;
-template <int N, int NB, bool kChained>
-__global__ void __launch_bounds__(kGemvMaxThreads, NB <= 2 ? 4 : 1)
+constexpr int kMmaPerSm = 4;
+template <int N, int NB, bool kChained, bool kDot>
+__global__ void __launch_bounds__(kGemvMaxThreads, NB <= 2 ? kMmaPerSm : 1)
 gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* __restrict__ x, int batch,
                 size_t ldx, int* dev_status, int lg_ksplit, int bpp, long long wait_limit, int copies_off) {
   // A programmatic dependent of whatever ran before it: prepared while that drains.  Only within a chain (stb_layer_stack,
@@ -361,7 +362,7 @@ gemv_mma_kernel(const __grid_constant__ GemvLayers layers, int m, const __half* 
     LaneTile<N> lt;
     load_lane_tile<N>(tile, lane, lt);
     refill();
-    FastRows<N, N == 5 && NB == 1> fr;
+    FastRows<N, kDot> fr;
     fr.init(lt, lt.A, lt.B);
     uint32_t XL[4] = {0, 0, 0, 0}, XH[4] = {0, 0, 0, 0};
     if (N == 5) {
@@ -898,7 +899,8 @@ static void gemv_shape(int n, int m, int& ksplit, int& warps) {
 
 // kChained: nobody writes the packed layer while the kernel before it on the stream runs.  That is another GEMV of the same
 // stb_layer_stack call (`early`: a programmatic dependent of it), or the kernel is launched in stream order.
-template <int N, int NB, bool kChained>
+// kDot: 5:8 picks halves and bytes by dot products (stb_decode.cuh).
+template <int N, int NB, bool kChained, bool kDot = N == 5 && NB == 1>
 static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, int batch, size_t ldx,
                               int* dev_status, cudaStream_t s, bool early, bool wait_selftest) {
   const int ntile = layers.tile_start[layers.count], nblk = m / kBlock;
@@ -912,7 +914,7 @@ static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices || !attr_done[dev]) {
-    e = cudaFuncSetAttribute(gemv_mma_kernel<N, NB, kChained>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(gemv_mma_kernel<N, NB, kChained, kDot>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < kMaxDevices) attr_done[dev] = true;
   }
@@ -938,12 +940,26 @@ static cudaError_t launch_mma(const GemvLayers& layers, int m, const __half* x, 
   int lg = 0;
   while ((1 << lg) < ksplit) ++lg;
   const long long limit = wait_selftest ? kSelftestWaitLimit : kWaitLimit;
-  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB, kChained>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, gemv_mma_kernel<N, NB, kChained, kDot>, layers, m, x, batch, ldx, dev_status, lg, bpp, limit, wait_selftest ? 1 : 0);
+}
+
+// Whether a launch is one full wave of CTAs and a small second one with few blocks each: the CTAs of the second have an SM almost to
+// themselves, and the longer latency of the dot products outweighs what they spare the full wave (5:8, 22000 x 768, four rows, 9.97 us
+// with products, 9.75 with shifts, 19500 x 512 7.94 and 7.77; from 12 blocks or one more CTA per SM on products are level or faster:
+// 19500 x 2048 14.2 and 14.6, 25000 x 1408 12.9 and 13.3, 17500 x 768 6.5 and 6.7).
+static bool short_second_wave(int ctas, int bpp) {
+  int dev = 0, sms = 0;
+  if (bpp > 11 || cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+  return ctas > kMmaPerSm * sms && ctas <= (kMmaPerSm + 1) * sms;
 }
 
 template <int NB>
 static cudaError_t launch_mma_n(int N, const GemvLayers& layers, int m, const __half* x, int batch, size_t ldx,
                                 int* dev_status, cudaStream_t s, bool chained, bool selftest) {
+  if constexpr (NB == 1) {            // (such a launch has no split)
+    if (N == 5 && !chained && short_second_wave(layers.tile_start[layers.count], m / kBlock))
+      return launch_mma<5, 1, false, false>(layers, m, x, batch, ldx, dev_status, s, true, selftest);
+  }
   // On its own a launch is a programmatic dependent as well, which hides 2 to 4 us of launch but keeps the compiler from reading
   // the weights through the read-only path: with more than eight rows 12% of the time (28672 x 8192 5:8, 16 rows: 99 against
   // 88 us), so that from 16384 tiles on such a launch keeps the stream's order.

@@ -850,6 +850,22 @@ def test_gemv_of_larger_layers(stb, N, n, m, batch):
     assert torch.equal(stb.gemv(layer, x, out_dtype=torch.float16), y.half())
 
 
+@pytest.mark.parametrize("batch", [1, 8])
+@pytest.mark.parametrize("tail,blocks", [(0, 4), (1, 4), (1, 11), (1, 12), (74, 1), (148, 11), (149, 4)])
+def test_gemv_with_a_short_second_wave(stb, tail, blocks, batch):
+    """5:8, four row tiles per SM and `tail` more: a launch whose second wave of CTAs is short takes a kernel of its own."""
+    import torch
+    n, m = 32 * (4 * torch.cuda.get_device_properties(0).multi_processor_count + tail) - 3, 128 * blocks
+    d = si.logical_layer(n, m, 5, 1500 + blocks, max_salient=9)
+    layer, L, rows = stb.pack_numpy(d), wl.as_logical(d), _sampled_rows(n, 5)
+    x = si.activations(batch, m, 1510)
+    y = stb.gemv(layer, torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    assert int(layer.dev_status.item()) == 0
+    ref = oracle.layer_rows(L, rows, x.astype(np.float64))
+    assert np.abs(y.double().cpu().numpy()[:, rows] - ref).max() <= TOL * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("N,batch,h,f", [(6, 3, 1024, 20000), (6, 16, 1024, 20000), (5, 9, 2048, 25603), (4, 1, 512, 6000)])
 def test_chain_takes_one_gemv_kernel(stb, N, batch, h, f):
     """stb_layer_stack over layers on both sides of its choice of kernel (means of 2500 tiles at 6:8, 6000 otherwise): two projections of

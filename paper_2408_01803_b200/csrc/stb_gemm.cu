@@ -236,10 +236,10 @@ __device__ __forceinline__ void load_gemm_tile(const uint8_t* tile, int lane, Ge
 
 // Decode role of one warp: packed row tile 4 mt + q, every fourth block of the CTA's K range, written into the A stages.
 // kF16: the stages hold fp16 (the scales as stored); otherwise bf16 (the scales rounded to nearest even).
-// kPairs (6:8): the position selectors of two rows by one look-up with the tile's pair field, whose upper twelve bits are the address of their entry: 32 bits
-// of selectors per row, two copies of every entry for even and odd lanes.  Splitting the field into two mask indices and looking
-// each up took 60 of the 760 instructions of a tile (28672 x 8192 at 64 tokens 96.5 -> 94.1 us, 11008 x 4096 27.6 -> 27.1).  For
-// calls of up to 64 tokens, where the decode is what takes the time and the boxes leave room for the table's 12 KB.
+// kPairs (6:8): the position selectors of two rows by one look-up with the tile's pair field, whose upper twelve bits are the address of
+// their entry: 32 bits of selectors per row, two copies of every entry for even and odd lanes.  Splitting the field into two mask
+// indices and looking each up took 60 of the 760 instructions of a tile (28672 x 8192 at 64 tokens 96.5 -> 94.1 us, 11008 x 4096 27.6 ->
+// 27.1).  For calls of up to 64 tokens, where the decode is what takes the time and the boxes leave room for the table's 12 KB.
 template <int N, bool kF16, int kStagesA, bool kPairs>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
   const int nblk = da.nblk, q = da.q, b0 = da.b0, b1 = da.b1, w = da.w;
@@ -312,7 +312,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs& da) {
     uint32_t fld[8];
     if constexpr (kPairs) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) fld[k] = nxt.fld[k] & 0xFFF0u;        // (a multiple of 16 in any packed layer; in one altered since, a wrong entry and no misaligned load)
+      for (int k = 0; k < 8; ++k) fld[k] = nxt.fld[k] & 0xFFF0u;        // (nothing to mask in a layer as packed: what altered it since makes no misaligned load)
     } else if constexpr (mask_pairs(N)) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) {                    // rows 2 mt, 2 mt + 1, slot s: k = 4 mt + s (multiply-adds: the integer pipe is the busy one)
